@@ -52,18 +52,6 @@ __device__ __forceinline__ real block_scalar(const double *src)
     }
 }
 
-// A float as a double, exactly, built from its bits on the integer pipe
-// (zero and normal floats; subnormal, infinite and NaN ones take the
-// conversion instruction).
-__device__ __forceinline__ double f2d_bits(float f)
-{
-    const uint32_t b = __float_as_uint(f);
-    const uint32_t e = (b >> 23) & 0xffu;
-    if ((b & 0x7fffffffu) == 0u) return __hiloint2double((int)(b & 0x80000000u), 0);
-    if (e == 0u || e == 0xffu) return (double)f;
-    return __hiloint2double((int)((b & 0x80000000u) | ((e + 896u) << 20) | ((b & 0x7fffffu) >> 3)), (int)(b << 29));
-}
-
 // Sites per thread of the two per-iteration BLAS kernels: every load of a
 // thread's sites is issued before any of them is used (memory-level
 // parallelism for these short, latency-bound kernels).  Four sites a thread

@@ -81,6 +81,45 @@ __device__ __forceinline__ float i20_to_f(uint32_t u)
     return __fsub_rn(__uint_as_float((u & 0xfffffu) ^ 0x4B080000u), 8912896.0f);  // 2^23 + 2^19
 }
 
+// FP64 <-> FP32 on the integer pipe.  GB300 converts at its FP64 rate (1/64 of
+// FP32), which bounded the format conversions: six conversions a site took
+// longer than the site's bytes.  Both give the bits of the conversion
+// instruction; values outside the ranges named take that instruction.
+//
+// A float as a double: zero and normal floats (subnormal, infinite and NaN ones
+// are converted by the instruction).
+__device__ __forceinline__ double f2d_bits(float f)
+{
+    const uint32_t b = __float_as_uint(f);
+    const uint32_t e = (b >> 23) & 0xffu;
+    if ((b & 0x7fffffffu) == 0u) return __hiloint2double((int)(b & 0x80000000u), 0);
+    if (e == 0u || e == 0xffu) return (double)f;
+    return __hiloint2double((int)((b & 0x80000000u) | ((e + 896u) << 20) | ((b & 0x7fffffu) >> 3)), (int)(b << 29));
+}
+
+// A double rounded to the nearest float (ties to even): zero and doubles with
+// 2^-126 <= |d| < 2^127 (the rest by the instruction).  The 29 dropped bits are
+// rounded away by adding half a unit less one plus the last kept bit; a carry
+// runs into the exponent as it should.
+__device__ __forceinline__ float d2f_bits(double d)
+{
+    const uint32_t hi = (uint32_t)__double2hiint(d), lo = (uint32_t)__double2loint(d);
+    const uint32_t e = (hi >> 20) & 0x7ffu;
+    if (e - 897u >= 253u) {  // not in [2^-126, 2^127)
+        if (((hi & 0x7fffffffu) | lo) == 0u) return __uint_as_float(hi);
+        return (float)d;
+    }
+    // the magnitude's top 32 bits below the sign, rebiased: (e - 896) and 23 fraction bits
+    const uint32_t t = __funnelshift_l(lo, (hi & 0x7fffffffu) - (896u << 20), 3);
+    const uint32_t rest = lo & 0x1fffffffu;
+    const uint32_t up = (rest + 0x0fffffffu + (t & 1u)) >> 29;  // 0 or 1
+    return __uint_as_float((hi & 0x80000000u) | (t + up));
+}
+
+// a compute-precision value rounded to FP32 (the FP32-based formats' first step)
+__device__ __forceinline__ float to_f32(float v) { return v; }
+__device__ __forceinline__ float to_f32(double v) { return d2f_bits(v); }
+
 // ---------------------------------------------------------------------------
 // spinor codecs
 // ---------------------------------------------------------------------------
@@ -111,16 +150,31 @@ struct Spinor<S_F64> {
         gather(b, n, i, c);
         decode(c, v);
     }
+    // encode: values -> record chunks (false: not storable); put: chunks -> field; store: both
+    template <typename real>
+    __device__ static bool encode(const real v[6], uint4 c[chunks])
+    {
+        bool ok = true;
+#pragma unroll
+        for (int k = 0; k < 3; k++) {
+            const double x = (double)v[2 * k], y = (double)v[2 * k + 1];
+            c[k] = make_uint4((unsigned)__double2loint(x), (unsigned)__double2hiint(x), (unsigned)__double2loint(y),
+                              (unsigned)__double2hiint(y));
+            ok = ok && isfinite(x) && isfinite(y);
+        }
+        return ok;
+    }
+    __device__ static void put(char *b, int n, int i, const uint4 c[chunks])
+    {
+#pragma unroll
+        for (int k = 0; k < 3; k++) reinterpret_cast<uint4 *>(b)[(size_t)k * n + i] = c[k];
+    }
     template <typename real>
     __device__ static bool store(char *b, int n, int i, const real v[6])
     {
-        double2 *p = reinterpret_cast<double2 *>(b);
-        bool ok = true;
-#pragma unroll
-        for (int c = 0; c < 3; c++) {
-            p[(size_t)c * n + i] = make_double2((double)v[2 * c], (double)v[2 * c + 1]);
-            ok = ok && isfinite((double)v[2 * c]) && isfinite((double)v[2 * c + 1]);
-        }
+        uint4 c[chunks];
+        const bool ok = encode(v, c);
+        put(b, n, i, c);
         return ok;
     }
 };
@@ -149,17 +203,30 @@ struct Spinor<S_F32> {
         decode(c, v);
     }
     template <typename real>
-    __device__ static bool store(char *b, int n, int i, const real v[6])
+    __device__ static bool encode(const real v[6], uint4 c[chunks])
     {
         float f[6];
         bool ok = true;
 #pragma unroll
         for (int k = 0; k < 6; k++) {
-            f[k] = (float)v[k];
+            f[k] = to_f32(v[k]);
             ok = ok && isfinite(f[k]);
         }
-        reinterpret_cast<float4 *>(b)[i] = make_float4(f[0], f[1], f[2], f[3]);
-        reinterpret_cast<float2 *>(b + (size_t)16 * n)[i] = make_float2(f[4], f[5]);
+        c[0] = make_uint4(__float_as_uint(f[0]), __float_as_uint(f[1]), __float_as_uint(f[2]), __float_as_uint(f[3]));
+        c[1] = make_uint4(__float_as_uint(f[4]), __float_as_uint(f[5]), 0u, 0u);
+        return ok;
+    }
+    __device__ static void put(char *b, int n, int i, const uint4 c[chunks])
+    {
+        reinterpret_cast<uint4 *>(b)[i] = c[0];
+        reinterpret_cast<uint2 *>(b + (size_t)16 * n)[i] = make_uint2(c[1].x, c[1].y);
+    }
+    template <typename real>
+    __device__ static bool store(char *b, int n, int i, const real v[6])
+    {
+        uint4 c[chunks];
+        const bool ok = encode(v, c);
+        put(b, n, i, c);
         return ok;
     }
 };
@@ -193,15 +260,14 @@ struct Spinor<S_HALF> {
         decode(c, v);
     }
     template <typename real>
-    __device__ static bool store(char *b, int n, int i, const real v[6])
+    __device__ static bool encode(const real v[6], uint4 c[chunks])
     {
-        (void)n;
         float f[6];
         float mx = 0.0f;
         bool ok = true;
 #pragma unroll
         for (int k = 0; k < 6; k++) {
-            f[k] = (float)v[k];
+            f[k] = to_f32(v[k]);
             ok = ok && isfinite(f[k]);
             mx = fmaxf(mx, fabsf(f[k]));
         }
@@ -213,12 +279,21 @@ struct Spinor<S_HALF> {
 #pragma unroll
             for (int k = 0; k < 6; k++) q[k] = max(-32767, min(32767, __float2int_rn(fmul(f[k], inv))));
         }
-        int4 r;
-        r.x = (int)(lo16(q[0]) | (lo16(q[1]) << 16));
-        r.y = (int)(lo16(q[2]) | (lo16(q[3]) << 16));
-        r.z = (int)(lo16(q[4]) | (lo16(q[5]) << 16));
-        r.w = __float_as_int(mx);
-        reinterpret_cast<int4 *>(b)[i] = r;
+        c[0] = make_uint4(lo16(q[0]) | (lo16(q[1]) << 16), lo16(q[2]) | (lo16(q[3]) << 16),
+                          lo16(q[4]) | (lo16(q[5]) << 16), __float_as_uint(mx));
+        return ok;
+    }
+    __device__ static void put(char *b, int n, int i, const uint4 c[chunks])
+    {
+        (void)n;
+        reinterpret_cast<uint4 *>(b)[i] = c[0];
+    }
+    template <typename real>
+    __device__ static bool store(char *b, int n, int i, const real v[6])
+    {
+        uint4 c[chunks];
+        const bool ok = encode(v, c);
+        put(b, n, i, c);
         return ok;
     }
 };
@@ -255,15 +330,14 @@ struct Spinor<S_INT20> {
         decode(c, v);
     }
     template <typename real>
-    __device__ static bool store(char *b, int n, int i, const real v[6])
+    __device__ static bool encode(const real v[6], uint4 c[chunks])
     {
-        (void)n;
         float f[6];
         float mx = 0.0f;
         bool ok = true;
 #pragma unroll
         for (int k = 0; k < 6; k++) {
-            f[k] = (float)v[k];
+            f[k] = to_f32(v[k]);
             ok = ok && isfinite(f[k]);
             mx = fmaxf(mx, fabsf(f[k]));
         }
@@ -281,7 +355,20 @@ struct Spinor<S_INT20> {
         w.y = (u[1] & 0xffu) | ((u[2] & 0xfffffu) << 8) | (((u[3] >> 16) & 0xfu) << 28);
         w.z = (u[3] & 0xffffu) | (((u[4] >> 4) & 0xffffu) << 16);
         w.w = (u[4] & 0xfu) | ((u[5] & 0xfffffu) << 4) | (E << 24);
-        reinterpret_cast<uint4 *>(b)[i] = w;
+        c[0] = w;
+        return ok;
+    }
+    __device__ static void put(char *b, int n, int i, const uint4 c[chunks])
+    {
+        (void)n;
+        reinterpret_cast<uint4 *>(b)[i] = c[0];
+    }
+    template <typename real>
+    __device__ static bool store(char *b, int n, int i, const real v[6])
+    {
+        uint4 c[chunks];
+        const bool ok = encode(v, c);
+        put(b, n, i, c);
         return ok;
     }
 };
@@ -326,14 +413,14 @@ struct Spinor<S_INT14> {
         decode(c, v);
     }
     template <typename real>
-    __device__ static bool store(char *b, int n, int i, const real v[6])
+    __device__ static bool encode(const real v[6], uint4 c[chunks])
     {
         float f[6];
         float mx = 0.0f;
         bool ok = true;
 #pragma unroll
         for (int k = 0; k < 6; k++) {
-            f[k] = (float)v[k];
+            f[k] = to_f32(v[k]);
             ok = ok && isfinite(f[k]);
             mx = fmaxf(mx, fabsf(f[k]));
         }
@@ -348,8 +435,20 @@ struct Spinor<S_INT14> {
         }
 #pragma unroll
         for (int k = 0; k < 4; k++) h[k] |= (E >> (2 * k)) & 3u;
-        reinterpret_cast<uint2 *>(b)[i] = make_uint2(h[0] | (h[1] << 16), h[2] | (h[3] << 16));
-        reinterpret_cast<uint32_t *>(b + (size_t)8 * n)[i] = h[4] | (h[5] << 16);
+        c[0] = make_uint4(h[0] | (h[1] << 16), h[2] | (h[3] << 16), h[4] | (h[5] << 16), 0u);
+        return ok;
+    }
+    __device__ static void put(char *b, int n, int i, const uint4 c[chunks])
+    {
+        reinterpret_cast<uint2 *>(b)[i] = make_uint2(c[0].x, c[0].y);
+        reinterpret_cast<uint32_t *>(b + (size_t)8 * n)[i] = c[0].z;
+    }
+    template <typename real>
+    __device__ static bool store(char *b, int n, int i, const real v[6])
+    {
+        uint4 c[chunks];
+        const bool ok = encode(v, c);
+        put(b, n, i, c);
         return ok;
     }
 };
@@ -406,7 +505,7 @@ struct Spinor<S_INT30> {
     // 2^(f-155) (m (1 + 2^-29) < 2 - 2^-53), so its exponent gives E = f - 28
     // (subnormal or small mx: E = 1); v 2^(127-E) is then exact in FP32 (a
     // power of two, magnitude below 2^29) and rounds to the same integer.
-    __device__ static bool store_f32(char *b, int n, int i, const float v[6])
+    __device__ static bool encode_f32(const float v[6], uint4 c[chunks])
     {
         float mx = 0.0f;
         bool ok = true;
@@ -425,24 +524,31 @@ struct Spinor<S_INT30> {
 #pragma unroll
             for (int k = 0; k < 6; k++) u[k] = (uint32_t)__float2int_rn(fmul(v[k], down));
         }
-        pack(b, n, i, E, u);
+        pack(c, E, u);
         return ok;
     }
 
     // FP32-pair values (FP64-class compute), the 30-bit rule on the exact value
-    // hi + lo without FP64 arithmetic.  Exponent: as store_f32 from hi's
+    // hi + lo without FP64 arithmetic.  Exponent: as encode_f32 from hi's
     // exponent field f (E = f - 28), except that a power-of-two hi with an
     // opposite-sign lo larger than 2^(p-29) (p the exponent of hi) lies in
     // the binade below (E = f - 29).  Integer: round-to-nearest-even of the
     // scaled pair, exactly: r = rint(hi'), then the exact remainder
     // (hi' - r) + lo' (TwoSum) rounded the same way in a second stage.
-    __device__ static bool store_ff(char *b, int n, int i, const ff v[6])
+    __device__ static bool encode_ff(const ff v[6], uint4 c[chunks])
     {
         uint32_t u[6], E;
-        return store_ff_q(b, n, i, v, u, E);
+        return encode_ff_q(v, c, u, E);
     }
-    // the same, returning the stored integers (signed, in u) and exponent field
+    // the same stored, returning the stored integers (signed, in u) and exponent field
     __device__ static bool store_ff_q(char *b, int n, int i, const ff v[6], uint32_t u[6], uint32_t &E)
+    {
+        uint4 c[chunks];
+        const bool ok = encode_ff_q(v, c, u, E);
+        put(b, n, i, c);
+        return ok;
+    }
+    __device__ static bool encode_ff_q(const ff v[6], uint4 c[chunks], uint32_t u[6], uint32_t &E)
     {
         bool ok = true;
         int km = 0;
@@ -485,26 +591,39 @@ struct Spinor<S_INT30> {
                 u[k] = (uint32_t)q;
             }
         }
-        pack(b, n, i, E, u);
+        pack(c, E, u);
         return ok;
     }
 
-    __device__ static void pack(char *b, int n, int i, uint32_t E, const uint32_t u[6])
+    __device__ static void pack(uint4 c[chunks], uint32_t E, const uint32_t u[6])
     {
         uint4 a;
         a.x = (u[0] & 0x3fffffffu) | ((E & 3u) << 30);
         a.y = (u[1] & 0x3fffffffu) | (((E >> 2) & 3u) << 30);
         a.z = (u[2] & 0x3fffffffu) | (((E >> 4) & 3u) << 30);
         a.w = (u[3] & 0x3fffffffu) | (((E >> 6) & 3u) << 30);
-        reinterpret_cast<uint4 *>(b)[i] = a;
-        reinterpret_cast<uint2 *>(b + (size_t)16 * n)[i] = make_uint2(u[4] & 0x3fffffffu, u[5] & 0x3fffffffu);
+        c[0] = a;
+        c[1] = make_uint4(u[4] & 0x3fffffffu, u[5] & 0x3fffffffu, 0u, 0u);
     }
-
+    __device__ static void put(char *b, int n, int i, const uint4 c[chunks])
+    {
+        reinterpret_cast<uint4 *>(b)[i] = c[0];
+        reinterpret_cast<uint2 *>(b + (size_t)16 * n)[i] = make_uint2(c[1].x, c[1].y);
+    }
     template <typename real>
     __device__ static bool store(char *b, int n, int i, const real v[6])
     {
-        if constexpr (std::is_same<real, float>::value) return store_f32(b, n, i, v);
-        if constexpr (is_ff<real>::value) return store_ff(b, n, i, v);
+        uint4 c[chunks];
+        const bool ok = encode(v, c);
+        put(b, n, i, c);
+        return ok;
+    }
+
+    template <typename real>
+    __device__ static bool encode(const real v[6], uint4 c[chunks])
+    {
+        if constexpr (std::is_same<real, float>::value) return encode_f32(v, c);
+        if constexpr (is_ff<real>::value) return encode_ff(v, c);
         double d[6];
         double mx = 0.0;
         bool ok = true;
@@ -529,7 +648,7 @@ struct Spinor<S_INT30> {
                 for (int k = 0; k < 6; k++) u[k] = (uint32_t)(int32_t)__double2ll_rn(__dmul_rn(d[k], down));
             }
         }
-        pack(b, n, i, E, u);
+        pack(c, E, u);
         return ok;
     }
 };
@@ -658,6 +777,60 @@ __device__ __forceinline__ void rebuild_row2_phase(real U[18], real fr, real fi)
     RE(8) = fr * c2r + fi * c2i; IM(8) = fi * c2r - fr * c2i;
 #undef RE
 #undef IM
+}
+
+// A warp's sites (lane l: site i0 + l of n) between registers and an FP64 or FP32
+// array [site][6], through shared memory so that every global access is a
+// full line (the lanes' own 48-byte strides touch twelve lines an access and
+// write half sectors).  sh: 192 values of this warp, 16-byte aligned; every
+// lane calls; i0 < n.
+template <typename T>
+__device__ __forceinline__ void warp_load_sites(const T *in, int64_t i0, int64_t n, T v[6], T *sh)
+{
+    const int lane = threadIdx.x & 31;
+    const int m = 6 * (int)(n - i0 < 32 ? n - i0 : 32);
+#pragma unroll
+    for (int k = 0; k < 6; k++) {
+        const int j = lane + 32 * k;
+        if (j < m) sh[j] = __ldcs(in + 6 * i0 + j);
+    }
+    __syncwarp();
+#pragma unroll
+    for (int k = 0; k < 3; k++) {
+        v[2 * k] = sh[6 * lane + 2 * k];
+        v[2 * k + 1] = sh[6 * lane + 2 * k + 1];
+    }
+    __syncwarp();  // sh may be written again
+}
+
+__device__ __forceinline__ void warp_store_sites(double *out, int64_t i0, int64_t n, const double v[6], double *sh)
+{
+    const int lane = threadIdx.x & 31;
+#pragma unroll
+    for (int k = 0; k < 3; k++) reinterpret_cast<double2 *>(sh)[3 * lane + k] = make_double2(v[2 * k], v[2 * k + 1]);
+    __syncwarp();
+    const int m = 6 * (int)(n - i0 < 32 ? n - i0 : 32);
+#pragma unroll
+    for (int k = 0; k < 6; k++) {
+        const int j = lane + 32 * k;
+        if (j < m) out[6 * i0 + j] = sh[j];
+    }
+    __syncwarp();  // sh may be written again
+}
+
+// The decoded value of a record as FP64 (FP32 compute decodes to FP32, widened
+// on the integer pipe).
+template <int SF, typename real>
+__device__ __forceinline__ void decode_f64(const uint4 *c, double v[6])
+{
+    if constexpr (std::is_same<real, float>::value) {
+        float f[6];
+        Spinor<SF>::decode(c, f);
+#pragma unroll
+        for (int k = 0; k < 6; k++) v[k] = f2d_bits(f[k]);
+    } else {
+        Spinor<SF>::decode(c, v);
+    }
 }
 
 template <int GF, int RECON>

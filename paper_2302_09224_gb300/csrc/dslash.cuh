@@ -143,8 +143,47 @@ using SiteAcc = std::conditional_t<std::is_same<real, float>::value, SiteAccPack
 constexpr int kNumStencilConfigs = 5;
 __host__ __device__ constexpr bool stencil_config_valid(int cfg, int gf) { return cfg >= 0 && cfg < kNumStencilConfigs && gf >= 0; }
 __host__ __device__ constexpr int stencil_block(int cfg) { return cfg == 3 ? 256 : 128; }
+// Threads a block is launched with.  The FP64 stencil runs at the FP64 pipe's
+// rate, so its time is that of the fullest SM: with few blocks an SM the grid
+// is cut finer (down to 32 threads a block) while that lowers the most sites
+// any SM gets.  16^3x32 (65536 sites, 152 SMs): blocks of 128 leave up to four
+// blocks on an SM where 3.4 is the mean.
+inline int stencil_threads(int cfg, int gf, int vh)
+{
+    const int b = stencil_block(cfg);
+    if (gf != G_F64) return b;
+    constexpr int sms = 152;
+    int best = b;
+    long long most = 0;
+    for (int t = b; t >= 32; t /= 2) {
+        const long long nb = (vh + t - 1) / t;
+        const long long m = (nb + sms - 1) / sms * t;  // sites on the fullest SM
+        if (t == b || m * 100 < most * 97) {  // at least 3 % fewer
+            best = t;
+            most = m;
+        }
+    }
+    return best;
+}
 __host__ __device__ constexpr int stencil_minb(int cfg) { return cfg == 2 ? 8 : cfg == 3 ? 4 : cfg == 4 ? 8 : 1; }
 __host__ __device__ constexpr bool stencil_unrolled(int cfg) { return cfg == 0 || cfg == 4; }
+
+// The fields of one pass: input, output and xpay (output parity po).
+struct StencilIO {
+    const char *in;
+    char *out;
+    const char *y;
+    int po;
+};
+__device__ __forceinline__ StencilIO stencil_io(const DslashArgs &a) { return {a.in, a.out, a.y, a.out_parity}; }
+// Both parities in one launch: parity blockIdx.y, every field pointer that of the even half and the
+// odd half half_bytes after it.
+__device__ __forceinline__ StencilIO stencil_io_full(const DslashArgs &a)
+{
+    const int po = (int)blockIdx.y;
+    const size_t own = po ? a.half_bytes : 0, other = po ? 0 : a.half_bytes;
+    return {a.in + other, a.out + own, a.y + own, po};
+}
 
 // One direction mu of the stencil at site x (coordinates c, lex), accumulated
 // into acc.  Fixed-point links are applied unscaled and the sum is kept in
@@ -211,9 +250,9 @@ __device__ __forceinline__ void rebuild_r8(float U[18], float es, float as)
 }
 
 template <int GF, int SF, typename real, int LREC, bool COH = false, bool KEEP = false>
-__device__ __forceinline__ void stencil_direction(const DslashArgs &a, int mu, int cmu, int c3, int lex, int cb,
-                                                  int po, size_t pstride, real lsc, real ratio, int phase_sum,
-                                                  SiteAcc<real> &acc)
+__device__ __forceinline__ void stencil_direction(const DslashArgs &a, const char *in, int mu, int cmu, int c3,
+                                                  int lex, int cb, int po, size_t pstride, real lsc, real ratio,
+                                                  int phase_sum, SiteAcc<real> &acc)
 {
     constexpr bool kScaled = LinkScaled<GF>::value;
     const Geom &g = a.g;
@@ -227,11 +266,11 @@ __device__ __forceinline__ void stencil_direction(const DslashArgs &a, int mu, i
     real U[18], s[6];
 
     Link<GF, 18>::template load<real, KEEP>(a.gv.fat, pstride, (po * 4 + mu) * vh + cb, U);
-    load_neighbour<real, SF, COH>(a.in, vh, np1, s);
+    load_neighbour<real, SF, COH>(in, vh, np1, s);
     acc.add(U, s);
 
     Link<GF, 18>::template load<real, KEEP>(a.gv.fat, pstride, (pi * 4 + mu) * vh + nm1, U);
-    load_neighbour<real, SF, COH>(a.in, vh, nm1, s);
+    load_neighbour<real, SF, COH>(in, vh, nm1, s);
     acc.adj_sub(U, s);
 
     // row 2 of an r12 link in the units of rows 0 and 1: sign * lsc * conj(row0 x row1)
@@ -245,7 +284,7 @@ __device__ __forceinline__ void stencil_direction(const DslashArgs &a, int mu, i
     }
     // an 8-real link comes back in true units with its sign removed: the spinor takes the sign and 1/fsc
     if constexpr (LREC == 8) rebuild_r8(U, lsc, kScaled ? 1.0f / 32767.0f : 1.0f);
-    load_neighbour<real, SF, COH>(a.in, vh, np3, s);
+    load_neighbour<real, SF, COH>(in, vh, np3, s);
     if constexpr (LREC == 8) {
         const real r8s = kScaled ? ratio / lsc : real(1);
         const bool flip = g.antiperiodic_t && mu == 3 && c3 + 3 >= L;
@@ -266,7 +305,7 @@ __device__ __forceinline__ void stencil_direction(const DslashArgs &a, int mu, i
         rebuild_row2_r13(U, lsc);
     }
     if constexpr (LREC == 8) rebuild_r8(U, lsc, kScaled ? 1.0f / 32767.0f : 1.0f);
-    load_neighbour<real, SF, COH>(a.in, vh, nm3, s);
+    load_neighbour<real, SF, COH>(in, vh, nm3, s);
     if constexpr (LREC == 8) {
         const real r8s = kScaled ? ratio / lsc : real(1);
         const bool flip = g.antiperiodic_t && mu == 3 && cm3 + 3 >= L;
@@ -449,8 +488,8 @@ __device__ __forceinline__ unsigned load_int30_raw(const char *b, int n, int i, 
 }
 
 template <bool COH, bool KEEP, int LREC>
-__device__ __forceinline__ void stencil_direction_i30(const DslashArgs &a, int mu, int cmu, int lex, int cb, int po,
-                                                      size_t pstride, int phase_sum, SiteAccI30 &acc)
+__device__ __forceinline__ void stencil_direction_i30(const DslashArgs &a, const char *in, int mu, int cmu, int lex,
+                                                      int cb, int po, size_t pstride, int phase_sum, SiteAccI30 &acc)
 {
     const Geom &g = a.g;
     const int vh = g.vh, pi = 1 - po;
@@ -461,10 +500,10 @@ __device__ __forceinline__ void stencil_direction_i30(const DslashArgs &a, int m
     int u[18], q[6];
     unsigned E;
     load_link_ints<KEEP>(a.gv.fat, pstride, (po * 4 + mu) * vh + cb, u);
-    E = load_int30_raw<COH>(a.in, vh, np1, q);
+    E = load_int30_raw<COH>(in, vh, np1, q);
     acc.term<false>(0, u, q, E);
     load_link_ints<KEEP>(a.gv.fat, pstride, (pi * 4 + mu) * vh + nm1, u);
-    E = load_int30_raw<COH>(a.in, vh, nm1, q);
+    E = load_int30_raw<COH>(in, vh, nm1, q);
     acc.term<true>(0, u, q, E);
     if constexpr (LREC == 12) {
         // the sign of a long link: its staggered phase, flipped across an antiperiodic t boundary
@@ -474,17 +513,17 @@ __device__ __forceinline__ void stencil_direction_i30(const DslashArgs &a, int m
         const bool flipb = g.antiperiodic_t && mu == 3 && cm3 + 3 >= L;
         load_link_ints_r12<KEEP>(a.gv.lng, pstride, (po * 4 + mu) * vh + cb, u, flipf ? -eta : eta,
                                  a.gv.lng_r2_mul, a.gv.lng_r2_shift);
-        E = load_int30_raw<COH>(a.in, vh, np3, q);
+        E = load_int30_raw<COH>(in, vh, np3, q);
         acc.term<false>(1, u, q, E);
         load_link_ints_r12<KEEP>(a.gv.lng, pstride, (pi * 4 + mu) * vh + nm3, u, flipb ? -eta : eta,
                                  a.gv.lng_r2_mul, a.gv.lng_r2_shift);
     } else {
         load_link_ints<KEEP>(a.gv.lng, pstride, (po * 4 + mu) * vh + cb, u);
-        E = load_int30_raw<COH>(a.in, vh, np3, q);
+        E = load_int30_raw<COH>(in, vh, np3, q);
         acc.term<false>(1, u, q, E);
         load_link_ints<KEEP>(a.gv.lng, pstride, (pi * 4 + mu) * vh + nm3, u);
     }
-    E = load_int30_raw<COH>(a.in, vh, nm3, q);
+    E = load_int30_raw<COH>(in, vh, nm3, q);
     acc.term<true>(1, u, q, E);
 }
 
@@ -493,16 +532,12 @@ struct UsesIntPath {
     static constexpr bool value = GF == G_FIX32 && SF == S_INT30 && is_ff<real>::value && (LREC == 18 || LREC == 12);
 };
 
-// One output site cb: the stencil, the optional xpay, the store and, when
-// reducing, this site's Re<y, out> and |out|^2 added to rv (in the compute
-// precision; reduce_grid sums the threads).
-template <int GF, int SF, typename real, int LREC, bool RED, int CFG, bool COH = false, bool KEEP = false>
-__device__ __forceinline__ void stencil_site(const DslashArgs &a, int cb, size_t pstride, real fsc, real lsc,
-                                             real ratio, real rv[2])
+// sign * D in at output site cb.
+template <int GF, int SF, typename real, int LREC, int CFG, bool COH = false, bool KEEP = false>
+__device__ __forceinline__ void stencil_value(const DslashArgs &a, const char *in, int po, int cb, size_t pstride,
+                                              real fsc, real lsc, real ratio, real o[6])
 {
     const Geom &g = a.g;
-    const int vh = g.vh;
-    const int po = a.out_parity;
     int r = cb / g.xh;
     const int xh = cb - r * g.xh;
     const int y = r % g.L[1];
@@ -512,7 +547,6 @@ __device__ __forceinline__ void stencil_site(const DslashArgs &a, int cb, size_t
     const int x = 2 * xh + ((y + z + t + po) & 1);
     const int c[4] = {x, y, z, t};
     const int lex = 2 * cb + (x & 1);
-    real o[6];
     if constexpr (UsesIntPath<GF, SF, real, LREC>::value) {
         SiteAccI30 acc;
         acc.zero();
@@ -520,7 +554,7 @@ __device__ __forceinline__ void stencil_site(const DslashArgs &a, int cb, size_t
             int phase_sum = 0;  // x + y + ... below mu: the staggered phase eta_mu(x)
 #pragma unroll
             for (int mu = 0; mu < 4; mu++) {
-                stencil_direction_i30<COH, KEEP, LREC>(a, mu, c[mu], lex, cb, po, pstride, phase_sum, acc);
+                stencil_direction_i30<COH, KEEP, LREC>(a, in, mu, c[mu], lex, cb, po, pstride, phase_sum, acc);
                 phase_sum += c[mu];
             }
         } else {
@@ -528,7 +562,7 @@ __device__ __forceinline__ void stencil_site(const DslashArgs &a, int cb, size_t
 #pragma unroll 1
             for (int mu = 0; mu < 4; mu++) {
                 const int cmu = mu == 0 ? x : mu == 1 ? y : mu == 2 ? z : t;
-                stencil_direction_i30<COH, KEEP, LREC>(a, mu, cmu, lex, cb, po, pstride, phase_sum, acc);
+                stencil_direction_i30<COH, KEEP, LREC>(a, in, mu, cmu, lex, cb, po, pstride, phase_sum, acc);
                 phase_sum += cmu;
             }
         }
@@ -542,7 +576,7 @@ __device__ __forceinline__ void stencil_site(const DslashArgs &a, int cb, size_t
         int phase_sum = 0;  // x + y + ... below mu: the staggered phase eta_mu(x)
 #pragma unroll
         for (int mu = 0; mu < 4; mu++) {
-            stencil_direction<GF, SF, real, LREC, COH, KEEP>(a, mu, c[mu], t, lex, cb, po, pstride, lsc, ratio,
+            stencil_direction<GF, SF, real, LREC, COH, KEEP>(a, in, mu, c[mu], t, lex, cb, po, pstride, lsc, ratio,
                                                              phase_sum, acc);
             phase_sum += c[mu];
         }
@@ -551,7 +585,7 @@ __device__ __forceinline__ void stencil_site(const DslashArgs &a, int cb, size_t
 #pragma unroll 1
         for (int mu = 0; mu < 4; mu++) {
             const int cmu = mu == 0 ? x : mu == 1 ? y : mu == 2 ? z : t;
-            stencil_direction<GF, SF, real, LREC, COH, KEEP>(a, mu, cmu, t, lex, cb, po, pstride, lsc, ratio,
+            stencil_direction<GF, SF, real, LREC, COH, KEEP>(a, in, mu, cmu, t, lex, cb, po, pstride, lsc, ratio,
                                                              phase_sum, acc);
             phase_sum += cmu;
         }
@@ -561,13 +595,25 @@ __device__ __forceinline__ void stencil_site(const DslashArgs &a, int cb, size_t
 #pragma unroll
     for (int k = 0; k < 6; k++) o[k] = sf * acc.get(k);
     }
+}
+
+// One output site cb: the stencil, the optional xpay, the store and, when
+// reducing, this site's Re<y, out> and |out|^2 added to rv (in the compute
+// precision; reduce_grid sums the threads).
+template <int GF, int SF, typename real, int LREC, bool RED, int CFG, bool COH = false, bool KEEP = false>
+__device__ __forceinline__ void stencil_site(const DslashArgs &a, const StencilIO io, int cb, size_t pstride, real fsc,
+                                             real lsc, real ratio, real rv[2])
+{
+    const int vh = a.g.vh;
+    real o[6];
+    stencil_value<GF, SF, real, LREC, CFG, COH, KEEP>(a, io.in, io.po, cb, pstride, fsc, lsc, ratio, o);
     if constexpr (RED && UsesIntPath<GF, SF, real, LREC>::value) {
         // FP64-class: Re<y, out> and |out|^2 exactly in integers from the stored 30-bit records
         int32_t qy[6] = {0, 0, 0, 0, 0, 0};
         uint32_t Ey = 0;
         if (a.xpay) {
             uint4 cy[Spinor<S_INT30>::chunks];
-            Spinor<S_INT30>::gather(a.y, vh, cb, cy);
+            Spinor<S_INT30>::gather(io.y, vh, cb, cy);
             Ey = Spinor<S_INT30>::raw(cy, qy);
             real yv[6];
             Spinor<S_INT30>::decode(cy, yv);
@@ -576,7 +622,7 @@ __device__ __forceinline__ void stencil_site(const DslashArgs &a, int cb, size_t
             for (int k = 0; k < 6; k++) o[k] = aa * yv[k] + o[k];
         }
         uint32_t qo[6], Eo;
-        if (!Spinor<S_INT30>::store_ff_q(a.out, vh, cb, o, qo, Eo)) atomicExch(a.err, 1);
+        if (!Spinor<S_INT30>::store_ff_q(io.out, vh, cb, o, qo, Eo)) atomicExch(a.err, 1);
         long long d = 0, n2 = 0;
 #pragma unroll
         for (int k = 0; k < 6; k++) {
@@ -589,7 +635,7 @@ __device__ __forceinline__ void stencil_site(const DslashArgs &a, int cb, size_t
     }
     if (a.xpay) {
         real yv[6];
-        Spinor<SF>::load(a.y, vh, cb, yv);
+        Spinor<SF>::load(io.y, vh, cb, yv);
         const real aa = (real)a.a;
 #pragma unroll
         for (int k = 0; k < 6; k++) o[k] = aa * yv[k] + o[k];
@@ -606,7 +652,7 @@ __device__ __forceinline__ void stencil_site(const DslashArgs &a, int cb, size_t
         for (int k = 0; k < 6; k++) n2 += o[k] * o[k];
         rv[1] += n2;
     }
-    if (!Spinor<SF>::store(a.out, vh, cb, o)) atomicExch(a.err, 1);
+    if (!Spinor<SF>::store(io.out, vh, cb, o)) atomicExch(a.err, 1);
 }
 
 // One thread per site.  A reducing pass ends each block with its block sum
@@ -628,11 +674,51 @@ __global__ void __launch_bounds__(stencil_block(CFG), stencil_minb(CFG))
     const real ratio = lsc / fsc;
     real rv[2] = {real(0), real(0)};
     const int cb = blockIdx.x * blockDim.x + threadIdx.x;
-    if (cb < vh) stencil_site<GF, SF, real, LREC, RED, CFG>(a, cb, pstride, fsc, lsc, ratio, rv);
+    if (cb < vh) stencil_site<GF, SF, real, LREC, RED, CFG>(a, stencil_io(a), cb, pstride, fsc, lsc, ratio, rv);
     if constexpr (RED) {  // summed by stencil_finish_kernel or by the CG's residual update
         const red_t<real> r2[2] = {(red_t<real>)rv[0], (red_t<real>)rv[1]};
         store_block_partial<2>(r2, a.red);
     }
+}
+
+// The pass whose output goes to the caller: the site is rounded to the storage
+// format as the other passes store it, decoded and written as FP64 [site][6]
+// (a separate unpack pass read the stored field again and wrote it: at
+// 32^3x64, both parities, 2 x 19 us).  FULL: both parities in one launch.
+// Nothing is written when the packing of the inputs has flagged them (a.bad).
+template <int GF, int SF, typename real, int LREC, bool FULL, int CFG>
+__global__ void __launch_bounds__(stencil_block(CFG), stencil_minb(CFG))
+    dslash_out_kernel(const __grid_constant__ DslashArgs a)
+{
+    __shared__ __align__(16) double sh[stencil_block(CFG) / 32][192];
+    pdl_wait();
+    if (*(volatile const int *)a.bad != 0) return;  // uniform over the grid
+    const int vh = a.g.vh;
+    const size_t pstride = (size_t)8 * vh * 16;
+    constexpr bool kScaled = LinkScaled<GF>::value;
+    const real fsc = kScaled ? (sizeof(real) == 8 ? (real)a.gv.fat_scale_d : (real)a.gv.fat_scale_f) : real(1);
+    const real lsc = kScaled ? (sizeof(real) == 8 ? (real)a.gv.lng_scale_d : (real)a.gv.lng_scale_f) : real(1);
+    const real ratio = lsc / fsc;
+    const int cb = blockIdx.x * blockDim.x + threadIdx.x;
+    const StencilIO io = FULL ? stencil_io_full(a) : stencil_io(a);
+    double *out64 = a.out64 + (FULL ? (size_t)blockIdx.y * 6 * vh : 0);
+    double v[6];
+    if (cb < vh) {
+        real o[6];
+        stencil_value<GF, SF, real, LREC, CFG>(a, io.in, io.po, cb, pstride, fsc, lsc, ratio, o);
+        if (a.xpay) {
+            real yv[6];
+            Spinor<SF>::load(io.y, vh, cb, yv);
+            const real aa = (real)a.a;
+#pragma unroll
+            for (int k = 0; k < 6; k++) o[k] = aa * yv[k] + o[k];
+        }
+        uint4 c[Spinor<SF>::chunks];
+        if (!Spinor<SF>::encode(o, c)) *(volatile int *)a.err = 1;
+        decode_f64<SF, real>(c, v);
+    }
+    const int i0 = cb & ~31;
+    if (i0 < vh) warp_store_sites(out64, i0, vh, v, sh[threadIdx.x >> 5]);
 }
 
 // After a reducing pass: one block sums the pass's block partials and runs the
@@ -657,7 +743,7 @@ __global__ void __launch_bounds__(1024) stencil_finish_kernel(RedBuf red, unsign
 template <int GF, int SF, typename real, int LREC, bool RED, int CFG>
 void launch_cfg(const DslashArgs &a, cudaStream_t s)
 {
-    constexpr int B = stencil_block(CFG);
+    const int B = stencil_threads(CFG, GF, a.g.vh);
     const int nb = (a.g.vh + B - 1) / B;
     launch_chained(dslash_kernel<GF, SF, real, LREC, RED, CFG>, dim3(nb), dim3(B), s, a);
     if constexpr (RED)
@@ -666,9 +752,39 @@ void launch_cfg(const DslashArgs &a, cudaStream_t s)
                            a.slot, a.active);
 }
 
+template <int GF, int SF, typename real, int LREC, int CFG>
+void launch_out_cfg(const DslashArgs &a, cudaStream_t s)
+{
+    const int B = stencil_threads(CFG, GF, a.g.vh);
+    const int nb = (a.g.vh + B - 1) / B;
+    if (a.half_bytes)
+        launch_chained(dslash_out_kernel<GF, SF, real, LREC, true, CFG>, dim3(nb, 2), dim3(B), s, a);
+    else
+        launch_chained(dslash_out_kernel<GF, SF, real, LREC, false, CFG>, dim3(nb), dim3(B), s, a);
+}
+
+// The pass to the caller's FP64 array: the plain pass's launch shapes.
+template <int GF, int SF, typename real, int LREC>
+void launch_out(int cfg, const DslashArgs &a, cudaStream_t s)
+{
+    switch (cfg) {
+    case 1: launch_out_cfg<GF, SF, real, LREC, 1>(a, s); break;
+    case 2: launch_out_cfg<GF, SF, real, LREC, 2>(a, s); break;
+    case 3: launch_out_cfg<GF, SF, real, LREC, 3>(a, s); break;
+    case 4: launch_out_cfg<GF, SF, real, LREC, 4>(a, s); break;
+    default: launch_out_cfg<GF, SF, real, LREC, 0>(a, s); break;
+    }
+}
+
 template <int GF, int SF, typename real, int LREC, bool RED>
 void launch_any(int cfg, const DslashArgs &a, cudaStream_t s)
 {
+    if constexpr (!RED) {
+        if (a.out64 != nullptr) {
+            launch_out<GF, SF, real, LREC>(cfg, a, s);
+            return;
+        }
+    }
     switch (cfg) {
     case 1: launch_cfg<GF, SF, real, LREC, RED, 1>(a, s); break;
     case 2: launch_cfg<GF, SF, real, LREC, RED, 2>(a, s); break;
@@ -804,7 +920,7 @@ __global__ void __launch_bounds__(stencil_block(CFG), stencil_minb(CFG))
         const int cb = slice * vs + off;
         if (kind == 0) {
             // links stay in L2 for D_eo a few slices later
-            if (off < vs) stencil_site<GF, SF, real, LREC, false, CFG, false, true>(a1, cb, pstride, fsc, lsc, ratio, rv);
+            if (off < vs) stencil_site<GF, SF, real, LREC, false, CFG, false, true>(a1, stencil_io(a1), cb, pstride, fsc, lsc, ratio, rv);
             __syncthreads();  // every thread's tmp stores precede the release below
             if (threadIdx.x == 0) red_release_add(done + slice, 1u);
         } else {
@@ -823,7 +939,7 @@ __global__ void __launch_bounds__(stencil_block(CFG), stencil_minb(CFG))
             }
             __syncthreads();
             // tmp is written by other blocks of this kernel: read through L2
-            if (off < vs) stencil_site<GF, SF, real, LREC, true, CFG, true>(a2, cb, pstride, fsc, lsc, ratio, rv);
+            if (off < vs) stencil_site<GF, SF, real, LREC, true, CFG, true>(a2, stencil_io(a2), cb, pstride, fsc, lsc, ratio, rv);
         }
     }
     __shared__ double tot[2];

@@ -8,7 +8,8 @@ namespace hisq {
 unsigned dslash_partials(int gf, int sf, int cf, int long_recon, const Geom &g)
 {
     const int cfg = stencil_config(gf, sf, cf, long_recon, true, g);
-    return (unsigned)((g.vh + stencil_block(cfg) - 1) / stencil_block(cfg));
+    const int b = stencil_threads(cfg, gf, g.vh);
+    return (unsigned)((g.vh + b - 1) / b);
 }
 
 bool launch_dslash_finish(int gf, int sf, int cf, int long_recon, const DslashArgs &a, cudaStream_t s)

@@ -220,6 +220,11 @@ struct DslashArgs {
     void *st;               // CGState or MSState, per finisher
     int slot;               // ring slot handed to the finisher
     int defer_finish;       // reducing pass: leave the summing launch to launch_dslash_finish
+    // the pass to a caller's array (plain pass only, out unused): the stored value decoded to FP64
+    // [site][6]; nothing is written when *bad != 0 (device int); err may be host-mapped
+    double *out64;
+    const int *bad;
+    size_t half_bytes;      // with out64, non-zero: both parities, the odd half this far after the even
 };
 
 // The fused M_ee pass (d1: D_oe into tmp; d2: D_eo from tmp with xpay and the
@@ -292,6 +297,16 @@ bool launch_mee_fused(int gf, int sf, int cf, int long_recon, const MeeArgs &m, 
 int stencil_config_in_use(int gf, int sf, int cf, int long_recon, bool reduce, const Geom &g);
 
 void launch_pack_spinor(int sf, int64_t n, const double *in, char *out, int *err, cudaStream_t s);
+// Up to four fields of n sites in one launch, chained to the stream's kernels; a site that cannot be
+// encoded sets *bad and *bad_host to 1.
+struct PackFields {
+    const double *in[4];
+    char *out[4];
+    int nfields;
+    int *bad;
+    int *bad_host;
+};
+void launch_pack_fields(int sf, int64_t n, const PackFields &f, cudaStream_t s);
 void launch_pack32_spinor(int sf, int64_t n, const float *in, char *out, int *err, cudaStream_t s);
 void launch_pack_pair_int30(int64_t n, const float *in, char *out, int *err, cudaStream_t s);
 void launch_unpack_spinor(int sf, int cf, int64_t n, const char *in, double *out, cudaStream_t s);
@@ -368,6 +383,8 @@ struct hisq_ctx {
     cudaStream_t stream = nullptr;
     hisq::RedBuf red{};
     int *err_flag = nullptr;         // device int
+    int *bad_flag = nullptr;         // device int: the stencil entry point's inputs, zero between calls
+    int *host_flags = nullptr;       // mapped host ints: [0] bad input, [1] unstorable output, zero between calls
     std::string last_error;
     std::mutex mu;
     std::vector<hisq_gauge *> gauges;
@@ -442,6 +459,21 @@ cudaError_t graph_kernel_nodes(cudaGraph_t g, size_t *n);
 // A validated triplet: returns HISQ_OK and the device view of the gauge copy.
 hisq_status gauge_view_for(hisq_ctx *c, hisq_gauge *g, const hisq_prec &p, GaugeView *v);
 hisq_status check_prec(hisq_ctx *c, const hisq_prec &p);
+// One call of the stencil entry points on device arrays: in_s, y_s hold the packed inputs (one or two
+// halves); tune_out, one half field, lets a first call time the launch shapes (null: not tuned here).
+struct StencilCall {
+    const hisq_gauge *g;
+    GaugeView gv;
+    hisq_prec prec;
+    int out_parity;
+    double a;
+    const double *y;
+    const double *in;
+    double *out;
+    char *in_s, *y_s, *tune_out;
+};
+// host_out: where the result is copied for a call on host arrays, or null.
+hisq_status run_stencil_call(hisq_ctx *c, const StencilCall &k, double *host_out, cudaStream_t s, const char *who);
 // The same view without building a missing copy (never allocates).
 hisq_status gauge_view_existing(hisq_ctx *c, const hisq_gauge *g, const hisq_prec &p, GaugeView *v);
 

@@ -1,7 +1,6 @@
 // noalloc.cu -- hisq_dslash_noalloc: the stencil entry point for callers that
-// must not allocate device memory.  Its scratch (the input, xpay and output
-// fields in the storage format and a non-finite counter) is one file-scope
-// device array sized for at most HISQ_NOALLOC_MAX_SITES sites per parity;
+// must not allocate device memory.  Its scratch (the input and xpay fields in
+// the storage format) is one file-scope device array sized for at most HISQ_NOALLOC_MAX_SITES sites per parity;
 // every GPU that loads the library holds it until the process exits.
 #include <cuda_runtime.h>
 
@@ -15,7 +14,7 @@ namespace {
 
 constexpr int64_t kMaxSites = HISQ_NOALLOC_MAX_SITES;
 constexpr size_t kFieldBytes = (size_t)48 * 2 * kMaxSites;  // one full-lattice field, widest format
-constexpr size_t kScratchBytes = 3 * kFieldBytes + 256;
+constexpr size_t kScratchBytes = 2 * kFieldBytes;
 
 static __device__ __align__(256) unsigned char noalloc_scratch[kScratchBytes];
 
@@ -61,7 +60,7 @@ extern "C" hisq_status hisq_dslash_noalloc(hisq_ctx *c, const hisq_gauge *g, his
     cudaError_t e = cudaSetDevice(c->device);
     if (e != cudaSuccess) return cuda_fail(c, e, "hisq_dslash_noalloc: cudaSetDevice");
     cudaStream_t s = pick_stream(c, stream);
-    // the counter read-back and the synchronisation below cannot be captured
+    // the synchronisation below cannot be captured
     if (stream_capturing(s))
         return fail(c, HISQ_EINVAL, "hisq_dslash_noalloc cannot be called while its stream is being captured");
     GaugeView gv{};
@@ -70,58 +69,6 @@ extern "C" hisq_status hisq_dslash_noalloc(hisq_ctx *c, const hisq_gauge *g, his
     char *sc = nullptr;
     st = scratch_address(c, &sc);
     if (st) return st;
-    const int nhalf = out_parity == 2 ? 2 : 1;
-    const size_t bs = spinor_field_bytes(prec.spinor, vh);
-    char *in_s = sc, *y_s = sc + kFieldBytes, *out_s = sc + 2 * kFieldBytes;
-    int *bad = reinterpret_cast<int *>(sc + 3 * kFieldBytes);
-    // the array keeps the previous call's contents: the counter starts at zero
-    e = cudaMemsetAsync(bad, 0, sizeof(int), s);
-    if (e != cudaSuccess) return cuda_fail(c, e, "hisq_dslash_noalloc");
-    for (int h = 0; h < nhalf; h++) {
-        launch_pack_spinor(prec.spinor, vh, in + h * vh * 6, in_s + h * bs, bad, s);
-        c->launches++;
-        if (xpay) {
-            launch_pack_spinor(prec.spinor, vh, xpay_in + h * vh * 6, y_s + h * bs, bad, s);
-            c->launches++;
-        }
-    }
-    int bad_in = 0;
-    e = cudaMemcpyAsync(&bad_in, bad, sizeof bad_in, cudaMemcpyDeviceToHost, s);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-    if (e != cudaSuccess) return cuda_fail(c, e, "hisq_dslash_noalloc pack");
-    if (bad_in) return fail(c, HISQ_EINVAL, "non-finite input spinor");
-    for (int h = 0; h < nhalf; h++) {
-        const int po = out_parity == 2 ? h : out_parity;
-        const int oi = out_parity == 2 ? po : 0, ii = out_parity == 2 ? 1 - po : 0;
-        DslashArgs da{};
-        da.g = g->geom;
-        da.gv = gv;
-        da.out_parity = po;
-        da.in = in_s + ii * bs;
-        da.out = out_s + oi * bs;
-        da.y = xpay ? y_s + oi * bs : nullptr;
-        da.a = a;
-        da.sign = xpay ? -1 : 1;
-        da.xpay = xpay ? 1 : 0;
-        da.err = bad;
-        da.fin = FIN_NONE;
-        if (!launch_dslash(prec.gauge, prec.spinor, prec.compute, prec.long_recon, false, da, s))
-            return fail(c, HISQ_EINVAL, "no stencil kernel for this triplet");
-        c->launches++;
-    }
-    for (int h = 0; h < nhalf; h++) {
-        launch_unpack_spinor(prec.spinor, prec.compute, vh, out_s + h * bs, out + h * vh * 6, s);
-        c->launches++;
-    }
-    // the stencil flags output sites it could not store
-    int bad_out = 0;
-    e = cudaMemcpyAsync(&bad_out, bad, sizeof bad_out, cudaMemcpyDeviceToHost, s);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-    if (e == cudaSuccess) e = cudaGetLastError();
-    if (e != cudaSuccess) return cuda_fail(c, e, "hisq_dslash_noalloc");
-    if (bad_out)
-        return fail(c, HISQ_ERANGE,
-                    "hisq_dslash_noalloc: output sites not storable in the spinor format (overflow or beyond its "
-                    "exponent range)");
-    return HISQ_OK;
+    StencilCall call{g, gv, prec, out_parity, a, xpay ? xpay_in : nullptr, in, out, sc, sc + kFieldBytes, nullptr};
+    return run_stencil_call(c, call, nullptr, s, "hisq_dslash_noalloc");
 }
