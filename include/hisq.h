@@ -263,7 +263,9 @@ typedef struct {
  * graphs: the event pairs are then recorded as graph nodes and read after
  * each block of iterations, and launches of iterations the device skipped
  * (the block stopped early) are not counted; the other solvers run without
- * graphs while profiling.  Reading synchronises on the events. */
+ * graphs while profiling.  The CG of a lattice small enough to iterate in one
+ * launch per run of iterations has each timed launch counted as its stencil
+ * passes, two an iteration.  Reading synchronises on the events. */
 HISQ_API void hisq_profile_enable(hisq_ctx *ctx, int on);
 HISQ_API void hisq_profile_reset(hisq_ctx *ctx);
 HISQ_API hisq_status hisq_profile_read(hisq_ctx *ctx, int kind, hisq_kernel_stats *out);

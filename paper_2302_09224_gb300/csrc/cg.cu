@@ -143,12 +143,19 @@ struct CGRun {
     double *r64 = nullptr, *ax64 = nullptr, *tmp64 = nullptr;
     CGState *st = nullptr;
     CGState *st_h = nullptr;
+    ulonglong2 *inbox = nullptr;  // resident iterations: the sums' words and their next tag
     GaugeView gv_s{}, gv_d{};
     double diag = 0;
     int ru = 0, mv_hi = 0;
     // one mode for the whole solve (its graph is captured once); the FP64 triplet keeps the one-block
     // sums: its split r_update (82 registers, one 512-thread block a SM) measured 0.2 % slower
     const bool split = split_mode.load() != 0 && cfg.sloppy.spinor != S_F64;
+
+    // a lattice that fits on the chip iterates in one launch per run of iterations
+    CGBlockShape resident = split && !mee_fused_asked()
+                                      ? cg_block_shape(cfg.sloppy.gauge, cfg.sloppy.spinor, cfg.sloppy.compute,
+                                                       cfg.sloppy.long_recon, vh)
+                                      : CGBlockShape{0, 0, 0};
 
     CGRun(hisq_ctx *c_, hisq_gauge *g_, const CGConfig &cfg_, cudaStream_t s_)
         : c(c_), g(g_), cfg(cfg_), s(s_), ws(c_, s_), vh(g_->geom.vh)
@@ -189,6 +196,15 @@ struct CGRun {
         if (e) return e;
         if (cudaMallocHost(&st_h, sizeof(CGState)) != cudaSuccess)
             return fail(c, HISQ_ENOMEM, "pinned host state");
+        if (resident.lanes > 0) {
+            const size_t words = 2 * (size_t)resident.blocks * resident.blocks;
+            if (ws.alloc((words + 1) * sizeof *inbox, (void **)&inbox) == HISQ_OK) {
+                cudaMemsetAsync(inbox, 0, words * sizeof *inbox, s);
+                cudaMemsetAsync(inbox + words, 1, sizeof *inbox, s);  // a first tag that is not zero
+            } else {
+                resident.lanes = 0;  // no room: the separate kernels
+            }
+        }
         cudaMemsetAsync(ring, 0, sb * cfg.nbuf, s);
         diag = 4.0 * cfg.mass * cfg.mass + cfg.sigma;
         tune_stencil(c, g->geom, cfg.sloppy, gv_s, ap_s, tmp_s, s);
@@ -280,6 +296,44 @@ struct CGRun {
         set_prof_tag(-1);
     }
 
+    // The same iterations, resident: up to iters of them (a multiple of nbuf) in one launch.
+    // timed: the profiler's event pair around it, counted as its stencil passes (two an iteration).
+    cudaError_t iterate_resident(double *x64, int iters, bool timed)
+    {
+        CGBlockArgs a{};
+        a.d.g = g->geom;
+        a.d.gv = gv_s;
+        a.r = r_s;
+        a.tmp = tmp_s;
+        a.ring = ring;
+        a.slot_bytes = sb;
+        a.nslots = cfg.nbuf;
+        a.iters = iters;
+        a.diag = diag;
+        a.x64 = x64;
+        a.st = st;
+        a.err = cur_err(c);
+        a.inbox = inbox;
+        a.seq = (unsigned *)(inbox + 2 * resident.blocks * resident.blocks);
+        a.bar = cur_red(c).sync + 8;
+        auto go = [&]() {
+            return launch_cg_block(cfg.sloppy.gauge, cfg.sloppy.spinor, cfg.sloppy.long_recon, resident, a, s)
+                       ? cudaSuccess
+                       : cudaGetLastError();
+        };
+        if (!timed) {
+            c->launches++;
+            return go();
+        }
+        set_prof_tag(kProfResident);
+        LaunchScope ls(c, s, PROF_STENCIL,
+                       iters * (stencil_bytes(cfg.sloppy, vh, false) + stencil_bytes(cfg.sloppy, vh, true)),
+                       2 * iters);
+        set_prof_tag(-1);
+        c->launches += 1 - 2 * iters;  // one kernel
+        return go();
+    }
+
     hisq_status run(const double *b64, double *x64, bool x_zero, hisq_solve_info *info)
     {
         hisq_status e = setup();
@@ -340,6 +394,7 @@ struct CGRun {
         cudaGraphExec_t exec = nullptr, exec_plain = nullptr;
         int64_t nodes = 0;
         int64_t block = 0;
+        int run_iters = 0;  // iterations asked of the last resident launch
         std::vector<Profiler::Rec> grecs;
         auto capture = [&](bool record, cudaGraphExec_t *out) -> cudaError_t {
             cudaGraph_t gr = nullptr;
@@ -366,7 +421,18 @@ struct CGRun {
             }
             const int k0 = st_h->k;
             const bool timed = !graph || block % every == 0;
-            if (graph) {
+            if (resident.lanes > 0) {
+                // several blocks of nbuf iterations a launch: the host looks at the state once per launch
+                // (once per nbuf iterations while profiling); where a run is cut changes no bit
+                const int left = (cfg.maxiter - k0 + cfg.nbuf - 1) / cfg.nbuf, most = c->prof.on ? 1 : 64 / cfg.nbuf;
+                const int iters = cfg.nbuf * std::min(left, most);
+                const cudaError_t ce = iterate_resident(x64, iters, c->prof.on && block % every == 0);
+                if (ce != cudaSuccess) {
+                    e = cuda_fail(c, ce, "resident CG launch");
+                    break;
+                }
+                run_iters = iters;
+            } else if (graph) {
                 cudaGraphExec_t *ex = (timed || !c->prof.on) ? &exec : &exec_plain;
                 if (!*ex) {
                     const cudaError_t ce = capture(c->prof.on && ex == &exec, ex);
@@ -385,7 +451,9 @@ struct CGRun {
             block++;
             e = pull_state();
             if (e) break;
-            if (!graph)
+            if (resident.lanes > 0)
+                prof_settle_resident(c, st_h->k - k0, run_iters);
+            else if (!graph)
                 prof_settle(c, st_h->k - k0);
             else if (timed)
                 prof_graph_account(c, grecs, st_h->k - k0);
@@ -397,7 +465,7 @@ struct CGRun {
                 break;
             }
             if (reason == REASON_RELIABLE || reason == REASON_CONVERGED) {
-                const int j = st_h->k - k0 - 1;
+                const int j = (st_h->k - k0 - 1) % cfg.nbuf;
                 flush(j + 1, nullptr, x64);
                 e = reliable_update(b64, x64, false, j);
                 if (e) break;
@@ -430,8 +498,8 @@ struct CGRun {
         info->matvecs_hi += mv_hi;
         info->reliable_updates += ru;
         info->true_residual = std::sqrt(st_h->hi_rr / bb);
-        if (herr & 2)  // a bounded wait of the fused M_ee pass gave up: its results are not trusted
-            return fail(c, HISQ_ECUDA, "fused M_ee pass: a wait for earlier t-slices reached its limit");
+        if (herr & 2)  // a bounded wait (fused M_ee pass, resident iterations) gave up: the results are not trusted
+            return fail(c, HISQ_ECUDA, "a wait between the blocks of a launch reached its limit");
         if (status == HISQ_ENOTCONV)
             fail(c, HISQ_ENOTCONV, "CG reached maxiter=%d with true residual %.3e", cfg.maxiter, info->true_residual);
         return status;

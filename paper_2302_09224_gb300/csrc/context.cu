@@ -174,6 +174,18 @@ void prof_settle(hisq_ctx *c, int n_exec)
     p.resize(w);
 }
 
+void prof_settle_resident(hisq_ctx *c, int n_exec, int n_asked)
+{
+    std::lock_guard<std::mutex> lk(c->prof_mu);
+    for (auto &r : c->prof.pending) {
+        if (r.tag != kProfResident) continue;
+        r.tag = -1;
+        if (n_exec >= n_asked) continue;
+        r.bytes *= (double)n_exec / n_asked;
+        r.nl = r.nl / n_asked * n_exec;
+    }
+}
+
 void prof_graph_account(hisq_ctx *c, const std::vector<Profiler::Rec> &recs, int n_exec)
 {
     std::lock_guard<std::mutex> lk(c->prof_mu);

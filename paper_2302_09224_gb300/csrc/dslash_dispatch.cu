@@ -4,6 +4,7 @@
 // the fastest is kept for the rest of the process.
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <array>
 #include <atomic>
 #include <map>
@@ -29,6 +30,8 @@ bool launch_mee_int20(int, int, const MeeArgs &, cudaStream_t);
 bool launch_mee_int30f(int, int, const MeeArgs &, cudaStream_t);
 
 std::atomic<int> fused_mode{0};
+
+bool mee_fused_asked() { return fused_mode.load() != 0; }
 
 bool mee_fused_available(int gf, int sf, int cf, const Geom &g)
 {
@@ -198,6 +201,57 @@ bool launch_dslash_mrhs(int gf, int sf, int cf, int long_recon, bool reduce, int
     if (gf == G_FIX16 && sf == S_HALF) return launch_mrhs_half(long_recon, reduce, T, variant, a, s);
     if (gf == G_FIX16 && sf == S_INT20) return launch_mrhs_int20(long_recon, reduce, T, variant, a, s);
     return false;
+}
+
+}  // namespace hisq
+
+namespace hisq {
+
+bool launch_cg_block_f32(int, const CGBlockShape &, const CGBlockArgs &, cudaStream_t);
+bool launch_cg_block_half(int, const CGBlockShape &, const CGBlockArgs &, cudaStream_t);
+bool launch_cg_block_int20(int, const CGBlockShape &, const CGBlockArgs &, cudaStream_t);
+
+// The most lanes a site (4, 2 or 1) with at most 512 threads on each SM (128
+// registers a thread: no spills), else one lane and up to 1024 threads while
+// the links of both passes are at most 160 MB (beyond the L2 the passes are
+// bound by HBM either way, and the separate ones hold more loads in flight);
+// the threads are spread over every SM.  Per iteration, here against the
+// separate kernels, 20-bit: 8^4 9.8 us against 21.8, 12^4 12.1 / 21.8, 16^4
+// 15.3 / 26.1, 16^3x32 21.1 / 33.0, 16^3x64 33.6 / 46.5, 20^3x36 38.1 / 47.5;
+// FP32: 16^3x32 18.8 / 35.2, but 16^3x64 (252 MB) 59.5 / 56.7.  Two lanes on
+// 864 threads (64 registers) lost to one lane on 431: 24.7 against 22.9 us on
+// 16^3x32, in an earlier form.
+CGBlockShape cg_block_shape(int gf, int sf, int cf, int long_recon, int vh)
+{
+    const bool has = cf == HISQ_COMPUTE_F32 && (long_recon == 12 || long_recon == 18) &&
+                     ((gf == G_F32 && sf == S_F32) || (gf == G_FIX16 && (sf == S_HALF || sf == S_INT20)));
+    static const int sms = [] {
+        int dev = 0, n = 0, coop = 0;
+        cudaGetDevice(&dev);
+        cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev);
+        cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev);
+        return coop ? n : 0;
+    }();
+    for (int lanes = 4; has && lanes >= 1; lanes /= 2) {
+        const long long all = (long long)vh * lanes;
+        if (all > (long long)sms * (lanes > 1 ? 512 : 1024)) continue;
+        if (all > (long long)sms * 512 && 16LL * vh * (link_bytes(gf, 18) + link_bytes(gf, long_recon)) > 160000000LL)
+            continue;
+        const int per = (int)((all + sms - 1) / sms);
+        const int threads = per <= 64 ? 64 : (per + 31) / 32 * 32;
+        return {lanes, threads, (int)((all + threads - 1) / threads)};
+    }
+    return {0, 0, 0};
+}
+
+bool launch_cg_block(int gf, int sf, int long_recon, const CGBlockShape &sh, const CGBlockArgs &args, cudaStream_t s)
+{
+    CGBlockArgs a = args;
+    a.wait_polls = std::min(fused_wait_polls.load(), 1u << 20);  // about half a second of L2 round trips
+    a.wait_extra = fused_wait_extra.load();
+    if (gf == G_F32) return launch_cg_block_f32(long_recon, sh, a, s);
+    if (sf == S_HALF) return launch_cg_block_half(long_recon, sh, a, s);
+    return launch_cg_block_int20(long_recon, sh, a, s);
 }
 
 }  // namespace hisq

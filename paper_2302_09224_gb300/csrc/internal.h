@@ -238,6 +238,30 @@ struct MeeArgs {
     unsigned wait_extra;    // added to every wait's target: nonzero only to test the bound
 };
 
+// Blocks of CG iterations of a lattice resident on the chip (cg_block.cuh): d holds the lattice and
+// links, ring nslots gradient vectors slot_bytes apart (slot 0 the current one at the launch).
+struct CGBlockArgs {
+    DslashArgs d;
+    char *r, *tmp, *ring;
+    size_t slot_bytes;
+    int nslots;
+    int iters;          // iterations at most (a multiple of nslots)
+    double diag;
+    double *x64;
+    CGState *st;
+    int *err;
+    ulonglong2 *inbox;  // the sums' words: two sets of blocks x blocks, zero before the first launch
+    unsigned *seq;      // tag of the next launch's first sum (not zero)
+    unsigned *bar;      // [0] arrivals, [8] blocks that have left; zero between launches
+    unsigned wait_polls;    // polls before a wait gives up, each at least one L2 round trip (set by the launcher)
+    unsigned wait_extra;    // added to every wait's target: nonzero only to test the bound
+};
+// Lanes per site, threads per block and blocks of such a launch; lanes 0: the lattice or the triplet
+// does not take it.
+struct CGBlockShape {
+    int lanes, threads, blocks;
+};
+
 // A tile of right-hand sides for the batched stencil: right-hand side t lives
 // in the fields at in/out/y + t * field_bytes.
 constexpr int kMaxRHS = 16;
@@ -292,8 +316,11 @@ void tune_dslash(int gf, int sf, int cf, int long_recon, const DslashArgs &a, cu
 int stencil_config(int gf, int sf, int cf, int long_recon, bool reduce, const Geom &g);
 // The fused M_ee pass (red.sync must be set); false when the triplet or the
 // lattice has none, or it is switched off (hisq_mee_fused).
+bool mee_fused_asked();  // hisq_mee_fused is on
 bool mee_fused_available(int gf, int sf, int cf, const Geom &g);
 bool launch_mee_fused(int gf, int sf, int cf, int long_recon, const MeeArgs &m, cudaStream_t s);
+CGBlockShape cg_block_shape(int gf, int sf, int cf, int long_recon, int vh);
+bool launch_cg_block(int gf, int sf, int long_recon, const CGBlockShape &sh, const CGBlockArgs &a, cudaStream_t s);
 int stencil_config_in_use(int gf, int sf, int cf, int long_recon, bool reduce, const Geom &g);
 
 void launch_pack_spinor(int sf, int64_t n, const double *in, char *out, int *err, cudaStream_t s);
@@ -444,6 +471,9 @@ void prof_flush_locked(hisq_ctx *c);
 // After a block of iterations of which n_exec ran: drop the pending records
 // tagged with a later iteration (launches that returned at once).
 void prof_settle(hisq_ctx *c, int n_exec);
+// The same for a launch of n_asked iterations (tagged kProfResident) that did n_exec of them.
+constexpr int kProfResident = -2;
+void prof_settle_resident(hisq_ctx *c, int n_exec, int n_asked);
 // Profiling inside a captured graph: while a recorder is set on the capturing
 // thread, launch scopes record their event pairs as graph nodes (external
 // event records) into it; after each replay of the graph and a synchronise,
