@@ -236,7 +236,8 @@ BatchSession::~BatchSession()
 {
     for (auto &kv : graphs)
         if (kv.second.exec) cudaGraphExecDestroy(kv.second.exec);
-    if (sth) cudaFreeHost(sth);
+    cudaStreamSynchronize(s);  // no copy into the state block is in flight
+    pinned_put(c, sth);
 }
 
 char *BatchSession::slot(int j, int t) { return ring + ((size_t)j * nr + t) * fb; }
@@ -386,7 +387,9 @@ hisq_status BatchSession::setup()
     if (!e) e = ws.alloc((size_t)48 * vh, (void **)&tmp64);
     if (!e) e = ws.alloc(sizeof(CGState) * nr, (void **)&st);
     if (e) return e;
-    if (cudaMallocHost(&sth, sizeof(CGState) * nr) != cudaSuccess) return fail(c, HISQ_ENOMEM, "pinned state");
+    static_assert(sizeof(CGState) * kMaxRHS <= kPinnedBytes, "a batch's states fit a pinned block");
+    sth = (CGState *)pinned_get(c, sizeof(CGState) * nr);
+    if (!sth) return fail(c, HISQ_ENOMEM, "pinned state");
     mv_hi.assign(nr, 0);
     ru.assign(nr, 0);
     k0.assign(nr, 0);

@@ -481,7 +481,8 @@ struct BRun {
     }
     ~BRun()
     {
-        if (bh) cudaFreeHost(bh);
+        cudaStreamSynchronize(st);  // no copy into the state block is in flight
+        pinned_put(c, bh);
     }
 
     BArgs args() const
@@ -627,7 +628,8 @@ struct BRun {
         if (!e) e = ws.alloc(f64b, (void **)&r64);
         if (!e) e = ws.alloc(sizeof(BState), (void **)&b);
         if (e) return e;
-        if (cudaMallocHost(&bh, sizeof(BState)) != cudaSuccess) return fail(c, HISQ_ENOMEM, "pinned host state");
+        bh = (BState *)pinned_get(c, sizeof(BState));
+        if (!bh) return fail(c, HISQ_ENOMEM, "pinned host state");
         tune_stencil(c, g->geom, p.sloppy, gv_s, U, R, st);
         tune_stencil(c, g->geom, prec_f64(), gv_d, (char *)ax64, (char *)r64, st);
         cudaMemsetAsync(U, 0, fb * (l + 1), st);

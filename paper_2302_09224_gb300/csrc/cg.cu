@@ -163,7 +163,8 @@ struct CGRun {
     }
     ~CGRun()
     {
-        if (st_h) cudaFreeHost(st_h);
+        cudaStreamSynchronize(s);  // no copy into the state block is in flight
+        pinned_put(c, st_h);
     }
 
     char *slot(int j) { return ring + (size_t)j * sb; }
@@ -194,7 +195,8 @@ struct CGRun {
         if (!e) e = ws.alloc(b64, (void **)&tmp64);
         if (!e) e = ws.alloc(sizeof(CGState), (void **)&st);
         if (e) return e;
-        if (cudaMallocHost(&st_h, sizeof(CGState)) != cudaSuccess)
+        st_h = (CGState *)pinned_get(c, sizeof(CGState));
+        if (!st_h)
             return fail(c, HISQ_ENOMEM, "pinned host state");
         if (resident.lanes > 0) {
             const size_t words = 2 * (size_t)resident.blocks * resident.blocks;

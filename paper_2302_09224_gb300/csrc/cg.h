@@ -10,8 +10,8 @@
 
 namespace hisq {
 
-// Device allocations owned by one solve; freed (after the stream drains) on
-// destruction.
+// Device allocations owned by one solve; given back (after the stream drains)
+// on destruction.
 struct Workspace {
     hisq_ctx *c;
     cudaStream_t s;

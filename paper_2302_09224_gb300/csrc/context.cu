@@ -63,6 +63,29 @@ int *cur_err(hisq_ctx *c) { return tl_lane ? tl_lane->err : c->err_flag; }
 void set_thread_capturing(bool on) { tl_capturing = on; }
 bool thread_capturing() { return tl_capturing; }
 
+// Device buffers of finished calls stay with the context for the next one, by
+// exact size: a solve allocates the same dozen fields each time, and
+// cudaMalloc and cudaFree of them took 10 to 740 us each (4 KB to 1 GB; the
+// latter also waits for the whole device).  Kept buffers are never in use: each
+// is given back after its stream has been waited for.  They are bounded
+// (kKeepBytes, and an eighth of the budget), count against the budget but not
+// as used, and are released, oldest first, when an allocation needs the room,
+// and with the context.
+namespace {
+constexpr size_t kKeepBytes = (size_t)4 << 30;
+
+void release_kept(hisq_ctx *c, size_t until)  // alloc_mu held
+{
+    size_t n = 0;
+    while (n < c->kept.size() && c->kept_bytes > until) {
+        cudaFree(c->kept[n].first);
+        c->kept_bytes -= c->kept[n].second;
+        n++;
+    }
+    c->kept.erase(c->kept.begin(), c->kept.begin() + n);
+}
+}  // namespace
+
 hisq_status ctx_alloc(hisq_ctx *c, size_t bytes, void **p)
 {
     *p = nullptr;
@@ -70,7 +93,21 @@ hisq_status ctx_alloc(hisq_ctx *c, size_t bytes, void **p)
     std::lock_guard<std::mutex> lk(c->alloc_mu);
     if (c->used + bytes > c->budget)
         return fail(c, HISQ_ENOMEM, "device budget exceeded: %zu + %zu > %zu bytes", c->used, bytes, c->budget);
-    const cudaError_t e = cudaMalloc(p, bytes);
+    for (size_t k = c->kept.size(); k-- > 0;)
+        if (c->kept[k].second == bytes) {
+            *p = c->kept[k].first;
+            c->kept.erase(c->kept.begin() + k);
+            c->kept_bytes -= bytes;
+            c->used += bytes;
+            return HISQ_OK;
+        }
+    if (c->used + c->kept_bytes + bytes > c->budget) release_kept(c, c->budget - c->used - bytes);
+    cudaError_t e = cudaMalloc(p, bytes);
+    if (e != cudaSuccess && !c->kept.empty()) {
+        (void)cudaGetLastError();
+        release_kept(c, 0);
+        e = cudaMalloc(p, bytes);
+    }
     if (e != cudaSuccess) {
         (void)cudaGetLastError();
         *p = nullptr;
@@ -80,12 +117,54 @@ hisq_status ctx_alloc(hisq_ctx *c, size_t bytes, void **p)
     return HISQ_OK;
 }
 
+// The buffer's last use has completed (its stream was waited for).
 void ctx_free(hisq_ctx *c, void *p, size_t bytes)
 {
     if (!p) return;
     std::lock_guard<std::mutex> lk(c->alloc_mu);
-    cudaFree(p);
     c->used -= std::min(c->used, bytes);
+    const size_t most = std::min(kKeepBytes, c->budget / 8);
+    if (bytes > most) {
+        cudaFree(p);
+        return;
+    }
+    release_kept(c, most - bytes);
+    c->kept.emplace_back(p, bytes);
+    c->kept_bytes += bytes;
+}
+
+// Pinned host blocks of kPinnedBytes for the solvers' state (allocating and
+// freeing one takes 255 us); a few are kept with the context.
+void *pinned_get(hisq_ctx *c, size_t bytes)
+{
+    if (bytes > kPinnedBytes) return nullptr;
+    {
+        std::lock_guard<std::mutex> lk(c->alloc_mu);
+        if (!c->pinned.empty()) {
+            void *p = c->pinned.back();
+            c->pinned.pop_back();
+            return p;
+        }
+    }
+    void *p = nullptr;
+    if (cudaMallocHost(&p, kPinnedBytes) != cudaSuccess) {
+        (void)cudaGetLastError();
+        return nullptr;
+    }
+    return p;
+}
+
+void pinned_put(hisq_ctx *c, void *p)
+{
+    if (!p) return;
+    {
+        std::lock_guard<std::mutex> lk(c->alloc_mu);
+        if (c->pinned.size() < 8) {
+            c->pinned.push_back(p);
+            return;
+        }
+    }
+    cudaFreeHost(p);
 }
 
 cudaStream_t pick_stream(hisq_ctx *c, void *s) { return s ? (cudaStream_t)s : c->stream; }
@@ -521,6 +600,8 @@ void hisq_destroy(hisq_ctx *c)
     if (c->scratch) cudaFree(c->scratch);
     if (c->red.partials) cudaFree(c->red.partials);
     if (c->host_flags) cudaFreeHost(c->host_flags);
+    for (auto &k : c->kept) cudaFree(k.first);
+    for (void *h : c->pinned) cudaFreeHost(h);
     if (c->stream) cudaStreamDestroy(c->stream);
     delete c;
 }
@@ -602,7 +683,7 @@ void hisq_free_gauge(hisq_ctx *c, hisq_gauge *g)
 {
     if (!c || !g) return;
     cudaSetDevice(c->device);
-    cudaStreamSynchronize(c->stream);
+    cudaStreamSynchronize(c->stream);  // every call that reads the links waits for its own stream
     {
         std::lock_guard<std::mutex> lk(c->mu);
         c->gauges.erase(std::remove(c->gauges.begin(), c->gauges.end(), g), c->gauges.end());
@@ -631,7 +712,7 @@ static hisq_status grow_scratch(hisq_ctx *c, size_t bytes)
 {
     if (c->scratch_bytes >= bytes) return HISQ_OK;
     if (c->scratch) {
-        cudaStreamSynchronize(c->stream);
+        cudaStreamSynchronize(c->stream);  // every call that uses it waits for its own stream
         ctx_free(c, c->scratch, c->scratch_bytes);
         c->scratch = nullptr;
         c->scratch_bytes = 0;

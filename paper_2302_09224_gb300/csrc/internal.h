@@ -11,6 +11,7 @@
 #include <atomic>
 #include <mutex>
 #include <string>
+#include <utility>
 #include <vector>
 
 #include "hisq.h"
@@ -419,7 +420,10 @@ struct hisq_ctx {
     char *scratch = nullptr;
     size_t scratch_bytes = 0;
     std::atomic<int64_t> launches{0};  // kernels launched (graph replays count their nodes)
-    std::mutex alloc_mu;               // device allocations and lazily built gauge copies
+    std::mutex alloc_mu;               // device allocations and the buffers kept below
+    std::vector<std::pair<void *, size_t>> kept;  // device buffers of finished calls, oldest first
+    size_t kept_bytes = 0;
+    std::vector<void *> pinned;        // pinned host blocks of finished solves
     std::mutex err_mu;                 // last_error
     hisq::Server *server = nullptr;    // request loop, started by the first hisq_submit
     std::mutex prof_mu;
@@ -450,6 +454,10 @@ hisq_status fail(hisq_ctx *c, hisq_status s, const char *fmt, ...);
 hisq_status cuda_fail(hisq_ctx *c, cudaError_t e, const char *what);
 hisq_status ctx_alloc(hisq_ctx *c, size_t bytes, void **p);
 void ctx_free(hisq_ctx *c, void *p, size_t bytes);
+// A pinned host block of at least `bytes` (at most kPinnedBytes; null: none to be had) and its return.
+constexpr size_t kPinnedBytes = 16384;
+void *pinned_get(hisq_ctx *c, size_t bytes);
+void pinned_put(hisq_ctx *c, void *p);
 cudaStream_t pick_stream(hisq_ctx *c, void *s);
 
 // launch bookkeeping: call before / after every kernel launch on stream s

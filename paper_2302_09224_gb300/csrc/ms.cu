@@ -189,7 +189,8 @@ struct MSRun {
     }
     ~MSRun()
     {
-        if (mh) cudaFreeHost(mh);
+        cudaStreamSynchronize(s);  // no copy into the state block is in flight
+        pinned_put(c, mh);
     }
 
     double *x64(int i) { return X + (size_t)i * 6 * vh; }
@@ -323,7 +324,8 @@ struct MSRun {
         if (!e) e = ws.alloc(b48, (void **)&tmp64);
         if (!e) e = ws.alloc(sizeof(MSState), (void **)&m);
         if (e) return e;
-        if (cudaMallocHost(&mh, sizeof(MSState)) != cudaSuccess) return fail(c, HISQ_ENOMEM, "pinned host state");
+        mh = (MSState *)pinned_get(c, sizeof(MSState));
+        if (!mh) return fail(c, HISQ_ENOMEM, "pinned host state");
         cudaMemsetAsync(ACC, 0, accb * ns, s);
         cudaMemsetAsync(X, 0, b48 * ns, s);
         tune_stencil(c, g->geom, p.sloppy, gv_s, w_s, tmp_s, s);
