@@ -22,10 +22,12 @@
 
 #include "bcg.h"
 #include "blas.h"
+#include "blas_update.cuh"
 #include "cg.h"
 #include "codecs.cuh"
 #include "finish.cuh"
 #include "internal.h"
+#include "launch.cuh"
 #include "reduce.cuh"
 
 namespace hisq {
@@ -33,6 +35,10 @@ namespace hisq {
 namespace {
 
 constexpr int kBlock = 256;
+
+constexpr int kRBlock = 512;        // residual update: threads, and blocks per right-hand side at most
+constexpr int kRMaxBlocks = 304;
+constexpr int kUSites = 2;          // sites a thread of the updates loads before using any
 
 struct BBArgs {
     int n, nrhs;
@@ -42,105 +48,207 @@ struct BBArgs {
     char *ring;         // [nbuf][nrhs] fields
     int nslots;
     int clear_ring;
+    int slot;           // ring slot of the iteration
+    int T;              // tile of the stencil pass that left its block sums
+    int nstencil, nr_blocks;  // block sums per right-hand side: the stencil pass's, the residual update's
+    const float2 *stencil_sums;
+    float2 *r_sums;     // [nrhs][nr_blocks]
     double *x64;        // [nrhs] FP64 planar fields (48 n bytes each)
     CGState *st;
     int *err;
-    RedBuf red;
 };
 
-// r_t -= alpha_t Ap_t for active t; per-RHS |r_t|^2 and Re<r_t new, r_t old>
-template <int SF, typename real>
-__global__ void __launch_bounds__(kBlock) b_r_update_kernel(BBArgs a)
+// An iteration's updates, blockIdx.y the right-hand side: each runs the split
+// form of the single system's (blas.cu: every block sums the previous
+// kernel's partials of its right-hand side and takes its step from them; block
+// 0 runs the finisher), so no one-block launch and no last-block tail is left.
+// One kernel over all right-hand sides with 32 sums a thread and a last block
+// took 183 us for 16 right-hand sides of 331776 sites (34 us of bytes).  The
+// grid of one right-hand side depends on the lattice alone, so its sums do not
+// depend on its companions.
+__device__ __forceinline__ BlasArgs rhs_args(const BBArgs &a, int t)
 {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    real v[2 * kMaxRHS];
+    BlasArgs b{};
+    b.n = a.n;
+    b.err = a.err;
+    b.v0 = a.r + (size_t)t * a.fb;
+    return b;
+}
+
+// The sums of right-hand side t over the stencil pass's blocks, FP32 pairs in a fixed order (thread 0).
+__device__ __forceinline__ void sum_stencil_partials(const BBArgs &a, int t, double tot[2])
+{
+    __shared__ FF sh[32][2];
+    const int t0 = t / a.T * a.T;
+    const float2 *part = a.stencil_sums + (size_t)t0 * a.nstencil + (t - t0);
+    FF w[2] = {{0.0f, 0.0f}, {0.0f, 0.0f}};
+    constexpr int U = 8;
+    for (int b0 = threadIdx.x; b0 < a.nstencil; b0 += U * kRBlock) {
+        float2 v[U];
 #pragma unroll
-    for (int k = 0; k < 2 * kMaxRHS; k++) v[k] = 0;
-    if (i < a.n) {
+        for (int u = 0; u < U; u++) {
+            const int b = b0 + u * kRBlock;
+            v[u] = b < a.nstencil ? __ldcg(part + (size_t)b * a.T) : make_float2(0.0f, 0.0f);
+        }
 #pragma unroll
-        for (int t = 0; t < kMaxRHS; t++) {
-            if (t >= a.nrhs || !a.st[t].active) continue;
-            real r[6], ap[6];
-            char *rf = a.r + (size_t)t * a.fb;
-            Spinor<SF>::load(rf, a.n, i, r);
-            Spinor<SF>::load(a.ap + (size_t)t * a.fb, a.n, i, ap);
-            const real alpha = (real)a.st[t].alpha;
-            real n2 = 0, d = 0;
-#pragma unroll
-            for (int k = 0; k < 6; k++) {
-                const real rn = r[k] - alpha * ap[k];
-                n2 += rn * rn;
-                d += rn * r[k];
-                r[k] = rn;
-            }
-            v[2 * t] = n2;
-            v[2 * t + 1] = d;
-            if (!Spinor<SF>::store(rf, a.n, i, r)) atomicExch(a.err, 1);
+        for (int u = 0; u < U; u++) {
+            w[0] = ff_add(w[0], FF{v[u].x, 0.0f});
+            w[1] = ff_add(w[1], FF{v[u].y, 0.0f});
         }
     }
-    __shared__ double tot[2 * kMaxRHS];
-    if (reduce_grid<2 * kMaxRHS>(v, a.red, tot) && threadIdx.x == 0)
-        run_batch_finisher(FIN_CG_BETA, tot, a.st, 0, a.nrhs, 0);
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    warp_sum_ff<2>(w);
+    if (lane == 0) {
+        sh[wid][0] = w[0];
+        sh[wid][1] = w[1];
+    }
+    __syncthreads();
+    if (wid == 0) {
+        w[0] = lane < kRBlock / 32 ? sh[lane][0] : FF{0.0f, 0.0f};
+        w[1] = lane < kRBlock / 32 ? sh[lane][1] : FF{0.0f, 0.0f};
+        warp_sum_ff<2>(w);
+        tot[0] = (double)w[0].hi + (double)w[0].lo;
+        tot[1] = (double)w[1].hi + (double)w[1].lo;
+    }
+}
+
+// r_t -= alpha_t Ap_t for active t; block sums of |r_t|^2 and Re<r_t new, r_t old>
+template <int SF, typename real>
+__global__ void __launch_bounds__(kRBlock) b_r_update_kernel(const __grid_constant__ BBArgs a)
+{
+    pdl_wait();
+    pdl_launch_dependents();
+    const int t = (int)blockIdx.y;
+    CGState *st = a.st + t;
+    if (*(volatile const int *)&st->active == 0) return;
+    constexpr int U = kUSites, C = Spinor<SF>::chunks;
+    BlasArgs b = rhs_args(a, t);
+    b.v1 = a.ap + (size_t)t * a.fb;
+    const int step = (int)gridDim.x * kRBlock * U;
+    int i0 = (int)blockIdx.x * kRBlock * U + (int)threadIdx.x;
+    uint4 cr[U][C], ca[U][C];
+    r_load<SF>(b, i0, cr, ca);
+    __shared__ real al_sh;
+    __shared__ int ok_sh;
+    double tot[2] = {0.0, 0.0};
+    sum_stencil_partials(a, t, tot);
+    if (threadIdx.x == 0) {
+        const double al = st->rr / tot[0];
+        const bool ok = tot[0] > 0.0 && isfinite(al);  // else the finisher stops this system
+        al_sh = ok ? real(al) : real(0);
+        ok_sh = ok;
+    }
+    __syncthreads();
+    if (ok_sh) {
+        const real alpha = al_sh;
+        real v[2] = {0, 0};
+        for (; i0 < a.n; i0 += step) {
+            r_group<SF, real>(b, i0, cr, ca, alpha, v);
+            r_load<SF>(b, i0 + step, cr, ca);
+        }
+        store_partial_at<2, float>(v, reinterpret_cast<float *>(a.r_sums + (size_t)t * a.nr_blocks), blockIdx.x);
+    }
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+        st->rr_den = st->rr;
+        run_finisher(FIN_CG_ALPHA, tot, st, a.slot);
+    }
 }
 
 // p_out_t = r_t + beta_t p_in_t for active t
 template <int SF, typename real>
-__global__ void __launch_bounds__(kBlock) b_p_update_kernel(BBArgs a)
+__global__ void __launch_bounds__(kBlock) b_p_update_kernel(const __grid_constant__ BBArgs a)
 {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (a.clear_ring && i == 0)
-        for (int t = 0; t < a.nrhs; t++)
-            if (a.st[t].active)
-                for (int j = 0; j < kMaxBuf; j++) a.st[t].alpha_ring[j] = 0.0;
-    if (i >= a.n) return;
-    for (int t = 0; t < a.nrhs; t++) {
-        if (!a.st[t].active) continue;
-        real r[6], p[6];
-        Spinor<SF>::load(a.r + (size_t)t * a.fb, a.n, i, r);
-        Spinor<SF>::load(a.p_in + (size_t)t * a.fb, a.n, i, p);
-        const real beta = (real)a.st[t].beta;
-#pragma unroll
-        for (int k = 0; k < 6; k++) p[k] = r[k] + beta * p[k];
-        if (!Spinor<SF>::store(a.p_out + (size_t)t * a.fb, a.n, i, p)) atomicExch(a.err, 1);
+    pdl_wait();
+    pdl_launch_dependents();
+    const int t = (int)blockIdx.y;
+    CGState *st = a.st + t;
+    if (*(volatile const int *)&st->active == 0) return;
+    constexpr int U = kUSites, C = Spinor<SF>::chunks;
+    if (a.clear_ring && blockIdx.x == 0 && threadIdx.x == 0)
+        for (int j = 0; j < kMaxBuf; j++) st->alpha_ring[j] = 0.0;
+    BlasArgs b = rhs_args(a, t);
+    b.v1 = a.p_in + (size_t)t * a.fb;
+    b.v2 = a.p_out + (size_t)t * a.fb;
+    const int i0 = (int)blockIdx.x * kBlock * U + (int)threadIdx.x;
+    uint4 cr[U][C], cp[U][C];
+    p_load<SF>(b, i0, cr, cp);
+    __shared__ double tot[2];
+    __shared__ real be_sh;
+    __shared__ int ok_sh;
+    RedBuf rb{};
+    rb.partials = reinterpret_cast<double *>(a.r_sums + (size_t)t * a.nr_blocks);
+    warp0_sum_partials<2, float>(rb, (unsigned)a.nr_blocks, tot);
+    if (threadIdx.x == 0) {
+        const double rr_new = tot[0];
+        const double be = (st->pr ? rr_new - tot[1] : rr_new) / st->rr_den;
+        const bool ok = isfinite(rr_new) && isfinite(be);  // else the finisher stops this system
+        be_sh = ok ? real(be) : real(0);
+        ok_sh = ok;
     }
+    __syncthreads();
+    if (ok_sh) p_group<SF, real>(b, i0, cr, cp, be_sh);
+    if (blockIdx.x == 0 && threadIdx.x == 0) run_finisher(FIN_CG_BETA, tot, st, a.slot);
 }
 
 // x_t += sum_j alpha_{t,j} p_{t,j} for active t (increment in the compute precision)
 template <int SF, typename real>
-__global__ void __launch_bounds__(kBlock) b_flush_kernel(BBArgs a)
+__global__ void __launch_bounds__(kBlock) b_flush_kernel(const __grid_constant__ BBArgs a)
 {
+    pdl_wait();
+    pdl_launch_dependents();
+    const int t = (int)blockIdx.y;
+    if (*(volatile const int *)&a.st[t].active == 0) return;
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    __shared__ real al_s[kMaxBuf];
+    if (threadIdx.x < kMaxBuf)
+        al_s[threadIdx.x] = threadIdx.x < a.nslots ? (real)a.st[t].alpha_ring[threadIdx.x] : real(0);
+    __syncthreads();
     if (i >= a.n) return;
-    for (int t = 0; t < a.nrhs; t++) {
-        if (!a.st[t].active) continue;
-        real dx[6] = {0, 0, 0, 0, 0, 0};
-        for (int j = 0; j < a.nslots; j++) {
-            const real al = (real)a.st[t].alpha_ring[j];
-            if (al == real(0)) continue;
-            real p[6];
-            Spinor<SF>::load(a.ring + ((size_t)j * a.nrhs + t) * a.fb, a.n, i, p);
+    constexpr int G = 4, C = Spinor<SF>::chunks;  // slots whose loads are in flight together
+    char *xf = reinterpret_cast<char *>(a.x64) + (size_t)t * 48 * a.n;
+    uint4 cx[Spinor<S_F64>::chunks];
+    Spinor<S_F64>::gather(xf, a.n, i, cx);
+    real dx[6] = {0, 0, 0, 0, 0, 0};
+    for (int j0 = 0; j0 < a.nslots; j0 += G) {
+        uint4 cp[G][C];
+        real al[G];
 #pragma unroll
-            for (int k = 0; k < 6; k++) dx[k] += al * p[k];
+        for (int q = 0; q < G; q++) {
+            al[q] = j0 + q < a.nslots ? al_s[j0 + q] : real(0);
+            if (al[q] != real(0)) Spinor<SF>::gather(a.ring + ((size_t)(j0 + q) * a.nrhs + t) * a.fb, a.n, i, cp[q]);
         }
-        char *xf = reinterpret_cast<char *>(a.x64) + (size_t)t * 48 * a.n;
-        double x[6];
-        Spinor<S_F64>::load(xf, a.n, i, x);
 #pragma unroll
-        for (int k = 0; k < 6; k++) x[k] += (double)dx[k];
-        Spinor<S_F64>::store(xf, a.n, i, x);
+        for (int q = 0; q < G; q++) {
+            if (al[q] == real(0)) continue;
+            real p[6];
+            Spinor<SF>::decode(cp[q], p);
+#pragma unroll
+            for (int k = 0; k < 6; k++) dx[k] += al[q] * p[k];
+        }
     }
+    double x[6];
+    Spinor<S_F64>::decode(cx, x);
+#pragma unroll
+    for (int k = 0; k < 6; k++) x[k] += f2d_bits(dx[k]);
+    Spinor<S_F64>::store(xf, a.n, i, x);
 }
 
-#define BB_DISPATCH(SF_, CF_, KERNEL)                                                             \
+#define BB_DISPATCH(SF_, KERNEL, NB, BS)                                                          \
     do {                                                                                         \
-        const int nb_ = (a.n + kBlock - 1) / kBlock;                                             \
+        const dim3 nb_(NB, a.nrhs), bs_(BS);                                                     \
         switch (SF_) {                                                                           \
-        case S_F32: KERNEL<S_F32, float><<<nb_, kBlock, 0, s>>>(a); break;                       \
-        case S_HALF: KERNEL<S_HALF, float><<<nb_, kBlock, 0, s>>>(a); break;                     \
-        case S_INT20: KERNEL<S_INT20, float><<<nb_, kBlock, 0, s>>>(a); break;                   \
+        case S_F32: launch_chained(KERNEL<S_F32, float>, nb_, bs_, s, a); break;                 \
+        case S_HALF: launch_chained(KERNEL<S_HALF, float>, nb_, bs_, s, a); break;               \
+        case S_INT20: launch_chained(KERNEL<S_INT20, float>, nb_, bs_, s, a); break;             \
         default: break;                                                                          \
         }                                                                                        \
     } while (0)
+
+int r_blocks(int n)
+{
+    const int need = (n + kRBlock * kUSites - 1) / (kRBlock * kUSites);
+    return need < kRMaxBlocks ? need : kRMaxBlocks;
+}
 
 using TileKey = std::array<int, 10>;
 // The fastest (T, variant) for a full batch, and per tile size (index log2 T)
@@ -179,7 +287,6 @@ TileChoice tune_tile(hisq_ctx *c, const Geom &geom, const hisq_prec &p, const Ga
         d.sign = 1;
         d.nrhs = nrhs;
         d.err = cur_err(c);
-        d.red = cur_red(c);
         cudaEvent_t e0, e1;
         cudaEventCreate(&e0);
         cudaEventCreate(&e1);
@@ -259,13 +366,17 @@ BBArgs bb_args(const BatchSession &b)
     a.ring = b.ring;
     a.st = b.st;
     a.err = cur_err(b.c);
-    a.red = cur_red(b.c);
+    a.T = b.T;
+    a.nstencil = (b.vh + kMrhsBlock - 1) / kMrhsBlock;
+    a.nr_blocks = r_blocks(b.vh);
+    a.stencil_sums = b.sums;
+    a.r_sums = b.sums + (size_t)b.nr * a.nstencil;
     return a;
 }
 
 }  // namespace
 
-void BatchSession::stencil_pass(int parity_out, const char *in, char *out, const char *y, bool red, int slot_i)
+void BatchSession::stencil_pass(int parity_out, const char *in, char *out, const char *y, bool red)
 {
     DslashMArgs d{};
     d.g = g->geom;
@@ -277,14 +388,12 @@ void BatchSession::stencil_pass(int parity_out, const char *in, char *out, const
     d.field_bytes = fb;
     d.nrhs = nr;
     d.err = cur_err(c);
-    d.red = cur_red(c);
     d.st = st;
-    d.slot = slot_i;
+    d.partials = sums;
     d.tile_mask = tile_mask;
     if (y) {
         d.xpay = 1;
         d.sign = -1;
-        d.fin = FIN_CG_ALPHA;
     } else {
         d.sign = 1;
     }
@@ -299,24 +408,25 @@ void BatchSession::iterate_block()
 {
     const double sb = (double)spinor_site_bytes(cfg.sloppy.spinor) * vh;
     for (int i = 0; i < N; i++) {
-        stencil_pass(1, slot(i, 0), tmp_s, nullptr, false, i);
-        stencil_pass(0, tmp_s, ap_s, slot(i, 0), true, i);
+        stencil_pass(1, slot(i, 0), tmp_s, nullptr, false);
+        stencil_pass(0, tmp_s, ap_s, slot(i, 0), true);
         BBArgs a = bb_args(*this);
+        a.slot = i;
         {
             LaunchScope ls(c, s, PROF_BLAS, 3.0 * sb * nr);
-            BB_DISPATCH(cfg.sloppy.spinor, cfg.sloppy.compute, b_r_update_kernel);
+            BB_DISPATCH(cfg.sloppy.spinor, b_r_update_kernel, a.nr_blocks, kRBlock);
         }
         if (i == N - 1) {
             a.x64 = x64;
             a.nslots = N;
             LaunchScope ls(c, s, PROF_BLAS, (96.0 + N * spinor_site_bytes(cfg.sloppy.spinor)) * vh * nr);
-            BB_DISPATCH(cfg.sloppy.spinor, cfg.sloppy.compute, b_flush_kernel);
+            BB_DISPATCH(cfg.sloppy.spinor, b_flush_kernel, (vh + kBlock - 1) / kBlock, kBlock);
         }
         a.p_in = slot(i, 0);
         a.p_out = slot((i + 1) % N, 0);
         a.clear_ring = i == N - 1;
         LaunchScope ls(c, s, PROF_BLAS, 3.0 * sb * nr);
-        BB_DISPATCH(cfg.sloppy.spinor, cfg.sloppy.compute, b_p_update_kernel);
+        BB_DISPATCH(cfg.sloppy.spinor, b_p_update_kernel, (vh + kBlock * kUSites - 1) / (kBlock * kUSites), kBlock);
     }
 }
 
@@ -386,6 +496,9 @@ hisq_status BatchSession::setup()
     if (!e) e = ws.alloc((size_t)48 * vh, (void **)&ax64);
     if (!e) e = ws.alloc((size_t)48 * vh, (void **)&tmp64);
     if (!e) e = ws.alloc(sizeof(CGState) * nr, (void **)&st);
+    // block sums of a reducing stencil pass and of the residual update, per right-hand side
+    if (!e)
+        e = ws.alloc(sizeof(float2) * nr * ((vh + kMrhsBlock - 1) / kMrhsBlock + r_blocks(vh)), (void **)&sums);
     if (e) return e;
     static_assert(sizeof(CGState) * kMaxRHS <= kPinnedBytes, "a batch's states fit a pinned block");
     sth = (CGState *)pinned_get(c, sizeof(CGState) * nr);

@@ -41,6 +41,7 @@ struct BatchSession {
     char *r_s = nullptr, *ap_s = nullptr, *tmp_s = nullptr, *ring = nullptr;
     double *b64 = nullptr, *x64 = nullptr, *r64 = nullptr, *ax64 = nullptr, *tmp64 = nullptr;
     CGState *st = nullptr, *sth = nullptr;
+    float2 *sums = nullptr;
     GaugeView gv_s{}, gv_d{};
     std::vector<int> mv_hi, ru, k0, occupied, status;
     std::vector<double> bb, stop2, diag;
@@ -73,7 +74,7 @@ struct BatchSession {
 
   private:
     char *slot(int j, int t);
-    void stencil_pass(int parity_out, const char *in, char *out, const char *y, bool red, int slot_i);
+    void stencil_pass(int parity_out, const char *in, char *out, const char *y, bool red);
     void iterate_block();
     void choose_tile();
     hisq_status pull();

@@ -30,6 +30,7 @@
 #include "dslash.cuh"
 #include "finish.cuh"
 #include "internal.h"
+#include "launch.cuh"
 #include "reduce.cuh"
 
 namespace hisq {
@@ -185,13 +186,20 @@ __device__ __forceinline__ void term_mv(V re[3], V im[3], const V ur[9], const V
 // Whether any right-hand side of the tile [t0, t0 + T) is still iterating
 // (solver states present); a tile of stopped or empty slots is skipped.
 template <int T>
-__device__ __forceinline__ bool tile_active(const DslashMArgs &a)
+__device__ __forceinline__ bool tile_active(const DslashMArgs &a, int t0)
 {
     if (a.st == nullptr) return true;
     bool any = false;
 #pragma unroll
-    for (int j = 0; j < T; j++) any = any || *(volatile const int *)&a.st[a.t0 + j].active != 0;
+    for (int j = 0; j < T; j++) any = any || *(volatile const int *)&a.st[t0 + j].active != 0;
     return any;
+}
+
+// The index of the k-th set bit of mask.
+__device__ __forceinline__ int nth_tile(unsigned mask, int k)
+{
+    for (; k > 0; k--) mask &= mask - 1u;
+    return __ffs((int)mask) - 1;
 }
 
 // ---------------------------------------------------------------------------
@@ -280,12 +288,16 @@ __global__ void __launch_bounds__(kMrhsBlock, mrhs_min_blocks(T)) dslash_mrhs_ke
     constexpr int SC = Spinor<SF>::chunks;
     static_assert(!STAGED || SC == 1, "staged tiles take 16-byte spinor records");
     extern __shared__ __align__(16) uint4 stage_smem[];
-    if (a.active_any != nullptr && *(volatile const int *)a.active_any == 0) return;
-    if (!tile_active<T>(a)) return;  // every system of this tile stopped or empty: uniform over the grid
+    pdl_wait();
+    pdl_launch_dependents();
+    // the tiles of one block of sites are neighbours in the launch: their links are read from HBM once
+    const int site_block = (int)blockIdx.x / a.ntiles;
+    const int t0 = T * nth_tile(a.tile_mask, (int)blockIdx.x - site_block * a.ntiles);
+    if (!tile_active<T>(a, t0)) return;  // every system of this tile stopped or empty
     const Geom &g = a.g;
     const int vh = g.vh;
     const int tid = threadIdx.x;
-    const int cb = blockIdx.x * blockDim.x + tid;
+    const int cb = site_block * blockDim.x + tid;
     const int po = a.out_parity;
     const size_t pstride = (size_t)8 * vh * 16;
     constexpr bool kScaled = LinkScaled<GF>::value;
@@ -325,7 +337,7 @@ __global__ void __launch_bounds__(kMrhsBlock, mrhs_min_blocks(T)) dslash_mrhs_ke
 #pragma unroll
                 for (int j = 0; j < T; j++)
                     cp_async_16(slot(stage, kLinkSlots + j),
-                                a.in + (size_t)(a.t0 + j) * a.field_bytes + (size_t)ti.nb * 16);
+                                a.in + (size_t)(t0 + j) * a.field_bytes + (size_t)ti.nb * 16);
             }
         };
         // staged: each term's indices are computed once, when its copies are
@@ -362,7 +374,7 @@ __global__ void __launch_bounds__(kMrhsBlock, mrhs_min_blocks(T)) dslash_mrhs_ke
                         // the xpay records of every right-hand side, in flight during the last term
 #pragma unroll
                         for (int j = 0; j < T; j++)
-                            cp_async_16(slot(0, kLinkSlots + j), a.y + (size_t)(a.t0 + j) * a.field_bytes + (size_t)cb * 16);
+                            cp_async_16(slot(0, kLinkSlots + j), a.y + (size_t)(t0 + j) * a.field_bytes + (size_t)cb * 16);
                     }
                     cp_async_commit();  // possibly empty: keeps one group per term
                     cp_async_wait_1();  // this term's copies have landed (this thread's)
@@ -379,7 +391,7 @@ __global__ void __launch_bounds__(kMrhsBlock, mrhs_min_blocks(T)) dslash_mrhs_ke
                         Link<GF, LREC>::gather(a.gv.lng, pstride, cur.li, lc);
 #pragma unroll
                     for (int j = 0; j < T; j++)
-                        Spinor<SF>::gather(a.in + (size_t)(a.t0 + j) * a.field_bytes, vh, cur.nb, sc + j * SC);
+                        Spinor<SF>::gather(a.in + (size_t)(t0 + j) * a.field_bytes, vh, cur.nb, sc + j * SC);
                 }
 
                 // the link, unscaled (fat) or in units of the fat scale (long)
@@ -434,7 +446,7 @@ __global__ void __launch_bounds__(kMrhsBlock, mrhs_min_blocks(T)) dslash_mrhs_ke
                     if constexpr (STAGED)
                         yc[j] = *slot(0, kLinkSlots + e0 + j);
                     else
-                        Spinor<SF>::gather(a.y + (size_t)(a.t0 + e0 + j) * a.field_bytes, vh, cb, yc + j * SC);
+                        Spinor<SF>::gather(a.y + (size_t)(t0 + e0 + j) * a.field_bytes, vh, cb, yc + j * SC);
                 }
             }
 #pragma unroll
@@ -446,12 +458,12 @@ __global__ void __launch_bounds__(kMrhsBlock, mrhs_min_blocks(T)) dslash_mrhs_ke
                     o[2 * i] = fmul(sf, lane_of(re[gi][i], l));
                     o[2 * i + 1] = fmul(sf, lane_of(im[gi][i], l));
                 }
-                const size_t off = (size_t)(a.t0 + j) * a.field_bytes;
+                const size_t off = (size_t)(t0 + j) * a.field_bytes;
                 if (a.xpay) {
                     float yv[6];
                     Spinor<SF>::decode(yc + (j - e0) * SC, yv);
                     // a solver's per-system coefficient lives in its state (slots change hands)
-                    const float aa = a.st ? (float)a.st[a.t0 + j].diag : (float)a.a[a.t0 + j];
+                    const float aa = a.st ? (float)a.st[t0 + j].diag : (float)a.a[t0 + j];
 #pragma unroll
                     for (int k = 0; k < 6; k++) o[k] = __fmaf_rn(aa, yv[k], o[k]);
                     if constexpr (RED) {
@@ -472,27 +484,10 @@ __global__ void __launch_bounds__(kMrhsBlock, mrhs_min_blocks(T)) dslash_mrhs_ke
         }
     }
 
-    if constexpr (RED) store_block_partial<2 * T, float>(rv, a.red);  // summed by mrhs_finish_kernel
-}
-
-// After a reducing tile launch: one block sums the launch's block partials
-// and runs the finisher of each active right-hand side of the tile.  The
-// same thread count for every tile keeps each right-hand side's summation
-// order, and so its iterates, independent of the tile.
-constexpr int kMrhsFinishThreads = 1024;
-
-template <int T>
-__global__ void __launch_bounds__(kMrhsFinishThreads) mrhs_finish_kernel(const __grid_constant__ DslashMArgs a, unsigned nblocks)
-{
-    if (a.active_any != nullptr && *(volatile const int *)a.active_any == 0) return;
-    if (!tile_active<T>(a)) return;
-    __shared__ double tot[2 * T];
-    sum_partials<2 * T, float>(a.red, nblocks, tot);
-    if (threadIdx.x == 0) {
-#pragma unroll
-        for (int k = 0; k < 2 * T; k++) a.red.result[k] = tot[k];
-        run_batch_finisher(a.fin, tot, a.st, a.t0, T, a.slot);
-    }
+    // block sums, summed by the residual update's blocks: [t0 * blocks + block * T + j]
+    if constexpr (RED)
+        store_partial_at<2 * T, float>(rv, reinterpret_cast<float *>(a.partials + (size_t)t0 * a.nblocks),
+                                       (unsigned)site_block);
 }
 
 template <int GF, int SF, int LREC, int T, bool RED, bool STAGED>
@@ -505,10 +500,7 @@ bool launch_mrhs_kernel(const DslashMArgs &a, cudaStream_t s)
                                cudaSuccess;  // once per kernel
         if (!ok) return false;
     }
-    const int nb = (a.g.vh + kMrhsBlock - 1) / kMrhsBlock;
-    kern<<<nb, kMrhsBlock, smem, s>>>(a);
-    if constexpr (RED) mrhs_finish_kernel<T><<<1, kMrhsFinishThreads, 0, s>>>(a, (unsigned)nb);
-    return true;
+    return launch_chained_smem(kern, dim3(a.nblocks * a.ntiles), dim3(kMrhsBlock), smem, s, a) == cudaSuccess;
 }
 
 template <int GF, int SF, int LREC, bool RED, bool STAGED>
@@ -533,28 +525,24 @@ bool launch_mrhs_variant(int T, int variant, const DslashMArgs &a, cudaStream_t 
     return launch_mrhs_tile<GF, SF, LREC, RED, false>(T, a, s);
 }
 
-// All nrhs right-hand sides in tiles of T (T divides nrhs; one launch per
-// tile); variant 0 the register kernel, 1 the staged one (16-byte records).
+// All nrhs right-hand sides in tiles of T (T divides nrhs), in one launch;
+// variant 0 the register kernel, 1 the staged one (16-byte records).
 template <int GF, int SF, typename real>
 bool launch_mrhs_t(int long_recon, bool reduce, int T, int variant, const DslashMArgs &args, cudaStream_t s)
 {
     static_assert(std::is_same<real, float>::value, "the batched stencil computes in FP32");
     if (long_recon != 12 && long_recon != 18) return false;  // 18- and 12-real long links only
-    if (reduce && !red_fits(args.g.vh, kMrhsBlock, 2 * T)) return false;
-    for (int t0 = 0; t0 < args.nrhs; t0 += T) {
-        if (args.tile_mask != 0u && !((args.tile_mask >> (t0 / T)) & 1u)) continue;  // no system of it iterates
-        DslashMArgs a = args;
-        a.t0 = t0;
-        bool ok;
-        if (long_recon == 12)
-            ok = reduce ? launch_mrhs_variant<GF, SF, 12, true>(T, variant, a, s)
-                        : launch_mrhs_variant<GF, SF, 12, false>(T, variant, a, s);
-        else
-            ok = reduce ? launch_mrhs_variant<GF, SF, 18, true>(T, variant, a, s)
-                        : launch_mrhs_variant<GF, SF, 18, false>(T, variant, a, s);
-        if (!ok) return false;
-    }
-    return true;
+    DslashMArgs a = args;
+    const unsigned every = args.nrhs / T >= 32 ? ~0u : (1u << (args.nrhs / T)) - 1u;
+    a.tile_mask = args.tile_mask != 0u ? args.tile_mask & every : every;  // only tiles with a system that iterates
+    a.ntiles = __builtin_popcount(a.tile_mask);
+    a.nblocks = (a.g.vh + kMrhsBlock - 1) / kMrhsBlock;
+    if (a.ntiles == 0) return true;
+    if (long_recon == 12)
+        return reduce ? launch_mrhs_variant<GF, SF, 12, true>(T, variant, a, s)
+                      : launch_mrhs_variant<GF, SF, 12, false>(T, variant, a, s);
+    return reduce ? launch_mrhs_variant<GF, SF, 18, true>(T, variant, a, s)
+                  : launch_mrhs_variant<GF, SF, 18, false>(T, variant, a, s);
 }
 
 }  // namespace hisq

@@ -186,13 +186,4 @@ __device__ __forceinline__ void run_finisher(int fin, const double *sums, void *
     }
 }
 
-// Batched solver: the CG finisher for each active right-hand side of a tile
-// (stopped right-hand sides keep their state untouched).
-__device__ __forceinline__ void run_batch_finisher(int fin, const double *sums, CGState *st, int t0, int T, int slot)
-{
-    if (st == nullptr) return;
-    for (int j = 0; j < T; j++)
-        if (st[t0 + j].active) run_finisher(fin, sums + 2 * j, &st[t0 + j], slot);
-}
-
 }  // namespace hisq

@@ -280,14 +280,11 @@ struct DslashMArgs {
     int sign;
     int xpay;
     int nrhs;
-    int t0;                 // first right-hand side of the tile (set by the launcher)
     unsigned tile_mask;     // bit k: launch tile k (0: every tile)
-    const int *active_any;  // skip when *active_any == 0 (null: always run)
+    int ntiles, nblocks;    // tiles launched and blocks of sites (set by the launcher)
     int *err;
-    RedBuf red;
-    int fin;
     CGState *st;            // per right-hand side states (st[t])
-    int slot;
+    float2 *partials;       // a reducing pass's block sums, nblocks per right-hand side (see the kernel)
 };
 
 // ---------------------------------------------------------------------------

@@ -28,12 +28,13 @@ __device__ __forceinline__ void pdl_launch_dependents() { asm volatile("griddepc
 // kernel<<<grid, block, 0, s>>>(args...) with programmatic stream
 // serialisation when pdl_mode is on
 template <typename... P, typename... A>
-inline cudaError_t launch_chained(void (*kernel)(P...), dim3 grid, dim3 block, cudaStream_t s, A &&...args)
+inline cudaError_t launch_chained_smem(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s,
+                                       A &&...args)
 {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = grid;
     cfg.blockDim = block;
-    cfg.dynamicSmemBytes = 0;
+    cfg.dynamicSmemBytes = smem;
     cfg.stream = s;
     cudaLaunchAttribute at[1];
     at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -41,6 +42,11 @@ inline cudaError_t launch_chained(void (*kernel)(P...), dim3 grid, dim3 block, c
     cfg.attrs = at;
     cfg.numAttrs = 1;
     return cudaLaunchKernelEx(&cfg, kernel, std::forward<A>(args)...);
+}
+template <typename... P, typename... A>
+inline cudaError_t launch_chained(void (*kernel)(P...), dim3 grid, dim3 block, cudaStream_t s, A &&...args)
+{
+    return launch_chained_smem(kernel, grid, block, 0, s, std::forward<A>(args)...);
 }
 
 }  // namespace hisq

@@ -382,10 +382,9 @@ int wave_blocks(K kernel, int block)
     return (per > 0 ? per : 1) * (sms > 0 ? sms : 1);
 }
 
-// Only this block's share: its sums stored at its index of rb.partials, no
-// completion counter (a separate one-block kernel sums them after the launch).
+// A block's sums stored at row `row` of part.
 template <int NR, typename T>
-__device__ void store_block_partial(const T vin[NR], const RedBuf &rb)
+__device__ __forceinline__ void store_partial_at(const T vin[NR], T *part, unsigned row)
 {
     __shared__ T sh[32][NR];
     T v[NR];
@@ -393,11 +392,17 @@ __device__ void store_block_partial(const T vin[NR], const RedBuf &rb)
     for (int k = 0; k < NR; k++) v[k] = vin[k];
     block_sum<NR, T>(v, sh);
     if (threadIdx.x == 0) {
-        T *part = reinterpret_cast<T *>(rb.partials);
-        const unsigned bid = blockIdx.y * gridDim.x + blockIdx.x;
 #pragma unroll
-        for (int k = 0; k < NR; k++) part[(size_t)bid * NR + k] = v[k];
+        for (int k = 0; k < NR; k++) part[(size_t)row * NR + k] = v[k];
     }
+}
+
+// Only this block's share: its sums stored at its index of rb.partials, no
+// completion counter (a separate one-block kernel sums them after the launch).
+template <int NR, typename T>
+__device__ __forceinline__ void store_block_partial(const T vin[NR], const RedBuf &rb)
+{
+    store_partial_at<NR, T>(vin, reinterpret_cast<T *>(rb.partials), blockIdx.y * gridDim.x + blockIdx.x);
 }
 
 }  // namespace hisq
