@@ -143,7 +143,7 @@ __global__ void __launch_bounds__(kRBlock) b_r_update_kernel(const __grid_consta
         const real alpha = al_sh;
         real v[2] = {0, 0};
         for (; i0 < a.n; i0 += step) {
-            r_group<SF, real>(b, i0, cr, ca, alpha, v);
+            r_group<SF, real>(b, i0, cr, ca, alpha, v, b.v0);
             r_load<SF>(b, i0 + step, cr, ca);
         }
         store_partial_at<2, float>(v, reinterpret_cast<float *>(a.r_sums + (size_t)t * a.nr_blocks), blockIdx.x);

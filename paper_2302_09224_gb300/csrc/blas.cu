@@ -36,23 +36,6 @@ __device__ __forceinline__ bool nonzero(float v) { return v != 0.0f; }
 __device__ __forceinline__ bool nonzero(double v) { return v != 0.0; }
 __device__ __forceinline__ bool nonzero(ff v) { return v.hi != 0.0f || v.lo != 0.0f; }
 
-// A solver scalar (FP64 in the state) in the compute precision.  For FP32
-// pairs the conversion runs on GB300's narrow FP64 pipe, so one thread of the
-// block converts and the block reads the pair from shared memory.  Every
-// thread of the block calls it, at most once per kernel.
-template <typename real>
-__device__ __forceinline__ real block_scalar(const double *src)
-{
-    if constexpr (is_ff<real>::value) {
-        __shared__ ff sh;
-        if (threadIdx.x == 0) sh = ff(*src);
-        __syncthreads();
-        return sh;
-    } else {
-        return (real)*src;
-    }
-}
-
 // Sites per thread of the two per-iteration BLAS kernels: every load of a
 // thread's sites is issued before any of them is used (memory-level
 // parallelism for these short, latency-bound kernels).  Four sites a thread
@@ -74,7 +57,7 @@ __global__ void __launch_bounds__(kBlock) r_update_kernel(BlasArgs a)
     for (int i0 = blockIdx.x * blockDim.x * U + threadIdx.x; i0 < a.n; i0 += gridDim.x * blockDim.x * U) {
         uint4 cr[U][C], ca[U][C];
         r_load<SF>(a, i0, cr, ca);
-        r_group<SF, real>(a, i0, cr, ca, alpha, v);
+        r_group<SF, real>(a, i0, cr, ca, alpha, v, a.v0);
     }
     __shared__ double tot[2];
     if (reduce_grid<2>(v, a.red, tot) && threadIdx.x == 0) {
@@ -114,12 +97,6 @@ __global__ void __launch_bounds__(kBlock) p_update_kernel(BlasArgs a)
 // update, which is then partial; the solver never reads that ring slot before
 // rewriting it (the slot's alpha is zero until then).  Each block's first
 // loads are issued before its partial sums, so the sums overlap them.
-inline __device__ RedBuf split_half(RedBuf rb)
-{
-    rb.partials += kSplitHalf;
-    return rb;
-}
-
 template <int SF, typename real, int BS>
 __global__ void __launch_bounds__(BS) r_update_split_kernel(BlasArgs a)
 {
@@ -147,7 +124,7 @@ __global__ void __launch_bounds__(BS) r_update_split_kernel(BlasArgs a)
         const real alpha = al_sh;
         red_t<real> v[2] = {0, 0};
         for (; i0 < a.n; i0 += step) {
-            r_group<SF, real>(a, i0, cr, ca, alpha, v);
+            r_group<SF, real>(a, i0, cr, ca, alpha, v, a.v0);
             r_load<SF>(a, i0 + step, cr, ca);
         }
         store_block_partial<2>(v, split_half(a.red));

@@ -11,6 +11,31 @@
 
 namespace hisq {
 
+// A solver scalar (FP64 in the state) in the compute precision.  For FP32
+// pairs the conversion runs on GB300's narrow FP64 pipe, so one thread of the
+// block converts and the block reads the pair from shared memory.  Every
+// thread of the block calls it, at most once per kernel.
+template <typename real>
+__device__ __forceinline__ real block_scalar(const double *src)
+{
+    if constexpr (is_ff<real>::value) {
+        __shared__ ff sh;
+        if (threadIdx.x == 0) sh = ff(*src);
+        __syncthreads();
+        return sh;
+    } else {
+        return (real)*src;
+    }
+}
+
+// The partials' second half: the split chain's residual update leaves its block
+// sums there while it reads the stencil pass's from the first.
+inline __device__ RedBuf split_half(RedBuf rb)
+{
+    rb.partials += kSplitHalf;
+    return rb;
+}
+
 // Loads of r (v0) and Ap (v1) at the U sites i0 + u * blockDim.x.
 template <int SF, int U, int C>
 __device__ __forceinline__ void r_load(const BlasArgs &a, int i0, uint4 (&cr)[U][C], uint4 (&ca)[U][C])
@@ -25,10 +50,10 @@ __device__ __forceinline__ void r_load(const BlasArgs &a, int i0, uint4 (&cr)[U]
     }
 }
 
-// r <- r - alpha Ap at those sites, stored; |r_new|^2 and Re<r_new, r_old> added to v.
+// r - alpha Ap at those sites, stored in out (r itself or another field); |r_new|^2 and Re<r_new, r_old> added to v.
 template <int SF, typename real, int U, int C>
 __device__ __forceinline__ void r_group(const BlasArgs &a, int i0, const uint4 (&cr)[U][C], const uint4 (&ca)[U][C],
-                                        real alpha, red_t<real> v[2])
+                                        real alpha, red_t<real> v[2], char *out)
 {
 #pragma unroll
     for (int u = 0; u < U; u++) {
@@ -45,7 +70,7 @@ __device__ __forceinline__ void r_group(const BlasArgs &a, int i0, const uint4 (
 #pragma unroll
             for (int k = 0; k < 6; k++) rn[k] = r[k] - alpha * ap[k];
             uint32_t qn[6], En;
-            if (!Spinor<S_INT30>::store_ff_q(a.v0, a.n, i, rn, qn, En)) atomicExch(a.err, 1);
+            if (!Spinor<S_INT30>::store_ff_q(out, a.n, i, rn, qn, En)) atomicExch(a.err, 1);
             long long n2 = 0, d = 0;
 #pragma unroll
             for (int k = 0; k < 6; k++) {
@@ -68,7 +93,7 @@ __device__ __forceinline__ void r_group(const BlasArgs &a, int i0, const uint4 (
             }
             v[0] += (red_t<real>)n2;
             v[1] += (red_t<real>)d;
-            if (!Spinor<SF>::store(a.v0, a.n, i, rn)) atomicExch(a.err, 1);
+            if (!Spinor<SF>::store(out, a.n, i, rn)) atomicExch(a.err, 1);
         }
     }
 }

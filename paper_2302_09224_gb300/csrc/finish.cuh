@@ -25,6 +25,100 @@ __device__ __forceinline__ void ms_stop(MSState *m, int reason)
 // hep-lat/9612014): r_i = zeta_i r with
 //   zeta_i' = zeta_i zeta_i^- a^- / (a b^- (zeta_i^- - zeta_i) + zeta_i^- a^- (1 + s_i a))
 //   alpha_i = a zeta_i'/zeta_i,  beta_i = b (zeta_i'/zeta_i)^2.
+// One shift's step at alpha = a.
+__device__ __forceinline__ void ms_alpha_shift(MSState *m, int i, double a)
+{
+    if (!m->live[i]) {
+        m->alpha_i[i] = 0.0;
+        return;
+    }
+    const double z = m->zeta[i], zm = m->zeta_prev[i];
+    const double den = a * m->beta_prev * (zm - z) + zm * m->alpha_prev * (1.0 + m->shift[i] * a);
+    const double zn = z * zm * m->alpha_prev / den;
+    if (!isfinite(zn) || zn == 0.0) {  // the shift has converged beyond representability
+        m->live[i] = 0;
+        m->frozen_at[i] = m->k;
+        m->alpha_i[i] = 0.0;
+        return;
+    }
+    m->zeta_new[i] = zn;
+    m->alpha_i[i] = a * zn / z;
+}
+
+// The recurrence's scalars run by one warp, a lane a shift (a thread's loop
+// over twelve shifts' FP64 divisions took 12 us a kernel).  ms_alpha_warp after
+// <p0, A p0> is known.
+static_assert(kMaxShift <= 32, "a lane per shift");
+__device__ __forceinline__ void ms_alpha_warp(MSState *m, double pAp)
+{
+    const int i = threadIdx.x & 31;
+    const double a = m->rr / pAp;
+    if (!(pAp > 0.0) || !isfinite(a)) {
+        if (i == 0) {
+            m->alpha = 0.0;
+            ms_stop(m, REASON_BREAKDOWN);
+        }
+        return;
+    }
+    if (i < m->nshift) ms_alpha_shift(m, i, a);
+    __syncwarp();
+    if (i == 0) {
+        m->pAp = pAp;
+        m->alpha = a;
+    }
+}
+
+// After |r_new|^2 is known: beta, every shift's step recorded in slot j of the
+// ring (applied later by shift_ring_kernel), freezing, and the decisions.
+__device__ __forceinline__ void ms_beta_warp(MSState *m, MSRing *ring, int j, double rr_new)
+{
+    const int i = threadIdx.x & 31;
+    const int ns = m->nshift;
+    const double rr = m->rr, b = rr_new / rr;
+    const bool ok = isfinite(rr_new) && isfinite(b);
+    bool frozen = true;
+    if (ok && i < ns) {
+        if (m->live[i]) {
+            const double q = m->zeta_new[i] / m->zeta[i];
+            m->beta_i[i] = b * q * q;
+            m->zeta_prev[i] = m->zeta[i];
+            m->zeta[i] = m->zeta_new[i];
+            const double zr2 = m->zeta[i] * m->zeta[i] * rr_new;
+            frozen = zr2 <= m->stop2[i];
+            m->freeze_next[i] = frozen;
+        }
+        ring->a[j][i] = m->alpha_i[i];
+        ring->z[j][i] = m->zeta[i];
+        ring->b[j][i] = m->beta_i[i];
+        ring->live[j][i] = m->live[i];
+        // a shift that reached its target takes no part in later iterations
+        if (m->live[i] && m->freeze_next[i] && (i > 0 || ns == 1)) {
+            m->live[i] = 0;
+            m->frozen_at[i] = m->k + 1;
+        }
+    }
+    // the stage ends when every shift but the base (the base, if alone) has stopped
+    const bool all_frozen = __all_sync(0xffffffffu, (i == 0 && ns > 1) || frozen);
+    if (i != 0) return;
+    m->k += 1;
+    ring->n = ok ? j + 1 : j;
+    if (!ok) {
+        ms_stop(m, REASON_BREAKDOWN);
+        return;
+    }
+    m->beta = b;
+    m->alpha_prev = m->alpha;
+    m->beta_prev = b;
+    m->rr_prev = rr;
+    m->rr = rr_new;
+    if (rr_new > m->rr_max) m->rr_max = rr_new;
+    if (all_frozen)
+        ms_stop(m, REASON_CONVERGED);
+    else if (rr_new < m->delta2 * m->rr_max)
+        ms_stop(m, REASON_RELIABLE);
+}
+
+// The scalar recurrence's steps that a reducing kernel's one thread runs.
 __device__ __forceinline__ void run_ms_finisher(int fin, const double *sums, MSState *m)
 {
     if (fin == FIN_MS_ALPHA) {
@@ -37,63 +131,7 @@ __device__ __forceinline__ void run_ms_finisher(int fin, const double *sums, MSS
         }
         m->pAp = pAp;
         m->alpha = a;
-        for (int i = 0; i < m->nshift; i++) {
-            if (!m->live[i]) {
-                m->alpha_i[i] = 0.0;
-                continue;
-            }
-            const double z = m->zeta[i], zm = m->zeta_prev[i];
-            const double den = a * m->beta_prev * (zm - z) + zm * m->alpha_prev * (1.0 + m->shift[i] * a);
-            const double zn = z * zm * m->alpha_prev / den;
-            if (!isfinite(zn) || zn == 0.0) {  // the shift has converged beyond representability
-                m->live[i] = 0;
-                m->frozen_at[i] = m->k;
-                m->alpha_i[i] = 0.0;
-                continue;
-            }
-            m->zeta_new[i] = zn;
-            m->alpha_i[i] = a * zn / z;
-        }
-    } else if (fin == FIN_MS_BETA) {
-        const double rr_new = sums[0];
-        const double b = rr_new / m->rr;
-        m->k += 1;
-        if (!isfinite(rr_new) || !isfinite(b)) {
-            ms_stop(m, REASON_BREAKDOWN);
-            return;
-        }
-        m->beta = b;
-        bool all_frozen = true;
-        for (int i = 0; i < m->nshift; i++) {
-            if (!m->live[i]) continue;
-            const double q = m->zeta_new[i] / m->zeta[i];
-            m->beta_i[i] = b * q * q;
-            m->zeta_prev[i] = m->zeta[i];
-            m->zeta[i] = m->zeta_new[i];
-            const double zr2 = m->zeta[i] * m->zeta[i] * rr_new;
-            m->freeze_next[i] = zr2 <= m->stop2[i];
-            if (i > 0 && !m->freeze_next[i]) all_frozen = false;
-        }
-        if (m->nshift == 1) all_frozen = m->freeze_next[0] != 0;
-        m->alpha_prev = m->alpha;
-        m->beta_prev = b;
-        m->rr_prev = m->rr;
-        m->rr = rr_new;
-        if (rr_new > m->rr_max) m->rr_max = rr_new;
-        if (all_frozen)
-            m->pending = REASON_CONVERGED;
-        else if (rr_new < m->delta2 * m->rr_max)
-            m->pending = REASON_RELIABLE;
-    } else if (fin == FIN_MS_APPLY) {
-        for (int i = 0; i < m->nshift; i++)
-            if (m->live[i] && m->freeze_next[i] && (i > 0 || m->nshift == 1)) {
-                m->live[i] = 0;
-                m->frozen_at[i] = m->k;
-            }
-        if (m->pending != REASON_NONE) {
-            ms_stop(m, m->pending);
-            m->pending = REASON_NONE;
-        }
+        for (int i = 0; i < m->nshift; i++) ms_alpha_shift(m, i, a);
     } else if (fin == FIN_MS_TRUE) {
         m->rr = sums[0];
         m->rr_max = sums[0];

@@ -157,10 +157,18 @@ struct MSState {
     int live[kMaxShift];               // shift still updated
     int freeze_next[kMaxShift];        // freeze after this iteration's update
     int frozen_at[kMaxShift];
+    double rr_den;                     // |r_k|^2 as the residual update read it (beta's denominator)
     int nshift;
-    int active, reason, pending;
+    int active, reason;
     int k;
-    int pad;
+};
+
+// The steps of up to kMaxBuf iterations of the shifted recurrences, not yet
+// applied to the shifts' fields: n iterations of part `part` of a block.
+struct MSRing {
+    double a[kMaxBuf][kMaxShift], z[kMaxBuf][kMaxShift], b[kMaxBuf][kMaxShift];
+    int live[kMaxBuf][kMaxShift];
+    int n, part;
 };
 
 // Finisher selected by a reducing kernel: what the last block does with the
@@ -172,9 +180,7 @@ enum FinOp {
     FIN_CG_TRUE = 3,      // values: |r_hi|^2, Re/Im <r_hi, p>   -> projection, coef, beta
     FIN_STORE = 4,        // copy the sums to RedBuf::result only
     FIN_MS_ALPHA = 5,     // values: Re<p0,Ap0>                  -> alpha, zeta_i', alpha_i
-    FIN_MS_BETA = 6,      // values: |r_new|^2                   -> beta, beta_i, freezing, decisions
-    FIN_MS_TRUE = 7,      // values: |r_hi|^2                    -> restart after a reliable update
-    FIN_MS_APPLY = 8      // no values: apply pending freezes and stop decisions
+    FIN_MS_TRUE = 7       // values: |r_hi|^2                    -> restart after a reliable update
 };
 
 // ---------------------------------------------------------------------------

@@ -2,10 +2,10 @@
 // C-ABI entry point.
 //
 // Stage 1 (sloppy triplet): one base recurrence on A = M_ee + sigma_0 (the
-// smallest shift) with reliable updates on the base system; every shift's
-// solution and gradient vector are updated in one fused kernel per iteration
-// that reads r once (x_i accumulators in the compute precision, flushed into
-// FP64 at each reliable update).  Shift i stops updating once its iterated
+// smallest shift) with reliable updates on the base system; the other shifts'
+// solutions and gradient vectors, which only need the residuals, are brought up
+// to date in one kernel per block of iterations (x_i accumulators in the compute
+// precision, flushed into FP64 at each reliable update).  Shift i stops updating once its iterated
 // residual zeta_i |r| reaches max(tol_i, 10 eps of the sloppy format); the
 // stage ends when every shift other than the base has stopped.
 // Stage 2 (refinement triplet): CG on the base system continuing from its
@@ -18,12 +18,15 @@
 #include <chrono>
 #include <cmath>
 #include <numeric>
+#include <type_traits>
 #include <vector>
 
 #include "blas.h"
+#include "blas_update.cuh"
 #include "cg.h"
 #include "codecs.cuh"
 #include "internal.h"
+#include "launch.cuh"
 #include "reduce.cuh"
 #include "finish.cuh"
 
@@ -32,62 +35,215 @@ namespace hisq {
 struct MSArgs {
     int n;
     int nshift;
-    const char *r;        // sloppy residual
     char *p;              // nshift sloppy fields, p_bytes apart
     size_t p_bytes;
     char *acc;            // nshift accumulator fields (F32 or F64 planar), acc_bytes apart
     size_t acc_bytes;
     double *x64;          // nshift FP64 planar fields, 48*n apart
-    MSState *m;
-    const int *active;
     int *err;
-    RedBuf red;
 };
 
 namespace {
 
 constexpr int kBlock = 256;
 
-// For every live shift: acc_i += alpha_i p_i, p_i = zeta_i r + beta_i p_i.
-template <int SF, typename real>
-__global__ void __launch_bounds__(kBlock) shift_update_kernel(MSArgs a)
+// An iteration of the stage after the two stencil passes: the residual update
+// (every block sums the reducing pass's partials and takes alpha), then the base
+// system's gradient vector and accumulator (every block sums the residual
+// update's partials and takes beta).  The last block of each grid has no sites:
+// its first warp runs the scalar recurrences of all shifts meanwhile.
+struct MSIter {
+    BlasArgs b;      // n, err, red; v0, v1: r and A p, then r and p of the base; nparts
+    char *out;       // the new residual (its own ring slot); then the base's accumulator
+    MSState *m;
+    MSRing *ring;
+    int slot, part;  // the iteration's ring slot, and the part of the block that fills the ring
+};
+
+template <typename real>
+constexpr int ms_block()
 {
-    if (a.active && *(volatile const int *)a.active == 0) return;
-    constexpr int AF = is_ff<real>::value ? S_FF : sizeof(real) == 8 ? S_F64 : S_F32;
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    const MSState *m = a.m;
-    // the shifts' step sizes in the compute precision, converted once per block (for FP32 pairs
-    // the conversion runs on the narrow FP64 pipe)
-    __shared__ real cs[3][kMaxShift];
-    if (threadIdx.x < a.nshift) {
-        cs[0][threadIdx.x] = (real)m->alpha_i[threadIdx.x];
-        cs[1][threadIdx.x] = (real)m->zeta[threadIdx.x];
-        cs[2][threadIdx.x] = (real)m->beta_i[threadIdx.x];
+    return std::is_same<real, float>::value ? 1024 : 512;
+}
+
+template <int SF, typename real>
+__global__ void __launch_bounds__(ms_block<real>()) ms_r_update_kernel(const __grid_constant__ MSIter a)
+{
+    constexpr int BS = ms_block<real>(), U = 2, C = Spinor<SF>::chunks;
+    pdl_wait();
+    pdl_launch_dependents();
+    MSState *m = a.m;
+    if (*(volatile const int *)&m->active == 0) return;
+    const bool scalars = blockIdx.x == gridDim.x - 1;
+    const int step = (int)(gridDim.x - 1) * BS * U;
+    int i0 = scalars ? a.b.n : (int)blockIdx.x * BS * U + (int)threadIdx.x;
+    uint4 cr[U][C], ca[U][C];
+    r_load<SF>(a.b, i0, cr, ca);
+    __shared__ double tot[2];
+    __shared__ real al_sh;
+    __shared__ int ok_sh;
+    if (a.b.nparts > 0) sum_partials<2, part_t<real>>(a.b.red, a.b.nparts, tot);
+    if (scalars) {
+        if (threadIdx.x >= 32) return;
+        __syncwarp();
+        if (threadIdx.x == 0) {
+            m->rr_den = m->rr;
+            if (a.slot == 0) {
+                a.ring->n = 0;
+                a.ring->part = a.part;
+            }
+        }
+        if (a.b.nparts > 0) ms_alpha_warp(m, tot[0]);
+        return;
+    }
+    if (threadIdx.x == 0) {
+        // without partials the pass ran the finisher itself
+        const double al = a.b.nparts > 0 ? m->rr / tot[0] : m->alpha;
+        const bool ok = (a.b.nparts == 0 || tot[0] > 0.0) && isfinite(al);
+        al_sh = ok ? real(al) : real(0);
+        ok_sh = ok;
     }
     __syncthreads();
-    if (i < a.n) {
-        real r[6];
-        Spinor<SF>::load(a.r, a.n, i, r);
-        for (int s = 0; s < a.nshift; s++) {
-            if (!m->live[s]) continue;
+    if (!ok_sh) return;
+    const real alpha = al_sh;
+    red_t<real> v[2] = {0, 0};
+    for (; i0 < a.b.n; i0 += step) {
+        r_group<SF, real>(a.b, i0, cr, ca, alpha, v, a.out);
+        r_load<SF>(a.b, i0 + step, cr, ca);
+    }
+    store_block_partial<2>(v, split_half(a.b.red));
+}
+
+template <int SF, typename real>
+__global__ void __launch_bounds__(kBlock) ms_p_update_kernel(const __grid_constant__ MSIter a)
+{
+    constexpr int C = Spinor<SF>::chunks;
+    constexpr int AF = is_ff<real>::value ? S_FF : sizeof(real) == 8 ? S_F64 : S_F32;
+    pdl_wait();
+    pdl_launch_dependents();
+    MSState *m = a.m;
+    if (*(volatile const int *)&m->active == 0) return;
+    const bool scalars = blockIdx.x == gridDim.x - 1;
+    const int n = a.b.n, i = (int)(blockIdx.x * blockDim.x + threadIdx.x);
+    const bool mine = !scalars && i < n;
+    uint4 cr[C], cp[C], cx[Spinor<AF>::chunks];
+    if (mine) {
+        Spinor<SF>::gather(a.b.v0, n, i, cr);
+        Spinor<SF>::gather(a.b.v1, n, i, cp);
+        Spinor<AF>::gather(a.out, n, i, cx);
+    }
+    __shared__ double tot[2];
+    __shared__ real al_sh, be_sh;
+    __shared__ int ok_sh;
+    warp0_sum_partials<2, part_t<real>>(split_half(a.b.red), a.b.nparts, tot);
+    if (scalars) {
+        if (threadIdx.x >= 32) return;
+        __syncwarp();
+        ms_beta_warp(m, a.ring, a.slot, tot[0]);
+        return;
+    }
+    if (threadIdx.x == 0) {
+        const double be = tot[0] / m->rr_den;
+        ok_sh = isfinite(tot[0]) && isfinite(be);
+        be_sh = real(be);
+        al_sh = real(m->alpha);
+    }
+    __syncthreads();
+    if (!mine || !ok_sh) return;
+    const real al = al_sh, be = be_sh;
+    real r[6], p[6], x[6];
+    Spinor<SF>::decode(cr, r);
+    Spinor<SF>::decode(cp, p);
+    Spinor<AF>::decode(cx, x);
+#pragma unroll
+    for (int k = 0; k < 6; k++) {
+        x[k] += al * p[k];
+        p[k] = r[k] + be * p[k];
+    }
+    if (!Spinor<SF>::store(a.b.v1, n, i, p)) atomicExch(a.b.err, 1);
+    Spinor<AF>::store(a.out, n, i, x);
+}
+
+// The recorded iterations of every shift but the base, whose gradient vectors
+// and accumulators need nothing but the residuals r_1, r_2, ... of the block (kept
+// in a ring): per iteration j in which the shift was live, acc_i += alpha_ij p_i,
+// p_i = zeta_ij r_j + beta_ij p_i.  A shift's fields are read and written once
+// per block of iterations instead of every one (12 shifts at 16^3x32, FP64-class:
+// 36.8 us an iteration before), and p_i stays in the compute precision between
+// the block's iterations.  The last residual goes to r0, where the next part
+// starts.
+template <int SF, typename real>
+__global__ void __launch_bounds__(kBlock) shift_ring_kernel(MSArgs a, const MSRing *ring, int part, char *r0,
+                                                              char *r_ring)
+{
+    pdl_wait();
+    pdl_launch_dependents();
+    if (ring->part != part) return;  // the block stopped before this part (uniform over the grid)
+    constexpr int AF = is_ff<real>::value ? S_FF : sizeof(real) == 8 ? S_F64 : S_F32;
+    // iterations whose residuals a thread holds at once: decoded for FP32, as records otherwise
+    constexpr bool kDecoded = std::is_same<real, float>::value;
+    constexpr int RB = 8, C = Spinor<SF>::chunks;
+    __shared__ real cs[3][kMaxBuf][kMaxShift];
+    __shared__ unsigned live[kMaxBuf];
+    const int n = ring->n;
+    for (int k = threadIdx.x; k < n * kMaxShift; k += blockDim.x) {
+        const int j = k / kMaxShift, s = k % kMaxShift;
+        const bool on = s < a.nshift && ring->live[j][s] != 0;
+        const unsigned bits = __ballot_sync(__activemask(), on);
+        if (s == 0) live[j] = bits;
+        if (on) {
+            cs[0][j][s] = (real)ring->a[j][s];
+            cs[1][j][s] = (real)ring->z[j][s];
+            cs[2][j][s] = (real)ring->b[j][s];
+        }
+    }
+    __syncthreads();
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= a.n || n == 0) return;
+    for (int j0 = 0; j0 < n; j0 += RB) {
+        const int m = n - j0 < RB ? n - j0 : RB;
+        uint4 cr[RB][C];
+        real r[kDecoded ? RB : 1][6];
+        unsigned any = 0;
+#pragma unroll
+        for (int j = 0; j < RB; j++)
+            if (j < m) {
+                Spinor<SF>::gather(r_ring + (size_t)(j0 + j) * a.p_bytes, a.n, i, cr[j]);
+                any |= live[j0 + j];
+            }
+        if (j0 + m == n) {
+#pragma unroll
+            for (int j = 0; j < RB; j++)
+                if (j == m - 1) Spinor<SF>::put(r0, a.n, i, cr[j]);
+        }
+        if constexpr (kDecoded) {
+#pragma unroll
+            for (int j = 0; j < RB; j++)
+                if (j < m) Spinor<SF>::decode(cr[j], r[j]);
+        }
+        for (int s = 1; s < a.nshift; s++) {
+            if (!((any >> s) & 1u)) continue;
             real p[6], x[6];
             char *ps = a.p + (size_t)s * a.p_bytes;
             char *xs = a.acc + (size_t)s * a.acc_bytes;
             Spinor<SF>::load(ps, a.n, i, p);
             Spinor<AF>::load(xs, a.n, i, x);
-            const real al = cs[0][s], z = cs[1][s], be = cs[2][s];
 #pragma unroll
-            for (int k = 0; k < 6; k++) {
-                x[k] += al * p[k];
-                p[k] = z * r[k] + be * p[k];
+            for (int j = 0; j < RB; j++) {
+                if (j >= m || !((live[j0 + j] >> s) & 1u)) continue;
+                const real al = cs[0][j0 + j][s], z = cs[1][j0 + j][s], be = cs[2][j0 + j][s];
+                real rv[6];
+                if constexpr (!kDecoded) Spinor<SF>::decode(cr[j], rv);
+#pragma unroll
+                for (int k = 0; k < 6; k++) {
+                    x[k] += al * p[k];
+                    p[k] = z * (kDecoded ? r[j][k] : rv[k]) + be * p[k];
+                }
             }
             if (!Spinor<SF>::store(ps, a.n, i, p)) atomicExch(a.err, 1);
             Spinor<AF>::store(xs, a.n, i, x);
         }
     }
-    double v[1] = {0.0};
-    __shared__ double tot[1];
-    if (reduce_grid<1>(v, a.red, tot) && threadIdx.x == 0) run_finisher(FIN_MS_APPLY, tot, a.m, 0);
 }
 
 // x64_i += acc_i and acc_i = 0 for every shift.
@@ -180,8 +336,10 @@ struct MSRun {
     char *r_s = nullptr, *w_s = nullptr, *tmp_s = nullptr, *P = nullptr, *ACC = nullptr;
     double *X = nullptr, *r64 = nullptr, *ax64 = nullptr, *tmp64 = nullptr;
     MSState *m = nullptr, *mh = nullptr;
+    MSRing *ring = nullptr;
     GaugeView gv_s{}, gv_d{};
     int ru = 0, mv_hi = 0;
+    int parts = 1;  // iterations whose residuals are kept before the shifts are brought up to date
 
     MSRun(hisq_ctx *c_, hisq_gauge *g_, const hisq_solver_params &p_, cudaStream_t s_)
         : c(c_), g(g_), p(p_), s(s_), ws(c_, s_), vh(g_->geom.vh), ns(0)
@@ -201,15 +359,12 @@ struct MSRun {
         MSArgs a{};
         a.n = vh;
         a.nshift = ns;
-        a.r = r_s;
         a.p = P;
         a.p_bytes = sb;
         a.acc = ACC;
         a.acc_bytes = accb;
         a.x64 = X;
-        a.m = m;
         a.err = cur_err(c);
-        a.red = cur_red(c);
         return a;
     }
 
@@ -256,46 +411,75 @@ struct MSRun {
 
     const double *b64 = nullptr;
 
+    // SF and compute type of the sloppy triplet
+    template <typename F>
+    void dispatch(F f)
+    {
+        const bool f64 = p.sloppy.compute == HISQ_COMPUTE_F64;
+        switch (p.sloppy.spinor) {
+        case S_F64: f(std::integral_constant<int, S_F64>{}, double{}); break;
+        case S_F32: f(std::integral_constant<int, S_F32>{}, float{}); break;
+        case S_HALF: f(std::integral_constant<int, S_HALF>{}, float{}); break;
+        case S_INT20: f(std::integral_constant<int, S_INT20>{}, float{}); break;
+        case S_INT14: f(std::integral_constant<int, S_INT14>{}, float{}); break;
+        case S_INT30:
+            if (f64) f(std::integral_constant<int, S_INT30>{}, ff{});  // FP64-class compute in FP32 pairs
+            else f(std::integral_constant<int, S_INT30>{}, float{});
+            break;
+        }
+    }
+
+    // the residual a part starts from (0) and those of its iterations, in the FP64 work fields
+    char *r_slot(int j) { return j == 0 ? r_s : (char *)r64 + (size_t)(j - 1) * sb; }
+
     void iterate_block(int nit)
     {
         const double diag0 = 4.0 * p.mass * p.mass + sig[0];
         const int *act = &m->active;
         for (int it = 0; it < nit; it++) {
-            apply_mee(c, g->geom, p.sloppy, gv_s, diag0, pf(0), tmp_s, w_s, FIN_MS_ALPHA, m, 0, act, PROF_STENCIL, s);
-            BlasArgs b{};
-            b.n = vh;
-            b.err = cur_err(c);
-            b.red = cur_red(c);
-            b.v0 = r_s;
-            b.v1 = w_s;
-            b.active = act;
-            b.alpha_src = &m->alpha;
-            b.fin = FIN_MS_BETA;
-            b.fst = m;
-            {
-                LaunchScope ls(c, s, PROF_BLAS, 3.0 * spinor_site_bytes(p.sloppy.spinor) * vh);
-                launch_r_update(p.sloppy.spinor, p.sloppy.compute, b, s);
-            }
-            MSArgs a = args();
-            a.active = act;
+            const unsigned np = apply_mee(c, g->geom, p.sloppy, gv_s, diag0, pf(0), tmp_s, w_s, FIN_MS_ALPHA, m, 0, act,
+                                          PROF_STENCIL, s, true);
+            MSIter a{};
+            a.b.n = vh;
+            a.b.err = cur_err(c);
+            a.b.red = cur_red(c);
+            a.m = m;
+            a.ring = ring;
+            a.slot = it % parts;
+            a.part = it / parts;
+            dispatch([&](auto sf, auto rl) {
+                constexpr int SF = decltype(sf)::value;
+                using real = decltype(rl);
+                constexpr int BS = ms_block<real>();
+                static const int wave = wave_blocks(ms_r_update_kernel<SF, real>, BS);
+                const int need = (vh + 2 * BS - 1) / (2 * BS);
+                const int nb = std::max(1, std::min(need, wave - 1));
+                a.b.v0 = r_slot(a.slot);
+                a.b.v1 = w_s;
+                a.out = r_slot(a.slot + 1);
+                a.b.nparts = np;
+                {
+                    LaunchScope ls(c, s, PROF_BLAS, 3.0 * spinor_site_bytes(SF) * vh);
+                    launch_chained(ms_r_update_kernel<SF, real>, dim3(nb + 1), dim3(BS), s, a);
+                }
+                a.b.v0 = r_slot(a.slot + 1);
+                a.b.v1 = pf(0);
+                a.out = ACC;
+                a.b.nparts = nb;
+                LaunchScope ls(c, s, PROF_BLAS, (3.0 * spinor_site_bytes(SF) + 2.0 * spinor_site_bytes(acc_fmt)) * vh);
+                launch_chained(ms_p_update_kernel<SF, real>, dim3(nblk(vh) + 1), dim3(kBlock), s, a);
+            });
+            if (a.slot != parts - 1 && it != nit - 1) continue;
             int live = 0;
-            for (int i = 0; i < ns; i++) live += mh->live[i];
-            LaunchScope ls(c, s, PROF_BLAS,
-                           (spinor_site_bytes(p.sloppy.spinor) +
-                            live * (2.0 * spinor_site_bytes(p.sloppy.spinor) + 2.0 * spinor_site_bytes(acc_fmt))) * vh);
-            const bool f64 = p.sloppy.compute == HISQ_COMPUTE_F64;
-            switch (p.sloppy.spinor) {
-            case S_F64: shift_update_kernel<S_F64, double><<<nblk(vh), kBlock, 0, s>>>(a); break;
-            case S_F32: shift_update_kernel<S_F32, float><<<nblk(vh), kBlock, 0, s>>>(a); break;
-            case S_HALF: shift_update_kernel<S_HALF, float><<<nblk(vh), kBlock, 0, s>>>(a); break;
-            case S_INT20: shift_update_kernel<S_INT20, float><<<nblk(vh), kBlock, 0, s>>>(a); break;
-            case S_INT14: shift_update_kernel<S_INT14, float><<<nblk(vh), kBlock, 0, s>>>(a); break;
-            case S_INT30:
-                if (f64)  // FP64-class compute in FP32 pairs, pair accumulators
-                    shift_update_kernel<S_INT30, ff><<<nblk(vh), kBlock, 0, s>>>(a);
-                else shift_update_kernel<S_INT30, float><<<nblk(vh), kBlock, 0, s>>>(a);
-                break;
-            }
+            for (int i = 1; i < ns; i++) live += mh->live[i];
+            dispatch([&](auto sf, auto rl) {
+                constexpr int SF = decltype(sf)::value;
+                LaunchScope ls(c, s, PROF_BLAS,
+                               ((a.slot + 2.0) * spinor_site_bytes(SF) +
+                                live * 2.0 * (spinor_site_bytes(SF) + spinor_site_bytes(acc_fmt))) * vh);
+                launch_chained(shift_ring_kernel<SF, decltype(rl)>, dim3(nblk(vh)), dim3(kBlock), s, args(),
+                               (const MSRing *)ring, a.part, r_s, (char *)r64);
+            });
         }
     }
 
@@ -313,15 +497,19 @@ struct MSRun {
         acc_fmt = p.sloppy.compute != HISQ_COMPUTE_F64 ? S_F32 : p.sloppy.spinor == S_INT30 ? S_FF : S_F64;
         accb = spinor_field_bytes(acc_fmt, vh);
         const size_t b48 = (size_t)48 * vh;
+        const int N = std::max(1, p.nbuf);
         e = ws.alloc(sb, (void **)&r_s);
+        if (!e) e = ws.alloc(sizeof(MSRing), (void **)&ring);
         if (!e) e = ws.alloc(sb, (void **)&w_s);
         if (!e) e = ws.alloc(sb, (void **)&tmp_s);
         if (!e) e = ws.alloc(sb * ns, (void **)&P);
         if (!e) e = ws.alloc(accb * ns, (void **)&ACC);
         if (!e) e = ws.alloc(b48 * ns, (void **)&X);
-        if (!e) e = ws.alloc(b48, (void **)&r64);
-        if (!e) e = ws.alloc(b48, (void **)&ax64);
-        if (!e) e = ws.alloc(b48, (void **)&tmp64);
+        // true residuals' work fields; between them, a block's residuals (as many as fit)
+        if (!e) e = ws.alloc(3 * b48, (void **)&r64);
+        ax64 = r64 + (size_t)6 * vh;
+        tmp64 = ax64 + (size_t)6 * vh;
+        parts = std::min(N, (int)(3 * b48 / sb));
         if (!e) e = ws.alloc(sizeof(MSState), (void **)&m);
         if (e) return e;
         mh = (MSState *)pinned_get(c, sizeof(MSState));
@@ -370,7 +558,6 @@ struct MSRun {
         *mh = init;
         cudaMemcpyAsync(m, &init, sizeof init, cudaMemcpyHostToDevice, s);
         const bool graph = p.use_graph && !c->prof.on;
-        const int N = std::max(1, p.nbuf);
         cudaGraphExec_t exec = nullptr;
         int64_t nodes = 0;
         hisq_status status = HISQ_OK;
