@@ -6,14 +6,15 @@
 // Vectors r_0..r_l, u_0..u_l and the shadow residual live in the sloppy
 // format; x, b and true residuals in FP64; every scalar (rho, alpha, omega,
 // the Gram-Schmidt coefficients tau, sigma, gamma) is computed on the device
-// by the reducing kernels' finishers, so a cycle is one fixed kernel sequence
-// (captured once as a CUDA graph).  A reliable update (FP64 true residual)
+// by the kernels that use it, so a cycle is one fixed kernel sequence (captured
+// once as a CUDA graph).  A reliable update (FP64 true residual)
 // ends a cycle when |r| has dropped below delta times its maximum since the
 // previous one, or when the iterated residual meets the target.
 #include <cuda_runtime.h>
 
 #include <chrono>
 #include <cmath>
+#include <type_traits>
 #include <vector>
 
 #include "blas.h"
@@ -29,26 +30,31 @@ namespace {
 
 constexpr int kMaxL = 8;
 constexpr int kBlock = 256;
-constexpr int kBSites = 2;  // sites a thread of the reductions loads before using any (in flight together)
+constexpr int kMaxBlocks = 304;   // blocks with sites of the vector kernels (two a SM; more rows cost the next kernel's sums)
+constexpr int kGroup = 4;         // fields of a kind whose loads a thread issues before it stores any
+constexpr int kMaxRows = 4096;    // stencil block sums that the next kernel's blocks sum themselves
 
 struct BState {
-    double rho_re, rho_im;         // rho_0
-    double alpha_re, alpha_im;
-    double omega_re, omega_im;
-    double beta_re, beta_im;
+    double rho_re[kMaxL], rho_im[kMaxL];          // rho_j of the cycle's steps
+    double al_re[kMaxL], al_im[kMaxL];            // alpha_j
+    double rhoc_re, rhoc_im, alc_re, alc_im;      // -omega rho and alpha carried from the previous cycle
+    double dot[3];                                // Re, Im <rt, v> and |v|^2 where they are summed once
     double tau_re[kMaxL + 1][kMaxL + 1], tau_im[kMaxL + 1][kMaxL + 1];
-    double sigma[kMaxL + 1];
     double gp_re[kMaxL + 1], gp_im[kMaxL + 1];    // gamma'
-    double g_re[kMaxL + 1], g_im[kMaxL + 1];      // gamma
-    double gpp_re[kMaxL + 1], gpp_im[kMaxL + 1];  // gamma''
     double rr, rr_max, delta2, stop2, tiny2;
     double rt2;   // |rt|^2 of the shadow residual
     double brk2;  // breakdown when |<rt, v>|^2 <= brk2 |rt|^2 |v|^2
     int active, reason, cycles, l;
 };
 
-enum { OP_RHO = 1, OP_GAMMA = 2, OP_TAU = 3, OP_SIGMA = 4, OP_FINAL = 5 };
-
+// A cycle is a chain of kernels each of which sums its predecessor's block
+// partials itself (every block, one fixed order) and takes its scalars from
+// them, so no completion counter, last-block tail or one-thread launch lies
+// between: u update (beta from <rt, r_j>), M u_j with <rt, u_{j+1}> in its
+// epilogue, r and x update (alpha), M r_j with <rt, r_{j+1}>, the l
+// Gram-Schmidt passes, and the final update.  The last block of each grid has
+// no sites and writes the scalars to the state.  16^3x32 sites, 20-bit: 45
+// launches of about 10 us a cycle before, 21 now.
 struct BArgs {
     int vh;
     size_t hb;               // bytes of one half-lattice sloppy field
@@ -57,8 +63,9 @@ struct BArgs {
     char *U;                 // u_0..u_l
     const char *rt;          // shadow residual
     double *x64;             // FP64 full field (two planar halves, 48*vh bytes each)
-    int j, i;                // step indices
-    int op;
+    int j;                   // step
+    int rows;                // rows of partials to sum; 0: the sums are in the state
+    double *part_in, *part_out;
     BState *b;
     const int *active;
     int *err;
@@ -69,9 +76,9 @@ __device__ __forceinline__ bool skip(const int *active) { return active && *(vol
 
 __device__ __forceinline__ void cdiv(double ar, double ai, double br, double bi, double &qr, double &qi)
 {
-    const double d = br * br + bi * bi;
-    qr = (ar * br + ai * bi) / d;
-    qi = (ai * br - ar * bi) / d;
+    const double d = 1.0 / (br * br + bi * bi);
+    qr = (ar * br + ai * bi) * d;
+    qi = (ai * br - ar * bi) * d;
 }
 
 __device__ void b_stop(BState *b, int reason)
@@ -80,51 +87,487 @@ __device__ void b_stop(BState *b, int reason)
     b->active = 0;
 }
 
-// finishers of the reducing kernels; sums = {Re<x,y>, Im<x,y>, extra}
-__device__ void b_finish(BArgs &a, const double *s)
+// a value in the compute precision as FP64
+__device__ __forceinline__ double widen(float v) { return f2d_bits(v); }
+__device__ __forceinline__ double widen(double v) { return v; }
+
+// site s of the full lattice: half s / vh, index s % vh of it
+struct Site {
+    int h, i;
+};
+__device__ __forceinline__ Site site_of(int s, int vh) { return s < vh ? Site{0, s} : Site{1, s - vh}; }
+
+// The type of the stencil's block partials for spinor format SF with BLAS in `real`.
+template <int SF, typename real>
+using stencil_part_t = std::conditional_t<SF == S_INT30 && std::is_same<real, double>::value, FF, part_t<real>>;
+
+// The three sums of the pass or kernel before: the state's, or summed here (thread 0 of tot).
+template <int SF, typename real>
+__device__ __forceinline__ void dot_sums(const BArgs &a, double *tot)
 {
+    if (a.rows == 0) {
+        if (threadIdx.x < 3) tot[threadIdx.x] = a.b->dot[threadIdx.x];
+        __syncthreads();
+        return;
+    }
+    RedBuf rb{};
+    rb.partials = a.part_in;
+    sum_partials<3, stencil_part_t<SF, real>>(rb, (unsigned)a.rows, tot);
+}
+
+// NR sums over `rows` rows, a warp a value: FP32 rows in FP32 pairs, FP64 rows in FP64; every thread
+// may read tot afterwards.
+template <int NR, typename real>
+__device__ __forceinline__ void sum_rows(const real *part, int rows, double *tot)
+{
+    constexpr int U = 5;
+    const int lane = threadIdx.x & 31;
+    for (int v = threadIdx.x >> 5; v < NR; v += kBlock / 32) {
+        if constexpr (std::is_same<real, double>::value) {
+            double w[1] = {0.0};
+            for (int r = lane; r < rows; r += 32) w[0] += __ldcg(part + (size_t)r * NR + v);
+            warp_sum<1, double>(w);
+            if (lane == 0) tot[v] = w[0];
+        } else {
+            FF w[1] = {{0.0f, 0.0f}};
+            for (int r0 = lane; r0 < rows; r0 += 32 * U) {
+                float t[U];
+#pragma unroll
+                for (int u = 0; u < U; u++) t[u] = r0 + 32 * u < rows ? __ldcg(part + (size_t)(r0 + 32 * u) * NR + v) : 0.0f;
+#pragma unroll
+                for (int u = 0; u < U; u++) w[0] = ff_add(w[0], FF{t[u], 0.0f});
+            }
+            warp_sum_ff<1>(w);
+            if (lane == 0) tot[v] = (double)w[0].hi + (double)w[0].lo;
+        }
+    }
+    __syncthreads();
+}
+
+// one site's <x, y> = conj(x) y and |y|^2 added to v
+template <typename real>
+__device__ __forceinline__ void dot_site(const real x[6], const real y[6], real v[3])
+{
+#pragma unroll
+    for (int c = 0; c < 3; c++) {
+        const real xr = x[2 * c], xi = x[2 * c + 1], yr = y[2 * c], yi = y[2 * c + 1];
+        v[0] += xr * yr + xi * yi;
+        v[1] += xr * yi - xi * yr;
+        v[2] += yr * yr + yi * yi;
+    }
+}
+
+// The dot sums of many rows once, into the state (one block): a large lattice's stencil pass, whose rows
+// every block of the next kernel would read.
+template <typename T>
+__global__ void __launch_bounds__(1024) dot_rows_kernel(BArgs a)
+{
+    pdl_wait();
+    pdl_launch_dependents();
+    if (skip(a.active)) return;
+    __shared__ double tot[3];
+    RedBuf rb{};
+    rb.partials = a.part_in;
+    sum_partials<3, T>(rb, (unsigned)a.rows, tot);
+    if (threadIdx.x == 0)
+        for (int k = 0; k < 3; k++) a.b->dot[k] = tot[k];
+}
+
+// <rt, v> and |v|^2 over the full lattice, into the state: r_0 at a start or restart, and the stencil's
+// output where its block sums would not fit their buffer
+template <int SF, typename real>
+__global__ void __launch_bounds__(kBlock) dot_kernel(BArgs a, const char *v)
+{
+    pdl_wait();
+    pdl_launch_dependents();
+    if (skip(a.active)) return;
+    real s3[3] = {0, 0, 0};
+    for (int s = blockIdx.x * blockDim.x + threadIdx.x; s < 2 * a.vh; s += gridDim.x * blockDim.x) {
+        const Site q = site_of(s, a.vh);
+        real x[6], y[6];
+        Spinor<SF>::load(a.rt + q.h * a.hb, a.vh, q.i, x);
+        Spinor<SF>::load(v + q.h * a.hb, a.vh, q.i, y);
+        dot_site(x, y, s3);
+    }
+    __shared__ double tot[3];
+    if (reduce_grid<3>(s3, a.red, tot) && threadIdx.x == 0)
+        for (int k = 0; k < 3; k++) a.b->dot[k] = tot[k];
+}
+
+// u_i = r_i - beta u_i, i = 0..j, with rho1 = <rt, r_j>, beta = alpha rho1 / rho0.
+// Breakdown: rho1 (nearly) orthogonal relative to |rt| |r_j|, or a rho0 too small to divide by.
+template <int SF, typename real>
+__global__ void __launch_bounds__(kBlock) u_multi_kernel(BArgs a)
+{
+    pdl_wait();
+    pdl_launch_dependents();
+    if (skip(a.active)) return;
+    __shared__ double tot[3];
+    __shared__ real be_sh[2];
+    __shared__ int ok_sh;
+    dot_sums<SF, real>(a, tot);
+    if (threadIdx.x == 0) {
+        BState *b = a.b;
+        const int j = a.j;
+        const double pr = j ? b->rho_re[j - 1] : b->rhoc_re, pi = j ? b->rho_im[j - 1] : b->rhoc_im;
+        const double lr = j ? b->al_re[j - 1] : b->alc_re, li = j ? b->al_im[j - 1] : b->alc_im;
+        const double n2 = tot[0] * tot[0] + tot[1] * tot[1];
+        const bool ok = pr * pr + pi * pi > b->tiny2 && !(tot[2] > 0.0 && !(n2 > b->brk2 * b->rt2 * tot[2])) &&
+                        isfinite(n2);
+        if (blockIdx.x == gridDim.x - 1) {
+            if (ok) {
+                b->rho_re[j] = tot[0];
+                b->rho_im[j] = tot[1];
+            } else {
+                b_stop(b, REASON_BREAKDOWN);
+            }
+        }
+        double qr = 0.0, qi = 0.0;
+        if (ok) cdiv(tot[0], tot[1], pr, pi, qr, qi);
+        be_sh[0] = (real)(lr * qr - li * qi);
+        be_sh[1] = (real)(lr * qi + li * qr);
+        ok_sh = ok;
+    }
+    __syncthreads();
+    if (!ok_sh || blockIdx.x == gridDim.x - 1) return;
+    const real br = be_sh[0], bi = be_sh[1];
+    constexpr int G = kGroup, C = Spinor<SF>::chunks;
+    for (int s = blockIdx.x * blockDim.x + threadIdx.x; s < 2 * a.vh; s += (gridDim.x - 1) * blockDim.x) {
+        const Site q = site_of(s, a.vh);
+        const char *rf = a.R + q.h * a.hb;
+        char *uf = a.U + q.h * a.hb;
+        for (int i0 = 0; i0 <= a.j; i0 += G) {
+            uint4 cr[G][C], cu[G][C];
+#pragma unroll
+            for (int g = 0; g < G; g++)
+                if (i0 + g <= a.j) {
+                    Spinor<SF>::gather(rf + (i0 + g) * a.fb, a.vh, q.i, cr[g]);
+                    Spinor<SF>::gather(uf + (i0 + g) * a.fb, a.vh, q.i, cu[g]);
+                }
+#pragma unroll
+            for (int g = 0; g < G; g++) {
+                if (i0 + g > a.j) continue;
+                real r[6], u[6];
+                Spinor<SF>::decode(cr[g], r);
+                Spinor<SF>::decode(cu[g], u);
+#pragma unroll
+                for (int c = 0; c < 3; c++) {
+                    const real ur = u[2 * c], ui = u[2 * c + 1];
+                    u[2 * c] = r[2 * c] - (br * ur - bi * ui);
+                    u[2 * c + 1] = r[2 * c + 1] - (br * ui + bi * ur);
+                }
+                if (!Spinor<SF>::store(uf + (i0 + g) * a.fb, a.vh, q.i, u)) atomicExch(a.err, 1);
+            }
+        }
+    }
+}
+
+// r_i -= alpha u_{i+1}, i = 0..j; x += alpha u_0 (FP64), with gamma = <rt, u_{j+1}>, alpha = rho / gamma;
+// breakdown relative to |rt| |u_{j+1}|
+template <int SF, typename real>
+__global__ void __launch_bounds__(kBlock) r_multi_kernel(BArgs a)
+{
+    pdl_wait();
+    pdl_launch_dependents();
+    if (skip(a.active)) return;
+    __shared__ double tot[3];
+    __shared__ real al_sh[2];
+    __shared__ int ok_sh;
+    dot_sums<SF, real>(a, tot);
+    if (threadIdx.x == 0) {
+        BState *b = a.b;
+        const double n2 = tot[0] * tot[0] + tot[1] * tot[1];
+        const bool ok = !(n2 <= b->tiny2) && n2 > b->brk2 * b->rt2 * tot[2] && isfinite(tot[0]) && isfinite(tot[1]);
+        double qr = 0.0, qi = 0.0;
+        if (ok) cdiv(b->rho_re[a.j], b->rho_im[a.j], tot[0], tot[1], qr, qi);
+        if (blockIdx.x == gridDim.x - 1) {
+            if (ok) {
+                b->al_re[a.j] = qr;
+                b->al_im[a.j] = qi;
+            } else {
+                b_stop(b, REASON_BREAKDOWN);
+            }
+        }
+        al_sh[0] = (real)qr;
+        al_sh[1] = (real)qi;
+        ok_sh = ok;
+    }
+    __syncthreads();
+    if (!ok_sh || blockIdx.x == gridDim.x - 1) return;
+    const real ar = al_sh[0], ai = al_sh[1];
+    constexpr int G = kGroup, C = Spinor<SF>::chunks;
+    for (int s = blockIdx.x * blockDim.x + threadIdx.x; s < 2 * a.vh; s += (gridDim.x - 1) * blockDim.x) {
+        const Site q = site_of(s, a.vh);
+        // x += alpha u_0: the increment in the compute precision, the sum in FP64
+        real u0[6];
+        uint4 cx[Spinor<S_F64>::chunks];
+        char *xf = reinterpret_cast<char *>(a.x64) + q.h * (size_t)48 * a.vh;
+        Spinor<SF>::load(a.U + q.h * a.hb, a.vh, q.i, u0);
+        Spinor<S_F64>::gather(xf, a.vh, q.i, cx);
+        char *rf = a.R + q.h * a.hb;
+        const char *uf = a.U + a.fb + q.h * a.hb;
+        for (int i0 = 0; i0 <= a.j; i0 += G) {
+            uint4 cr[G][C], cu[G][C];
+#pragma unroll
+            for (int g = 0; g < G; g++)
+                if (i0 + g <= a.j) {
+                    Spinor<SF>::gather(uf + (i0 + g) * a.fb, a.vh, q.i, cu[g]);
+                    Spinor<SF>::gather(rf + (i0 + g) * a.fb, a.vh, q.i, cr[g]);
+                }
+#pragma unroll
+            for (int g = 0; g < G; g++) {
+                if (i0 + g > a.j) continue;
+                real u[6], r[6];
+                Spinor<SF>::decode(cu[g], u);
+                Spinor<SF>::decode(cr[g], r);
+#pragma unroll
+                for (int c = 0; c < 3; c++) {
+                    const real ur = u[2 * c], ui = u[2 * c + 1];
+                    r[2 * c] -= ar * ur - ai * ui;
+                    r[2 * c + 1] -= ar * ui + ai * ur;
+                }
+                if (!Spinor<SF>::store(rf + (i0 + g) * a.fb, a.vh, q.i, r)) atomicExch(a.err, 1);
+            }
+        }
+        double x[6];
+        Spinor<S_F64>::decode(cx, x);
+#pragma unroll
+        for (int c = 0; c < 3; c++) {
+            x[2 * c] += widen(ar * u0[2 * c] - ai * u0[2 * c + 1]);
+            x[2 * c + 1] += widen(ar * u0[2 * c + 1] + ai * u0[2 * c]);
+        }
+        Spinor<S_F64>::store(xf, a.vh, q.i, x);
+    }
+}
+
+// The most vectors after r_k that pass k's kernel is compiled for.
+__host__ __device__ constexpr int mgs_nj(int rest) { return rest == 0 ? 0 : rest == 1 ? 1 : rest <= 3 ? 3 : 7; }
+
+// The sums that pass k - 1 of l left.
+template <typename real>
+__device__ __forceinline__ void sum_prev(const BArgs &a, int k, int l, double *tot)
+{
+    const real *part = reinterpret_cast<const real *>(a.part_in);
+    switch (mgs_nj(l - k + 1)) {
+    case 1: sum_rows<5, real>(part, a.rows, tot); break;
+    case 3: sum_rows<9, real>(part, a.rows, tot); break;
+    default: sum_rows<17, real>(part, a.rows, tot); break;
+    }
+}
+
+// Gram-Schmidt pass k = a.j of r_1..r_l, modified in the right-looking order:
+// r_i -= tau_{k-1,i} r_{k-1} for i = k..l (k >= 2), each r_i thus projected
+// against r_1, r_2, ... one after another as the left-looking order does, then
+// the sums of sigma_k = |r_k|^2, <r_k, r_0> and <r_k, r_i>, i > k: l passes
+// over the vectors instead of l (l + 1) / 2 (16^3x32, l = 4: ten of 9.9 us).
+// NJ: the most vectors after r_k.
+template <int SF, typename real, int NJ>
+__global__ void __launch_bounds__(kBlock) mgs_kernel(BArgs a)
+{
+    constexpr int NR = 3 + 2 * NJ, C = Spinor<SF>::chunks;
+    pdl_wait();
+    pdl_launch_dependents();
+    if (skip(a.active)) return;
     BState *b = a.b;
-    if (a.op == OP_RHO) {
-        // rho1 = <rt, r_j>; beta = alpha rho1 / rho0; rho0 = rho1.  Breakdown:
-        // rho1 (nearly) orthogonal relative to |rt| |r_j| (sums[2] = |r_j|^2),
-        // or a rho0 too small to divide by
-        const double n2 = s[0] * s[0] + s[1] * s[1];
-        if (b->rho_re * b->rho_re + b->rho_im * b->rho_im <= b->tiny2 ||
-            (s[2] > 0.0 && !(n2 > b->brk2 * b->rt2 * s[2])) || !isfinite(n2)) {
-            b_stop(b, REASON_BREAKDOWN);
-            return;
+    const int k = a.j, rest = b->l - k;  // vectors after r_k
+    const bool scalars = blockIdx.x == gridDim.x - 1;
+    __shared__ double tot[3 + 2 * kMaxL];
+    __shared__ real tau[2 * (NJ + 1)];
+    __shared__ int ok_sh;
+    if (k >= 2) {
+        // the previous pass left 3 + 2 * (its NJ) values a row; tau_{k-1,i} = <r_{k-1}, r_i> / sigma_{k-1}
+        sum_prev<real>(a, k, b->l, tot);
+        const double sg = tot[0];
+        const bool ok = sg > 0.0 && isfinite(sg);
+        if (threadIdx.x <= rest) {
+            const int i = threadIdx.x;  // r_{k+i}
+            const double inv = ok ? 1.0 / sg : 0.0, tr = tot[3 + 2 * i] * inv, ti = tot[4 + 2 * i] * inv;
+            tau[2 * i] = (real)tr;
+            tau[2 * i + 1] = (real)ti;
+            if (scalars) {
+                b->tau_re[k - 1][k + i] = tr;
+                b->tau_im[k - 1][k + i] = ti;
+                if (i == 0) {
+                    b->gp_re[k - 1] = tot[1] * inv;
+                    b->gp_im[k - 1] = tot[2] * inv;
+                    if (!ok) b_stop(b, REASON_BREAKDOWN);
+                }
+            }
         }
-        double qr, qi;
-        cdiv(s[0], s[1], b->rho_re, b->rho_im, qr, qi);
-        b->beta_re = b->alpha_re * qr - b->alpha_im * qi;
-        b->beta_im = b->alpha_re * qi + b->alpha_im * qr;
-        b->rho_re = s[0];
-        b->rho_im = s[1];
-    } else if (a.op == OP_GAMMA) {
-        // gamma = <rt, u_{j+1}>; alpha = rho0 / gamma; breakdown relative to |rt| |u_{j+1}|
-        const double n2 = s[0] * s[0] + s[1] * s[1];
-        if (n2 <= b->tiny2 || !(n2 > b->brk2 * b->rt2 * s[2]) || !isfinite(s[0]) || !isfinite(s[1])) {
-            b_stop(b, REASON_BREAKDOWN);
-            return;
+        if (threadIdx.x == 0) ok_sh = ok;
+        __syncthreads();
+        if (!ok_sh) return;
+    }
+    if (scalars) return;
+    real v[NR];
+#pragma unroll
+    for (int q = 0; q < NR; q++) v[q] = 0;
+    for (int s = blockIdx.x * blockDim.x + threadIdx.x; s < 2 * a.vh; s += (gridDim.x - 1) * blockDim.x) {
+        const Site q = site_of(s, a.vh);
+        auto field = [&](int i) { return a.R + i * a.fb + q.h * a.hb; };
+        uint4 c0[C], cp[C], cr[NJ + 1][C];
+        Spinor<SF>::gather(field(0), a.vh, q.i, c0);
+        if (k >= 2) Spinor<SF>::gather(field(k - 1), a.vh, q.i, cp);
+#pragma unroll
+        for (int i = 0; i <= NJ; i++)
+            if (i <= rest) Spinor<SF>::gather(field(k + i), a.vh, q.i, cr[i]);
+        real r0[6], rp[6], rk[6];
+        Spinor<SF>::decode(c0, r0);
+        if (k >= 2) Spinor<SF>::decode(cp, rp);
+#pragma unroll
+        for (int i = 0; i <= NJ; i++) {
+            if (i > rest) continue;
+            real r[6];
+            Spinor<SF>::decode(cr[i], r);
+            if (k >= 2) {
+                const real tr = tau[2 * i], ti = tau[2 * i + 1];
+#pragma unroll
+                for (int c = 0; c < 3; c++) {
+                    const real pr = rp[2 * c], pi = rp[2 * c + 1];
+                    r[2 * c] -= tr * pr - ti * pi;
+                    r[2 * c + 1] -= tr * pi + ti * pr;
+                }
+                if (!Spinor<SF>::store(field(k + i), a.vh, q.i, r)) atomicExch(a.err, 1);
+            }
+            if (i == 0) {
+                real w[3] = {0, 0, 0};
+                dot_site(r, r0, w);
+                v[1] += w[0];
+                v[2] += w[1];
+                real n2 = 0;
+#pragma unroll
+                for (int c = 0; c < 6; c++) {
+                    rk[c] = r[c];
+                    n2 += r[c] * r[c];
+                }
+                v[0] += n2;
+            } else {
+                real w[3] = {0, 0, 0};
+                dot_site(rk, r, w);
+                v[1 + 2 * i] += w[0];
+                v[2 + 2 * i] += w[1];
+            }
         }
-        cdiv(b->rho_re, b->rho_im, s[0], s[1], b->alpha_re, b->alpha_im);
-    } else if (a.op == OP_TAU) {
-        // tau_ij = <r_i, r_j> / sigma_i
-        b->tau_re[a.i][a.j] = s[0] / b->sigma[a.i];
-        b->tau_im[a.i][a.j] = s[1] / b->sigma[a.i];
-    } else if (a.op == OP_SIGMA) {
-        // sums = {Re<r_j, r_0>, Im<r_j, r_0>, |r_j|^2}: sigma_j, gamma'_j
-        const double sg = s[2];
-        if (!(sg > 0.0) || !isfinite(sg)) {
-            b_stop(b, REASON_BREAKDOWN);
-            return;
+    }
+    store_partial_at<NR, real>(v, reinterpret_cast<real *>(a.part_out), blockIdx.x);
+}
+
+// x += gamma_1 r_0 + sum gamma''_j r_j;  r_0 -= gamma'_l r_l + sum gamma'_j r_j;
+// u_0 -= gamma_l u_l + sum gamma_j u_j; then <rt, r_0>, |r_0|^2 and the cycle's decisions, with
+// gamma_l = gamma'_l, omega = gamma_l; gamma_j = gamma'_j - sum_{i>j} tau_ji gamma_i;
+// gamma''_j = gamma_{j+1} + sum_{i=j+1}^{l-1} tau_ji gamma_{i+1}
+template <int SF, typename real>
+__global__ void __launch_bounds__(kBlock) final_kernel(BArgs a)
+{
+    pdl_wait();
+    pdl_launch_dependents();
+    if (skip(a.active)) return;
+    BState *b = a.b;
+    const int l = b->l;
+    __shared__ double tot[3];
+    __shared__ double g_re[kMaxL + 1], g_im[kMaxL + 1];
+    __shared__ real g[kMaxL + 1][2], gp[kMaxL + 1][2], gpp[kMaxL + 1][2];
+    __shared__ int ok_sh;
+    sum_rows<3, real>(reinterpret_cast<const real *>(a.part_in), a.rows, tot);
+    if (threadIdx.x == 0) {
+        const double sg = tot[0];
+        const bool ok = sg > 0.0 && isfinite(sg);
+        ok_sh = ok;
+        const double gr = ok ? tot[1] / sg : 0.0, gi = ok ? tot[2] / sg : 0.0;
+        g_re[l] = gr;
+        g_im[l] = gi;
+        for (int j = l - 1; j >= 1; j--) {
+            double sr = b->gp_re[j], si = b->gp_im[j];
+            for (int i = j + 1; i <= l; i++) {
+                sr -= b->tau_re[j][i] * g_re[i] - b->tau_im[j][i] * g_im[i];
+                si -= b->tau_re[j][i] * g_im[i] + b->tau_im[j][i] * g_re[i];
+            }
+            g_re[j] = sr;
+            g_im[j] = si;
         }
-        b->sigma[a.j] = sg;
-        b->gp_re[a.j] = s[0] / sg;
-        b->gp_im[a.j] = s[1] / sg;
-    } else if (a.op == OP_FINAL) {
-        // sums = {|r_0|^2}
-        const double rr = s[0];
+        for (int j = 1; j <= l; j++) {
+            g[j][0] = (real)g_re[j];
+            g[j][1] = (real)g_im[j];
+            gp[j][0] = (real)(j < l ? b->gp_re[j] : gr);
+            gp[j][1] = (real)(j < l ? b->gp_im[j] : gi);
+            if (j == l) continue;
+            double sr = g_re[j + 1], si = g_im[j + 1];
+            for (int i = j + 1; i <= l - 1; i++) {
+                sr += b->tau_re[j][i] * g_re[i + 1] - b->tau_im[j][i] * g_im[i + 1];
+                si += b->tau_re[j][i] * g_im[i + 1] + b->tau_im[j][i] * g_re[i + 1];
+            }
+            gpp[j][0] = (real)sr;
+            gpp[j][1] = (real)si;
+        }
+        if (!ok && blockIdx.x == 0) b_stop(b, REASON_BREAKDOWN);
+    }
+    __syncthreads();
+    if (!ok_sh) return;
+    real v[3] = {0, 0, 0};
+    for (int s = blockIdx.x * blockDim.x + threadIdx.x; s < 2 * a.vh; s += gridDim.x * blockDim.x) {
+        const Site q = site_of(s, a.vh);
+        // updates in the compute precision; x's increment is added in FP64
+        real dx[6] = {0, 0, 0, 0, 0, 0}, r0[6], u0[6], t[6];
+        char *xf = reinterpret_cast<char *>(a.x64) + q.h * (size_t)48 * a.vh;
+        char *r0f = a.R + q.h * a.hb, *u0f = a.U + q.h * a.hb;
+        uint4 cx[Spinor<S_F64>::chunks];
+        constexpr int G = kGroup - 1, C = Spinor<SF>::chunks;  // l - 1 = 3 fields of a kind at the usual l = 4
+        uint4 ct[C];
+        Spinor<S_F64>::gather(xf, a.vh, q.i, cx);
+        Spinor<SF>::gather(a.rt + q.h * a.hb, a.vh, q.i, ct);
+        Spinor<SF>::load(r0f, a.vh, q.i, r0);
+        Spinor<SF>::load(u0f, a.vh, q.i, u0);
+        auto cax = [](real *y, const real *c2, const real *z, real sgn) {
+            const real c_r = c2[0] * sgn, c_i = c2[1] * sgn;
+#pragma unroll
+            for (int c = 0; c < 3; c++) {
+                y[2 * c] += c_r * z[2 * c] - c_i * z[2 * c + 1];
+                y[2 * c + 1] += c_r * z[2 * c + 1] + c_i * z[2 * c];
+            }
+        };
+        cax(dx, g[1], r0, real(1));
+        Spinor<SF>::load(a.R + l * a.fb + q.h * a.hb, a.vh, q.i, t);
+        cax(r0, gp[l], t, real(-1));
+        Spinor<SF>::load(a.U + l * a.fb + q.h * a.hb, a.vh, q.i, t);
+        cax(u0, g[l], t, real(-1));
+        for (int j0 = 1; j0 <= l - 1; j0 += G) {
+            uint4 cr[G][C], cu[G][C];
+#pragma unroll
+            for (int w = 0; w < G; w++)
+                if (j0 + w <= l - 1) {
+                    Spinor<SF>::gather(u0f + (j0 + w) * a.fb, a.vh, q.i, cu[w]);
+                    Spinor<SF>::gather(r0f + (j0 + w) * a.fb, a.vh, q.i, cr[w]);
+                }
+#pragma unroll
+            for (int w = 0; w < G; w++) {
+                const int j = j0 + w;
+                if (j > l - 1) continue;
+                Spinor<SF>::decode(cu[w], t);
+                cax(u0, g[j], t, real(-1));
+                Spinor<SF>::decode(cr[w], t);
+                cax(dx, gpp[j], t, real(1));
+                cax(r0, gp[j], t, real(-1));
+            }
+        }
+        real rt[6];
+        Spinor<SF>::decode(ct, rt);
+        double x[6];
+        Spinor<S_F64>::decode(cx, x);
+#pragma unroll
+        for (int k = 0; k < 6; k++) x[k] += widen(dx[k]);
+        Spinor<S_F64>::store(xf, a.vh, q.i, x);
+        if (!Spinor<SF>::store(r0f, a.vh, q.i, r0)) atomicExch(a.err, 1);
+        if (!Spinor<SF>::store(u0f, a.vh, q.i, u0)) atomicExch(a.err, 1);
+        dot_site(rt, r0, v);
+    }
+    if (reduce_grid<3>(v, a.red, tot) && threadIdx.x == 0) {
+        for (int k = 0; k < 3; k++) b->dot[k] = tot[k];
+        // the next cycle's rho_0 starts from -omega rho
+        const double rr = tot[2], lr = b->rho_re[l - 1], li = b->rho_im[l - 1];
+        b->rhoc_re = -(g_re[l] * lr - g_im[l] * li);
+        b->rhoc_im = -(g_re[l] * li + g_im[l] * lr);
+        b->alc_re = b->al_re[l - 1];
+        b->alc_im = b->al_im[l - 1];
         b->rr = rr;
         b->cycles += 1;
         if (!isfinite(rr)) {
@@ -139,276 +582,6 @@ __device__ void b_finish(BArgs &a, const double *s)
     }
 }
 
-// a field of the full lattice = two half-lattice fields; blockIdx.y = parity
-__device__ __forceinline__ const char *half(const char *f, size_t hb) { return f + blockIdx.y * hb; }
-__device__ __forceinline__ char *half(char *f, size_t hb) { return f + blockIdx.y * hb; }
-
-// rho_0 <- -omega rho_0 (start of a cycle)
-__global__ void cycle_start_kernel(BState *b, const int *active)
-{
-    pdl_wait();
-    pdl_launch_dependents();
-    if (skip(active)) return;
-    const double r = -(b->omega_re * b->rho_re - b->omega_im * b->rho_im);
-    const double i = -(b->omega_re * b->rho_im + b->omega_im * b->rho_re);
-    b->rho_re = r;
-    b->rho_im = i;
-}
-
-// <x, y> = sum conj(x) y over the full lattice (+ |y|^2), then the finisher
-template <int SF, typename real>
-__global__ void __launch_bounds__(kBlock) dot_kernel(BArgs a, const char *x, const char *y)
-{
-    pdl_wait();
-    pdl_launch_dependents();
-    if (skip(a.active)) return;
-    constexpr int U = kBSites, C = Spinor<SF>::chunks;
-    const char *xf = half(x, a.hb), *yf = half(y, a.hb);
-    real v[3] = {0, 0, 0};
-    for (int s0 = blockIdx.x * blockDim.x * U + threadIdx.x; s0 < a.vh; s0 += gridDim.x * blockDim.x * U) {
-        uint4 cx[U][C], cy[U][C];
-#pragma unroll
-        for (int u = 0; u < U; u++) {
-            const int s = s0 + u * blockDim.x;
-            if (s < a.vh) {
-                Spinor<SF>::gather(xf, a.vh, s, cx[u]);
-                Spinor<SF>::gather(yf, a.vh, s, cy[u]);
-            }
-        }
-#pragma unroll
-        for (int u = 0; u < U; u++) {
-            if (s0 + u * (int)blockDim.x >= a.vh) continue;
-            real xv[6], yv[6];
-            Spinor<SF>::decode(cx[u], xv);
-            Spinor<SF>::decode(cy[u], yv);
-            real d0 = 0, d1 = 0, d2 = 0;  // one site in the compute precision (see reduce_grid)
-#pragma unroll
-            for (int c = 0; c < 3; c++) {
-                const real xr = xv[2 * c], xi = xv[2 * c + 1], yr = yv[2 * c], yi = yv[2 * c + 1];
-                d0 += xr * yr + xi * yi;
-                d1 += xr * yi - xi * yr;
-                d2 += yr * yr + yi * yi;
-            }
-            v[0] += d0;
-            v[1] += d1;
-            v[2] += d2;
-        }
-    }
-    __shared__ double tot[3];
-    if (reduce_grid<3>(v, a.red, tot) && threadIdx.x == 0) b_finish(a, tot);
-}
-
-// u_i = r_i - beta u_i, i = 0..j
-template <int SF, typename real>
-__global__ void __launch_bounds__(kBlock) u_multi_kernel(BArgs a)
-{
-    pdl_wait();
-    pdl_launch_dependents();
-    if (skip(a.active)) return;
-    const real br = (real)a.b->beta_re, bi = (real)a.b->beta_im;
-    for (int s = blockIdx.x * blockDim.x + threadIdx.x; s < a.vh; s += gridDim.x * blockDim.x)
-    for (int i = 0; i <= a.j; i++) {
-        real r[6], u[6];
-        Spinor<SF>::load(half(a.R + i * a.fb, a.hb), a.vh, s, r);
-        char *uf = half(a.U + i * a.fb, a.hb);
-        Spinor<SF>::load(uf, a.vh, s, u);
-#pragma unroll
-        for (int c = 0; c < 3; c++) {
-            const real ur = u[2 * c], ui = u[2 * c + 1];
-            u[2 * c] = r[2 * c] - (br * ur - bi * ui);
-            u[2 * c + 1] = r[2 * c + 1] - (br * ui + bi * ur);
-        }
-        if (!Spinor<SF>::store(uf, a.vh, s, u)) atomicExch(a.err, 1);
-    }
-}
-
-// r_i -= alpha u_{i+1}, i = 0..j; x += alpha u_0 (FP64)
-template <int SF, typename real>
-__global__ void __launch_bounds__(kBlock) r_multi_kernel(BArgs a)
-{
-    pdl_wait();
-    pdl_launch_dependents();
-    if (skip(a.active)) return;
-    const real ar = (real)a.b->alpha_re, ai = (real)a.b->alpha_im;
-    for (int s = blockIdx.x * blockDim.x + threadIdx.x; s < a.vh; s += gridDim.x * blockDim.x) {
-    for (int i = 0; i <= a.j; i++) {
-        real u[6], r[6];
-        Spinor<SF>::load(half(a.U + (i + 1) * a.fb, a.hb), a.vh, s, u);
-        char *rf = half(a.R + i * a.fb, a.hb);
-        Spinor<SF>::load(rf, a.vh, s, r);
-#pragma unroll
-        for (int c = 0; c < 3; c++) {
-            const real ur = u[2 * c], ui = u[2 * c + 1];
-            r[2 * c] -= ar * ur - ai * ui;
-            r[2 * c + 1] -= ar * ui + ai * ur;
-        }
-        if (!Spinor<SF>::store(rf, a.vh, s, r)) atomicExch(a.err, 1);
-    }
-    // x += alpha u_0: the increment in the compute precision, the sum in FP64
-    real u0[6];
-    double x[6];
-    Spinor<SF>::load(half(a.U, a.hb), a.vh, s, u0);
-    char *xf = reinterpret_cast<char *>(a.x64) + blockIdx.y * (size_t)48 * a.vh;
-    Spinor<S_F64>::load(xf, a.vh, s, x);
-#pragma unroll
-    for (int c = 0; c < 3; c++) {
-        x[2 * c] += (double)(ar * u0[2 * c] - ai * u0[2 * c + 1]);
-        x[2 * c + 1] += (double)(ar * u0[2 * c + 1] + ai * u0[2 * c]);
-    }
-    Spinor<S_F64>::store(xf, a.vh, s, x);
-    }
-}
-
-// Modified Gram-Schmidt step (j, i): r_j -= tau_{i-1,j} r_{i-1} (i >= 2), then
-// tau_ij = <r_i, r_j>/sigma_i (i < j) or sigma_j, gamma'_j (i == j).
-template <int SF, typename real>
-__global__ void __launch_bounds__(kBlock) mgs_kernel(BArgs a)
-{
-    pdl_wait();
-    pdl_launch_dependents();
-    if (skip(a.active)) return;
-    constexpr int U = kBSites, C = Spinor<SF>::chunks;
-    char *rjf = half(a.R + a.j * a.fb, a.hb);
-    const char *rpf = half(a.R + (a.i >= 2 ? a.i - 1 : 0) * a.fb, a.hb);
-    const int other = a.i < a.j ? a.i : 0;  // <r_i, r_j>, or <r_j, r_0> at i == j
-    const char *rof = half(a.R + other * a.fb, a.hb);  // never r_j or r_{i-1}: read before r_j is stored
-    const real tr = a.i >= 2 ? (real)a.b->tau_re[a.i - 1][a.j] : real(0);
-    const real ti = a.i >= 2 ? (real)a.b->tau_im[a.i - 1][a.j] : real(0);
-    real v[3] = {0, 0, 0};
-    for (int s0 = blockIdx.x * blockDim.x * U + threadIdx.x; s0 < a.vh; s0 += gridDim.x * blockDim.x * U) {
-        uint4 cj[U][C], cp[U][C], co[U][C];
-#pragma unroll
-        for (int u = 0; u < U; u++) {
-            const int s = s0 + u * blockDim.x;
-            if (s < a.vh) {
-                Spinor<SF>::gather(rjf, a.vh, s, cj[u]);
-                if (a.i >= 2) Spinor<SF>::gather(rpf, a.vh, s, cp[u]);
-                Spinor<SF>::gather(rof, a.vh, s, co[u]);
-            }
-        }
-#pragma unroll
-        for (int u = 0; u < U; u++) {
-        const int s = s0 + u * blockDim.x;
-        if (s >= a.vh) continue;
-        real rj[6], ri[6];
-        Spinor<SF>::decode(cj[u], rj);
-        if (a.i >= 2) {
-            real rp[6];
-            Spinor<SF>::decode(cp[u], rp);
-#pragma unroll
-            for (int c = 0; c < 3; c++) {
-                const real pr = rp[2 * c], pi = rp[2 * c + 1];
-                rj[2 * c] -= tr * pr - ti * pi;
-                rj[2 * c + 1] -= tr * pi + ti * pr;
-            }
-            if (!Spinor<SF>::store(rjf, a.vh, s, rj)) atomicExch(a.err, 1);
-        }
-        Spinor<SF>::decode(co[u], ri);
-        real d0 = 0, d1 = 0, d2 = 0;
-#pragma unroll
-        for (int c = 0; c < 3; c++) {
-            const real jr = rj[2 * c], ji = rj[2 * c + 1], or_ = ri[2 * c], oi = ri[2 * c + 1];
-            if (a.i < a.j) {  // conj(r_i) r_j
-                d0 += or_ * jr + oi * ji;
-                d1 += or_ * ji - oi * jr;
-            } else {          // conj(r_j) r_0
-                d0 += jr * or_ + ji * oi;
-                d1 += jr * oi - ji * or_;
-            }
-            d2 += jr * jr + ji * ji;
-        }
-        v[0] += d0;
-        v[1] += d1;
-        v[2] += d2;
-        }
-    }
-    __shared__ double tot[3];
-    if (reduce_grid<3>(v, a.red, tot) && threadIdx.x == 0) b_finish(a, tot);
-}
-
-// gamma_l = gamma'_l, omega = gamma_l; gamma_j = gamma'_j - sum_{i>j} tau_ji gamma_i;
-// gamma''_j = gamma_{j+1} + sum_{i=j+1}^{l-1} tau_ji gamma_{i+1}
-__global__ void gamma_kernel(BState *b, const int *active)
-{
-    pdl_wait();
-    pdl_launch_dependents();
-    if (skip(active)) return;
-    const int l = b->l;
-    b->g_re[l] = b->gp_re[l];
-    b->g_im[l] = b->gp_im[l];
-    b->omega_re = b->g_re[l];
-    b->omega_im = b->g_im[l];
-    for (int j = l - 1; j >= 1; j--) {
-        double sr = 0, si = 0;
-        for (int i = j + 1; i <= l; i++) {
-            sr += b->tau_re[j][i] * b->g_re[i] - b->tau_im[j][i] * b->g_im[i];
-            si += b->tau_re[j][i] * b->g_im[i] + b->tau_im[j][i] * b->g_re[i];
-        }
-        b->g_re[j] = b->gp_re[j] - sr;
-        b->g_im[j] = b->gp_im[j] - si;
-    }
-    for (int j = 1; j <= l - 1; j++) {
-        double sr = 0, si = 0;
-        for (int i = j + 1; i <= l - 1; i++) {
-            sr += b->tau_re[j][i] * b->g_re[i + 1] - b->tau_im[j][i] * b->g_im[i + 1];
-            si += b->tau_re[j][i] * b->g_im[i + 1] + b->tau_im[j][i] * b->g_re[i + 1];
-        }
-        b->gpp_re[j] = b->g_re[j + 1] + sr;
-        b->gpp_im[j] = b->g_im[j + 1] + si;
-    }
-}
-
-// x += gamma_1 r_0 + sum gamma''_j r_j;  r_0 -= gamma'_l r_l + sum gamma'_j r_j;
-// u_0 -= gamma_l u_l + sum gamma_j u_j;  |r_0|^2 -> OP_FINAL
-template <int SF, typename real>
-__global__ void __launch_bounds__(kBlock) final_kernel(BArgs a)
-{
-    pdl_wait();
-    pdl_launch_dependents();
-    if (skip(a.active)) return;
-    const BState *b = a.b;
-    const int l = b->l;
-    real v[1] = {0};
-    for (int s = blockIdx.x * blockDim.x + threadIdx.x; s < a.vh; s += gridDim.x * blockDim.x) {
-        // updates in the compute precision; x's increment is added in FP64
-        real dx[6] = {0, 0, 0, 0, 0, 0}, r0[6], u0[6], t[6];
-        char *xf = reinterpret_cast<char *>(a.x64) + blockIdx.y * (size_t)48 * a.vh;
-        char *r0f = half(a.R, a.hb), *u0f = half(a.U, a.hb);
-        Spinor<SF>::load(r0f, a.vh, s, r0);
-        Spinor<SF>::load(u0f, a.vh, s, u0);
-        auto cax = [](real *y, double cr, double ci, const real *z, real sgn) {
-            const real c_r = (real)cr * sgn, c_i = (real)ci * sgn;
-            for (int c = 0; c < 3; c++) {
-                y[2 * c] += c_r * z[2 * c] - c_i * z[2 * c + 1];
-                y[2 * c + 1] += c_r * z[2 * c + 1] + c_i * z[2 * c];
-            }
-        };
-        cax(dx, b->g_re[1], b->g_im[1], r0, real(1));
-        Spinor<SF>::load(half(a.R + l * a.fb, a.hb), a.vh, s, t);
-        cax(r0, b->gp_re[l], b->gp_im[l], t, real(-1));
-        Spinor<SF>::load(half(a.U + l * a.fb, a.hb), a.vh, s, t);
-        cax(u0, b->g_re[l], b->g_im[l], t, real(-1));
-        for (int j = 1; j <= l - 1; j++) {
-            Spinor<SF>::load(half(a.U + j * a.fb, a.hb), a.vh, s, t);
-            cax(u0, b->g_re[j], b->g_im[j], t, real(-1));
-            Spinor<SF>::load(half(a.R + j * a.fb, a.hb), a.vh, s, t);
-            cax(dx, b->gpp_re[j], b->gpp_im[j], t, real(1));
-            cax(r0, b->gp_re[j], b->gp_im[j], t, real(-1));
-        }
-        double x[6];
-        Spinor<S_F64>::load(xf, a.vh, s, x);
-        for (int k = 0; k < 6; k++) x[k] += (double)dx[k];
-        Spinor<S_F64>::store(xf, a.vh, s, x);
-        if (!Spinor<SF>::store(r0f, a.vh, s, r0)) atomicExch(a.err, 1);
-        if (!Spinor<SF>::store(u0f, a.vh, s, u0)) atomicExch(a.err, 1);
-        real n2 = 0;
-        for (int k = 0; k < 6; k++) n2 += r0[k] * r0[k];
-        v[0] += n2;
-    }
-    __shared__ double tot[1];
-    if (reduce_grid<1>(v, a.red, tot) && threadIdx.x == 0) b_finish(a, tot);
-}
-
 // after a reliable update: rr = |r_hi|^2 (sums[0]) and iterate again
 __global__ void restart_kernel(BState *b, const double *sum)
 {
@@ -421,44 +594,30 @@ __global__ void restart_kernel(BState *b, const double *sum)
     if (!b->active) b->reason = REASON_BREAKDOWN;
 }
 
-// Two rows (parities) of blocks that loop over their parity's sites: one wave
-// at kernel K's occupancy (at most 4 blocks per SM per row), so that the end
-// of a reducing block is paid once per resident block and no partial second
-// wave trails the first (at 47 registers, five blocks fit a SM, not eight).
-template <auto K>
-dim3 grid2(int vh)
+// Blocks with sites of a vector kernel over the full lattice.
+int vec_blocks(int vh)
 {
-    static const int per_row = [] {
-        int dev = 0, n = 0, occ = 0;
-        cudaGetDevice(&dev);
-        cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev);
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, K, kBlock, 0);
-        const int per_sm = occ < 1 ? 1 : occ > 8 ? 8 : occ;
-        const int rows_total = (n > 0 ? n : 1) * per_sm;
-        return rows_total / 2 > 0 ? rows_total / 2 : 1;
-    }();
-    const int need = (vh + kBlock - 1) / kBlock;
-    return dim3(need < per_row ? need : per_row, 2);
+    const int need = (2 * vh + kBlock - 1) / kBlock;
+    return need < kMaxBlocks ? need : kMaxBlocks;
 }
 
-// KERNEL<spinor format, compute type> over both parities of vh sites each.
-#define B_LAUNCH(KERNEL, SF, REAL, VH, ...) \
-    launch_chained(KERNEL<SF, REAL>, grid2<&KERNEL<SF, REAL>>(VH), dim3(kBlock), st, __VA_ARGS__)
-#define B_DISPATCH(SF_, CF_, KERNEL, VH, ...)                                               \
-    do {                                                                                    \
-        const bool f64_ = (CF_) == HISQ_COMPUTE_F64;                                        \
-        switch (SF_) {                                                                      \
-        case S_F64: B_LAUNCH(KERNEL, S_F64, double, VH, __VA_ARGS__); break;                \
-        case S_F32: B_LAUNCH(KERNEL, S_F32, float, VH, __VA_ARGS__); break;                 \
-        case S_HALF: B_LAUNCH(KERNEL, S_HALF, float, VH, __VA_ARGS__); break;               \
-        case S_INT20: B_LAUNCH(KERNEL, S_INT20, float, VH, __VA_ARGS__); break;             \
-        case S_INT14: B_LAUNCH(KERNEL, S_INT14, float, VH, __VA_ARGS__); break;             \
-        case S_INT30:                                                                       \
-            if (f64_) B_LAUNCH(KERNEL, S_INT30, double, VH, __VA_ARGS__);                   \
-            else B_LAUNCH(KERNEL, S_INT30, float, VH, __VA_ARGS__);                         \
-            break;                                                                          \
-        }                                                                                   \
-    } while (0)
+// f(integral_constant<spinor format>, a value of the compute type)
+template <typename F>
+void b_dispatch(const hisq_prec &p, F f)
+{
+    const bool f64 = p.compute == HISQ_COMPUTE_F64;
+    switch (p.spinor) {
+    case S_F64: f(std::integral_constant<int, S_F64>{}, double{}); break;
+    case S_F32: f(std::integral_constant<int, S_F32>{}, float{}); break;
+    case S_HALF: f(std::integral_constant<int, S_HALF>{}, float{}); break;
+    case S_INT20: f(std::integral_constant<int, S_INT20>{}, float{}); break;
+    case S_INT14: f(std::integral_constant<int, S_INT14>{}, float{}); break;
+    case S_INT30:
+        if (f64) f(std::integral_constant<int, S_INT30>{}, double{});
+        else f(std::integral_constant<int, S_INT30>{}, float{});
+        break;
+    }
+}
 
 struct BRun {
     hisq_ctx *c;
@@ -527,56 +686,110 @@ struct BRun {
         }
     }
 
-    void dot(const char *x, const char *y, int op, int j, int i)
+    // <rt, v> and |v|^2 into the state
+    void dot_to_state(const char *v, const int *act)
     {
         BArgs a = args();
-        a.op = op;
-        a.j = j;
-        a.i = i;
+        a.active = act;
         LaunchScope ls(c, st, PROF_BLAS, 2.0 * sbytes());
-        B_DISPATCH(p.sloppy.spinor, p.sloppy.compute, dot_kernel, vh, a, x, y);
+        b_dispatch(p.sloppy, [&](auto sf, auto rl) {
+            launch_chained(dot_kernel<decltype(sf)::value, decltype(rl)>, dim3(vec_blocks(vh)), dim3(kBlock), st, a, v);
+        });
+    }
+
+    // out = M in with <rt, out> and |out|^2; returns the rows of partials left at red.partials (0: the sums are
+    // in the state)
+    int mfull_dot(const char *in, char *out)
+    {
+        const int rows = dslash_full_rows(p.sloppy.gauge, vh);
+        const size_t row_bytes = 3 * (p.sloppy.compute == HISQ_COMPUTE_F64 ? 8 : 4);
+        const bool fits = rows * row_bytes <= kSplitHalf * sizeof(double);
+        DslashArgs d{};
+        d.g = g->geom;
+        d.gv = gv_s;
+        d.err = cur_err(c);
+        d.red = cur_red(c);
+        if (!fits) d.red.partials = nullptr;
+        d.active = &b->active;
+        d.in = in;
+        d.out = out;
+        d.y = in;
+        d.a = 2.0 * p.mass;
+        d.sign = 1;
+        d.xpay = 1;
+        d.half_bytes = hb;
+        d.dot = rt;
+        {
+            LaunchScope ls(c, st, PROF_STENCIL, 2.0 * stencil_bytes(p.sloppy, vh, true));
+            launch_dslash(p.sloppy.gauge, p.sloppy.spinor, p.sloppy.compute, p.sloppy.long_recon, false, d, st);
+        }
+        if (!fits) {
+            dot_to_state(out, &b->active);
+            return 0;
+        }
+        if (rows <= kMaxRows) return rows;
+        BArgs a = args();
+        a.rows = rows;
+        a.part_in = cur_red(c).partials;
+        LaunchScope ls(c, st, PROF_BLAS, 0.0);
+        if (p.sloppy.compute != HISQ_COMPUTE_F64)
+            launch_chained(dot_rows_kernel<float>, dim3(1), dim3(1024), st, a);
+        else if (p.sloppy.spinor == S_F64)
+            launch_chained(dot_rows_kernel<double>, dim3(1), dim3(1024), st, a);
+        else
+            launch_chained(dot_rows_kernel<FF>, dim3(1), dim3(1024), st, a);
+        return 0;
     }
 
     void cycle()
     {
-        const int *act = &b->active;
-        {
-            LaunchScope ls(c, st, PROF_BLAS, 0.0);
-            launch_chained(cycle_start_kernel, dim3(1), dim3(1), st, b, act);
-        }
+        const int nb = vec_blocks(vh);
+        double *half[2] = {cur_red(c).partials, cur_red(c).partials + kSplitHalf};
+        int rows = 0;  // <rt, r_0> is in the state
         for (int j = 0; j < l; j++) {
-            dot(rt, R + j * fb, OP_RHO, j, 0);
             BArgs a = args();
             a.j = j;
-            {
+            a.rows = rows;
+            a.part_in = half[0];
+            b_dispatch(p.sloppy, [&](auto sf, auto rl) {
                 LaunchScope ls(c, st, PROF_BLAS, 3.0 * (j + 1) * sbytes());
-                B_DISPATCH(p.sloppy.spinor, p.sloppy.compute, u_multi_kernel, vh, a);
-            }
-            mfull(p.sloppy, gv_s, U + j * fb, U + (j + 1) * fb, hb, act, PROF_STENCIL);
-            dot(rt, U + (j + 1) * fb, OP_GAMMA, j, 0);
-            {
+                launch_chained(u_multi_kernel<decltype(sf)::value, decltype(rl)>, dim3(nb + 1), dim3(kBlock), st, a);
+            });
+            a.rows = mfull_dot(U + j * fb, U + (j + 1) * fb);
+            b_dispatch(p.sloppy, [&](auto sf, auto rl) {
                 LaunchScope ls(c, st, PROF_BLAS, (3.0 * (j + 1) + 1) * sbytes() + 96.0 * 2 * vh);
-                B_DISPATCH(p.sloppy.spinor, p.sloppy.compute, r_multi_kernel, vh, a);
-            }
-            mfull(p.sloppy, gv_s, R + j * fb, R + (j + 1) * fb, hb, act, PROF_STENCIL);
+                launch_chained(r_multi_kernel<decltype(sf)::value, decltype(rl)>, dim3(nb + 1), dim3(kBlock), st, a);
+            });
+            rows = mfull_dot(R + j * fb, R + (j + 1) * fb);
         }
-        for (int j = 1; j <= l; j++)
-            for (int i = 1; i <= j; i++) {
-                BArgs a = args();
-                a.j = j;
-                a.i = i;
-                a.op = i < j ? OP_TAU : OP_SIGMA;
-                LaunchScope ls(c, st, PROF_BLAS, (i >= 2 ? 4.0 : 2.0) * sbytes());
-                B_DISPATCH(p.sloppy.spinor, p.sloppy.compute, mgs_kernel, vh, a);
-            }
-        {
-            LaunchScope ls(c, st, PROF_BLAS, 0.0);
-            launch_chained(gamma_kernel, dim3(1), dim3(1), st, b, act);
+        for (int k = 1; k <= l; k++) {
+            BArgs a = args();
+            a.j = k;
+            a.rows = nb;
+            a.part_in = half[(k - 1) & 1];
+            a.part_out = half[k & 1];
+            b_dispatch(p.sloppy, [&](auto sf, auto rl) {
+                constexpr int SF = decltype(sf)::value;
+                using real = decltype(rl);
+                LaunchScope ls(c, st, PROF_BLAS, ((l - k + 2.0) + (k >= 2 ? l - k + 2.0 : 0.0)) * sbytes());
+                const dim3 grid(nb + 1), block(kBlock);
+                switch (mgs_nj(l - k)) {
+                case 0: launch_chained(mgs_kernel<SF, real, 0>, grid, block, st, a); break;
+                case 1: launch_chained(mgs_kernel<SF, real, 1>, grid, block, st, a); break;
+                case 3: launch_chained(mgs_kernel<SF, real, 3>, grid, block, st, a); break;
+                default: launch_chained(mgs_kernel<SF, real, 7>, grid, block, st, a); break;
+                }
+            });
         }
         BArgs a = args();
-        a.op = OP_FINAL;
-        LaunchScope ls(c, st, PROF_BLAS, (2.0 * l + 4.0) * sbytes() + 96.0 * 2 * vh);
-        B_DISPATCH(p.sloppy.spinor, p.sloppy.compute, final_kernel, vh, a);
+        a.rows = nb;
+        a.part_in = half[l & 1];
+        // the final update's own sums go to the other half
+        a.red.partials = half[(l + 1) & 1];
+        b_dispatch(p.sloppy, [&](auto sf, auto rl) {
+            LaunchScope ls(c, st, PROF_BLAS, (2.0 * l + 5.0) * sbytes() + 96.0 * 2 * vh);
+            launch_chained(final_kernel<decltype(sf)::value, decltype(rl)>, dim3(nb), dim3(kBlock), st, a);
+        });
     }
 
     hisq_status pull()
@@ -669,8 +882,7 @@ struct BRun {
         if (e) return e;
         cudaMemcpyAsync(rt, R, fb, cudaMemcpyDeviceToDevice, st);
         BState init{};
-        init.rho_re = 1.0;
-        init.omega_re = 1.0;
+        init.rhoc_re = -1.0;  // rho = omega = 1
         init.rr = rr;
         init.rr_max = rr;
         init.delta2 = p.delta * p.delta;
@@ -682,6 +894,7 @@ struct BRun {
         init.l = l;
         *bh = init;
         cudaMemcpyAsync(b, &init, sizeof init, cudaMemcpyHostToDevice, st);
+        dot_to_state(R, nullptr);
         hisq_status status = HISQ_OK;
         bool done = rr <= init.stop2;
         const bool graph = p.use_graph && !c->prof.on;
@@ -731,6 +944,7 @@ struct BRun {
                     cudaMemcpyAsync(cur_red(c).result, &rr, sizeof rr, cudaMemcpyHostToDevice, st);
                     launch_chained(restart_kernel, dim3(1), dim3(1), st, b, (const double *)cur_red(c).result);
                 }
+                dot_to_state(R, nullptr);
                 e = pull();
                 if (e) break;
                 done = rr <= init.stop2;

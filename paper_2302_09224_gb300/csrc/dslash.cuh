@@ -721,6 +721,46 @@ __global__ void __launch_bounds__(stencil_block(CFG), stencil_minb(CFG))
     if (i0 < vh) warp_store_sites(out64, i0, vh, v, sh[threadIdx.x >> 5]);
 }
 
+// Both parities in one launch, out = a y + sign D in, with the block sums of
+// <dot, out> and |out|^2 (BiCGStab(l)'s next scalars; a pass of their own over
+// the two fields took 10 to 20 us).  On a small lattice one launch of both
+// parities also fills the chip better than two of one.
+template <int GF, int SF, typename real, int LREC, int CFG>
+__global__ void __launch_bounds__(stencil_block(CFG), stencil_minb(CFG))
+    dslash_full_dot_kernel(const __grid_constant__ DslashArgs a)
+{
+    pdl_wait();
+    pdl_launch_dependents();
+    if (a.active != nullptr && *(volatile const int *)a.active == 0) return;  // uniform over the grid
+    const int vh = a.g.vh;
+    const size_t pstride = (size_t)8 * vh * 16;
+    constexpr bool kScaled = LinkScaled<GF>::value;
+    const real fsc = kScaled ? (sizeof(real) == 8 ? (real)a.gv.fat_scale_d : (real)a.gv.fat_scale_f) : real(1);
+    const real lsc = kScaled ? (sizeof(real) == 8 ? (real)a.gv.lng_scale_d : (real)a.gv.lng_scale_f) : real(1);
+    const real ratio = lsc / fsc;
+    const int cb = blockIdx.x * blockDim.x + threadIdx.x;
+    const StencilIO io = stencil_io_full(a);
+    red_t<real> v[3] = {real(0), real(0), real(0)};
+    if (cb < vh) {
+        real o[6], t[6];
+        stencil_value<GF, SF, real, LREC, CFG>(a, io.in, io.po, cb, pstride, fsc, lsc, ratio, o);
+        Spinor<SF>::load(io.y, vh, cb, t);
+        const real aa = (real)a.a;
+#pragma unroll
+        for (int k = 0; k < 6; k++) o[k] = aa * t[k] + o[k];
+        if (!Spinor<SF>::store(io.out, vh, cb, o)) atomicExch(a.err, 1);
+        Spinor<SF>::load(a.dot + (io.po ? a.half_bytes : 0), vh, cb, t);
+#pragma unroll
+        for (int c = 0; c < 3; c++) {
+            const real xr = t[2 * c], xi = t[2 * c + 1], yr = o[2 * c], yi = o[2 * c + 1];
+            v[0] += xr * yr + xi * yi;
+            v[1] += xr * yi - xi * yr;
+            v[2] += yr * yr + yi * yi;
+        }
+    }
+    if (a.red.partials != nullptr) store_block_partial<3>(v, a.red);
+}
+
 // After a reducing pass: one block sums the pass's block partials and runs the
 // solver's finisher (a separate launch instead of a completion counter in
 // every block of the pass: no fence or atomic ends a stencil block).
@@ -782,6 +822,11 @@ void launch_any(int cfg, const DslashArgs &a, cudaStream_t s)
     if constexpr (!RED) {
         if (a.out64 != nullptr) {
             launch_out<GF, SF, real, LREC>(cfg, a, s);
+            return;
+        }
+        if (a.dot != nullptr) {  // the 64-register unrolled shape, the plain passes' usual choice
+            const int B = stencil_threads(4, GF, 2 * a.g.vh);
+            launch_chained(dslash_full_dot_kernel<GF, SF, real, LREC, 4>, dim3((a.g.vh + B - 1) / B, 2), dim3(B), s, a);
             return;
         }
     }

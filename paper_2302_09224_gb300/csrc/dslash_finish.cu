@@ -12,6 +12,12 @@ unsigned dslash_partials(int gf, int sf, int cf, int long_recon, const Geom &g)
     return (unsigned)((g.vh + b - 1) / b);
 }
 
+int dslash_full_rows(int gf, int vh)
+{
+    const int b = stencil_threads(4, gf, 2 * vh);
+    return 2 * ((vh + b - 1) / b);
+}
+
 bool launch_dslash_finish(int gf, int sf, int cf, int long_recon, const DslashArgs &a, cudaStream_t s)
 {
     const unsigned nb = dslash_partials(gf, sf, cf, long_recon, a.g);

@@ -231,8 +231,13 @@ struct DslashArgs {
     // [site][6]; nothing is written when *bad != 0 (device int); err may be host-mapped
     double *out64;
     const int *bad;
-    size_t half_bytes;      // with out64, non-zero: both parities, the odd half this far after the even
+    size_t half_bytes;      // non-zero (with out64 or dot): both parities, the odd half this far after the even
+    // both parities to out, with block partials of <dot, out> (Re, Im) and |out|^2 (none when
+    // red.partials is null): rows of dslash_full_rows
+    const char *dot;
 };
+// Blocks of the pass over both parities with dot.
+int dslash_full_rows(int gf, int vh);
 
 // The fused M_ee pass (d1: D_oe into tmp; d2: D_eo from tmp with xpay and the
 // reduction), scheduled in t-slices through red.sync.
