@@ -18,6 +18,7 @@
 #include <cmath>
 #include <map>
 #include <mutex>
+#include <type_traits>
 #include <vector>
 
 #include "bcg.h"
@@ -58,14 +59,11 @@ struct BBArgs {
     int *err;
 };
 
-// An iteration's updates, blockIdx.y the right-hand side: each runs the split
-// form of the single system's (blas.cu: every block sums the previous
-// kernel's partials of its right-hand side and takes its step from them; block
-// 0 runs the finisher), so no one-block launch and no last-block tail is left.
-// One kernel over all right-hand sides with 32 sums a thread and a last block
-// took 183 us for 16 right-hand sides of 331776 sites (34 us of bytes).  The
-// grid of one right-hand side depends on the lattice alone, so its sums do not
-// depend on its companions.
+// An iteration's updates, blockIdx.y the right-hand side.  One kernel over all
+// right-hand sides with 32 sums a thread and a last block took 183 us for 16
+// right-hand sides of 331776 sites (38 us of bytes).  The grid of one
+// right-hand side depends on the lattice alone, so its sums do not depend on its
+// companions.
 __device__ __forceinline__ BlasArgs rhs_args(const BBArgs &a, int t)
 {
     BlasArgs b{};
@@ -75,20 +73,32 @@ __device__ __forceinline__ BlasArgs rhs_args(const BBArgs &a, int t)
     return b;
 }
 
-// The sums of right-hand side t over the stencil pass's blocks, FP32 pairs in a fixed order (thread 0).
-__device__ __forceinline__ void sum_stencil_partials(const BBArgs &a, int t, double tot[2])
+// The step of right-hand side blockIdx.x from the block sums of the kernel
+// before (FP32 pairs, a fixed order): alpha after the stencil pass, beta after
+// the residual update.  A launch of its own: with a grid of several waves per
+// update, every block summing the partials itself cost more than the update
+// (16 right-hand sides of 331776 sites: 101 and 69 us against 38 us of bytes).
+template <int FIN>
+__global__ void __launch_bounds__(512) b_scalar_kernel(const __grid_constant__ BBArgs a)
 {
-    __shared__ FF sh[32][2];
+    pdl_wait();
+    pdl_launch_dependents();
+    const int t = (int)blockIdx.x;
+    CGState *st = a.st + t;
+    if (*(volatile const int *)&st->active == 0) return;
+    __shared__ FF sh[16][2];
     const int t0 = t / a.T * a.T;
-    const float2 *part = a.stencil_sums + (size_t)t0 * a.nstencil + (t - t0);
+    const float2 *part = FIN == FIN_CG_ALPHA ? a.stencil_sums + (size_t)t0 * a.nstencil + (t - t0)
+                                             : a.r_sums + (size_t)t * a.nr_blocks;
+    const int rows = FIN == FIN_CG_ALPHA ? a.nstencil : a.nr_blocks, stride = FIN == FIN_CG_ALPHA ? a.T : 1;
     FF w[2] = {{0.0f, 0.0f}, {0.0f, 0.0f}};
     constexpr int U = 8;
-    for (int b0 = threadIdx.x; b0 < a.nstencil; b0 += U * kRBlock) {
+    for (int b0 = threadIdx.x; b0 < rows; b0 += U * 512) {
         float2 v[U];
 #pragma unroll
         for (int u = 0; u < U; u++) {
-            const int b = b0 + u * kRBlock;
-            v[u] = b < a.nstencil ? __ldcg(part + (size_t)b * a.T) : make_float2(0.0f, 0.0f);
+            const int b = b0 + u * 512;
+            v[u] = b < rows ? __ldcg(part + (size_t)b * stride) : make_float2(0.0f, 0.0f);
         }
 #pragma unroll
         for (int u = 0; u < U; u++) {
@@ -103,12 +113,15 @@ __device__ __forceinline__ void sum_stencil_partials(const BBArgs &a, int t, dou
         sh[wid][1] = w[1];
     }
     __syncthreads();
-    if (wid == 0) {
-        w[0] = lane < kRBlock / 32 ? sh[lane][0] : FF{0.0f, 0.0f};
-        w[1] = lane < kRBlock / 32 ? sh[lane][1] : FF{0.0f, 0.0f};
-        warp_sum_ff<2>(w);
-        tot[0] = (double)w[0].hi + (double)w[0].lo;
-        tot[1] = (double)w[1].hi + (double)w[1].lo;
+    if (wid != 0) return;
+    w[0] = lane < 16 ? sh[lane][0] : FF{0.0f, 0.0f};
+    w[1] = lane < 16 ? sh[lane][1] : FF{0.0f, 0.0f};
+    warp_sum_ff<2>(w);
+    if (lane == 0) {
+        const double tot[2] = {(double)w[0].hi + (double)w[0].lo, (double)w[1].hi + (double)w[1].lo};
+        if (FIN == FIN_CG_BETA && a.clear_ring)
+            for (int j = 0; j < kMaxBuf; j++) st->alpha_ring[j] = 0.0;
+        run_finisher(FIN, tot, st, a.slot);
     }
 }
 
@@ -119,75 +132,39 @@ __global__ void __launch_bounds__(kRBlock) b_r_update_kernel(const __grid_consta
     pdl_wait();
     pdl_launch_dependents();
     const int t = (int)blockIdx.y;
-    CGState *st = a.st + t;
+    const CGState *st = a.st + t;
     if (*(volatile const int *)&st->active == 0) return;
     constexpr int U = kUSites, C = Spinor<SF>::chunks;
     BlasArgs b = rhs_args(a, t);
     b.v1 = a.ap + (size_t)t * a.fb;
     const int step = (int)gridDim.x * kRBlock * U;
-    int i0 = (int)blockIdx.x * kRBlock * U + (int)threadIdx.x;
-    uint4 cr[U][C], ca[U][C];
-    r_load<SF>(b, i0, cr, ca);
-    __shared__ real al_sh;
-    __shared__ int ok_sh;
-    double tot[2] = {0.0, 0.0};
-    sum_stencil_partials(a, t, tot);
-    if (threadIdx.x == 0) {
-        const double al = st->rr / tot[0];
-        const bool ok = tot[0] > 0.0 && isfinite(al);  // else the finisher stops this system
-        al_sh = ok ? real(al) : real(0);
-        ok_sh = ok;
+    const real alpha = (real)st->alpha;
+    real v[2] = {0, 0};
+    for (int i0 = (int)blockIdx.x * kRBlock * U + (int)threadIdx.x; i0 < a.n; i0 += step) {
+        uint4 cr[U][C], ca[U][C];
+        r_load<SF>(b, i0, cr, ca);
+        r_group<SF, real>(b, i0, cr, ca, alpha, v, b.v0);
     }
-    __syncthreads();
-    if (ok_sh) {
-        const real alpha = al_sh;
-        real v[2] = {0, 0};
-        for (; i0 < a.n; i0 += step) {
-            r_group<SF, real>(b, i0, cr, ca, alpha, v, b.v0);
-            r_load<SF>(b, i0 + step, cr, ca);
-        }
-        store_partial_at<2, float>(v, reinterpret_cast<float *>(a.r_sums + (size_t)t * a.nr_blocks), blockIdx.x);
-    }
-    if (blockIdx.x == 0 && threadIdx.x == 0) {
-        st->rr_den = st->rr;
-        run_finisher(FIN_CG_ALPHA, tot, st, a.slot);
-    }
+    store_partial_at<2, float>(v, reinterpret_cast<float *>(a.r_sums + (size_t)t * a.nr_blocks), blockIdx.x);
 }
 
-// p_out_t = r_t + beta_t p_in_t for active t
+// p_out_t = r_t + beta_t p_in_t
 template <int SF, typename real>
 __global__ void __launch_bounds__(kBlock) b_p_update_kernel(const __grid_constant__ BBArgs a)
 {
     pdl_wait();
     pdl_launch_dependents();
     const int t = (int)blockIdx.y;
-    CGState *st = a.st + t;
+    const CGState *st = a.st + t;
     if (*(volatile const int *)&st->active == 0) return;
     constexpr int U = kUSites, C = Spinor<SF>::chunks;
-    if (a.clear_ring && blockIdx.x == 0 && threadIdx.x == 0)
-        for (int j = 0; j < kMaxBuf; j++) st->alpha_ring[j] = 0.0;
     BlasArgs b = rhs_args(a, t);
     b.v1 = a.p_in + (size_t)t * a.fb;
     b.v2 = a.p_out + (size_t)t * a.fb;
     const int i0 = (int)blockIdx.x * kBlock * U + (int)threadIdx.x;
     uint4 cr[U][C], cp[U][C];
     p_load<SF>(b, i0, cr, cp);
-    __shared__ double tot[2];
-    __shared__ real be_sh;
-    __shared__ int ok_sh;
-    RedBuf rb{};
-    rb.partials = reinterpret_cast<double *>(a.r_sums + (size_t)t * a.nr_blocks);
-    warp0_sum_partials<2, float>(rb, (unsigned)a.nr_blocks, tot);
-    if (threadIdx.x == 0) {
-        const double rr_new = tot[0];
-        const double be = (st->pr ? rr_new - tot[1] : rr_new) / st->rr_den;
-        const bool ok = isfinite(rr_new) && isfinite(be);  // else the finisher stops this system
-        be_sh = ok ? real(be) : real(0);
-        ok_sh = ok;
-    }
-    __syncthreads();
-    if (ok_sh) p_group<SF, real>(b, i0, cr, cp, be_sh);
-    if (blockIdx.x == 0 && threadIdx.x == 0) run_finisher(FIN_CG_BETA, tot, st, a.slot);
+    p_group<SF, real>(b, i0, cr, cp, (real)st->beta);
 }
 
 // x_t += sum_j alpha_{t,j} p_{t,j} for active t (increment in the compute precision)
@@ -412,6 +389,12 @@ void BatchSession::iterate_block()
         stencil_pass(0, tmp_s, ap_s, slot(i, 0), true);
         BBArgs a = bb_args(*this);
         a.slot = i;
+        a.clear_ring = i == N - 1;
+        auto scalar = [&](auto fin) {
+            LaunchScope ls(c, s, PROF_BLAS, 0.0);
+            launch_chained(b_scalar_kernel<decltype(fin)::value>, dim3(nr), dim3(512), s, a);
+        };
+        scalar(std::integral_constant<int, FIN_CG_ALPHA>{});
         {
             LaunchScope ls(c, s, PROF_BLAS, 3.0 * sb * nr);
             BB_DISPATCH(cfg.sloppy.spinor, b_r_update_kernel, a.nr_blocks, kRBlock);
@@ -422,9 +405,9 @@ void BatchSession::iterate_block()
             LaunchScope ls(c, s, PROF_BLAS, (96.0 + N * spinor_site_bytes(cfg.sloppy.spinor)) * vh * nr);
             BB_DISPATCH(cfg.sloppy.spinor, b_flush_kernel, (vh + kBlock - 1) / kBlock, kBlock);
         }
+        scalar(std::integral_constant<int, FIN_CG_BETA>{});
         a.p_in = slot(i, 0);
         a.p_out = slot((i + 1) % N, 0);
-        a.clear_ring = i == N - 1;
         LaunchScope ls(c, s, PROF_BLAS, 3.0 * sb * nr);
         BB_DISPATCH(cfg.sloppy.spinor, b_p_update_kernel, (vh + kBlock * kUSites - 1) / (kBlock * kUSites), kBlock);
     }
