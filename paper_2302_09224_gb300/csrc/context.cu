@@ -638,21 +638,23 @@ hisq_status hisq_load_gauge(hisq_ctx *c, const int dims[4], const double *fat, c
         delete g;
         return st;
     }
-    const cudaMemcpyKind kind = (flags & HISQ_GAUGE_ON_DEVICE) ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice;
-    cudaError_t e = cudaMemcpyAsync(g->fat64, fat, bytes, kind, c->stream);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(g->lng64, lng, bytes, kind, c->stream);
-    double *scal = cur_red(c).result;  // 5 scratch doubles: fat max, long max, fat dev, long dev, long U(3) dev
-    if (e == cudaSuccess) e = cudaMemsetAsync(scal, 0, 5 * sizeof(double), c->stream);
+    // host arrays are copied, then scanned; device arrays are copied by the scan
+    const bool on_device = (flags & HISQ_GAUGE_ON_DEVICE) != 0;
+    cudaError_t e = cudaSuccess;
+    if (!on_device) {
+        e = cudaMemcpyAsync(g->fat64, fat, bytes, cudaMemcpyHostToDevice, c->stream);
+        if (e == cudaSuccess) e = cudaMemcpyAsync(g->lng64, lng, bytes, cudaMemcpyHostToDevice, c->stream);
+    }
+    // per field: bits of max |element|, not 12 reals, not unitary
+    unsigned long long *scan = (unsigned long long *)cur_red(c).result, h[6] = {0, 0, 0, 0, 0, 0};
+    if (e == cudaSuccess) e = cudaMemsetAsync(scan, 0, sizeof h, c->stream);
     if (e == cudaSuccess) {
         LaunchScope ls(c, c->stream, PROF_CONVERT, 0.0);
-        launch_absmax(18 * 4 * V, g->fat64, scal + 0, c->stream);
-        launch_absmax(18 * 4 * V, g->lng64, scal + 1, c->stream);
-        launch_r12_check(g->geom, g->fat64, 1, scal + 2, c->stream);
-        launch_r12_check(g->geom, g->lng64, 3, scal + 3, c->stream);
-        launch_u3_check(g->geom, g->lng64, scal + 4, c->stream);
+        launch_gauge_scan(g->geom, false, on_device ? fat : g->fat64, on_device ? g->fat64 : nullptr, scan, c->stream);
+        launch_gauge_scan(g->geom, true, on_device ? lng : g->lng64, on_device ? g->lng64 : nullptr, scan + 3,
+                          c->stream);
     }
-    double h[5] = {0, 0, 0, 0, 0};
-    if (e == cudaSuccess) e = cudaMemcpyAsync(h, scal, sizeof h, cudaMemcpyDeviceToHost, c->stream);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(h, scan, sizeof h, cudaMemcpyDeviceToHost, c->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
     if (e != cudaSuccess) {
         ctx_free(c, g->fat64, bytes);
@@ -660,17 +662,20 @@ hisq_status hisq_load_gauge(hisq_ctx *c, const int dims[4], const double *fat, c
         delete g;
         return cuda_fail(c, e, "gauge upload");
     }
-    if (!std::isfinite(h[0]) || !std::isfinite(h[1])) {
+    double mx[2];
+    std::memcpy(&mx[0], &h[0], sizeof(double));
+    std::memcpy(&mx[1], &h[3], sizeof(double));
+    if (!std::isfinite(mx[0]) || !std::isfinite(mx[1])) {
         ctx_free(c, g->fat64, bytes);
         ctx_free(c, g->lng64, bytes);
         delete g;
         return fail(c, HISQ_EINVAL, "gauge field has non-finite entries");
     }
-    g->fat_max = h[0];
-    g->lng_max = h[1];
-    g->fat_r12_ok = std::isfinite(h[2]) && h[2] <= 1e-6;
-    g->lng_r12_ok = std::isfinite(h[3]) && h[3] <= 1e-6;
-    g->lng_u3_ok = std::isfinite(h[4]) && h[4] <= 1e-6;
+    g->fat_max = mx[0];
+    g->lng_max = mx[1];
+    g->fat_r12_ok = h[1] == 0;
+    g->lng_r12_ok = h[4] == 0;
+    g->lng_u3_ok = h[5] == 0;
     {
         std::lock_guard<std::mutex> lk(c->mu);
         c->gauges.push_back(g);

@@ -87,21 +87,6 @@ __device__ __forceinline__ void atomic_max_nonneg(double *addr, double v)
     atomicMax(reinterpret_cast<unsigned long long *>(addr), (unsigned long long)__double_as_longlong(v));
 }
 
-__global__ void absmax_kernel(int64_t n, const double *x, double *out)
-{
-    double m = 0.0;
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-        const double a = fabs(x[i]);
-        m = (a > m || a != a) ? a : m;
-    }
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1) {
-        const double o = __shfl_down_sync(0xffffffffu, m, off);
-        m = (o > m || o != o) ? o : m;
-    }
-    if ((threadIdx.x & 31) == 0) atomic_max_nonneg(out, m);
-}
-
 __device__ __forceinline__ void lex_coords(const Geom &g, int lex, int c[4])
 {
     c[0] = lex % g.L[0];
@@ -112,63 +97,232 @@ __device__ __forceinline__ void lex_coords(const Geom &g, int lex, int c[4])
     c[3] = r / g.L[2];
 }
 
-// Largest deviation of row 2 from sign * conj(row0 x row1) over all links of
-// a field (k = 1 fat, k = 3 long): zero to rounding when the field can be
-// stored as 12 reals (Sec. 1, 18 -> 12 compression).
-__global__ void r12_check_kernel(Geom g, const double *links, int k, double *out)
+// idx = mu V + lex, without a 64-bit division
+__device__ __forceinline__ void link_index(int64_t idx, int V, int &mu, int &lex)
 {
-    const int V = 2 * g.vh;
+    mu = (idx >= V) + (idx >= 2LL * V) + (idx >= 3LL * V);
+    lex = (int)(idx - (int64_t)mu * V);
+}
+
+// A warp's 32 consecutive links of an FP64 [mu][lex][18] field, from idx0 on
+// (fewer at the field's end), to shared memory in full lines; a link's 18 reals
+// are kLinkPad apart there (a lane's walk over its own link then meets no bank
+// conflict).  f(bits, address) sees every real once, by the lane that loaded it.
+constexpr int kLinkPad = 19;
+constexpr int kLinkBlock = 128;
+template <typename F>
+__device__ __forceinline__ void warp_load_links(const double *links, int64_t idx0, int64_t n, double *sh, F f)
+{
+    const int lane = threadIdx.x & 31;
+    const int m = 18 * (int)(n - idx0 < 32 ? n - idx0 : 32);
+    // as bit patterns: an absolute value written on doubles becomes an FP64 instruction
+    const unsigned long long *src = reinterpret_cast<const unsigned long long *>(links) + 18 * idx0;
+    unsigned long long v[18];
+#pragma unroll
+    for (int k = 0; k < 18; k++) {
+        const int j = lane + 32 * k;
+        v[k] = j < m ? __ldcs(src + j) : 0ull;
+    }
+#pragma unroll
+    for (int k = 0; k < 18; k++) {
+        const int j = lane + 32 * k;
+        if (j >= m) continue;
+        reinterpret_cast<unsigned long long *>(sh)[j / 18 * kLinkPad + j % 18] = v[k];
+        f(v[k], 18 * idx0 + j);
+    }
+    __syncwarp();
+}
+
+// Row 2's deviation from sign * conj(row0 x row1), and the deviation of U U^+
+// from 1, of one link in FP64.
+__device__ __noinline__ double r12_dev64(const double *u, double sign)
+{
+    double R[18], m = 0.0;
+    for (int j = 0; j < 18; j++) R[j] = u[j];
+    rebuild_row2(R, sign);
+    for (int j = 12; j < 18; j++) {
+        const double d = fabs(R[j] - u[j]);
+        m = (d > m || d != d) ? d : m;
+    }
+    return m;
+}
+
+__device__ __noinline__ double u3_dev64(const double *u)
+{
     double m = 0.0;
-    for (int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; idx < 4LL * V;
-         idx += (int64_t)gridDim.x * blockDim.x) {
-        const int mu = (int)(idx / V), lex = (int)(idx % V);
+    for (int i = 0; i < 3; i++)
+        for (int j = 0; j < 3; j++) {
+            double re = 0.0, im = 0.0;  // sum_k U_ik conj(U_jk)
+            for (int k = 0; k < 3; k++) {
+                const double ar = u[2 * (3 * i + k)], ai = u[2 * (3 * i + k) + 1];
+                const double br = u[2 * (3 * j + k)], bi = u[2 * (3 * j + k) + 1];
+                re += ar * br + ai * bi;
+                im += ai * br - ar * bi;
+            }
+            const double d = fmax(fabs(re - (i == j ? 1.0 : 0.0)), fabs(im));
+            m = (d > m || d != d) ? d : m;
+        }
+    return m;
+}
+
+// A double as an FP32 pair on the integer and FP32 pipes: the top 24 bits, and
+// the other 29 rounded to FP32 (below 2^-126 as zero); |d| < 2^127.
+__device__ __forceinline__ ff d2ff_bits(double d)
+{
+    const uint32_t hi = (uint32_t)__double2hiint(d), lo = (uint32_t)__double2loint(d);
+    const uint32_t e = (hi >> 20) & 0x7ffu, sg = hi & 0x80000000u;
+    if (e < 897u) return ff(0.0f);
+    const float h = __uint_as_float(sg | __funnelshift_l(lo, (hi & 0x7fffffffu) - (896u << 20), 3));
+    if (e < 950u) return ff(h);
+    const float sc = __uint_as_float(sg | ((e - 948u) << 23));  // 2^(e - 1075)
+    return ff(h, __fmul_rn(__uint2float_rn(lo & 0x1fffffffu), sc));
+}
+
+// The same two deviations in FP32 pairs (about 46 bits): FP64 arithmetic at
+// GB300's rate bounded the checks (70 and 171 us for a field of 524288 links,
+// 11 us of bytes).
+__device__ __forceinline__ float r12_dev_ff(const ff u[18], float sign)
+{
+    float m = 0.0f;
+#pragma unroll
+    for (int c = 0; c < 3; c++) {
+        const int k = (c + 1) % 3, l = (c + 2) % 3;
+        const ff *ak = u + 2 * k, *al = u + 2 * l, *bk = u + 6 + 2 * k, *bl = u + 6 + 2 * l;
+        const ff cr = (ak[0] * bl[0] - ak[1] * bl[1]) - (al[0] * bk[0] - al[1] * bk[1]);
+        const ff ci = (ak[0] * bl[1] + ak[1] * bl[0]) - (al[0] * bk[1] + al[1] * bk[0]);
+        const float dr = fabsf((ff_scale(cr, sign) - u[12 + 2 * c]).hi);
+        const float di = fabsf((ff_scale(ci, -sign) - u[13 + 2 * c]).hi);
+        m = fmaxf(m, fmaxf(dr, di));
+    }
+    return m;
+}
+
+__device__ __forceinline__ float u3_dev_ff(const ff u[18])
+{
+    float m = 0.0f;
+#pragma unroll
+    for (int i = 0; i < 3; i++)
+#pragma unroll
+        for (int j = i; j < 3; j++) {  // (j, i) is its conjugate
+            ff re(i == j ? -1.0f : 0.0f), im(0.0f);
+#pragma unroll
+            for (int k = 0; k < 3; k++) {
+                const ff *a = u + 2 * (3 * i + k), *b = u + 2 * (3 * j + k);
+                re += a[0] * b[0] + a[1] * b[1];
+                if (i != j) im += a[1] * b[0] - a[0] * b[1];
+            }
+            m = fmaxf(m, fmaxf(fabsf(re.hi), fabsf(im.hi)));
+        }
+    return m;
+}
+
+// A gauge field at load, in one pass over its links (five passes before, two of
+// them bound by FP64 arithmetic): the resident copy (COPY), the bits of the
+// largest |element| (out[0]; non-negative doubles order like their bits, NaN
+// above infinity), whether some link's row 2 is not sign * conj(row0 x row1)
+// to 1e-6 (out[1], k = 1 fat, k = 3 long) and, for the long links, whether some
+// link is not unitary to 1e-6 (out[2]).  The deviations are taken in FP32 pairs;
+// a link whose deviation comes within 0.1 % of the bound, or whose elements
+// exceed 16, is decided in FP64.
+constexpr double kCompressTol = 1e-6;
+template <bool LONG, bool COPY>
+__global__ void __launch_bounds__(kLinkBlock) gauge_scan_kernel(Geom g, const double *links, double *copy,
+                                                                unsigned long long *out)
+{
+    __shared__ double sh[kLinkBlock / 32][32 * kLinkPad];
+    __shared__ unsigned long long mx_sh[kLinkBlock / 32];
+    const int V = 2 * g.vh, lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    const int64_t n = 4LL * V;
+    const int64_t idx = (int64_t)blockIdx.x * kLinkBlock + threadIdx.x, idx0 = idx - lane;
+    unsigned long long mx = 0;
+    if (idx0 < n) {
+        warp_load_links(links, idx0, n, sh[wid], [&](unsigned long long v, int64_t at) {
+            const unsigned long long b = v & 0x7fffffffffffffffull;
+            mx = b > mx ? b : mx;
+            if constexpr (COPY) reinterpret_cast<unsigned long long *>(copy)[at] = v;
+        });
+    }
+    bool bad12 = false, bad3 = false;
+    if (idx < n) {
+        const double *u = sh[wid] + lane * kLinkPad;
+        int mu, lex;
+        link_index(idx, V, mu, lex);
         int c[4];
         lex_coords(g, lex, c);
         int ps = 0;
         for (int nu = 0; nu < mu; nu++) ps += c[nu];
-        double sign = (ps & 1) ? -1.0 : 1.0;
-        if (g.antiperiodic_t && mu == 3 && c[3] + k >= g.L[3]) sign = -sign;
-        double U[18];
-        const double *src = links + idx * 18;
-        for (int j = 0; j < 18; j++) U[j] = src[j];
-        double R[18];
-        for (int j = 0; j < 18; j++) R[j] = U[j];
-        rebuild_row2(R, sign);
-        for (int j = 12; j < 18; j++) {
-            const double d = fabs(R[j] - U[j]);
-            m = (d > m || d != d) ? d : m;
+        const bool flip = g.antiperiodic_t && mu == 3 && c[3] + (LONG ? 3 : 1) >= g.L[3];
+        const float sign = ((ps & 1) != 0) != flip ? -1.0f : 1.0f;
+        ff w[18];
+        unsigned top = 0;
+#pragma unroll
+        for (int k = 0; k < 18; k++) {
+            const double v = u[k];
+            const unsigned h = (unsigned)__double2hiint(v) & 0x7fffffffu;
+            top = h > top ? h : top;
+            w[k] = d2ff_bits(v);
+        }
+        const bool big = top >= 0x40300000u;  // 16
+        const float lo = (float)(0.999 * kCompressTol), hi = (float)(1.001 * kCompressTol);
+        const float d12 = r12_dev_ff(w, sign);
+        bad12 = big || !(d12 < lo);
+        if (bad12 && (big || d12 <= hi)) {
+            const double d = r12_dev64(u, (double)sign);
+            bad12 = !(isfinite(d) && d <= kCompressTol);
+        }
+        if constexpr (LONG) {
+            const float d3 = u3_dev_ff(w);
+            bad3 = big || !(d3 < lo);
+            if (bad3 && (big || d3 <= hi)) {
+                const double d = u3_dev64(u);
+                bad3 = !(isfinite(d) && d <= kCompressTol);
+            }
         }
     }
 #pragma unroll
     for (int off = 16; off > 0; off >>= 1) {
-        const double o = __shfl_down_sync(0xffffffffu, m, off);
-        m = (o > m || o != o) ? o : m;
+        const unsigned long long o = __shfl_down_sync(0xffffffffu, mx, off);
+        mx = o > mx ? o : mx;
     }
-    if ((threadIdx.x & 31) == 0) atomic_max_nonneg(out, m);
+    if (lane == 0) mx_sh[wid] = mx;
+    const int any12 = __syncthreads_or(bad12), any3 = __syncthreads_or(bad3);
+    if (threadIdx.x == 0) {
+        // (a field that does not compress has bad links everywhere: one store, not one per link)
+        volatile unsigned long long *flag = out;
+        if (any12 && flag[1] == 0) flag[1] = 1ull;
+        if (any3 && flag[2] == 0) flag[2] = 1ull;
+        for (int w = 1; w < kLinkBlock / 32; w++) mx = mx_sh[w] > mx ? mx_sh[w] : mx;
+        if (mx > *(volatile unsigned long long *)out) atomicMax(out, mx);
+    }
 }
 
 // FP64 [mu][lex][18] -> stored copy [plane][parity][mu][Vh] in format GF with
 // RECON reals per link.  Fixed point: q = rint(x * inv) clamped to +-qmax,
 // inv = qmax / global max (Sec. 2 footnote; Sec. 4 for 32 bits).
+// A thread a link in the caller's order, so that both the reads (through shared
+// memory) and the writes (16 consecutive links of each parity a warp) are full
+// lines.  The fixed-point integers take two FP64 operations a real: the product,
+// and the sum with 1.5 2^52, whose low word is the product rounded to the
+// nearest even integer (rint, two clamps and a conversion took five; 93 us for
+// 524288 18-real links to 16 bits).
 template <int GF, int RECON>
-__global__ void quantise_kernel(Geom g, const double *links, double inv, char *out)
+__global__ void __launch_bounds__(kLinkBlock) quantise_kernel(Geom g, const double *links, double inv, char *out)
 {
+    __shared__ double sh[kLinkBlock / 32][32 * kLinkPad];
     const int vh = g.vh;
     const int64_t n = 8LL * vh;
-    const int64_t li = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (li >= n) return;
-    const int cb = (int)(li % vh);
-    const int pm = (int)(li / vh);
-    const int par = pm >> 2, mu = pm & 3;
-    int r = cb / g.xh;
-    const int xh = cb - r * g.xh;
-    const int y = r % g.L[1];
-    r /= g.L[1];
-    const int z = r % g.L[2];
-    const int t = r / g.L[2];
-    const int x = 2 * xh + ((y + z + t + par) & 1);
-    const int lex = 2 * cb + (x & 1);
-    const double *src = links + ((int64_t)mu * 2 * vh + lex) * 18;
+    const int64_t idx = (int64_t)blockIdx.x * kLinkBlock + threadIdx.x;
+    const int lane = threadIdx.x & 31;
+    if (idx - lane < n) warp_load_links(links, idx - lane, n, sh[threadIdx.x >> 5], [](unsigned long long, int64_t) {});
+    if (idx >= n) return;
+    int mu, lex;
+    link_index(idx, 2 * vh, mu, lex);
+    int cc[4];
+    lex_coords(g, lex, cc);
+    const int t = cc[3];
+    const int par = (cc[0] + cc[1] + cc[2] + cc[3]) & 1;
+    const int64_t li = (int64_t)(par * 4 + mu) * vh + lex / 2;
+    const double *src = sh[threadIdx.x >> 5] + lane * kLinkPad;
     const size_t pstride = (size_t)n * 16;
     constexpr int n16 = link_n16(GF, RECON), tail = link_tail(GF, RECON);
     if constexpr (RECON == 8) {
@@ -176,7 +330,6 @@ __global__ void quantise_kernel(Geom g, const double *links, double inv, char *o
         // sign): arg V00 / pi, arg V20 / pi, V01, V02, V10.  Angles are stored as the format
         // stores a real in [-1, 1] (fixed point: rint(t qmax)), elements as every other element.
         int ps = 0;
-        const int cc[4] = {x, y, z, t};
         for (int nu = 0; nu < mu; nu++) ps += cc[nu];
         double sg = (ps & 1) ? -1.0 : 1.0;
         if (g.antiperiodic_t && mu == 3 && t + 3 >= g.L[3]) sg = -sg;
@@ -217,10 +370,11 @@ __global__ void quantise_kernel(Geom g, const double *links, double inv, char *o
     } else if constexpr (GF == G_F32) {
         for (int k = 0; k < n16; k++)
             reinterpret_cast<float4 *>(out + k * pstride)[li] =
-                make_float4((float)src[4 * k], (float)src[4 * k + 1], (float)src[4 * k + 2], (float)src[4 * k + 3]);
+                make_float4(d2f_bits(src[4 * k]), d2f_bits(src[4 * k + 1]), d2f_bits(src[4 * k + 2]),
+                            d2f_bits(src[4 * k + 3]));
         if constexpr (tail == 8)
             reinterpret_cast<float2 *>(out + n16 * pstride)[li] =
-                make_float2((float)src[4 * n16], (float)src[4 * n16 + 1]);
+                make_float2(d2f_bits(src[4 * n16]), d2f_bits(src[4 * n16 + 1]));
     } else if constexpr (GF == G_SE15) {
         // per link: 15-bit integers with one exponent, the 30-bit rule in FP64 with scale 2^14 - 1
         // (t = max |x| / (2^14 - 1), 2^(E-127) the power of two just above t); half k = q_k << 1 | bit k
@@ -254,11 +408,15 @@ __global__ void quantise_kernel(Geom g, const double *links, double inv, char *o
                 make_uint2(h[8 * n16] | (h[8 * n16 + 1] << 16), h[8 * n16 + 2] | (h[8 * n16 + 3] << 16));
     } else {
         constexpr double qmax = GF == G_FIX16 ? 32767.0 : 2147483647.0;
+        // |x inv| <= qmax (1 + 2^-52), so the rounded product stays within +-qmax (clamped where the field is
+        // so small that inv overflowed)
         int q[RECON];
-        for (int k = 0; k < RECON; k++) {
-            double v = rint(__dmul_rn(src[k], inv));
-            v = fmin(qmax, fmax(-qmax, v));
-            q[k] = (int)v;
+        if (isinf(inv)) {
+            for (int k = 0; k < RECON; k++) q[k] = (int)fmin(qmax, fmax(-qmax, rint(__dmul_rn(src[k], inv))));
+        } else {
+#pragma unroll
+            for (int k = 0; k < RECON; k++)
+                q[k] = __double2loint(__dadd_rn(__dmul_rn(src[k], inv), 6755399441055744.0));
         }
         if constexpr (GF == G_FIX16) {
             for (int k = 0; k < n16; k++) {
@@ -411,36 +569,6 @@ __global__ void r8_check_kernel(Geom g, const double *links, const char *stored,
     }
 }
 
-// Largest |(U U^+)_ij - delta_ij| over all links of a field: zero to rounding
-// when every link is unitary (the 13-real format applies).
-__global__ void u3_check_kernel(Geom g, const double *links, double *out)
-{
-    const int V = 2 * g.vh;
-    double m = 0.0;
-    for (int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; idx < 4LL * V;
-         idx += (int64_t)gridDim.x * blockDim.x) {
-        const double *u = links + idx * 18;
-        for (int i = 0; i < 3; i++)
-            for (int j = 0; j < 3; j++) {
-                double re = 0.0, im = 0.0;  // sum_k U_ik conj(U_jk)
-                for (int k = 0; k < 3; k++) {
-                    const double ar = u[2 * (3 * i + k)], ai = u[2 * (3 * i + k) + 1];
-                    const double br = u[2 * (3 * j + k)], bi = u[2 * (3 * j + k) + 1];
-                    re += ar * br + ai * bi;
-                    im += ai * br - ar * bi;
-                }
-                const double d = fmax(fabs(re - (i == j ? 1.0 : 0.0)), fabs(im));
-                m = (d > m || d != d) ? d : m;
-            }
-    }
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1) {
-        const double o = __shfl_down_sync(0xffffffffu, m, off);
-        m = (o > m || o != o) ? o : m;
-    }
-    if ((threadIdx.x & 31) == 0) atomic_max_nonneg(out, m);
-}
-
 int nblocks(int64_t n, int b) { return (int)((n + b - 1) / b); }
 
 }  // namespace
@@ -517,10 +645,18 @@ void launch_unpack_spinor(int sf, int cf, int64_t n, const char *in, double *out
     }
 }
 
-void launch_absmax(int64_t n, const double *x, double *out, cudaStream_t s)
+void launch_gauge_scan(const Geom &g, bool lng, const double *links, double *copy, unsigned long long *out,
+                       cudaStream_t s)
 {
-    const int nb = (int)std::min<int64_t>(nblocks(n, kBlock), 4096);
-    absmax_kernel<<<nb, kBlock, 0, s>>>(n, x, out);
+    const int nb = nblocks(8LL * g.vh, kLinkBlock);
+    if (lng && copy)
+        gauge_scan_kernel<true, true><<<nb, kLinkBlock, 0, s>>>(g, links, copy, out);
+    else if (lng)
+        gauge_scan_kernel<true, false><<<nb, kLinkBlock, 0, s>>>(g, links, copy, out);
+    else if (copy)
+        gauge_scan_kernel<false, true><<<nb, kLinkBlock, 0, s>>>(g, links, copy, out);
+    else
+        gauge_scan_kernel<false, false><<<nb, kLinkBlock, 0, s>>>(g, links, copy, out);
 }
 
 void launch_r8_check(const Geom &g, int gf, const double *links, const char *stored, double el, double an,
@@ -535,23 +671,11 @@ void launch_r8_check(const Geom &g, int gf, const double *links, const char *sto
     }
 }
 
-void launch_u3_check(const Geom &g, const double *links, double *out, cudaStream_t s)
-{
-    const int nb = (int)std::min<int64_t>(nblocks(8LL * g.vh, kBlock), 4096);
-    u3_check_kernel<<<nb, kBlock, 0, s>>>(g, links, out);
-}
-
-void launch_r12_check(const Geom &g, const double *links, int k, double *out, cudaStream_t s)
-{
-    const int nb = (int)std::min<int64_t>(nblocks(8LL * g.vh, kBlock), 4096);
-    r12_check_kernel<<<nb, kBlock, 0, s>>>(g, links, k, out);
-}
-
 void launch_quantise_links(const Geom &g, int gf, int recon, const double *links, double inv, char *out,
                            cudaStream_t s)
 {
-    const int nb = nblocks(8LL * g.vh, kBlock);
-#define Q(GF, R) quantise_kernel<GF, R><<<nb, kBlock, 0, s>>>(g, links, inv, out)
+    const int nb = nblocks(8LL * g.vh, kLinkBlock);
+#define Q(GF, R) quantise_kernel<GF, R><<<nb, kLinkBlock, 0, s>>>(g, links, inv, out)
     if (recon == 18) {
         switch (gf) {
         case G_F64: Q(G_F64, 18); break;

@@ -348,16 +348,16 @@ void launch_pack_pair_int30(int64_t n, const float *in, char *out, int *err, cud
 void launch_unpack_spinor(int sf, int cf, int64_t n, const char *in, double *out, cudaStream_t s);
 
 // gauge preparation
-// out_max / out_maxdev must be zeroed before the launch (atomic max)
-void launch_absmax(int64_t n, const double *x, double *out_max, cudaStream_t s);
-void launch_r12_check(const Geom &g, const double *links, int k, double *out_maxdev, cudaStream_t s);
+// One pass over a field: its resident copy (copy may be null), and in out (three words, zeroed before
+// the launch) the bits of max |element|, non-zero when it cannot be stored as 12 reals, and, for the long
+// links, non-zero when it is not unitary.
+void launch_gauge_scan(const Geom &g, bool lng, const double *links, double *copy, unsigned long long *out,
+                       cudaStream_t s);
 // FP64 rebuild error of a field stored with 8 reals: out[0] the largest
 // element error, out[1] the sum of squared element errors (both zeroed before
 // the launch); el / an: element and angle scales
 void launch_r8_check(const Geom &g, int gf, const double *links, const char *stored, double el, double an,
                      double *out, cudaStream_t s);
-// max over links of |U U^+ - 1| (out_maxdev zeroed before the launch)
-void launch_u3_check(const Geom &g, const double *links, double *out_maxdev, cudaStream_t s);
 void launch_quantise_links(const Geom &g, int gf, int recon, const double *links, double inv, char *out,
                            cudaStream_t s);
 
