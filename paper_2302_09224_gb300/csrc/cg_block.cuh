@@ -51,8 +51,8 @@ __device__ __forceinline__ void lane_stencil(const DslashArgs &a, const char *in
         const int mu = lane_s * (4 / S) + k;
         const int cmu = mu == 0 ? x : mu == 1 ? y : mu == 2 ? z : t;
         const int phase_sum = mu == 0 ? 0 : mu == 1 ? x : mu == 2 ? x + y : x + y + z;
-        // other blocks write `in` during the launch (L2 loads); the links are read every pass (kept in L2)
-        stencil_direction<GF, SF, float, LREC, true, true>(a, in, mu, cmu, t, lex, cb, po, pstride, lsc, ratio,
+        // other blocks write `in` between barriers (plain loads); the links are read every pass (kept in L2)
+        stencil_direction<GF, SF, float, LREC, 2, true>(a, in, mu, cmu, t, lex, cb, po, pstride, lsc, ratio,
                                                            phase_sum, acc);
     }
 #pragma unroll

@@ -759,6 +759,26 @@ __device__ __forceinline__ void gather_coherent(const char *b, int n, int i, uin
     }
 }
 
+// A spinor record by plain loads: for fields that other blocks write between
+// grid barriers (not the read-only path, but L1 serves the neighbours' reuse; a
+// barrier's acquire discards the lines of before).
+template <int SF>
+__device__ __forceinline__ void gather_plain(const char *b, int n, int i, uint4 c[Spinor<SF>::chunks])
+{
+    if constexpr (SF == S_INT14) {
+        const uint2 a = reinterpret_cast<const uint2 *>(b)[i];
+        c[0] = make_uint4(a.x, a.y, reinterpret_cast<const uint32_t *>(b + (size_t)8 * n)[i], 0u);
+        return;
+    }
+    constexpr int n16 = spinor_n16(SF), tail = spinor_tail(SF);
+#pragma unroll
+    for (int k = 0; k < n16; k++) c[k] = reinterpret_cast<const uint4 *>(b + (size_t)k * 16 * n)[i];
+    if constexpr (tail == 8) {
+        const uint2 t = reinterpret_cast<const uint2 *>(b + (size_t)n16 * 16 * n)[i];
+        c[n16] = make_uint4(t.x, t.y, 0u, 0u);
+    }
+}
+
 // Row 2 of a 13-real link: f * conj(row0 x row1) with the complex factor
 // f = (fr, fi) (the det phase e^{i pi t}, times the fixed-point scale).
 template <typename real>

@@ -189,12 +189,16 @@ __device__ __forceinline__ StencilIO stencil_io_full(const DslashArgs &a)
 // into acc.  Fixed-point links are applied unscaled and the sum is kept in
 // units of the fat scale: a long term's spinor is multiplied by lsc/fsc (one
 // accumulator for both fields keeps registers for loads in flight).
-template <typename real, int SF, bool COH>
+// COH: 0 the read-only path, 1 through L2 only, 2 plain loads
+template <typename real, int SF, int COH>
 __device__ __forceinline__ void load_neighbour(const char *b, int n, int i, real s[6])
 {
-    if constexpr (COH) {
+    if constexpr (COH != 0) {
         uint4 c[Spinor<SF>::chunks];
-        gather_coherent<SF>(b, n, i, c);
+        if constexpr (COH == 2)
+            gather_plain<SF>(b, n, i, c);
+        else
+            gather_coherent<SF>(b, n, i, c);
         Spinor<SF>::decode(c, s);
     } else {
         Spinor<SF>::load(b, n, i, s);
@@ -249,7 +253,7 @@ __device__ __forceinline__ void rebuild_r8(float U[18], float es, float as)
     U[17] = -((a1r * b2i + a1i * b2r) - (a2r * b1i + a2i * b1r));
 }
 
-template <int GF, int SF, typename real, int LREC, bool COH = false, bool KEEP = false>
+template <int GF, int SF, typename real, int LREC, int COH = 0, bool KEEP = false>
 __device__ __forceinline__ void stencil_direction(const DslashArgs &a, const char *in, int mu, int cmu, int c3,
                                                   int lex, int cb, int po, size_t pstride, real lsc, real ratio,
                                                   int phase_sum, SiteAcc<real> &acc)

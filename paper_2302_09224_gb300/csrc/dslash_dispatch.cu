@@ -212,15 +212,12 @@ bool launch_cg_block_half(int, const CGBlockShape &, const CGBlockArgs &, cudaSt
 bool launch_cg_block_int20(int, const CGBlockShape &, const CGBlockArgs &, cudaStream_t);
 
 // The most lanes a site (4, 2 or 1) with at most 512 threads on each SM (128
-// registers a thread: no spills), else one lane and up to 1024 threads while
-// the links of both passes are at most 160 MB (beyond the L2 the passes are
-// bound by HBM either way, and the separate ones hold more loads in flight);
-// the threads are spread over every SM.  Per iteration, here against the
-// separate kernels, 20-bit: 8^4 9.8 us against 21.8, 12^4 12.1 / 21.8, 16^4
-// 15.3 / 26.1, 16^3x32 21.1 / 33.0, 16^3x64 33.6 / 46.5, 20^3x36 38.1 / 47.5;
-// FP32: 16^3x32 18.8 / 35.2, but 16^3x64 (252 MB) 59.5 / 56.7.  Two lanes on
-// 864 threads (64 registers) lost to one lane on 431: 24.7 against 22.9 us on
-// 16^3x32, in an earlier form.
+// registers a thread: no spills), else one lane and up to 1024 threads, spread
+// over every SM.  Per iteration, here against the separate kernels, 20-bit: 8^4
+// 9.8 us against 22, 12^4 12.0 / 21.6, 16^4 15.4 / 24.4, 16^3x32 20.9 / 32.2,
+// 16^3x64 33.8 / 47.5, 20^3x36 39.0 / 47.5; FP32: 16^3x32 17.7 / 32.3, 16^3x64
+// 53.8 / 56.9, 20^3x36 58.4 / 61.4.  Two lanes on 864 threads (64 registers)
+// lost to one lane on 431: 24.7 against 22.9 us on 16^3x32, in an earlier form.
 CGBlockShape cg_block_shape(int gf, int sf, int cf, int long_recon, int vh)
 {
     const bool has = cf == HISQ_COMPUTE_F32 && (long_recon == 12 || long_recon == 18) &&
@@ -235,8 +232,6 @@ CGBlockShape cg_block_shape(int gf, int sf, int cf, int long_recon, int vh)
     for (int lanes = 4; has && lanes >= 1; lanes /= 2) {
         const long long all = (long long)vh * lanes;
         if (all > (long long)sms * (lanes > 1 ? 512 : 1024)) continue;
-        if (all > (long long)sms * 512 && 16LL * vh * (link_bytes(gf, 18) + link_bytes(gf, long_recon)) > 160000000LL)
-            continue;
         const int per = (int)((all + sms - 1) / sms);
         const int threads = per <= 64 ? 64 : (per + 31) / 32 * 32;
         return {lanes, threads, (int)((all + threads - 1) / threads)};
