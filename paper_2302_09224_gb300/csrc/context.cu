@@ -727,6 +727,26 @@ static hisq_status grow_scratch(hisq_ctx *c, size_t bytes)
     return st;
 }
 
+// Waits for a pack call's launch; the count of bad sites is read back only where there is one (the words
+// are zero between calls).
+static hisq_status pack_result(hisq_ctx *c, int64_t *n_bad, cudaStream_t s, const char *who)
+{
+    cudaError_t e = cudaStreamSynchronize(s);
+    if (e == cudaSuccess) e = cudaGetLastError();
+    if (e != cudaSuccess) return cuda_fail(c, e, who);
+    int h = 0;
+    volatile int *flag = c->host_flags;
+    if (*flag != 0) {
+        *flag = 0;
+        e = cudaMemcpyAsync(&h, c->bad_flag, sizeof h, cudaMemcpyDeviceToHost, s);
+        if (e == cudaSuccess) e = cudaMemsetAsync(c->bad_flag, 0, sizeof(int), s);
+        if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+        if (e != cudaSuccess) return cuda_fail(c, e, who);
+    }
+    if (n_bad) *n_bad = h;
+    return HISQ_OK;
+}
+
 hisq_status hisq_spinor_pack(hisq_ctx *c, int sfmt, int64_t n, const double *in, void *packed, int64_t *n_bad,
                              void *stream)
 {
@@ -734,18 +754,11 @@ hisq_status hisq_spinor_pack(hisq_ctx *c, int sfmt, int64_t n, const double *in,
         return fail(c, HISQ_EINVAL, "hisq_spinor_pack: bad argument");
     cudaSetDevice(c->device);
     cudaStream_t s = pick_stream(c, stream);
-    int *bad = cur_err(c);
-    cudaMemsetAsync(bad, 0, sizeof(int), s);
     {
         LaunchScope ls(c, s, PROF_CONVERT, (48.0 + spinor_site_bytes(sfmt)) * n);
-        launch_pack_spinor(sfmt, n, in, (char *)packed, bad, s);
+        launch_pack_spinor(sfmt, n, in, (char *)packed, c->bad_flag, s, c->host_flags);
     }
-    int h = 0;
-    cudaMemcpyAsync(&h, bad, sizeof h, cudaMemcpyDeviceToHost, s);
-    const cudaError_t e = cudaStreamSynchronize(s);
-    if (e != cudaSuccess) return cuda_fail(c, e, "hisq_spinor_pack");
-    if (n_bad) *n_bad = h;
-    return HISQ_OK;
+    return pack_result(c, n_bad, s, "hisq_spinor_pack");
 }
 
 hisq_status hisq_spinor_pack32(hisq_ctx *c, int sfmt, int64_t n, const float *in, void *packed, int64_t *n_bad,
@@ -755,18 +768,11 @@ hisq_status hisq_spinor_pack32(hisq_ctx *c, int sfmt, int64_t n, const float *in
         return fail(c, HISQ_EINVAL, "hisq_spinor_pack32: bad argument");
     cudaSetDevice(c->device);
     cudaStream_t s = pick_stream(c, stream);
-    int *bad = cur_err(c);
-    cudaMemsetAsync(bad, 0, sizeof(int), s);
     {
         LaunchScope ls(c, s, PROF_CONVERT, (24.0 + spinor_site_bytes(sfmt)) * n);
-        launch_pack32_spinor(sfmt, n, in, (char *)packed, bad, s);
+        launch_pack32_spinor(sfmt, n, in, (char *)packed, c->bad_flag, s, c->host_flags);
     }
-    int h = 0;
-    cudaMemcpyAsync(&h, bad, sizeof h, cudaMemcpyDeviceToHost, s);
-    const cudaError_t e = cudaStreamSynchronize(s);
-    if (e != cudaSuccess) return cuda_fail(c, e, "hisq_spinor_pack32");
-    if (n_bad) *n_bad = h;
-    return HISQ_OK;
+    return pack_result(c, n_bad, s, "hisq_spinor_pack32");
 }
 
 hisq_status hisq_spinor_pack_pair_int30(hisq_ctx *c, int64_t n, const float *in, void *packed, int64_t *n_bad,
@@ -776,18 +782,11 @@ hisq_status hisq_spinor_pack_pair_int30(hisq_ctx *c, int64_t n, const float *in,
         return fail(c, HISQ_EINVAL, "hisq_spinor_pack_pair_int30: bad argument");
     cudaSetDevice(c->device);
     cudaStream_t s = pick_stream(c, stream);
-    int *bad = cur_err(c);
-    cudaMemsetAsync(bad, 0, sizeof(int), s);
     {
         LaunchScope ls(c, s, PROF_CONVERT, (48.0 + spinor_site_bytes(S_INT30)) * n);
-        launch_pack_pair_int30(n, in, (char *)packed, bad, s);
+        launch_pack_pair_int30(n, in, (char *)packed, c->bad_flag, s, c->host_flags);
     }
-    int h = 0;
-    cudaMemcpyAsync(&h, bad, sizeof h, cudaMemcpyDeviceToHost, s);
-    const cudaError_t e = cudaStreamSynchronize(s);
-    if (e != cudaSuccess) return cuda_fail(c, e, "hisq_spinor_pack_pair_int30");
-    if (n_bad) *n_bad = h;
-    return HISQ_OK;
+    return pack_result(c, n_bad, s, "hisq_spinor_pack_pair_int30");
 }
 
 hisq_status hisq_spinor_unpack(hisq_ctx *c, int sfmt, int compute, int64_t n, const void *packed, double *out,

@@ -30,23 +30,31 @@ __device__ __forceinline__ bool pack_warp(int64_t n, const T *in, char *out, T *
     return i >= n || Spinor<SF>::store(out, (int)n, (int)i, v);
 }
 
+// Sites that cannot be encoded: counted on the device, and (host not null) reported to a host-mapped word,
+// which stays zero otherwise, so that the caller has nothing to copy back.
+__device__ __forceinline__ void report_bad(int *bad, int *host)
+{
+    atomicAdd(bad, 1);
+    if (host != nullptr) *(volatile int *)host = 1;
+}
+
 // FP64 input; FP32 input goes through the FP32 store (the one FP32-compute kernels use)
 template <int SF, typename T>
-__global__ void __launch_bounds__(kBlock) pack_kernel(int64_t n, const T *in, char *out, int *bad)
+__global__ void __launch_bounds__(kBlock) pack_kernel(int64_t n, const T *in, char *out, int *bad, int *host)
 {
     __shared__ __align__(16) T sh[kBlock / 32][192];
-    if (!pack_warp<SF>(n, in, out, sh[threadIdx.x >> 5])) atomicAdd(bad, 1);
+    if (!pack_warp<SF>(n, in, out, sh[threadIdx.x >> 5])) report_bad(bad, host);
 }
 
 // FP32-pair input [n][6][hi, lo] through the pair store (FP64-class kernels)
-__global__ void pack_pair_kernel(int64_t n, const float *in, char *out, int *bad)
+__global__ void pack_pair_kernel(int64_t n, const float *in, char *out, int *bad, int *host)
 {
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
     ff v[6];
 #pragma unroll
     for (int k = 0; k < 6; k++) v[k] = ff(in[12 * i + 2 * k], in[12 * i + 2 * k + 1]);
-    if (!Spinor<S_INT30>::store(out, (int)n, (int)i, v)) atomicAdd(bad, 1);
+    if (!Spinor<S_INT30>::store(out, (int)n, (int)i, v)) report_bad(bad, host);
 }
 
 // Field blockIdx.y of several (the halves of the stencil entry point's inputs)
@@ -573,17 +581,17 @@ int nblocks(int64_t n, int b) { return (int)((n + b - 1) / b); }
 
 }  // namespace
 
-void launch_pack_spinor(int sf, int64_t n, const double *in, char *out, int *bad, cudaStream_t s)
+void launch_pack_spinor(int sf, int64_t n, const double *in, char *out, int *bad, cudaStream_t s, int *host)
 {
     if (n <= 0) return;
     const int nb = nblocks(n, kBlock);
     switch (sf) {
-    case S_F64: pack_kernel<S_F64, double><<<nb, kBlock, 0, s>>>(n, in, out, bad); break;
-    case S_F32: pack_kernel<S_F32, double><<<nb, kBlock, 0, s>>>(n, in, out, bad); break;
-    case S_HALF: pack_kernel<S_HALF, double><<<nb, kBlock, 0, s>>>(n, in, out, bad); break;
-    case S_INT20: pack_kernel<S_INT20, double><<<nb, kBlock, 0, s>>>(n, in, out, bad); break;
-    case S_INT14: pack_kernel<S_INT14, double><<<nb, kBlock, 0, s>>>(n, in, out, bad); break;
-    case S_INT30: pack_kernel<S_INT30, double><<<nb, kBlock, 0, s>>>(n, in, out, bad); break;
+    case S_F64: pack_kernel<S_F64, double><<<nb, kBlock, 0, s>>>(n, in, out, bad, host); break;
+    case S_F32: pack_kernel<S_F32, double><<<nb, kBlock, 0, s>>>(n, in, out, bad, host); break;
+    case S_HALF: pack_kernel<S_HALF, double><<<nb, kBlock, 0, s>>>(n, in, out, bad, host); break;
+    case S_INT20: pack_kernel<S_INT20, double><<<nb, kBlock, 0, s>>>(n, in, out, bad, host); break;
+    case S_INT14: pack_kernel<S_INT14, double><<<nb, kBlock, 0, s>>>(n, in, out, bad, host); break;
+    case S_INT30: pack_kernel<S_INT30, double><<<nb, kBlock, 0, s>>>(n, in, out, bad, host); break;
     default: break;
     }
 }
@@ -603,24 +611,24 @@ void launch_pack_fields(int sf, int64_t n, const PackFields &f, cudaStream_t s)
     }
 }
 
-void launch_pack32_spinor(int sf, int64_t n, const float *in, char *out, int *bad, cudaStream_t s)
+void launch_pack32_spinor(int sf, int64_t n, const float *in, char *out, int *bad, cudaStream_t s, int *host)
 {
     if (n <= 0) return;
     const int nb = nblocks(n, kBlock);
     switch (sf) {
-    case S_F32: pack_kernel<S_F32, float><<<nb, kBlock, 0, s>>>(n, in, out, bad); break;
-    case S_HALF: pack_kernel<S_HALF, float><<<nb, kBlock, 0, s>>>(n, in, out, bad); break;
-    case S_INT20: pack_kernel<S_INT20, float><<<nb, kBlock, 0, s>>>(n, in, out, bad); break;
-    case S_INT14: pack_kernel<S_INT14, float><<<nb, kBlock, 0, s>>>(n, in, out, bad); break;
-    case S_INT30: pack_kernel<S_INT30, float><<<nb, kBlock, 0, s>>>(n, in, out, bad); break;
+    case S_F32: pack_kernel<S_F32, float><<<nb, kBlock, 0, s>>>(n, in, out, bad, host); break;
+    case S_HALF: pack_kernel<S_HALF, float><<<nb, kBlock, 0, s>>>(n, in, out, bad, host); break;
+    case S_INT20: pack_kernel<S_INT20, float><<<nb, kBlock, 0, s>>>(n, in, out, bad, host); break;
+    case S_INT14: pack_kernel<S_INT14, float><<<nb, kBlock, 0, s>>>(n, in, out, bad, host); break;
+    case S_INT30: pack_kernel<S_INT30, float><<<nb, kBlock, 0, s>>>(n, in, out, bad, host); break;
     default: break;
     }
 }
 
-void launch_pack_pair_int30(int64_t n, const float *in, char *out, int *bad, cudaStream_t s)
+void launch_pack_pair_int30(int64_t n, const float *in, char *out, int *bad, cudaStream_t s, int *host)
 {
     if (n <= 0) return;
-    pack_pair_kernel<<<nblocks(n, kBlock), kBlock, 0, s>>>(n, in, out, bad);
+    pack_pair_kernel<<<nblocks(n, kBlock), kBlock, 0, s>>>(n, in, out, bad, host);
 }
 
 void launch_unpack_spinor(int sf, int cf, int64_t n, const char *in, double *out, cudaStream_t s)

@@ -332,7 +332,8 @@ CGBlockShape cg_block_shape(int gf, int sf, int cf, int long_recon, int vh);
 bool launch_cg_block(int gf, int sf, int long_recon, const CGBlockShape &sh, const CGBlockArgs &a, cudaStream_t s);
 int stencil_config_in_use(int gf, int sf, int cf, int long_recon, bool reduce, const Geom &g);
 
-void launch_pack_spinor(int sf, int64_t n, const double *in, char *out, int *err, cudaStream_t s);
+// err counts the sites that cannot be encoded; host (host-mapped, may be null) is set to 1 by any
+void launch_pack_spinor(int sf, int64_t n, const double *in, char *out, int *err, cudaStream_t s, int *host = nullptr);
 // Up to four fields of n sites in one launch, chained to the stream's kernels; a site that cannot be
 // encoded sets *bad and *bad_host to 1.
 struct PackFields {
@@ -343,8 +344,8 @@ struct PackFields {
     int *bad_host;
 };
 void launch_pack_fields(int sf, int64_t n, const PackFields &f, cudaStream_t s);
-void launch_pack32_spinor(int sf, int64_t n, const float *in, char *out, int *err, cudaStream_t s);
-void launch_pack_pair_int30(int64_t n, const float *in, char *out, int *err, cudaStream_t s);
+void launch_pack32_spinor(int sf, int64_t n, const float *in, char *out, int *err, cudaStream_t s, int *host);
+void launch_pack_pair_int30(int64_t n, const float *in, char *out, int *err, cudaStream_t s, int *host);
 void launch_unpack_spinor(int sf, int cf, int64_t n, const char *in, double *out, cudaStream_t s);
 
 // gauge preparation
