@@ -163,6 +163,7 @@ __global__ void __launch_bounds__(T, 1) cg_block_kernel(const __grid_constant__ 
     const int vh = g.vh;
     for (int k = threadIdx.x; k < (int)(sizeof(CGState) / 4); k += blockDim.x)
         reinterpret_cast<unsigned *>(&st)[k] = reinterpret_cast<const unsigned *>(a.st)[k];
+    if (threadIdx.x < kMaxBuf) ring_sh[threadIdx.x] = 0.0f;  // a breakdown's flush reads every slot
     const unsigned tag0 = __ldcg(a.seq);  // of the launch's first sum
     unsigned tag = tag0;
     __syncthreads();

@@ -44,12 +44,14 @@ def solve(ctx, dims, m, b, name, recon=12, split=1, tol=1e-10, anti=False, **kw)
     return st, info, x, (fat.numpy(), lng.numpy())
 
 
-# sites per parity on both sides of the lane counts' limits on 152 SMs (38912, 77824 and 155648 sites for
-# four, two and one lane), and lattices that fill no whole block
+# sites per parity on both sides of the shapes' limits on 152 SMs (19456 and 38912 for four and two lanes,
+# 77824 and 155648 for one lane of 512 and 1024 threads), and lattices that fill no whole block
 @pytest.mark.parametrize("name,recon,dims,anti", [
     ("int20", 12, (2, 2, 2, 2), False),
     ("half", 18, (4, 6, 8, 10), True),
     ("f32", 12, (6, 4, 4, 22), False),
+    ("half", 18, (12, 12, 12, 22), True),
+    ("f32", 12, (12, 12, 12, 24), False),
     ("int20", 12, (16, 16, 10, 30), True),
     ("half", 12, (12, 20, 22, 16), False),
     ("int20", 18, (16, 18, 18, 30), False),
@@ -96,6 +98,28 @@ def test_repeatable_and_maxiter(ctx):
     assert st == hisq.HISQ_ENOTCONV and info.iters == 24  # whole blocks of nbuf = 8
     st, info, x, _ = solve(ctx, dims, m, b, "half", maxiter=0)
     assert st == hisq.HISQ_ENOTCONV and info.iters == 0 and not bool(x.any())
+
+
+def test_breakdown_leaves_a_finite_solution(ctx):
+    """m = 0 on a free field: a source of zero modes breaks the recurrence down at once; what the solve
+    reports is measured from x, which holds no step of an iteration that did not happen."""
+    dims = (4, 4, 4, 4)
+    fat, lng = synth.unit_gauge(dims, 0.5), synth.unit_gauge(dims, 0.5, long_link=True)
+    g = hisq.hisq_load_gauge(ctx, dims, fat.cuda(), lng.cuda())
+    try:
+        b = torch.ones((128, 3, 2), dtype=torch.float64, device="cuda")
+        p = hisq.hisq_default_params()
+        p.mass, p.tol, p.on_device, p.sloppy, p.maxiter = 0.0, 1e-10, 1, hisq.prec("f32", 18), 64
+        x = torch.zeros_like(b)
+        for _ in range(3):  # whatever an earlier solve left in the kept buffers
+            solve(ctx, (8, 8, 8, 8), 0.1, synth.spinor((8, 8, 8, 8), 1004, device="cuda"), "int20")
+            try:
+                hisq.hisq_cg(ctx, g, p, b, x)
+            except hisq.HisqError as e:
+                assert "EBREAKDOWN" in str(e)
+            assert bool(torch.isfinite(x).all())
+    finally:
+        hisq.hisq_free_gauge(ctx, g)
 
 
 def test_waits_end(ctx):
