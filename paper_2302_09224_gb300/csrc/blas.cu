@@ -292,7 +292,15 @@ __global__ void __launch_bounds__(kBlock) norm2_kernel(BlasArgs a)
     reduce_grid<1>(v, a.red, tot);
 }
 
-int nblk(int n) { return (n + kBlock - 1) / kBlock; }
+// Threads a block of the one-site-a-thread kernels, whose FP64 operations a few
+// SMs would otherwise do alone: down to 64 while blocks of more leave SMs idle.
+int threads_for(int n)
+{
+    int b = kBlock;
+    while (b > 64 && (n + b - 1) / b < 152) b /= 2;
+    return b;
+}
+int nblk(int n) { return (n + threads_for(n) - 1) / threads_for(n); }
 
 }  // namespace
 
@@ -389,25 +397,25 @@ void launch_p_update(int sf, int cf, const BlasArgs &a, cudaStream_t s)
 void launch_x_flush(int sf, int cf, const BlasArgs &a, cudaStream_t s)
 {
     if (sf == S_INT30 && cf == HISQ_COMPUTE_F64) {  // the increment in FP32 pairs, not on the FP64 pipe
-        launch_chained(x_flush_kernel<S_INT30, ff>, dim3(nblk(a.n)), dim3(kBlock), s, a);
+        launch_chained(x_flush_kernel<S_INT30, ff>, dim3(nblk(a.n)), dim3(threads_for(a.n)), s, a);
         return;
     }
-    HISQ_SF_DISPATCH(sf, cf, x_flush_kernel, dim3(nblk(a.n)), dim3(kBlock), s);
+    HISQ_SF_DISPATCH(sf, cf, x_flush_kernel, dim3(nblk(a.n)), dim3(threads_for(a.n)), s);
 }
 
 void launch_true_residual(int sf, int cf, const BlasArgs &a, cudaStream_t s)
 {
-    HISQ_SF_DISPATCH(sf, cf, true_residual_kernel, dim3(nblk(a.n)), dim3(kBlock), s);
+    HISQ_SF_DISPATCH(sf, cf, true_residual_kernel, dim3(nblk(a.n)), dim3(threads_for(a.n)), s);
 }
 
 void launch_p_reliable(int sf, int cf, const BlasArgs &a, cudaStream_t s)
 {
-    HISQ_SF_DISPATCH(sf, cf, p_reliable_kernel, dim3(nblk(a.n)), dim3(kBlock), s);
+    HISQ_SF_DISPATCH(sf, cf, p_reliable_kernel, dim3(nblk(a.n)), dim3(threads_for(a.n)), s);
 }
 
 void launch_norm2(const BlasArgs &a, cudaStream_t s)
 {
-    launch_chained(norm2_kernel, dim3(nblk(a.n)), dim3(kBlock), s, a);
+    launch_chained(norm2_kernel, dim3(nblk(a.n)), dim3(threads_for(a.n)), s, a);
 }
 
 }  // namespace hisq

@@ -685,6 +685,102 @@ __global__ void __launch_bounds__(stencil_block(CFG), stencil_minb(CFG))
     }
 }
 
+// FP64 passes with S lanes a site (one or more directions each, summed by
+// shuffles).  The FP64 pipe takes 64 cycles a warp instruction on each of an SM's
+// four partitions, so a pass takes as long as the partition with the most warps:
+// a site a thread leaves one to four warps on each at 8^4 to 16^3x32 (four where
+// 3.4 is the mean at 16^3x32: the FP64 entry point took 109 us there, 89 with two
+// lanes; 8^4 with four lanes 8 us a pass by ncu, 18 before).
+// OUT: the pass to the caller's array (see dslash_out_kernel), FULL: both parities.
+template <int LREC, int S, bool OUT, bool FULL>
+__global__ void __launch_bounds__(128, 4) dslash_lanes_kernel(const __grid_constant__ DslashArgs a)
+{
+    __shared__ __align__(16) double sh[OUT ? 128 / S : 1][6];
+    pdl_wait();
+    pdl_launch_dependents();
+    if (OUT ? *(volatile const int *)a.bad != 0 : a.active != nullptr && *(volatile const int *)a.active == 0)
+        return;  // uniform over the grid
+    const Geom &g = a.g;
+    const int vh = g.vh;
+    const size_t pstride = (size_t)8 * vh * 16;
+    const StencilIO io = FULL ? stencil_io_full(a) : stencil_io(a);
+    const int group = (int)(blockIdx.x * (blockDim.x / S) + threadIdx.x / S), lane_s = threadIdx.x % S;
+    const int cb = group < vh ? group : vh - 1;  // idle groups repeat the last site
+    int r = cb / g.xh;
+    const int xh = cb - r * g.xh;
+    const int y = r % g.L[1];
+    r /= g.L[1];
+    const int z = r % g.L[2];
+    const int t = r / g.L[2];
+    const int x = 2 * xh + ((y + z + t + io.po) & 1);
+    const int lex = 2 * cb + (x & 1);
+    SiteAccScalar<double> acc;
+    acc.zero();
+#pragma unroll
+    for (int k = 0; k < 4 / S; k++) {
+        const int mu = lane_s * (4 / S) + k;
+        const int cmu = mu == 0 ? x : mu == 1 ? y : mu == 2 ? z : t;
+        const int phase_sum = mu == 0 ? 0 : mu == 1 ? x : mu == 2 ? x + y : x + y + z;
+        stencil_direction<G_F64, S_F64, double, LREC>(a, io.in, mu, cmu, t, lex, cb, io.po, pstride, 1.0, 1.0, phase_sum,
+                                                      acc);
+    }
+    double o[6];
+#pragma unroll
+    for (int k = 0; k < 6; k++) {
+        o[k] = acc.get(k);
+#pragma unroll
+        for (int off = 1; off < S; off *= 2) o[k] += __shfl_xor_sync(0xffffffffu, o[k], off);
+    }
+    const double sg = (double)a.sign;
+    if (a.xpay) {
+        double yv[6];
+        Spinor<S_F64>::load(io.y, vh, cb, yv);
+#pragma unroll
+        for (int k = 0; k < 6; k++) o[k] = a.a * yv[k] + sg * o[k];
+    } else {
+#pragma unroll
+        for (int k = 0; k < 6; k++) o[k] *= sg;
+    }
+    bool ok = true;
+#pragma unroll
+    for (int k = 0; k < 6; k++) ok = ok && isfinite(o[k]);
+    const bool lead = group < vh && lane_s == 0;
+    if constexpr (OUT) {
+        if (lead && !ok) *(volatile int *)a.err = 1;
+        if (lane_s == 0)
+#pragma unroll
+            for (int k = 0; k < 6; k++) sh[threadIdx.x / S][k] = o[k];
+        __syncthreads();
+        const int g0 = (int)(blockIdx.x * (blockDim.x / S));
+        const int m = 6 * (vh - g0 < (int)blockDim.x / S ? vh - g0 : (int)blockDim.x / S);
+        double *out = a.out64 + (FULL ? (size_t)blockIdx.y * 6 * vh : 0) + (size_t)6 * g0;
+        for (int j = threadIdx.x; j < m; j += blockDim.x) out[j] = sh[0][j];
+    } else if (lead) {
+        Spinor<S_F64>::store(io.out, vh, cb, o);
+        if (!ok) atomicExch(a.err, 1);
+    }
+}
+
+// Lanes a site of an FP64 pass over n sites: the fewest of 1, 2 and 4 whose
+// fullest partition (608 of them) has at most 6 % more than the mean, else the
+// ones with the least.
+inline int f64_lanes(long long n)
+{
+    constexpr long long parts = 608;
+    int best = 1;
+    double least = 1e30;
+    for (int s = 1; s <= 4; s *= 2) {
+        const long long w = (n * s + 31) / 32;
+        const double over = (double)((w + parts - 1) / parts * parts) / (double)w;
+        if (over < least) {
+            least = over;
+            best = s;
+        }
+        if (least <= 1.06) break;
+    }
+    return best;
+}
+
 // The pass whose output goes to the caller: the site is rounded to the storage
 // format as the other passes store it, decoded and written as FP64 [site][6]
 // (a separate unpack pass read the stored field again and wrote it: at
@@ -820,9 +916,27 @@ void launch_out(int cfg, const DslashArgs &a, cudaStream_t s)
     }
 }
 
+template <int LREC, int S>
+void launch_lanes(const DslashArgs &a, cudaStream_t s)
+{
+    constexpr int B = 64;  // finer blocks even out the SMs' shares
+    const int nb = (a.g.vh + B / S - 1) / (B / S);
+    if (a.out64 == nullptr)
+        launch_chained(dslash_lanes_kernel<LREC, S, false, false>, dim3(nb), dim3(B), s, a);
+    else if (a.half_bytes)
+        launch_chained(dslash_lanes_kernel<LREC, S, true, true>, dim3(nb, 2), dim3(B), s, a);
+    else
+        launch_chained(dslash_lanes_kernel<LREC, S, true, false>, dim3(nb), dim3(B), s, a);
+}
+
 template <int GF, int SF, typename real, int LREC, bool RED>
 void launch_any(int cfg, const DslashArgs &a, cudaStream_t s)
 {
+    if constexpr (!RED && GF == G_F64) {
+        const int lanes = a.dot == nullptr ? f64_lanes((long long)a.g.vh * (a.out64 != nullptr && a.half_bytes ? 2 : 1)) : 1;
+        if (lanes == 4) return launch_lanes<LREC, 4>(a, s);
+        if (lanes == 2) return launch_lanes<LREC, 2>(a, s);
+    }
     if constexpr (!RED) {
         if (a.out64 != nullptr) {
             launch_out<GF, SF, real, LREC>(cfg, a, s);
