@@ -32,6 +32,18 @@ __device__ __forceinline__ bool skip(const int *active)
     return active != nullptr && *(volatile const int *)active == 0;
 }
 
+// a compute-precision value as FP64 and back, off the conversion instructions
+__device__ __forceinline__ double widen(float v) { return f2d_bits(v); }
+__device__ __forceinline__ double widen(double v) { return v; }
+template <typename real>
+__device__ __forceinline__ real narrow(double v)
+{
+    if constexpr (std::is_same<real, float>::value)
+        return d2f_bits(v);
+    else
+        return v;
+}
+
 __device__ __forceinline__ bool nonzero(float v) { return v != 0.0f; }
 __device__ __forceinline__ bool nonzero(double v) { return v != 0.0; }
 __device__ __forceinline__ bool nonzero(ff v) { return v.hi != 0.0f || v.lo != 0.0f; }
@@ -209,7 +221,7 @@ __global__ void __launch_bounds__(kBlock) x_flush_kernel(BlasArgs a)
         if constexpr (is_ff<real>::value)  // hi and lo widened on the integer pipe: two FP64 adds per real
             x[k] += f2d_bits(dx[k].hi) + f2d_bits(dx[k].lo);
         else
-            x[k] += (double)dx[k];
+            x[k] += widen(dx[k]);
     }
     Spinor<S_F64>::store(reinterpret_cast<char *>(a.x64), a.n, i, x);
 }
@@ -238,7 +250,7 @@ __global__ void __launch_bounds__(kBlock) true_residual_kernel(BlasArgs a)
         Spinor<SF>::load(a.v1, a.n, i, p);
 #pragma unroll
         for (int c = 0; c < 3; c++) {
-            const double rr = r[2 * c], ri = r[2 * c + 1], pr = p[2 * c], pi = p[2 * c + 1];
+            const double rr = r[2 * c], ri = r[2 * c + 1], pr = widen(p[2 * c]), pi = widen(p[2 * c + 1]);
             v[0] += rr * rr + ri * ri;
             v[1] += rr * pr + ri * pi;  // Re conj(r) p
             v[2] += rr * pi - ri * pr;  // Im conj(r) p
@@ -270,8 +282,8 @@ __global__ void __launch_bounds__(kBlock) p_reliable_kernel(BlasArgs a)
     const double cr = a.st->coef_re, ci = a.st->coef_im, beta = a.st->beta;
 #pragma unroll
     for (int c = 0; c < 3; c++) {
-        o[2 * c] = (real)(cr * r[2 * c] - ci * r[2 * c + 1] + beta * (double)p[2 * c]);
-        o[2 * c + 1] = (real)(cr * r[2 * c + 1] + ci * r[2 * c] + beta * (double)p[2 * c + 1]);
+        o[2 * c] = narrow<real>(cr * r[2 * c] - ci * r[2 * c + 1] + beta * widen(p[2 * c]));
+        o[2 * c + 1] = narrow<real>(cr * r[2 * c + 1] + ci * r[2 * c] + beta * widen(p[2 * c + 1]));
     }
     if (!Spinor<SF>::store(a.v2, a.n, i, o)) atomicExch(a.err, 1);
 }

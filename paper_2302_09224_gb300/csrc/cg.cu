@@ -209,7 +209,7 @@ struct CGRun {
         }
         cudaMemsetAsync(ring, 0, sb * cfg.nbuf, s);
         diag = 4.0 * cfg.mass * cfg.mass + cfg.sigma;
-        tune_stencil(c, g->geom, cfg.sloppy, gv_s, ap_s, tmp_s, s);
+        if (resident.lanes == 0) tune_stencil(c, g->geom, cfg.sloppy, gv_s, ap_s, tmp_s, s);
         tune_stencil(c, g->geom, prec_f64(), gv_d, (char *)ax64, (char *)tmp64, s);
         return HISQ_OK;
     }
@@ -235,17 +235,18 @@ struct CGRun {
         launch_x_flush(cfg.sloppy.spinor, cfg.sloppy.compute, a, s);
     }
 
-    // True residual and restart of the recurrence from p in slot j into slot 0.
-    hisq_status reliable_update(const double *b64, double *x64, bool x_zero, int j)
+    // True residual and restart of the recurrence from p in slot j into slot 0.  ax: A x where the caller
+    // has it (null: applied here).
+    hisq_status reliable_update(const double *b64, double *x64, bool x_zero, int j, const double *ax = nullptr)
     {
-        if (!x_zero) {
+        if (!x_zero && ax == nullptr) {
             apply_mee(c, g->geom, prec_f64(), gv_d, diag, (const char *)x64, (char *)tmp64, (char *)ax64, FIN_NONE,
                       nullptr, 0, nullptr, PROF_STENCIL_HI, s);
             mv_hi++;
         }
         BlasArgs a = blas();
         a.b64 = b64;
-        a.ax64 = x_zero ? nullptr : ax64;
+        a.ax64 = x_zero ? nullptr : ax != nullptr ? ax : ax64;
         a.r64 = r64;
         a.v0 = r_s;
         a.v1 = slot(j);
@@ -384,7 +385,7 @@ struct CGRun {
             init.rr_prev = cfg.rr_prev_init;
         }
         cudaMemcpyAsync(st, &init, sizeof init, cudaMemcpyHostToDevice, s);
-        e = reliable_update(b64, x64, x_zero, 0);
+        e = reliable_update(b64, x64, x_zero, 0, cfg.ax_init);
         if (e) return e;
         hisq_status status = HISQ_OK;
         bool done = st_h->hi_rr <= init.stop2;

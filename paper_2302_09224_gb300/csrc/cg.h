@@ -33,6 +33,7 @@ struct CGConfig {
     const char *p_init = nullptr;
     int p_init_fmt = 0;
     double rr_prev_init = 0.0;
+    const double *ax_init = nullptr;  // A x of the initial guess, FP64 planar, where the caller has it
     // error-estimate reliable-update trigger (dyn = 1) with the sloppy precision dyn_eps
     int dyn = 0;
     double dyn_eps = 0.0;

@@ -72,6 +72,14 @@ __device__ __forceinline__ float i16hi_to_f(uint32_t w)
     return f;
 }
 
+// Both halves of a word off the conversion unit: each placed, sign bit flipped,
+// in the mantissa of 2^23, the offset 2^23 + 2^15 subtracted (exact).
+__device__ __forceinline__ float2 i16pair_to_f(uint32_t w)
+{
+    const float lo = __uint_as_float((w & 0xffffu) ^ 0x4B008000u), hi = __uint_as_float((w >> 16) ^ 0x4B008000u);
+    return __fadd2_rn(make_float2(lo, hi), make_float2(-8421376.0f, -8421376.0f));
+}
+
 // 20-bit fields, exact on the FP32 and integer pipes: the two's-complement
 // field u, offset by 2^19, is placed in the mantissa of 2^23 and the offset
 // is subtracted; both operands are integers below 2^24, so the subtraction
@@ -908,7 +916,11 @@ struct Link {
         }
     }
 
-    template <typename real>
+    // KEEP (links that stay in L2): the kernel is then bound by instructions and the conversion unit (four
+    // lanes a clock a partition), not by HBM, so the 18-real 16-bit links take the FP32 and integer pipes;
+    // resident CG iterations, 16-bit 16^4: 13.2 -> 12.4 ms a solve, 20-bit 16^3x32 20.9 -> 20.4 us an
+    // iteration.  Streamed links (32^3x64 solve) lose by it: 620 -> 641 ms.
+    template <typename real, bool KEEP = false>
     __device__ static void decode(const uint4 c[chunks], real U[18])
     {
         if constexpr (GF == G_F64) {
@@ -958,6 +970,10 @@ struct Link {
                     if constexpr (sizeof(real) == 8) {
                         U[2 * k] = (double)(int)(short)(w[k] & 0xffffu);
                         U[2 * k + 1] = (double)((int)w[k] >> 16);
+                    } else if constexpr (RECON == 18 && KEEP) {
+                        const float2 f = i16pair_to_f(w[k]);
+                        U[2 * k] = f.x;
+                        U[2 * k + 1] = f.y;
                     } else {
                         U[2 * k] = i16lo_to_f(w[k]);
                         U[2 * k + 1] = i16hi_to_f(w[k]);
@@ -993,7 +1009,7 @@ struct Link {
     {
         uint4 c[chunks];
         gather<KEEP>(base, pstride, li, c);
-        decode(c, U);
+        decode<real, KEEP>(c, U);
         if constexpr (kPhase) U[12] = phase<real>(c);
     }
 };

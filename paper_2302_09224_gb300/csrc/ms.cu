@@ -610,30 +610,24 @@ struct MSRun {
         info->matvecs += mh->k;
         info->reliable_updates += ru;
         for (int i = 0; i < ns; i++) info->shift_iters[i] = mh->live[i] ? mh->k : mh->frozen_at[i];
-        // FP64 true residual of every shift after the multi-shift stage (Table 3's r_sigma)
-        std::vector<double> rs(ns);
+        // FP64 true residual of every shift after the multi-shift stage (Table 3's r_sigma), then its refinement:
+        // the base system keeps its gradient vector, the others restart
+        const double rr_base = mh->rr;
+        const bool refining = status != HISQ_EBREAKDOWN && refine;
+        hisq_status worst = status;
         for (int i = 0; i < ns; i++) {
             residual(i, FIN_STORE, nullptr);
             double rr = 0;
             cudaMemcpyAsync(&rr, cur_red(c).result, sizeof rr, cudaMemcpyDeviceToHost, s);
             if (cudaStreamSynchronize(s) != cudaSuccess) return cuda_fail(c, cudaGetLastError(), "residual");
-            rs[i] = std::sqrt(rr / bb);
-            info->shift_resid_ms[i] = rs[i];
-            info->shift_resid[i] = rs[i];
-        }
-        if (status == HISQ_EBREAKDOWN || !refine) {
-            info->matvecs_hi += mv_hi;
-            info->true_residual = info->shift_resid[0];
-            return status;
-        }
-        const double rr_base = mh->rr;
-        // refinement: the base system keeps its gradient vector, the others restart
-        hisq_status worst = status;
-        for (int i = 0; i < ns; i++) {
-            if (rs[i] <= tol[i]) continue;
+            const double rs = std::sqrt(rr / bb);
+            info->shift_resid_ms[i] = rs;
+            info->shift_resid[i] = rs;
+            if (!refining || rs <= tol[i]) continue;
             CGConfig cfg = config_from(&p, sig[i]);
             cfg.sloppy = p.refine;
             cfg.tol = tol[i];
+            cfg.ax_init = ax64;  // A x_i, just applied
             if (i == 0) {
                 cfg.p_init = pf(0);
                 cfg.p_init_fmt = p.sloppy.spinor;
@@ -651,6 +645,11 @@ struct MSRun {
             } else if (st != HISQ_OK) {
                 return st;
             }
+        }
+        if (!refining) {
+            info->matvecs_hi += mv_hi;
+            info->true_residual = info->shift_resid[0];
+            return status;
         }
         info->matvecs_hi += mv_hi;
         info->true_residual = info->shift_resid[0];
