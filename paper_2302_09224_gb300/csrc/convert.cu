@@ -205,13 +205,17 @@ __device__ __forceinline__ float r12_dev_ff(const ff u[18], float sign)
     return m;
 }
 
-__device__ __forceinline__ float u3_dev_ff(const ff u[18])
+// near: row 2 is the product of rows 0 and 1 to 1e-8.  Then U U^+ follows from
+// the first two rows (each further entry is off by at most a few times theirs
+// plus the row's own deviation), and only the first three pairs are formed.
+__device__ __forceinline__ float u3_dev_ff(const ff u[18], bool near)
 {
     float m = 0.0f;
 #pragma unroll
-    for (int i = 0; i < 3; i++)
+    for (int j = 0; j < 3; j++)
 #pragma unroll
-        for (int j = i; j < 3; j++) {  // (j, i) is its conjugate
+        for (int i = 0; i <= j; i++) {  // (j, i) is its conjugate
+            if (j == 2 && near && m < 1e-8f) continue;
             ff re(i == j ? -1.0f : 0.0f), im(0.0f);
 #pragma unroll
             for (int k = 0; k < 3; k++) {
@@ -279,7 +283,7 @@ __global__ void __launch_bounds__(kLinkBlock) gauge_scan_kernel(Geom g, const do
             bad12 = !(isfinite(d) && d <= kCompressTol);
         }
         if constexpr (LONG) {
-            const float d3 = u3_dev_ff(w);
+            const float d3 = u3_dev_ff(w, d12 < 1e-8f);
             bad3 = big || !(d3 < lo);
             if (bad3 && (big || d3 <= hi)) {
                 const double d = u3_dev64(u);
@@ -307,6 +311,27 @@ __global__ void __launch_bounds__(kLinkBlock) gauge_scan_kernel(Geom g, const do
 // FP64 [mu][lex][18] -> stored copy [plane][parity][mu][Vh] in format GF with
 // RECON reals per link.  Fixed point: q = rint(x * inv) clamped to +-qmax,
 // inv = qmax / global max (Sec. 2 footnote; Sec. 4 for 32 bits).
+// rint(fl(x inv)) for |x inv| <= 32767 (1 + 2^-52) without FP64 arithmetic, which
+// bounded the 16-bit quantisation (two operations a real, 44 us for 524288
+// 18-real links): the product in FP32 pairs is within 2^-30 of x inv, so its
+// nearest integer is the one wanted unless it lies that close to a tie, where
+// the FP64 rounding decides.
+// (The FP64 form is a function of its own, not inlined: written in place it is
+// evaluated for every real and then selected.)
+__device__ __noinline__ int quantise_f64(double x, double inv)
+{
+    return __double2loint(__dadd_rn(__dmul_rn(x, inv), 6755399441055744.0));
+}
+
+__device__ __forceinline__ int quantise16(double x, double inv, ff inv_ff)
+{
+    const ff v = d2ff_bits(x) * inv_ff;
+    const float t = __fadd_rn(v.hi, 12582912.0f);  // 1.5 2^23: its low bits are v.hi's nearest integer
+    const float rest = __fadd_rn(__fsub_rn(v.hi, __fsub_rn(t, 12582912.0f)), v.lo);
+    if (fabsf(fabsf(rest) - 0.5f) < 1e-6f) return quantise_f64(x, inv);
+    return (int)__float_as_uint(t) - 0x4B400000 + (rest > 0.5f ? 1 : rest < -0.5f ? -1 : 0);
+}
+
 // A thread a link in the caller's order, so that both the reads (through shared
 // memory) and the writes (16 consecutive links of each parity a warp) are full
 // lines.  The fixed-point integers take two FP64 operations a real: the product,
@@ -416,15 +441,16 @@ __global__ void __launch_bounds__(kLinkBlock) quantise_kernel(Geom g, const doub
                 make_uint2(h[8 * n16] | (h[8 * n16 + 1] << 16), h[8 * n16 + 2] | (h[8 * n16 + 3] << 16));
     } else {
         constexpr double qmax = GF == G_FIX16 ? 32767.0 : 2147483647.0;
-        // |x inv| <= qmax (1 + 2^-52), so the rounded product stays within +-qmax (clamped where the field is
-        // so small that inv overflowed)
+        // |x inv| <= qmax (1 + 2^-52), so the rounded product stays within +-qmax
         int q[RECON];
-        if (isinf(inv)) {
+        const ff inv_ff = GF == G_FIX16 ? d2ff_bits(inv) : ff(0.0f);
+        if (!(inv < 1e12)) {  // a field so small that inv overflows, or that a real's tail would leave FP32's range
             for (int k = 0; k < RECON; k++) q[k] = (int)fmin(qmax, fmax(-qmax, rint(__dmul_rn(src[k], inv))));
         } else {
 #pragma unroll
             for (int k = 0; k < RECON; k++)
-                q[k] = __double2loint(__dadd_rn(__dmul_rn(src[k], inv), 6755399441055744.0));
+                q[k] = GF == G_FIX16 ? quantise16(src[k], inv, inv_ff)
+                                     : __double2loint(__dadd_rn(__dmul_rn(src[k], inv), 6755399441055744.0));
         }
         if constexpr (GF == G_FIX16) {
             for (int k = 0; k < n16; k++) {

@@ -85,3 +85,56 @@ def test_large_links_are_decided_in_fp64(ctx):
     assert accepted(ctx, dims, fat.cuda(), lng.cuda(), 12)
     lng[1, 2, 1, 0, 3, 2, 2, 0] += 1e-3
     assert not accepted(ctx, dims, fat.cuda(), lng.cuda(), 12)
+
+
+@pytest.mark.parametrize("gmax", [1.0, 0.7310585786300049, 3.0e5, 2.0 ** -40, 1e-300, 5e-306])
+def test_sixteen_bit_integers_are_the_fp64_rule(ctx, gmax):
+    """q = rint(fl(x * fl(32767 / gmax))) in FP64 for every element, ties and neighbours of ties among them,
+    read back through the stencil: with one link element per site non-zero and a source that picks it,
+    the FP32 output is q * scale exactly representable."""
+    dims = (4, 4, 4, 4)
+    rng = np.random.default_rng(1)
+    fat = np.zeros((4, 4, 4, 4, 4, 3, 3, 2))
+    inv = np.float64(32767.0) / np.float64(gmax)
+    k = rng.integers(-32767, 32767, (4, 4, 4, 4))
+    off = rng.choice([0.5, 0.5 - 2.0 ** -36, 0.5 + 2.0 ** -36, 0.5 - 2.0 ** -21, 0.25, 0.0], k.shape)
+    with np.errstate(over="ignore", invalid="ignore"):
+        v = (k + off) / inv if np.isfinite(inv) else rng.choice([gmax, -gmax, gmax / 3, 0.0], k.shape)
+    fat[0, ..., 0, 0, 0] = v
+    fat[1, 0, 0, 0, 0, 2, 2, 1] = gmax  # the field's largest element
+    lng = synth.unit_gauge(dims, 1.0, long_link=True).numpy() * 0.0
+    lng[...] = 0.0
+    with np.errstate(over="ignore", invalid="ignore"):
+        want = np.clip(np.where(np.isnan(fat * inv), -32767.0, np.rint(fat * inv)), -32767, 32767)[0, ..., 0, 0, 0]
+    g = hisq.hisq_load_gauge(ctx, dims, torch.from_numpy(fat).cuda(), torch.from_numpy(lng).cuda())
+    try:
+        t, z, y, x = np.meshgrid(*(np.arange(4),) * 4, indexing="ij")
+        even = (x + y + z + t) % 2 == 0
+        # source 1 on colour 0 of every odd site: out(even, 0) = F_0(x) - F_0(x - 1), and the row of links on the
+        # even sites alone is recovered with the odd sites' set to zero in a second field
+        fat2 = fat.copy()
+        fat2[0, ~even] = 0.0
+        g2 = hisq.hisq_load_gauge(ctx, dims, torch.from_numpy(fat2).cuda(), torch.from_numpy(lng).cuda())
+        try:
+            src = torch.zeros((128, 3, 2), dtype=torch.float64, device="cuda")
+            src[:, 0, 0] = 1.0
+            out = torch.empty_like(src)
+            torch.cuda.synchronize()
+            scale = np.float32(np.float64(gmax) / 32767.0)
+            if scale == 0:  # below FP32: the pass's scale vanishes and with it the ratio of the fields' scales
+                with pytest.raises(hisq.HisqError, match="ERANGE"):
+                    hisq.hisq_dslash(ctx, g2, hisq.prec("half", 18), 0, 0.0, None, src, out, True)
+                return
+            hisq.hisq_dslash(ctx, g2, hisq.prec("half", 18), 0, 0.0, None, src, out, True)
+            got = out.cpu().numpy()[:, 0, 0]
+        finally:
+            hisq.hisq_free_gauge(ctx, g2)
+        w = want.reshape(-1)[even.reshape(-1)]
+        # the stencil's 16-bit store keeps the largest component of a site to 2^-16 of itself (here the only one)
+        ref = w * np.float64(scale)
+        assert np.all(np.abs(got - ref) <= 2.0 ** -15 * np.abs(ref))
+        # neighbouring integers differ by more than that below 2^14: there the integer itself is determined
+        small = np.abs(w) < 2 ** 14
+        assert np.array_equal(np.rint(got[small] / np.float64(scale)), w[small])
+    finally:
+        hisq.hisq_free_gauge(ctx, g)
