@@ -491,9 +491,14 @@ struct Spinor<S_INT30> {
 #pragma unroll
             for (int k = 0; k < 6; k++) v[k] = ff_scale(ff_from_int(q[k]), up);
         } else if constexpr (sizeof(real) == 8) {
-            const double up = __longlong_as_double((long long)(E + 896u) << 52);  // 2^(E-127)
 #pragma unroll
-            for (int k = 0; k < 6; k++) v[k] = __dmul_rn((double)q[k], up);
+            for (int k = 0; k < 6; k++) {  // q 2^(E-127), exact: its bits put together (no FP64 instruction)
+                const uint32_t mag = q[k] < 0 ? 0u - (uint32_t)q[k] : (uint32_t)q[k];
+                const int lz = __clz((int)mag);
+                const uint32_t frac = (mag << (lz & 31)) << 1;  // below the leading one
+                const uint32_t hi = ((uint32_t)q[k] & 0x80000000u) | ((E + 927u - (uint32_t)lz) << 20) | (frac >> 12);
+                v[k] = mag == 0u ? 0.0 : __hiloint2double((int)hi, (int)(frac << 20));
+            }
         } else {
             const float up = __uint_as_float(E << 23);
 #pragma unroll
@@ -632,28 +637,44 @@ struct Spinor<S_INT30> {
     {
         if constexpr (std::is_same<real, float>::value) return encode_f32(v, c);
         if constexpr (is_ff<real>::value) return encode_ff(v, c);
-        double d[6];
-        double mx = 0.0;
+        // the rule of the format in FP64, t = max / (2^29 - 1), E from t's exponent, q = rint(v 2^-(E-127)), on
+        // the integer pipe (its divisions, products and conversions at the FP64 rate took several times the
+        // site's bytes).  t's exponent is max's less 29, or less 28 from max = (2^29 - 1) 2^n on, where the
+        // correctly rounded quotient reaches the power of two: the top 28 fraction bits all ones.
+        uint32_t mh = 0, ml = 0;  // largest magnitude
         bool ok = true;
+        uint32_t h[6], l[6];
 #pragma unroll
         for (int k = 0; k < 6; k++) {
-            d[k] = (double)v[k];
-            ok = ok && isfinite(d[k]);
-            mx = fmax(mx, fabs(d[k]));
+            const double x = (double)v[k];
+            h[k] = (uint32_t)__double2hiint(x);
+            l[k] = (uint32_t)__double2loint(x);
+            const uint32_t a = h[k] & 0x7fffffffu;
+            ok = ok && a < 0x7ff00000u;
+            const bool more = a > mh || (a == mh && l[k] > ml);
+            mh = more ? a : mh;
+            ml = more ? l[k] : ml;
         }
         uint32_t E = 1;
         uint32_t u[6] = {0, 0, 0, 0, 0, 0};
         if (ok) {
-            const double t = __ddiv_rn(mx, 536870911.0);
-            const int biased = (int)((__double_as_longlong(t) >> 52) & 0x7ff);
-            int e = (t > 0.0 && biased > 0) ? biased - 895 : 1;  // frexp exponent + 127
+            const uint32_t top = ((mh & 0xfffffu) << 8) | (ml >> 24);
+            int e = (int)(mh >> 20) - 29 + (top == 0xfffffffu ? 1 : 0) - 895;  // frexp exponent + 127
             if (e < 1) e = 1;
             if (e > 254) ok = false;
             if (ok) {
                 E = (uint32_t)e;
-                const double down = __longlong_as_double((long long)(1150 - e) << 52);  // 2^-(E-127)
 #pragma unroll
-                for (int k = 0; k < 6; k++) u[k] = (uint32_t)(int32_t)__double2ll_rn(__dmul_rn(d[k], down));
+                for (int k = 0; k < 6; k++) {
+                    // v 2^-(E-127) = M 2^-s, M the 53-bit significand
+                    const int eb = (int)((h[k] >> 20) & 0x7ffu), sft = 948 - eb + e;
+                    uint32_t q = 0;
+                    if (eb > 0 && sft <= 53) {
+                        const uint64_t M = ((uint64_t)((h[k] & 0xfffffu) | 0x100000u) << 32) | l[k];
+                        q = (uint32_t)((M + ((1ull << (sft - 1)) - 1ull) + ((M >> sft) & 1ull)) >> sft);
+                    }
+                    u[k] = (h[k] & 0x80000000u) ? 0u - q : q;
+                }
             }
         }
         pack(c, E, u);
