@@ -18,7 +18,10 @@ OBJ = os.path.join(ROOT, "_build", "obj")
 LIB = os.path.join(HERE, "libhisq.so")
 
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
-NVFLAGS = ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", "-Xcompiler", "-fvisibility=hidden",
+# Device code stays uncompressed: above some size nvcc compresses a unit's code,
+# and the first kernel a process takes from it then waits 12 ms for that unit
+# (first hisq_dslash of a process, 20-bit at 8^4: 2585 us against 14352 us).
+NVFLAGS = ["-O3", "-lineinfo", "--no-compress", "-std=c++17", "-Xcompiler", "-fPIC", "-Xcompiler", "-fvisibility=hidden",
            "--expt-relaxed-constexpr", f"-I{INCLUDE}", f"-I{CSRC}"]
 
 

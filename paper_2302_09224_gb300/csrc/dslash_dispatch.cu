@@ -173,8 +173,9 @@ void tune_variant(int gf, int sf, int cf, int lrec, bool red, const DslashArgs &
         }
     }
     // three passes of 10 us are noisy: the two fastest are timed again, in turn (16^3x32 solves differed by
-    // up to 13 % between processes by the shape picked)
-    if (second >= 0 && ms_of[second] < 1.15f * ms_of[best]) {
+    // up to 13 % between processes by the shape picked).  From 40 us a pass on the first look decides: 16 more
+    // passes would cost a first call more than they tell it (FP64 16^3x32: 6.5 ms against 4.1 without).
+    if (second >= 0 && ms_of[best] < 0.04f && ms_of[second] < 1.15f * ms_of[best]) {
         float b2 = 1e30f, s2 = 1e30f;
         for (int r = 0; r < 2; r++) {
             b2 = std::min(b2, time_shape(best, 4));
