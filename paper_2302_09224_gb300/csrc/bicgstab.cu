@@ -12,6 +12,7 @@
 // previous one, or when the iterated residual meets the target.
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <chrono>
 #include <cmath>
 #include <type_traits>
@@ -31,7 +32,8 @@ namespace {
 constexpr int kMaxL = 8;
 constexpr int kBlock = 256;
 constexpr int kMaxBlocks = 304;   // blocks with sites of the vector kernels (two a SM; more rows cost the next kernel's sums)
-constexpr int kGroup = 4;         // fields of a kind whose loads a thread issues before it stores any
+constexpr int kGroup = 4;         // fields of a kind whose loads a thread issues before it stores any (template
+                                  // argument G of the u and r updates: one on large lattices, more threads instead)
 constexpr int kMaxRows = 4096;    // stencil block sums that the next kernel's blocks sum themselves
 
 struct BState {
@@ -157,19 +159,29 @@ __device__ __forceinline__ void dot_site(const real x[6], const real y[6], real 
     }
 }
 
-// The dot sums of many rows once, into the state (one block): a large lattice's stencil pass, whose rows
-// every block of the next kernel would read.
+// The dot sums of many rows once, into the state: a large lattice's stencil pass, whose rows every block of
+// the next kernel would read.  FP32 rows are summed in FP32 pairs.
 template <typename T>
-__global__ void __launch_bounds__(1024) dot_rows_kernel(BArgs a)
+__global__ void __launch_bounds__(kBlock) dot_rows_kernel(BArgs a)
 {
+    using V = std::conditional_t<std::is_same<T, double>::value, double, ff>;
     pdl_wait();
     pdl_launch_dependents();
     if (skip(a.active)) return;
+    const T *part = reinterpret_cast<const T *>(a.part_in);
+    V v[3] = {V(0), V(0), V(0)};
+    for (int r = blockIdx.x * blockDim.x + threadIdx.x; r < a.rows; r += gridDim.x * blockDim.x)
+#pragma unroll
+        for (int k = 0; k < 3; k++) {
+            if constexpr (std::is_same<T, FF>::value) {
+                const float2 t = __ldcg(reinterpret_cast<const float2 *>(part) + (size_t)r * 3 + k);
+                v[k] = v[k] + ff(t.x, t.y);
+            } else {
+                v[k] = v[k] + V(__ldcg(part + (size_t)r * 3 + k));
+            }
+        }
     __shared__ double tot[3];
-    RedBuf rb{};
-    rb.partials = a.part_in;
-    sum_partials<3, T>(rb, (unsigned)a.rows, tot);
-    if (threadIdx.x == 0)
+    if (reduce_grid<3>(v, a.red, tot) && threadIdx.x == 0)
         for (int k = 0; k < 3; k++) a.b->dot[k] = tot[k];
 }
 
@@ -196,7 +208,7 @@ __global__ void __launch_bounds__(kBlock) dot_kernel(BArgs a, const char *v)
 
 // u_i = r_i - beta u_i, i = 0..j, with rho1 = <rt, r_j>, beta = alpha rho1 / rho0.
 // Breakdown: rho1 (nearly) orthogonal relative to |rt| |r_j|, or a rho0 too small to divide by.
-template <int SF, typename real>
+template <int SF, typename real, int G>
 __global__ void __launch_bounds__(kBlock) u_multi_kernel(BArgs a)
 {
     pdl_wait();
@@ -231,7 +243,7 @@ __global__ void __launch_bounds__(kBlock) u_multi_kernel(BArgs a)
     __syncthreads();
     if (!ok_sh || blockIdx.x == gridDim.x - 1) return;
     const real br = be_sh[0], bi = be_sh[1];
-    constexpr int G = kGroup, C = Spinor<SF>::chunks;
+    constexpr int C = Spinor<SF>::chunks;
     for (int s = blockIdx.x * blockDim.x + threadIdx.x; s < 2 * a.vh; s += (gridDim.x - 1) * blockDim.x) {
         const Site q = site_of(s, a.vh);
         const char *rf = a.R + q.h * a.hb;
@@ -264,7 +276,7 @@ __global__ void __launch_bounds__(kBlock) u_multi_kernel(BArgs a)
 
 // r_i -= alpha u_{i+1}, i = 0..j; x += alpha u_0 (FP64), with gamma = <rt, u_{j+1}>, alpha = rho / gamma;
 // breakdown relative to |rt| |u_{j+1}|
-template <int SF, typename real>
+template <int SF, typename real, int G>
 __global__ void __launch_bounds__(kBlock) r_multi_kernel(BArgs a)
 {
     pdl_wait();
@@ -295,15 +307,17 @@ __global__ void __launch_bounds__(kBlock) r_multi_kernel(BArgs a)
     __syncthreads();
     if (!ok_sh || blockIdx.x == gridDim.x - 1) return;
     const real ar = al_sh[0], ai = al_sh[1];
-    constexpr int G = kGroup, C = Spinor<SF>::chunks;
+    constexpr int C = Spinor<SF>::chunks;
     for (int s = blockIdx.x * blockDim.x + threadIdx.x; s < 2 * a.vh; s += (gridDim.x - 1) * blockDim.x) {
         const Site q = site_of(s, a.vh);
         // x += alpha u_0: the increment in the compute precision, the sum in FP64
         real u0[6];
         uint4 cx[Spinor<S_F64>::chunks];
         char *xf = reinterpret_cast<char *>(a.x64) + q.h * (size_t)48 * a.vh;
-        Spinor<SF>::load(a.U + q.h * a.hb, a.vh, q.i, u0);
-        Spinor<S_F64>::gather(xf, a.vh, q.i, cx);
+        if (G > 1) {
+            Spinor<SF>::load(a.U + q.h * a.hb, a.vh, q.i, u0);
+            Spinor<S_F64>::gather(xf, a.vh, q.i, cx);
+        }
         char *rf = a.R + q.h * a.hb;
         const char *uf = a.U + a.fb + q.h * a.hb;
         for (int i0 = 0; i0 <= a.j; i0 += G) {
@@ -328,6 +342,10 @@ __global__ void __launch_bounds__(kBlock) r_multi_kernel(BArgs a)
                 }
                 if (!Spinor<SF>::store(rf + (i0 + g) * a.fb, a.vh, q.i, r)) atomicExch(a.err, 1);
             }
+        }
+        if (G == 1) {
+            Spinor<SF>::load(a.U + q.h * a.hb, a.vh, q.i, u0);
+            Spinor<S_F64>::gather(xf, a.vh, q.i, cx);
         }
         double x[6];
         Spinor<S_F64>::decode(cx, x);
@@ -594,11 +612,17 @@ __global__ void restart_kernel(BState *b, const double *sum)
     if (!b->active) b->reason = REASON_BREAKDOWN;
 }
 
-// Blocks with sites of a vector kernel over the full lattice.
-int vec_blocks(int vh)
+// Blocks with sites of a vector kernel over the full lattice: kMaxBlocks at most where the next kernel's blocks
+// sum its rows or the stencil's; on large lattices (more stencil rows than kMaxRows, summed once) one full wave
+// with the scalars' block, since two blocks a SM leave too few loads in flight.  32^3x64, 20-bit, us a launch at
+// 304 blocks of four fields at once and here: u update 66.6 and 46.3, r update 107.5 and 78.0, Gram-Schmidt passes
+// 66.5, 66.1, 42.3 and 52.1, 57.4, 32.8 (16^3x32 keeps 304: more rows cost the next kernel more than they give)
+template <typename K>
+int vec_blocks(K kernel, int vh, bool large)
 {
     const int need = (2 * vh + kBlock - 1) / kBlock;
-    return need < kMaxBlocks ? need : kMaxBlocks;
+    const int most = large ? std::max(wave_blocks(kernel, kBlock) - 1, 1) : kMaxBlocks;
+    return need < most ? need : most;
 }
 
 // f(integral_constant<spinor format>, a value of the compute type)
@@ -661,6 +685,7 @@ struct BRun {
         return a;
     }
 
+    bool large() const { return dslash_full_rows(p.sloppy.gauge, vh) > kMaxRows; }
     double sbytes() const { return spinor_site_bytes(p.sloppy.spinor) * 2.0 * vh; }
 
     // out = 2m in + D in on the full lattice (two half-lattice passes)
@@ -693,7 +718,8 @@ struct BRun {
         a.active = act;
         LaunchScope ls(c, st, PROF_BLAS, 2.0 * sbytes());
         b_dispatch(p.sloppy, [&](auto sf, auto rl) {
-            launch_chained(dot_kernel<decltype(sf)::value, decltype(rl)>, dim3(vec_blocks(vh)), dim3(kBlock), st, a, v);
+            auto k = dot_kernel<decltype(sf)::value, decltype(rl)>;
+            launch_chained(k, dim3(vec_blocks(k, vh, large())), dim3(kBlock), st, a, v);
         });
     }
 
@@ -731,19 +757,21 @@ struct BRun {
         BArgs a = args();
         a.rows = rows;
         a.part_in = cur_red(c).partials;
+        a.red.partials = cur_red(c).partials + kSplitHalf;
+        const dim3 grid(32), block(kBlock);
         LaunchScope ls(c, st, PROF_BLAS, 0.0);
         if (p.sloppy.compute != HISQ_COMPUTE_F64)
-            launch_chained(dot_rows_kernel<float>, dim3(1), dim3(1024), st, a);
+            launch_chained(dot_rows_kernel<float>, grid, block, st, a);
         else if (p.sloppy.spinor == S_F64)
-            launch_chained(dot_rows_kernel<double>, dim3(1), dim3(1024), st, a);
+            launch_chained(dot_rows_kernel<double>, grid, block, st, a);
         else
-            launch_chained(dot_rows_kernel<FF>, dim3(1), dim3(1024), st, a);
+            launch_chained(dot_rows_kernel<FF>, grid, block, st, a);
         return 0;
     }
 
     void cycle()
     {
-        const int nb = vec_blocks(vh);
+        int nb = 0;  // rows the Gram-Schmidt pass before left
         double *half[2] = {cur_red(c).partials, cur_red(c).partials + kSplitHalf};
         int rows = 0;  // <rt, r_0> is in the state
         for (int j = 0; j < l; j++) {
@@ -753,12 +781,18 @@ struct BRun {
             a.part_in = half[0];
             b_dispatch(p.sloppy, [&](auto sf, auto rl) {
                 LaunchScope ls(c, st, PROF_BLAS, 3.0 * (j + 1) * sbytes());
-                launch_chained(u_multi_kernel<decltype(sf)::value, decltype(rl)>, dim3(nb + 1), dim3(kBlock), st, a);
+                constexpr int SF = decltype(sf)::value;
+                using real = decltype(rl);
+                auto kern = large() ? u_multi_kernel<SF, real, 1> : u_multi_kernel<SF, real, kGroup>;
+                launch_chained(kern, dim3(vec_blocks(kern, vh, large()) + 1), dim3(kBlock), st, a);
             });
             a.rows = mfull_dot(U + j * fb, U + (j + 1) * fb);
             b_dispatch(p.sloppy, [&](auto sf, auto rl) {
                 LaunchScope ls(c, st, PROF_BLAS, (3.0 * (j + 1) + 1) * sbytes() + 96.0 * 2 * vh);
-                launch_chained(r_multi_kernel<decltype(sf)::value, decltype(rl)>, dim3(nb + 1), dim3(kBlock), st, a);
+                constexpr int SF = decltype(sf)::value;
+                using real = decltype(rl);
+                auto kern = large() ? r_multi_kernel<SF, real, 1> : r_multi_kernel<SF, real, kGroup>;
+                launch_chained(kern, dim3(vec_blocks(kern, vh, large()) + 1), dim3(kBlock), st, a);
             });
             rows = mfull_dot(R + j * fb, R + (j + 1) * fb);
         }
@@ -772,12 +806,15 @@ struct BRun {
                 constexpr int SF = decltype(sf)::value;
                 using real = decltype(rl);
                 LaunchScope ls(c, st, PROF_BLAS, ((l - k + 2.0) + (k >= 2 ? l - k + 2.0 : 0.0)) * sbytes());
-                const dim3 grid(nb + 1), block(kBlock);
+                auto pass = [&](auto kern) {
+                    nb = vec_blocks(kern, vh, large());
+                    launch_chained(kern, dim3(nb + 1), dim3(kBlock), st, a);
+                };
                 switch (mgs_nj(l - k)) {
-                case 0: launch_chained(mgs_kernel<SF, real, 0>, grid, block, st, a); break;
-                case 1: launch_chained(mgs_kernel<SF, real, 1>, grid, block, st, a); break;
-                case 3: launch_chained(mgs_kernel<SF, real, 3>, grid, block, st, a); break;
-                default: launch_chained(mgs_kernel<SF, real, 7>, grid, block, st, a); break;
+                case 0: pass(mgs_kernel<SF, real, 0>); break;
+                case 1: pass(mgs_kernel<SF, real, 1>); break;
+                case 3: pass(mgs_kernel<SF, real, 3>); break;
+                default: pass(mgs_kernel<SF, real, 7>); break;
                 }
             });
         }
@@ -788,7 +825,8 @@ struct BRun {
         a.red.partials = half[(l + 1) & 1];
         b_dispatch(p.sloppy, [&](auto sf, auto rl) {
             LaunchScope ls(c, st, PROF_BLAS, (2.0 * l + 5.0) * sbytes() + 96.0 * 2 * vh);
-            launch_chained(final_kernel<decltype(sf)::value, decltype(rl)>, dim3(nb), dim3(kBlock), st, a);
+            auto kern = final_kernel<decltype(sf)::value, decltype(rl)>;
+            launch_chained(kern, dim3(vec_blocks(kern, vh, large())), dim3(kBlock), st, a);
         });
     }
 
