@@ -130,7 +130,6 @@ template <int SF, typename real>
 __global__ void __launch_bounds__(kRBlock) b_r_update_kernel(const __grid_constant__ BBArgs a)
 {
     pdl_wait();
-    pdl_launch_dependents();
     const int t = (int)blockIdx.y;
     const CGState *st = a.st + t;
     if (*(volatile const int *)&st->active == 0) return;
@@ -145,6 +144,7 @@ __global__ void __launch_bounds__(kRBlock) b_r_update_kernel(const __grid_consta
         r_load<SF>(b, i0, cr, ca);
         r_group<SF, real>(b, i0, cr, ca, alpha, v, b.v0);
     }
+    pdl_launch_dependents();
     store_partial_at<2, float>(v, reinterpret_cast<float *>(a.r_sums + (size_t)t * a.nr_blocks), blockIdx.x);
 }
 
@@ -153,7 +153,6 @@ template <int SF, typename real>
 __global__ void __launch_bounds__(kBlock) b_p_update_kernel(const __grid_constant__ BBArgs a)
 {
     pdl_wait();
-    pdl_launch_dependents();
     const int t = (int)blockIdx.y;
     const CGState *st = a.st + t;
     if (*(volatile const int *)&st->active == 0) return;
@@ -165,6 +164,7 @@ __global__ void __launch_bounds__(kBlock) b_p_update_kernel(const __grid_constan
     uint4 cr[U][C], cp[U][C];
     p_load<SF>(b, i0, cr, cp);
     p_group<SF, real>(b, i0, cr, cp, (real)st->beta);
+    pdl_launch_dependents();
 }
 
 // x_t += sum_j alpha_{t,j} p_{t,j} for active t (increment in the compute precision)
@@ -172,7 +172,6 @@ template <int SF, typename real>
 __global__ void __launch_bounds__(kBlock) b_flush_kernel(const __grid_constant__ BBArgs a)
 {
     pdl_wait();
-    pdl_launch_dependents();
     const int t = (int)blockIdx.y;
     if (*(volatile const int *)&a.st[t].active == 0) return;
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
@@ -203,6 +202,7 @@ __global__ void __launch_bounds__(kBlock) b_flush_kernel(const __grid_constant__
             for (int k = 0; k < 6; k++) dx[k] += al[q] * p[k];
         }
     }
+    pdl_launch_dependents();
     double x[6];
     Spinor<S_F64>::decode(cx, x);
 #pragma unroll

@@ -191,7 +191,6 @@ template <int SF, typename real>
 __global__ void __launch_bounds__(kBlock) dot_kernel(BArgs a, const char *v)
 {
     pdl_wait();
-    pdl_launch_dependents();
     if (skip(a.active)) return;
     real s3[3] = {0, 0, 0};
     for (int s = blockIdx.x * blockDim.x + threadIdx.x; s < 2 * a.vh; s += gridDim.x * blockDim.x) {
@@ -201,6 +200,7 @@ __global__ void __launch_bounds__(kBlock) dot_kernel(BArgs a, const char *v)
         Spinor<SF>::load(v + q.h * a.hb, a.vh, q.i, y);
         dot_site(x, y, s3);
     }
+    pdl_launch_dependents();
     __shared__ double tot[3];
     if (reduce_grid<3>(s3, a.red, tot) && threadIdx.x == 0)
         for (int k = 0; k < 3; k++) a.b->dot[k] = tot[k];
@@ -212,7 +212,6 @@ template <int SF, typename real, int G>
 __global__ void __launch_bounds__(kBlock) u_multi_kernel(BArgs a)
 {
     pdl_wait();
-    pdl_launch_dependents();
     if (skip(a.active)) return;
     __shared__ double tot[3];
     __shared__ real be_sh[2];
@@ -272,6 +271,7 @@ __global__ void __launch_bounds__(kBlock) u_multi_kernel(BArgs a)
             }
         }
     }
+    pdl_launch_dependents();
 }
 
 // r_i -= alpha u_{i+1}, i = 0..j; x += alpha u_0 (FP64), with gamma = <rt, u_{j+1}>, alpha = rho / gamma;
@@ -280,7 +280,6 @@ template <int SF, typename real, int G>
 __global__ void __launch_bounds__(kBlock) r_multi_kernel(BArgs a)
 {
     pdl_wait();
-    pdl_launch_dependents();
     if (skip(a.active)) return;
     __shared__ double tot[3];
     __shared__ real al_sh[2];
@@ -356,6 +355,7 @@ __global__ void __launch_bounds__(kBlock) r_multi_kernel(BArgs a)
         }
         Spinor<S_F64>::store(xf, a.vh, q.i, x);
     }
+    pdl_launch_dependents();
 }
 
 // The most vectors after r_k that pass k's kernel is compiled for.
@@ -384,7 +384,6 @@ __global__ void __launch_bounds__(kBlock) mgs_kernel(BArgs a)
 {
     constexpr int NR = 3 + 2 * NJ, C = Spinor<SF>::chunks;
     pdl_wait();
-    pdl_launch_dependents();
     if (skip(a.active)) return;
     BState *b = a.b;
     const int k = a.j, rest = b->l - k;  // vectors after r_k
@@ -467,6 +466,7 @@ __global__ void __launch_bounds__(kBlock) mgs_kernel(BArgs a)
             }
         }
     }
+    pdl_launch_dependents();
     store_partial_at<NR, real>(v, reinterpret_cast<real *>(a.part_out), blockIdx.x);
 }
 
@@ -478,7 +478,6 @@ template <int SF, typename real>
 __global__ void __launch_bounds__(kBlock) final_kernel(BArgs a)
 {
     pdl_wait();
-    pdl_launch_dependents();
     if (skip(a.active)) return;
     BState *b = a.b;
     const int l = b->l;
@@ -578,6 +577,7 @@ __global__ void __launch_bounds__(kBlock) final_kernel(BArgs a)
         if (!Spinor<SF>::store(u0f, a.vh, q.i, u0)) atomicExch(a.err, 1);
         dot_site(rt, r0, v);
     }
+    pdl_launch_dependents();
     if (reduce_grid<3>(v, a.red, tot) && threadIdx.x == 0) {
         for (int k = 0; k < 3; k++) b->dot[k] = tot[k];
         // the next cycle's rho_0 starts from -omega rho

@@ -60,7 +60,6 @@ template <int SF, typename real>
 __global__ void __launch_bounds__(kBlock) r_update_kernel(BlasArgs a)
 {
     pdl_wait();
-    pdl_launch_dependents();
     if (skip(a.active)) return;
     constexpr int U = kRSites, C = Spinor<SF>::chunks;
     red_t<real> v[2] = {0, 0};
@@ -71,6 +70,7 @@ __global__ void __launch_bounds__(kBlock) r_update_kernel(BlasArgs a)
         r_load<SF>(a, i0, cr, ca);
         r_group<SF, real>(a, i0, cr, ca, alpha, v, a.v0);
     }
+    pdl_launch_dependents();
     __shared__ double tot[2];
     if (reduce_grid<2>(v, a.red, tot) && threadIdx.x == 0) {
         if (a.fin)
@@ -84,7 +84,6 @@ template <int SF, typename real>
 __global__ void __launch_bounds__(kBlock) p_update_kernel(BlasArgs a)
 {
     pdl_wait();
-    pdl_launch_dependents();
     if (skip(a.active)) return;
     constexpr int U = kPSites, C = Spinor<SF>::chunks;
     const int i0 = blockIdx.x * blockDim.x * U + threadIdx.x;
@@ -94,6 +93,7 @@ __global__ void __launch_bounds__(kBlock) p_update_kernel(BlasArgs a)
     p_load<SF>(a, i0, cr, cp);
     const real beta = block_scalar<real>(&a.st->beta);
     p_group<SF, real>(a, i0, cr, cp, beta);
+    pdl_launch_dependents();
 }
 
 // The CG iteration's scalar steps without one-block launches or last-block
@@ -113,7 +113,6 @@ template <int SF, typename real, int BS>
 __global__ void __launch_bounds__(BS) r_update_split_kernel(BlasArgs a)
 {
     pdl_wait();
-    pdl_launch_dependents();
     if (skip(a.active)) return;
     constexpr int U = kRSites, C = Spinor<SF>::chunks;
     const int step = gridDim.x * BS * U;
@@ -139,6 +138,7 @@ __global__ void __launch_bounds__(BS) r_update_split_kernel(BlasArgs a)
             r_group<SF, real>(a, i0, cr, ca, alpha, v, a.v0);
             r_load<SF>(a, i0 + step, cr, ca);
         }
+        pdl_launch_dependents();
         store_block_partial<2>(v, split_half(a.red));
     }
     if (blockIdx.x == 0 && threadIdx.x == 0) {
@@ -151,7 +151,6 @@ template <int SF, typename real>
 __global__ void __launch_bounds__(kBlock) p_update_split_kernel(BlasArgs a)
 {
     pdl_wait();
-    pdl_launch_dependents();
     if (skip(a.active)) return;
     constexpr int U = kPSites, C = Spinor<SF>::chunks;
     if (a.clear_ring && blockIdx.x == 0 && threadIdx.x == 0)
@@ -173,6 +172,7 @@ __global__ void __launch_bounds__(kBlock) p_update_split_kernel(BlasArgs a)
     }
     __syncthreads();
     if (ok_sh) p_group<SF, real>(a, i0, cr, cp, be_sh);
+    pdl_launch_dependents();
     // after the update: the finisher's registers are not live beside the loaded fields
     if (blockIdx.x == 0 && threadIdx.x == 0) run_finisher(FIN_CG_BETA, tot, a.st, a.slot);
 }
@@ -183,7 +183,6 @@ template <int SF, typename real>
 __global__ void __launch_bounds__(kBlock) x_flush_kernel(BlasArgs a)
 {
     pdl_wait();
-    pdl_launch_dependents();
     if (skip(a.active)) return;
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     __shared__ real al_s[kMaxBuf];  // the step sizes in the compute precision, converted once per block
@@ -214,6 +213,7 @@ __global__ void __launch_bounds__(kBlock) x_flush_kernel(BlasArgs a)
             for (int k = 0; k < 6; k++) dx[k] += al[g] * p[k];
         }
     }
+    pdl_launch_dependents();
     double x[6];
     Spinor<S_F64>::decode(cx, x);
 #pragma unroll
@@ -231,7 +231,6 @@ template <int SF, typename real>
 __global__ void __launch_bounds__(kBlock) true_residual_kernel(BlasArgs a)
 {
     pdl_wait();
-    pdl_launch_dependents();
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     double v[3] = {0.0, 0.0, 0.0};
     if (i < a.n) {
@@ -256,6 +255,7 @@ __global__ void __launch_bounds__(kBlock) true_residual_kernel(BlasArgs a)
             v[2] += rr * pi - ri * pr;  // Im conj(r) p
         }
     }
+    pdl_launch_dependents();
     __shared__ double tot[3];
     if (reduce_grid<3>(v, a.red, tot) && threadIdx.x == 0) {
         if (a.fin)
@@ -270,7 +270,6 @@ template <int SF, typename real>
 __global__ void __launch_bounds__(kBlock) p_reliable_kernel(BlasArgs a)
 {
     pdl_wait();
-    pdl_launch_dependents();
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i == 0)
         for (int j = 0; j < kMaxBuf; j++) a.st->alpha_ring[j] = 0.0;
@@ -285,6 +284,7 @@ __global__ void __launch_bounds__(kBlock) p_reliable_kernel(BlasArgs a)
         o[2 * c] = narrow<real>(cr * r[2 * c] - ci * r[2 * c + 1] + beta * widen(p[2 * c]));
         o[2 * c + 1] = narrow<real>(cr * r[2 * c + 1] + ci * r[2 * c] + beta * widen(p[2 * c + 1]));
     }
+    pdl_launch_dependents();
     if (!Spinor<SF>::store(a.v2, a.n, i, o)) atomicExch(a.err, 1);
 }
 

@@ -63,11 +63,12 @@ __global__ void __launch_bounds__(kBlock) pack_fields_kernel(int64_t n, const __
 {
     __shared__ __align__(16) double sh[kBlock / 32][192];
     pdl_wait();
-    pdl_launch_dependents();
     const int y = (int)blockIdx.y;
     const double *in = y == 0 ? f.in[0] : y == 1 ? f.in[1] : y == 2 ? f.in[2] : f.in[3];
     char *out = y == 0 ? f.out[0] : y == 1 ? f.out[1] : y == 2 ? f.out[2] : f.out[3];
-    if (!pack_warp<SF>(n, in, out, sh[threadIdx.x >> 5])) {
+    const bool ok = pack_warp<SF>(n, in, out, sh[threadIdx.x >> 5]);
+    pdl_launch_dependents();
+    if (!ok) {
         *(volatile int *)f.bad = 1;
         *(volatile int *)f.bad_host = 1;
     }

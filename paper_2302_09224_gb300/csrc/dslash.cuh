@@ -667,7 +667,6 @@ __global__ void __launch_bounds__(stencil_block(CFG), stencil_minb(CFG))
     dslash_kernel(const __grid_constant__ DslashArgs a)
 {
     pdl_wait();  // the input, xpay and state fields come from the previous kernel
-    pdl_launch_dependents();
     if (a.active != nullptr && *(volatile const int *)a.active == 0) return;  // uniform over the grid
     const int vh = a.g.vh;
     const size_t pstride = (size_t)8 * vh * 16;
@@ -679,6 +678,7 @@ __global__ void __launch_bounds__(stencil_block(CFG), stencil_minb(CFG))
     real rv[2] = {real(0), real(0)};
     const int cb = blockIdx.x * blockDim.x + threadIdx.x;
     if (cb < vh) stencil_site<GF, SF, real, LREC, RED, CFG>(a, stencil_io(a), cb, pstride, fsc, lsc, ratio, rv);
+    pdl_launch_dependents();
     if constexpr (RED) {  // summed by stencil_finish_kernel or by the CG's residual update
         const red_t<real> r2[2] = {(red_t<real>)rv[0], (red_t<real>)rv[1]};
         store_block_partial<2>(r2, a.red);
@@ -697,7 +697,6 @@ __global__ void __launch_bounds__(128, 4) dslash_lanes_kernel(const __grid_const
 {
     __shared__ __align__(16) double sh[OUT ? 128 / S : 1][6];
     pdl_wait();
-    pdl_launch_dependents();
     if (OUT ? *(volatile const int *)a.bad != 0 : a.active != nullptr && *(volatile const int *)a.active == 0)
         return;  // uniform over the grid
     const Geom &g = a.g;
@@ -759,6 +758,7 @@ __global__ void __launch_bounds__(128, 4) dslash_lanes_kernel(const __grid_const
         Spinor<S_F64>::store(io.out, vh, cb, o);
         if (!ok) atomicExch(a.err, 1);
     }
+    pdl_launch_dependents();
 }
 
 // Lanes a site of an FP64 pass over n sites: the fewest of 1, 2 and 4 whose
@@ -830,7 +830,6 @@ __global__ void __launch_bounds__(stencil_block(CFG), stencil_minb(CFG))
     dslash_full_dot_kernel(const __grid_constant__ DslashArgs a)
 {
     pdl_wait();
-    pdl_launch_dependents();
     if (a.active != nullptr && *(volatile const int *)a.active == 0) return;  // uniform over the grid
     const int vh = a.g.vh;
     const size_t pstride = (size_t)8 * vh * 16;
@@ -858,6 +857,7 @@ __global__ void __launch_bounds__(stencil_block(CFG), stencil_minb(CFG))
             v[2] += yr * yr + yi * yi;
         }
     }
+    pdl_launch_dependents();
     if (a.red.partials != nullptr) store_block_partial<3>(v, a.red);
 }
 

@@ -3,12 +3,21 @@
 // Every kernel of a solver iteration depends on the one before it (alpha,
 // beta and the vectors flow through device memory), so each used to start
 // only after the previous grid had drained.  Launched with programmatic
-// stream serialisation, a kernel's blocks are scheduled while its
-// predecessor's last wave is still running; each kernel calls pdl_wait()
-// before its first access to memory another kernel of the chain writes (the
-// wait returns once the predecessor grid has completed and its writes are
-// visible), then pdl_launch_dependents() so that its own successor can be
-// scheduled in turn.  Launched without the attribute, both are no-ops.
+// stream serialisation, a kernel's blocks are scheduled before its
+// predecessor has drained; each kernel calls pdl_wait() before its first
+// access to memory another kernel of the chain writes (the wait returns once
+// the predecessor grid has completed and its writes are visible), then
+// pdl_launch_dependents() so that its own successor can be scheduled in turn.
+// Launched without the attribute, both are no-ops.
+//
+// Kernels with work on every SM call pdl_launch_dependents() after that work,
+// not before it: a successor of about one wave that is scheduled beside
+// running blocks fills the SMs by the room these leave, unevenly, and a pass
+// bound by its fullest SM takes longer by more than the launch that was
+// hidden.  FP64 CG, 16^3x32: 43.1 ms with the early call, 29.9 without
+// programmatic launches, 29.8 with the late call; BiCGStab(4), 20-bit,
+// 16^3x32: 15.7, 13.9, 13.7; 20-bit CG, 24^3x48 (many waves a pass): 20.5,
+// 21.0, 20.5.  Kernels of a few blocks call it first.
 #pragma once
 
 #include <cuda_runtime.h>

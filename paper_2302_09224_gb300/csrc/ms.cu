@@ -71,7 +71,6 @@ __global__ void __launch_bounds__(ms_block<real>()) ms_r_update_kernel(const __g
 {
     constexpr int BS = ms_block<real>(), U = 2, C = Spinor<SF>::chunks;
     pdl_wait();
-    pdl_launch_dependents();
     MSState *m = a.m;
     if (*(volatile const int *)&m->active == 0) return;
     const bool scalars = blockIdx.x == gridDim.x - 1;
@@ -111,6 +110,7 @@ __global__ void __launch_bounds__(ms_block<real>()) ms_r_update_kernel(const __g
         r_group<SF, real>(a.b, i0, cr, ca, alpha, v, a.out);
         r_load<SF>(a.b, i0 + step, cr, ca);
     }
+    pdl_launch_dependents();
     store_block_partial<2>(v, split_half(a.b.red));
 }
 
@@ -120,7 +120,6 @@ __global__ void __launch_bounds__(kBlock) ms_p_update_kernel(const __grid_consta
     constexpr int C = Spinor<SF>::chunks;
     constexpr int AF = is_ff<real>::value ? S_FF : sizeof(real) == 8 ? S_F64 : S_F32;
     pdl_wait();
-    pdl_launch_dependents();
     MSState *m = a.m;
     if (*(volatile const int *)&m->active == 0) return;
     const bool scalars = blockIdx.x == gridDim.x - 1;
@@ -160,6 +159,7 @@ __global__ void __launch_bounds__(kBlock) ms_p_update_kernel(const __grid_consta
         x[k] += al * p[k];
         p[k] = r[k] + be * p[k];
     }
+    pdl_launch_dependents();
     if (!Spinor<SF>::store(a.b.v1, n, i, p)) atomicExch(a.b.err, 1);
     Spinor<AF>::store(a.out, n, i, x);
 }
