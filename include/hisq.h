@@ -133,7 +133,11 @@ HISQ_API void hisq_destroy(hisq_ctx *ctx);
 /* Message of the last failed call on this context (never NULL). */
 HISQ_API const char *hisq_last_error(hisq_ctx *ctx);
 
-/* Device bytes the context currently holds. */
+/* Device bytes of the context in use by gauge fields and running calls.
+ * Buffers of finished calls stay with the context for the next call of the same
+ * sizes (at most 4 GiB and an eighth of the budget, beside those in use and
+ * within the budget; released when an allocation needs the room); they are
+ * not counted. */
 HISQ_API size_t hisq_mem_used(hisq_ctx *ctx);
 
 /* Load a gauge configuration (Sec. 2 footnote, Sec. 4: one global scale per
@@ -307,12 +311,14 @@ HISQ_API void hisq_mee_fused_shape(int lag, int blocks_per_sm);
  * default, 2^22 polls of at least 64 ns each); unreachable = 1 raises every
  * wait's target past what the launch can reach, so each wait runs to its
  * limit, the kernel flags the error and goes on, and the solver returns
- * ECUDA.  Only for testing that a wait ends; 0 restores normal waits. */
+ * ECUDA.  The waits of a CG whose iterations run in one resident launch (small
+ * lattices; see hisq_cg_split_scalars) take the same two settings.  Only for
+ * testing that a wait ends; 0 restores normal waits. */
 HISQ_API void hisq_mee_fused_wait_test(unsigned polls, int unreachable);
 HISQ_API int hisq_stencil_config_reduce(int cfg);
 /* Programmatic dependent launch of the solvers' kernel chains (stencil
  * passes, their finish kernel and the fused BLAS kernels): 1 (default) lets
- * each kernel's blocks be scheduled while its predecessor's last wave runs
+ * each kernel's blocks be scheduled while its predecessor's last blocks end
  * (every kernel waits for its predecessor's results before touching them, so
  * results are identical either way); 0 launches them one after another.
  * Returns the previous setting, or -2 for an invalid value.  For benchmarking;
@@ -325,9 +331,11 @@ HISQ_API int hisq_programmatic_launch(int mode);
  * beta, so no one-block launch or last-block tail sits between the kernels;
  * 0 sums them once, in a one-block launch after the stencil pass and in the
  * last block of the residual update.  The sums are deterministic in both
- * modes; their rounding differs between the two (other block shapes).  The
- * FP64 triplet (FP64 sloppy storage) always takes the second form (faster
- * there).  Returns the previous setting, or -2 for an invalid value.  Read
+ * modes; their rounding differs between the two (other block shapes).  With
+ * 1 (and hisq_mee_fused off), a lattice whose sites fit on the chip's SMs runs
+ * a whole block of iterations in one resident cooperative launch instead
+ * (FP32, 16- and 20-bit triplets, 12- or 18-real long links).  The FP64 triplet
+ * (FP64 sloppy storage) always takes the second form (faster there).  Returns the previous setting, or -2 for an invalid value.  Read
  * when a solve starts.  For benchmarking; no counterpart in the paper. */
 HISQ_API int hisq_cg_split_scalars(int mode);
 /* The shape in use for triplet p on gauge g's lattice (plain pass, or the

@@ -479,10 +479,12 @@ hisq_status BatchSession::setup()
     if (!e) e = ws.alloc((size_t)48 * vh, (void **)&ax64);
     if (!e) e = ws.alloc((size_t)48 * vh, (void **)&tmp64);
     if (!e) e = ws.alloc(sizeof(CGState) * nr, (void **)&st);
-    // block sums of a reducing stencil pass and of the residual update, per right-hand side
-    if (!e)
-        e = ws.alloc(sizeof(float2) * nr * ((vh + kMrhsBlock - 1) / kMrhsBlock + r_blocks(vh)), (void **)&sums);
     if (e) return e;
+    // Block sums of a reducing stencil pass and of the residual update, per right-hand side: in a work field of
+    // the true residual, which no kernel uses between a pass and the scalars that take its sums (16 right-hand
+    // sides: 128 bytes for every 128 and every 1024 sites, under 48 a site on the smallest lattice of 8).
+    static_assert(kMaxRHS * sizeof(float2) * 2 <= 48 * 8, "the sums fit the field");
+    sums = (float2 *)tmp64;
     static_assert(sizeof(CGState) * kMaxRHS <= kPinnedBytes, "a batch's states fit a pinned block");
     sth = (CGState *)pinned_get(c, sizeof(CGState) * nr);
     if (!sth) return fail(c, HISQ_ENOMEM, "pinned state");

@@ -4,10 +4,11 @@
 // On a small lattice an iteration of four dependent kernels (two stencil
 // passes, the residual and the gradient update) is bound by their latencies:
 // 22 us an iteration on 8^4 and 26 us on 16^4 (20-bit), where the links read
-// from L2 take under 4 us.  This kernel: 9.8 and 15.3 us.  Here every thread group owns one site (of each parity) for
-// the whole launch: r, p, A p and the step of x stay in registers, only p and
-// the odd-site intermediate go through memory (L2), and the kernels' boundaries
-// become four grid-wide exchanges, two barriers and two sums:
+// from L2 take under 4 us.  This kernel: 9.8 and 15.3 us.  Every thread group
+// owns one site (of each parity) for the whole launch: r, p, A p and the step
+// of x stay in registers, only p and the odd-site intermediate go through
+// memory (L2), and the kernels' boundaries become four grid-wide exchanges, two
+// barriers and two sums:
 //   tmp = D_oe p | barrier | A p = diag p - D_eo tmp, <p, A p> | sum barrier |
 //   r -= alpha A p, |r|^2, <r, r_old> | sum barrier | p = r + beta p | barrier.
 // Every block sums the blocks' partials in one fixed order, takes alpha, beta and

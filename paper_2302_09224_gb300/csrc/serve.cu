@@ -9,7 +9,7 @@
 // soon as a slot frees up.  Sessions are admitted only while the context's
 // HBM budget allows their buffers; otherwise their requests wait.  A
 // multi-shift request runs its multi-shift stage (all shifts in one fused
-// update per iteration) on a worker; the refinement CG of each shift that has
+// update per block of iterations) on a worker; the refinement CG of each shift that has
 // not reached its target then enters the queue as an internal CG request
 // (its shifted diagonal, its target, the stage's solution as initial guess),
 // so the refinements join the batch sessions of their sloppy triplet beside
