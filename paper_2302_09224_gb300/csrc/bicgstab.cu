@@ -122,26 +122,37 @@ __device__ __forceinline__ void dot_sums(const BArgs &a, double *tot)
 template <int NR, typename real>
 __device__ __forceinline__ void sum_rows(const real *part, int rows, double *tot)
 {
-    constexpr int U = 5;
-    const int lane = threadIdx.x & 31;
-    for (int v = threadIdx.x >> 5; v < NR; v += kBlock / 32) {
-        if constexpr (std::is_same<real, double>::value) {
+    constexpr int U = 10, W = kBlock / 32, K = (NR + W - 1) / W;  // values a warp: v0, v0 + W, ..., loaded together
+    const int lane = threadIdx.x & 31, v0 = threadIdx.x >> 5;
+    if constexpr (std::is_same<real, double>::value) {
+        for (int v = v0; v < NR; v += W) {
             double w[1] = {0.0};
             for (int r = lane; r < rows; r += 32) w[0] += __ldcg(part + (size_t)r * NR + v);
             warp_sum<1, double>(w);
             if (lane == 0) tot[v] = w[0];
-        } else {
-            FF w[1] = {{0.0f, 0.0f}};
-            for (int r0 = lane; r0 < rows; r0 += 32 * U) {
-                float t[U];
-#pragma unroll
-                for (int u = 0; u < U; u++) t[u] = r0 + 32 * u < rows ? __ldcg(part + (size_t)(r0 + 32 * u) * NR + v) : 0.0f;
-#pragma unroll
-                for (int u = 0; u < U; u++) w[0] = ff_add(w[0], FF{t[u], 0.0f});
-            }
-            warp_sum_ff<1>(w);
-            if (lane == 0) tot[v] = (double)w[0].hi + (double)w[0].lo;
         }
+    } else {
+        FF w[K];
+#pragma unroll
+        for (int k = 0; k < K; k++) w[k] = {0.0f, 0.0f};
+        for (int r0 = lane; r0 < rows; r0 += 32 * U) {
+            float t[K][U];
+#pragma unroll
+            for (int k = 0; k < K; k++)
+#pragma unroll
+                for (int u = 0; u < U; u++)
+                    t[k][u] = v0 + k * W < NR && r0 + 32 * u < rows
+                                  ? __ldcg(part + (size_t)(r0 + 32 * u) * NR + v0 + k * W) : 0.0f;
+#pragma unroll
+            for (int u = 0; u < U; u++)
+#pragma unroll
+                for (int k = 0; k < K; k++) w[k] = ff_add(w[k], FF{t[k][u], 0.0f});
+        }
+        warp_sum_ff<K>(w);
+        if (lane == 0)
+#pragma unroll
+            for (int k = 0; k < K; k++)
+                if (v0 + k * W < NR) tot[v0 + k * W] = (double)w[k].hi + (double)w[k].lo;
     }
     __syncthreads();
 }
@@ -216,6 +227,23 @@ __global__ void __launch_bounds__(kBlock) u_multi_kernel(BArgs a)
     __shared__ double tot[3];
     __shared__ real be_sh[2];
     __shared__ int ok_sh;
+    // the first site's fields are loaded before the sums, and the next site's after a site's stores
+    constexpr int C = Spinor<SF>::chunks;
+    const int step = (int)(gridDim.x - 1) * kBlock;
+    int s = blockIdx.x == gridDim.x - 1 ? 2 * a.vh : (int)(blockIdx.x * kBlock + threadIdx.x);
+    uint4 cr[G][C], cu[G][C];
+    auto load = [&](int at, int i0) {
+        if (at >= 2 * a.vh) return;
+        const Site q = site_of(at, a.vh);
+        const size_t off = q.h * a.hb;
+#pragma unroll
+        for (int g = 0; g < G; g++)
+            if (i0 + g <= a.j) {
+                Spinor<SF>::gather(a.R + off + (i0 + g) * a.fb, a.vh, q.i, cr[g]);
+                Spinor<SF>::gather(a.U + off + (i0 + g) * a.fb, a.vh, q.i, cu[g]);
+            }
+    };
+    load(s, 0);
     dot_sums<SF, real>(a, tot);
     if (threadIdx.x == 0) {
         BState *b = a.b;
@@ -242,19 +270,11 @@ __global__ void __launch_bounds__(kBlock) u_multi_kernel(BArgs a)
     __syncthreads();
     if (!ok_sh || blockIdx.x == gridDim.x - 1) return;
     const real br = be_sh[0], bi = be_sh[1];
-    constexpr int C = Spinor<SF>::chunks;
-    for (int s = blockIdx.x * blockDim.x + threadIdx.x; s < 2 * a.vh; s += (gridDim.x - 1) * blockDim.x) {
+    for (; s < 2 * a.vh; s += step) {
         const Site q = site_of(s, a.vh);
-        const char *rf = a.R + q.h * a.hb;
         char *uf = a.U + q.h * a.hb;
         for (int i0 = 0; i0 <= a.j; i0 += G) {
-            uint4 cr[G][C], cu[G][C];
-#pragma unroll
-            for (int g = 0; g < G; g++)
-                if (i0 + g <= a.j) {
-                    Spinor<SF>::gather(rf + (i0 + g) * a.fb, a.vh, q.i, cr[g]);
-                    Spinor<SF>::gather(uf + (i0 + g) * a.fb, a.vh, q.i, cu[g]);
-                }
+            if (i0 > 0) load(s, i0);
 #pragma unroll
             for (int g = 0; g < G; g++) {
                 if (i0 + g > a.j) continue;
@@ -270,6 +290,7 @@ __global__ void __launch_bounds__(kBlock) u_multi_kernel(BArgs a)
                 if (!Spinor<SF>::store(uf + (i0 + g) * a.fb, a.vh, q.i, u)) atomicExch(a.err, 1);
             }
         }
+        load(s + step, 0);
     }
     pdl_launch_dependents();
 }
@@ -284,6 +305,29 @@ __global__ void __launch_bounds__(kBlock) r_multi_kernel(BArgs a)
     __shared__ double tot[3];
     __shared__ real al_sh[2];
     __shared__ int ok_sh;
+    // loads as in the u update; u_0 and x with them when several fields are in flight anyway (G > 1)
+    constexpr int C = Spinor<SF>::chunks;
+    const int step = (int)(gridDim.x - 1) * kBlock;
+    int s = blockIdx.x == gridDim.x - 1 ? 2 * a.vh : (int)(blockIdx.x * kBlock + threadIdx.x);
+    uint4 cr[G][C], cu[G][C], c0[C], cx[Spinor<S_F64>::chunks];
+    auto x_field = [&](int h) { return reinterpret_cast<char *>(a.x64) + h * (size_t)48 * a.vh; };
+    auto load_x = [&](const Site &q) {
+        Spinor<SF>::gather(a.U + q.h * a.hb, a.vh, q.i, c0);
+        Spinor<S_F64>::gather(x_field(q.h), a.vh, q.i, cx);
+    };
+    auto load = [&](int at, int i0) {
+        if (at >= 2 * a.vh) return;
+        const Site q = site_of(at, a.vh);
+        const size_t off = q.h * a.hb;
+        if (G > 1 && i0 == 0) load_x(q);
+#pragma unroll
+        for (int g = 0; g < G; g++)
+            if (i0 + g <= a.j) {
+                Spinor<SF>::gather(a.U + a.fb + off + (i0 + g) * a.fb, a.vh, q.i, cu[g]);
+                Spinor<SF>::gather(a.R + off + (i0 + g) * a.fb, a.vh, q.i, cr[g]);
+            }
+    };
+    load(s, 0);
     dot_sums<SF, real>(a, tot);
     if (threadIdx.x == 0) {
         BState *b = a.b;
@@ -306,27 +350,11 @@ __global__ void __launch_bounds__(kBlock) r_multi_kernel(BArgs a)
     __syncthreads();
     if (!ok_sh || blockIdx.x == gridDim.x - 1) return;
     const real ar = al_sh[0], ai = al_sh[1];
-    constexpr int C = Spinor<SF>::chunks;
-    for (int s = blockIdx.x * blockDim.x + threadIdx.x; s < 2 * a.vh; s += (gridDim.x - 1) * blockDim.x) {
+    for (; s < 2 * a.vh; s += step) {
         const Site q = site_of(s, a.vh);
-        // x += alpha u_0: the increment in the compute precision, the sum in FP64
-        real u0[6];
-        uint4 cx[Spinor<S_F64>::chunks];
-        char *xf = reinterpret_cast<char *>(a.x64) + q.h * (size_t)48 * a.vh;
-        if (G > 1) {
-            Spinor<SF>::load(a.U + q.h * a.hb, a.vh, q.i, u0);
-            Spinor<S_F64>::gather(xf, a.vh, q.i, cx);
-        }
         char *rf = a.R + q.h * a.hb;
-        const char *uf = a.U + a.fb + q.h * a.hb;
         for (int i0 = 0; i0 <= a.j; i0 += G) {
-            uint4 cr[G][C], cu[G][C];
-#pragma unroll
-            for (int g = 0; g < G; g++)
-                if (i0 + g <= a.j) {
-                    Spinor<SF>::gather(uf + (i0 + g) * a.fb, a.vh, q.i, cu[g]);
-                    Spinor<SF>::gather(rf + (i0 + g) * a.fb, a.vh, q.i, cr[g]);
-                }
+            if (i0 > 0) load(s, i0);
 #pragma unroll
             for (int g = 0; g < G; g++) {
                 if (i0 + g > a.j) continue;
@@ -342,18 +370,19 @@ __global__ void __launch_bounds__(kBlock) r_multi_kernel(BArgs a)
                 if (!Spinor<SF>::store(rf + (i0 + g) * a.fb, a.vh, q.i, r)) atomicExch(a.err, 1);
             }
         }
-        if (G == 1) {
-            Spinor<SF>::load(a.U + q.h * a.hb, a.vh, q.i, u0);
-            Spinor<S_F64>::gather(xf, a.vh, q.i, cx);
-        }
+        // x += alpha u_0: the increment in the compute precision, the sum in FP64
+        if (G == 1) load_x(q);
+        real u0[6];
         double x[6];
+        Spinor<SF>::decode(c0, u0);
         Spinor<S_F64>::decode(cx, x);
 #pragma unroll
         for (int c = 0; c < 3; c++) {
             x[2 * c] += widen(ar * u0[2 * c] - ai * u0[2 * c + 1]);
             x[2 * c + 1] += widen(ar * u0[2 * c + 1] + ai * u0[2 * c]);
         }
-        Spinor<S_F64>::store(xf, a.vh, q.i, x);
+        Spinor<S_F64>::store(x_field(q.h), a.vh, q.i, x);
+        load(s + step, 0);
     }
     pdl_launch_dependents();
 }
@@ -391,6 +420,21 @@ __global__ void __launch_bounds__(kBlock) mgs_kernel(BArgs a)
     __shared__ double tot[3 + 2 * kMaxL];
     __shared__ real tau[2 * (NJ + 1)];
     __shared__ int ok_sh;
+    // the first site's fields are loaded before the sums
+    const int step = (int)(gridDim.x - 1) * kBlock;
+    int s = scalars ? 2 * a.vh : (int)(blockIdx.x * kBlock + threadIdx.x);
+    uint4 c0[C], cp[C], cr[NJ + 1][C];
+    auto load = [&](int at) {
+        if (at >= 2 * a.vh) return;
+        const Site q = site_of(at, a.vh);
+        const char *f = a.R + q.h * a.hb;
+        Spinor<SF>::gather(f, a.vh, q.i, c0);
+        if (k >= 2) Spinor<SF>::gather(f + (k - 1) * a.fb, a.vh, q.i, cp);
+#pragma unroll
+        for (int i = 0; i <= NJ; i++)
+            if (i <= rest) Spinor<SF>::gather(f + (k + i) * a.fb, a.vh, q.i, cr[i]);
+    };
+    load(s);
     if (k >= 2) {
         // the previous pass left 3 + 2 * (its NJ) values a row; tau_{k-1,i} = <r_{k-1}, r_i> / sigma_{k-1}
         sum_prev<real>(a, k, b->l, tot);
@@ -419,15 +463,9 @@ __global__ void __launch_bounds__(kBlock) mgs_kernel(BArgs a)
     real v[NR];
 #pragma unroll
     for (int q = 0; q < NR; q++) v[q] = 0;
-    for (int s = blockIdx.x * blockDim.x + threadIdx.x; s < 2 * a.vh; s += (gridDim.x - 1) * blockDim.x) {
+    for (; s < 2 * a.vh; s += step) {
         const Site q = site_of(s, a.vh);
         auto field = [&](int i) { return a.R + i * a.fb + q.h * a.hb; };
-        uint4 c0[C], cp[C], cr[NJ + 1][C];
-        Spinor<SF>::gather(field(0), a.vh, q.i, c0);
-        if (k >= 2) Spinor<SF>::gather(field(k - 1), a.vh, q.i, cp);
-#pragma unroll
-        for (int i = 0; i <= NJ; i++)
-            if (i <= rest) Spinor<SF>::gather(field(k + i), a.vh, q.i, cr[i]);
         real r0[6], rp[6], rk[6];
         Spinor<SF>::decode(c0, r0);
         if (k >= 2) Spinor<SF>::decode(cp, rp);
@@ -465,6 +503,7 @@ __global__ void __launch_bounds__(kBlock) mgs_kernel(BArgs a)
                 v[2 + 2 * i] += w[1];
             }
         }
+        load(s + step);
     }
     pdl_launch_dependents();
     store_partial_at<NR, real>(v, reinterpret_cast<real *>(a.part_out), blockIdx.x);
