@@ -141,6 +141,7 @@ using SiteAcc = std::conditional_t<std::is_same<real, float>::value, SiteAccPack
 //   2: 128, <= 64 registers, rolled      3: 256, <= 64 registers, rolled
 //   4: 128, <= 64 registers, unrolled
 constexpr int kNumStencilConfigs = 5;
+constexpr long long kKeepLinkBytes = 90000000;  // links of both parities that an L2 of 129 MB keeps beside the fields
 __host__ __device__ constexpr bool stencil_config_valid(int cfg, int gf) { return cfg >= 0 && cfg < kNumStencilConfigs && gf >= 0; }
 __host__ __device__ constexpr int stencil_block(int cfg) { return cfg == 3 ? 256 : 128; }
 // Threads a block is launched with.  The FP64 stencil runs at the FP64 pipe's
@@ -825,7 +826,7 @@ __global__ void __launch_bounds__(stencil_block(CFG), stencil_minb(CFG))
 // <dot, out> and |out|^2 (BiCGStab(l)'s next scalars; a pass of their own over
 // the two fields took 10 to 20 us).  On a small lattice one launch of both
 // parities also fills the chip better than two of one.
-template <int GF, int SF, typename real, int LREC, int CFG>
+template <int GF, int SF, typename real, int LREC, int CFG, bool KEEP>
 __global__ void __launch_bounds__(stencil_block(CFG), stencil_minb(CFG))
     dslash_full_dot_kernel(const __grid_constant__ DslashArgs a)
 {
@@ -842,7 +843,7 @@ __global__ void __launch_bounds__(stencil_block(CFG), stencil_minb(CFG))
     red_t<real> v[3] = {real(0), real(0), real(0)};
     if (cb < vh) {
         real o[6], t[6];
-        stencil_value<GF, SF, real, LREC, CFG>(a, io.in, io.po, cb, pstride, fsc, lsc, ratio, o);
+        stencil_value<GF, SF, real, LREC, CFG, false, KEEP>(a, io.in, io.po, cb, pstride, fsc, lsc, ratio, o);
         Spinor<SF>::load(io.y, vh, cb, t);
         const real aa = (real)a.a;
 #pragma unroll
@@ -944,7 +945,13 @@ void launch_any(int cfg, const DslashArgs &a, cudaStream_t s)
         }
         if (a.dot != nullptr) {  // the 64-register unrolled shape, the plain passes' usual choice
             const int B = stencil_threads(4, GF, 2 * a.g.vh);
-            launch_chained(dslash_full_dot_kernel<GF, SF, real, LREC, 4>, dim3((a.g.vh + B - 1) / B, 2), dim3(B), s, a);
+            // Links that stay in the L2 from one application to the next are not loaded evict-first (BiCGStab(4),
+            // us a cycle: 12^4 half 142 -> 133, 16^4 FP32 185 -> 175, 30-bit 503 -> 480; 16^3x32 20-bit, 63 MB of
+            // links, 273 -> 272).
+            const bool keep = 16LL * a.g.vh * (link_bytes(GF, 18) + link_bytes(GF, LREC)) <= kKeepLinkBytes;
+            auto kern = keep ? dslash_full_dot_kernel<GF, SF, real, LREC, 4, true>
+                             : dslash_full_dot_kernel<GF, SF, real, LREC, 4, false>;
+            launch_chained(kern, dim3((a.g.vh + B - 1) / B, 2), dim3(B), s, a);
             return;
         }
     }
