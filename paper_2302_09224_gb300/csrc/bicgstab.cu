@@ -654,8 +654,8 @@ __global__ void restart_kernel(BState *b, const double *sum)
 // Blocks with sites of a vector kernel over the full lattice: kMaxBlocks at most where the next kernel's blocks
 // sum its rows or the stencil's; on large lattices (more stencil rows than kMaxRows, summed once) one full wave
 // with the scalars' block, since two blocks a SM leave too few loads in flight.  32^3x64, 20-bit, us a launch at
-// 304 blocks of four fields at once and here: u update 66.6 and 46.3, r update 107.5 and 78.0, Gram-Schmidt passes
-// 66.5, 66.1, 42.3 and 52.1, 57.4, 32.8 (16^3x32 keeps 304: more rows cost the next kernel more than they give)
+// 304 blocks of four fields at once and here: u update 66.6 and 48.6, r update 107.5 and 77.9, Gram-Schmidt passes
+// 66.5, 66.1, 42.3 and 52.0, 53.5, 32.7 (16^3x32 keeps 304: more rows cost the next kernel more than they give)
 template <typename K>
 int vec_blocks(K kernel, int vh, bool large)
 {
