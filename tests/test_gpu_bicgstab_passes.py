@@ -52,3 +52,9 @@ def test_every_l(ctx, l, name, recon):
 def test_sizes(ctx, dims):
     # 8 sites a parity; under one block; past 304 blocks' first round; 147456 sites: 2304 rows of stencil sums
     check(ctx, dims, "int20", 12, 4)
+
+
+@pytest.mark.parametrize("name,recon,l", [("int20", 12, 4), ("half", 12, 5), ("int30", 18, 2), ("f64", 18, 1)])
+def test_large_lattice(ctx, name, recon, l):
+    # 4804 rows of stencil sums, summed once by their own kernel; vector kernels on full waves, a field at a time
+    check(ctx, (10, 14, 36, 122), name, recon, l, m=0.5)
