@@ -160,6 +160,7 @@ struct MSState {
     double rr_den;                     // |r_k|^2 as the residual update read it (beta's denominator)
     int nshift;
     int active, reason;
+    int go;                            // the iteration's gradient update runs (its grid may clear active meanwhile)
     int k;
 };
 

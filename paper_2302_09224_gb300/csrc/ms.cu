@@ -52,6 +52,14 @@ constexpr int kBlock = 256;
 // system's gradient vector and accumulator (every block sums the residual
 // update's partials and takes beta).  The last block of each grid has no sites:
 // its first warp runs the scalar recurrences of all shifts meanwhile.
+//
+// No kernel tests at its head a word that a block of its own grid writes, where
+// a block that starts late would then skip work that counts.  The stage stops in
+// the gradient update (m->active), which therefore tests m->go, left by the
+// residual update before it: its sites are updated in place (the base's solution
+// and gradient vector), so none may be left out of the iteration that stops.  The
+// residual update tests m->active, which its own grid clears only on a breakdown,
+// where every other block finds the same sums and does nothing.
 struct MSIter {
     BlasArgs b;      // n, err, red; v0, v1: r and A p, then r and p of the base; nparts
     char *out;       // the new residual (its own ring slot); then the base's accumulator
@@ -72,8 +80,11 @@ __global__ void __launch_bounds__(ms_block<real>()) ms_r_update_kernel(const __g
     constexpr int BS = ms_block<real>(), U = 2, C = Spinor<SF>::chunks;
     pdl_wait();
     MSState *m = a.m;
-    if (*(volatile const int *)&m->active == 0) return;
     const bool scalars = blockIdx.x == gridDim.x - 1;
+    if (*(volatile const int *)&m->active == 0) {  // uniform over the grid but for a breakdown (see above)
+        if (scalars && threadIdx.x == 0) m->go = 0;
+        return;
+    }
     const int step = (int)(gridDim.x - 1) * BS * U;
     int i0 = scalars ? a.b.n : (int)blockIdx.x * BS * U + (int)threadIdx.x;
     uint4 cr[U][C], ca[U][C];
@@ -93,6 +104,7 @@ __global__ void __launch_bounds__(ms_block<real>()) ms_r_update_kernel(const __g
             }
         }
         if (a.b.nparts > 0) ms_alpha_warp(m, tot[0]);
+        if (threadIdx.x == 0) m->go = m->active;
         return;
     }
     if (threadIdx.x == 0) {
@@ -121,7 +133,7 @@ __global__ void __launch_bounds__(kBlock) ms_p_update_kernel(const __grid_consta
     constexpr int AF = is_ff<real>::value ? S_FF : sizeof(real) == 8 ? S_F64 : S_F32;
     pdl_wait();
     MSState *m = a.m;
-    if (*(volatile const int *)&m->active == 0) return;
+    if (m->go == 0) return;  // written by the kernel before, uniform over the grid
     const bool scalars = blockIdx.x == gridDim.x - 1;
     const int n = a.b.n, i = (int)(blockIdx.x * blockDim.x + threadIdx.x);
     const bool mine = !scalars && i < n;
