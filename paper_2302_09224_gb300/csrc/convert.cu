@@ -445,7 +445,9 @@ __global__ void __launch_bounds__(kLinkBlock) quantise_kernel(Geom g, const doub
         // |x inv| <= qmax (1 + 2^-52), so the rounded product stays within +-qmax
         int q[RECON];
         const ff inv_ff = GF == G_FIX16 ? d2ff_bits(inv) : ff(0.0f);
-        if (!(inv < 1e12)) {  // a field so small that inv overflows, or that a real's tail would leave FP32's range
+        // Outside [2^-73, 1e12) the FP64 form: a smaller field's inv overflows, or a real's tail leaves FP32's
+        // range; a larger one's inv loses its own tail (below 2^-73), and its elements leave d2ff_bits' (at 2^127).
+        if (!(inv >= 0x1p-73 && inv < 1e12)) {
             for (int k = 0; k < RECON; k++) q[k] = (int)fmin(qmax, fmax(-qmax, rint(__dmul_rn(src[k], inv))));
         } else {
 #pragma unroll
