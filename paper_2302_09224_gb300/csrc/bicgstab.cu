@@ -99,12 +99,8 @@ struct Site {
 };
 __device__ __forceinline__ Site site_of(int s, int vh) { return s < vh ? Site{0, s} : Site{1, s - vh}; }
 
-// The type of the stencil's block partials for spinor format SF with BLAS in `real`.
-template <int SF, typename real>
-using stencil_part_t = std::conditional_t<SF == S_INT30 && std::is_same<real, double>::value, FF, part_t<real>>;
-
 // The three sums of the pass or kernel before: the state's, or summed here (thread 0 of tot).
-template <int SF, typename real>
+template <typename real>
 __device__ __forceinline__ void dot_sums(const BArgs &a, double *tot)
 {
     if (a.rows == 0) {
@@ -114,7 +110,7 @@ __device__ __forceinline__ void dot_sums(const BArgs &a, double *tot)
     }
     RedBuf rb{};
     rb.partials = a.part_in;
-    sum_partials<3, stencil_part_t<SF, real>>(rb, (unsigned)a.rows, tot);
+    sum_partials<3, real>(rb, (unsigned)a.rows, tot);
 }
 
 // NR sums over `rows` rows, a warp a value: FP32 rows in FP32 pairs, FP64 rows in FP64; every thread
@@ -183,14 +179,7 @@ __global__ void __launch_bounds__(kBlock) dot_rows_kernel(BArgs a)
     V v[3] = {V(0), V(0), V(0)};
     for (int r = blockIdx.x * blockDim.x + threadIdx.x; r < a.rows; r += gridDim.x * blockDim.x)
 #pragma unroll
-        for (int k = 0; k < 3; k++) {
-            if constexpr (std::is_same<T, FF>::value) {
-                const float2 t = __ldcg(reinterpret_cast<const float2 *>(part) + (size_t)r * 3 + k);
-                v[k] = v[k] + ff(t.x, t.y);
-            } else {
-                v[k] = v[k] + V(__ldcg(part + (size_t)r * 3 + k));
-            }
-        }
+        for (int k = 0; k < 3; k++) v[k] = v[k] + V(__ldcg(part + (size_t)r * 3 + k));
     __shared__ double tot[3];
     if (reduce_grid<3>(v, a.red, tot) && threadIdx.x == 0)
         for (int k = 0; k < 3; k++) a.b->dot[k] = tot[k];
@@ -244,7 +233,7 @@ __global__ void __launch_bounds__(kBlock) u_multi_kernel(BArgs a)
             }
     };
     load(s, 0);
-    dot_sums<SF, real>(a, tot);
+    dot_sums<real>(a, tot);
     if (threadIdx.x == 0) {
         BState *b = a.b;
         const int j = a.j;
@@ -328,7 +317,7 @@ __global__ void __launch_bounds__(kBlock) r_multi_kernel(BArgs a)
             }
     };
     load(s, 0);
-    dot_sums<SF, real>(a, tot);
+    dot_sums<real>(a, tot);
     if (threadIdx.x == 0) {
         BState *b = a.b;
         const double n2 = tot[0] * tot[0] + tot[1] * tot[1];
@@ -801,10 +790,8 @@ struct BRun {
         LaunchScope ls(c, st, PROF_BLAS, 0.0);
         if (p.sloppy.compute != HISQ_COMPUTE_F64)
             launch_chained(dot_rows_kernel<float>, grid, block, st, a);
-        else if (p.sloppy.spinor == S_F64)
-            launch_chained(dot_rows_kernel<double>, grid, block, st, a);
         else
-            launch_chained(dot_rows_kernel<FF>, grid, block, st, a);
+            launch_chained(dot_rows_kernel<double>, grid, block, st, a);
         return 0;
     }
 

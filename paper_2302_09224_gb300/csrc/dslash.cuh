@@ -822,14 +822,47 @@ __global__ void __launch_bounds__(stencil_block(CFG), stencil_minb(CFG))
     if (i0 < vh) warp_store_sites(out64, i0, vh, v, sh[threadIdx.x >> 5]);
 }
 
+// Two 30-bit records' <x, y> = conj(x) y and |y|^2 in FP64 from their integers
+// and exponent fields, added to v: each component exact in 64-bit integers
+// (products below 2^58, six to a sum), one rounding to FP64, the scale
+// 2^(Ex + Ey - 254) put into the exponent (the converted value is at least 1 and
+// below 2^61, so it stays normal).
+__device__ __forceinline__ double int_dot_f64(long long p, int e)
+{
+    const double d = __ll2double_rn(p);
+    return p == 0 ? 0.0 : __hiloint2double(__double2hiint(d) + e * (1 << 20), __double2loint(d));
+}
+__device__ __forceinline__ void dot_records_f64(const int32_t x[6], uint32_t Ex, const uint32_t y[6], uint32_t Ey,
+                                                double v[3])
+{
+    long long re = 0, im = 0, n2 = 0;
+#pragma unroll
+    for (int c = 0; c < 3; c++) {
+        const int xr = x[2 * c], xi = x[2 * c + 1], yr = (int)y[2 * c], yi = (int)y[2 * c + 1];
+        asm("mad.wide.s32 %0, %1, %2, %0;" : "+l"(re) : "r"(xr), "r"(yr));
+        asm("mad.wide.s32 %0, %1, %2, %0;" : "+l"(re) : "r"(xi), "r"(yi));
+        asm("mad.wide.s32 %0, %1, %2, %0;" : "+l"(im) : "r"(xr), "r"(yi));
+        asm("mad.wide.s32 %0, %1, %2, %0;" : "+l"(im) : "r"(-xi), "r"(yr));
+        asm("mad.wide.s32 %0, %1, %1, %0;" : "+l"(n2) : "r"(yr));
+        asm("mad.wide.s32 %0, %1, %1, %0;" : "+l"(n2) : "r"(yi));
+    }
+    v[0] += int_dot_f64(re, (int)(Ex + Ey) - 254);
+    v[1] += int_dot_f64(im, (int)(Ex + Ey) - 254);
+    v[2] += int_dot_f64(n2, 2 * (int)Ey - 254);
+}
+
 // Both parities in one launch, out = a y + sign D in, with the block sums of
 // <dot, out> and |out|^2 (BiCGStab(l)'s next scalars; a pass of their own over
 // the two fields took 10 to 20 us).  On a small lattice one launch of both
-// parities also fills the chip better than two of one.
+// parities also fills the chip better than two of one.  The sums are in the
+// compute precision; those of the FP64-class triplet, whose stencil runs in
+// integers and FP32 pairs, in FP64 from the stored records.
 template <int GF, int SF, typename real, int LREC, int CFG, bool KEEP>
 __global__ void __launch_bounds__(stencil_block(CFG), stencil_minb(CFG))
     dslash_full_dot_kernel(const __grid_constant__ DslashArgs a)
 {
+    using sum = std::conditional_t<is_ff<real>::value, double, real>;
+    static_assert(!is_ff<real>::value || SF == S_INT30, "pairs are the 30-bit triplet's compute type");
     pdl_wait();
     if (a.active != nullptr && *(volatile const int *)a.active == 0) return;  // uniform over the grid
     const int vh = a.g.vh;
@@ -840,7 +873,7 @@ __global__ void __launch_bounds__(stencil_block(CFG), stencil_minb(CFG))
     const real ratio = lsc / fsc;
     const int cb = blockIdx.x * blockDim.x + threadIdx.x;
     const StencilIO io = stencil_io_full(a);
-    red_t<real> v[3] = {real(0), real(0), real(0)};
+    sum v[3] = {0, 0, 0};
     if (cb < vh) {
         real o[6], t[6];
         stencil_value<GF, SF, real, LREC, CFG, false, KEEP>(a, io.in, io.po, cb, pstride, fsc, lsc, ratio, o);
@@ -848,14 +881,25 @@ __global__ void __launch_bounds__(stencil_block(CFG), stencil_minb(CFG))
         const real aa = (real)a.a;
 #pragma unroll
         for (int k = 0; k < 6; k++) o[k] = aa * t[k] + o[k];
-        if (!Spinor<SF>::store(io.out, vh, cb, o)) atomicExch(a.err, 1);
-        Spinor<SF>::load(a.dot + (io.po ? a.half_bytes : 0), vh, cb, t);
+        const char *dot = a.dot + (io.po ? a.half_bytes : 0);
+        if constexpr (is_ff<real>::value) {
+            uint32_t qo[6], Eo;
+            if (!Spinor<SF>::store_ff_q(io.out, vh, cb, o, qo, Eo)) atomicExch(a.err, 1);
+            uint4 ct[Spinor<SF>::chunks];
+            int32_t qt[6];
+            Spinor<SF>::gather(dot, vh, cb, ct);
+            const uint32_t Et = Spinor<SF>::raw(ct, qt);
+            dot_records_f64(qt, Et, qo, Eo, v);
+        } else {
+            if (!Spinor<SF>::store(io.out, vh, cb, o)) atomicExch(a.err, 1);
+            Spinor<SF>::load(dot, vh, cb, t);
 #pragma unroll
-        for (int c = 0; c < 3; c++) {
-            const real xr = t[2 * c], xi = t[2 * c + 1], yr = o[2 * c], yi = o[2 * c + 1];
-            v[0] += xr * yr + xi * yi;
-            v[1] += xr * yi - xi * yr;
-            v[2] += yr * yr + yi * yi;
+            for (int c = 0; c < 3; c++) {
+                const real xr = t[2 * c], xi = t[2 * c + 1], yr = o[2 * c], yi = o[2 * c + 1];
+                v[0] += xr * yr + xi * yi;
+                v[1] += xr * yi - xi * yr;
+                v[2] += yr * yr + yi * yi;
+            }
         }
     }
     pdl_launch_dependents();
