@@ -167,8 +167,22 @@ __global__ void __launch_bounds__(T, 1) cg_block_kernel(const __grid_constant__ 
     if (threadIdx.x < kMaxBuf) ring_sh[threadIdx.x] = 0.0f;  // a breakdown's flush reads every slot
     const unsigned tag0 = __ldcg(a.seq);  // of the launch's first sum
     unsigned tag = tag0;
+    const unsigned nb = gridDim.x;
+    // Every block counts itself out, whichever way it ends; the last one zeroes the counters for the next launch
+    // and moves the first tag past every tag in the slots.  The fence: this block's arrivals precede its leaving.
+    auto leave = [&] {
+        if (threadIdx.x != 0) return;
+        __threadfence();
+        if (atomicAdd(a.bar + 8, 1u) != nb - 1) return;
+        a.bar[0] = 0u;
+        a.bar[8] = 0u;
+        *a.seq = tag0 + 2u * (unsigned)a.iters + 2u;
+    };
     __syncthreads();
-    if (st.active == 0) return;  // uniform over the grid
+    if (st.active == 0) {  // uniform over the grid, unless a wait of an earlier block has given up already
+        leave();
+        return;
+    }
     if (threadIdx.x == 0 && blockIdx.x != 0) st.hist = nullptr;  // block 0 keeps the history
 
     const int group = (int)((blockIdx.x * blockDim.x + threadIdx.x) / S), lane_s = threadIdx.x % S;
@@ -203,7 +217,6 @@ __global__ void __launch_bounds__(T, 1) cg_block_kernel(const __grid_constant__ 
         gather_coherent<SF>(a.ring, vh, cb, c);
         Spinor<SF>::decode(c, p);
     }
-    const unsigned nb = gridDim.x;
     unsigned arrived = 0;  // the target of the next barrier
     bool bad = false, gave_up = false;
     auto f64 = [](FF v) { return (double)v.hi + (double)v.lo; };
@@ -363,12 +376,7 @@ __global__ void __launch_bounds__(T, 1) cg_block_kernel(const __grid_constant__ 
     if (blockIdx.x == 0)
         for (int k = threadIdx.x; k < (int)(sizeof(CGState) / 4); k += blockDim.x)
             reinterpret_cast<unsigned *>(a.st)[k] = reinterpret_cast<const unsigned *>(&st)[k];
-    // the last block to leave zeroes the counters for the next launch
-    if (threadIdx.x == 0 && atomicAdd(a.bar + 8, 1u) == nb - 1) {
-        a.bar[0] = 0u;
-        a.bar[8] = 0u;
-        *a.seq = tag0 + 2u * (unsigned)a.iters + 2u;  // no later sum's tag is in the slots
-    }
+    leave();
 }
 
 template <int GF, int SF, int LREC, int S, int T>
