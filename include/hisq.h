@@ -312,8 +312,10 @@ HISQ_API void hisq_mee_fused_shape(int lag, int blocks_per_sm);
  * wait's target past what the launch can reach, so each wait runs to its
  * limit, the kernel flags the error and goes on, and the solver returns
  * ECUDA.  The waits of a CG whose iterations run in one resident launch (small
- * lattices; see hisq_cg_split_scalars) take the same two settings.  Only for
- * testing that a wait ends; 0 restores normal waits. */
+ * lattices; see hisq_cg_split_scalars) take the same two settings.
+ * unreachable = 2: that launch is refused, as on a device that cannot hold it,
+ * and the solve takes the separate kernels.  Only for testing; 0 restores
+ * normal waits and launches. */
 HISQ_API void hisq_mee_fused_wait_test(unsigned polls, int unreachable);
 HISQ_API int hisq_stencil_config_reduce(int cfg);
 /* Programmatic dependent launch of the solvers' kernel chains (stencil

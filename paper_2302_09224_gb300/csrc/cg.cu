@@ -300,8 +300,9 @@ struct CGRun {
     }
 
     // The same iterations, resident: up to iters of them (a multiple of nbuf) in one launch.
-    // timed: the profiler's event pair around it, counted as its stencil passes (two an iteration).
-    cudaError_t iterate_resident(double *x64, int iters, bool timed)
+    // timed: the profiler's event pair around it, counted as its stencil passes (two an iteration).  False: the
+    // launch was refused and nothing ran.
+    bool iterate_resident(double *x64, int iters, bool timed)
     {
         CGBlockArgs a{};
         a.d.g = g->geom;
@@ -320,21 +321,21 @@ struct CGRun {
         a.seq = (unsigned *)(inbox + 2 * resident.blocks * resident.blocks);
         a.bar = cur_red(c).sync + 8;
         auto go = [&]() {
-            return launch_cg_block(cfg.sloppy.gauge, cfg.sloppy.spinor, cfg.sloppy.long_recon, resident, a, s)
-                       ? cudaSuccess
-                       : cudaGetLastError();
+            return launch_cg_block(cfg.sloppy.gauge, cfg.sloppy.spinor, cfg.sloppy.long_recon, resident, a, s);
         };
         if (!timed) {
-            c->launches++;
-            return go();
+            const bool ok = go();
+            c->launches += ok;
+            return ok;
         }
         set_prof_tag(kProfResident);
         LaunchScope ls(c, s, PROF_STENCIL,
                        iters * (stencil_bytes(cfg.sloppy, vh, false) + stencil_bytes(cfg.sloppy, vh, true)),
                        2 * iters);
         set_prof_tag(-1);
-        c->launches += 1 - 2 * iters;  // one kernel
-        return go();
+        const bool ok = go();
+        c->launches += ok - 2 * iters;  // one kernel
+        return ok;
     }
 
     hisq_status run(const double *b64, double *x64, bool x_zero, hisq_solve_info *info)
@@ -429,10 +430,14 @@ struct CGRun {
                 // (once per nbuf iterations while profiling); where a run is cut changes no bit
                 const int left = (cfg.maxiter - k0 + cfg.nbuf - 1) / cfg.nbuf, most = c->prof.on ? 1 : 64 / cfg.nbuf;
                 const int iters = cfg.nbuf * std::min(left, most);
-                const cudaError_t ce = iterate_resident(x64, iters, c->prof.on && block % every == 0);
-                if (ce != cudaSuccess) {
-                    e = cuda_fail(c, ce, "resident CG launch");
-                    break;
+                if (!iterate_resident(x64, iters, c->prof.on && block % every == 0)) {
+                    // refused (the process has fewer SMs than the shape was chosen for): the separate kernels go on
+                    // from the same state; an error of the device shows in their launches and synchronisations
+                    (void)cudaGetLastError();
+                    prof_settle_resident(c, 0, iters);
+                    resident.lanes = 0;
+                    tune_stencil(c, g->geom, cfg.sloppy, gv_s, ap_s, tmp_s, s);
+                    continue;
                 }
                 run_iters = iters;
             } else if (graph) {

@@ -42,6 +42,7 @@ bool mee_fused_available(int gf, int sf, int cf, const Geom &g)
 
 extern std::atomic<int> fused_lag, fused_bps;
 extern std::atomic<unsigned> fused_wait_polls, fused_wait_extra;
+extern std::atomic<bool> resident_refused;
 
 bool launch_mee_fused(int gf, int sf, int cf, int long_recon, const MeeArgs &m_in, cudaStream_t s)
 {
@@ -266,6 +267,7 @@ bool launch_cg_block(int gf, int sf, int long_recon, const CGBlockShape &sh, con
     CGBlockArgs a = args;
     a.wait_polls = std::min(fused_wait_polls.load(), 1u << 20);  // about half a second of L2 round trips
     a.wait_extra = fused_wait_extra.load();
+    if (resident_refused.load()) return false;
     if (gf == G_F32) return launch_cg_block_f32(long_recon, sh, a, s);
     if (sf == S_HALF) return launch_cg_block_half(long_recon, sh, a, s);
     return launch_cg_block_int20(long_recon, sh, a, s);
@@ -294,12 +296,14 @@ extern "C" int hisq_mee_fused(int mode)
 namespace hisq {
 std::atomic<int> fused_lag{4}, fused_bps{0};
 std::atomic<unsigned> fused_wait_polls{kMeeWaitPolls}, fused_wait_extra{0};
+std::atomic<bool> resident_refused{false};
 }
 
 extern "C" void hisq_mee_fused_wait_test(unsigned polls, int unreachable)
 {
     hisq::fused_wait_polls.store(polls > 0 ? polls : hisq::kMeeWaitPolls);
-    hisq::fused_wait_extra.store(unreachable ? 1u : 0u);
+    hisq::fused_wait_extra.store(unreachable && unreachable != 2 ? 1u : 0u);
+    hisq::resident_refused.store(unreachable == 2);
 }
 
 extern "C" void hisq_mee_fused_shape(int lag, int blocks_per_sm)

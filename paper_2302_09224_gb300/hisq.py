@@ -337,8 +337,8 @@ def hisq_mee_fused_shape(lag: int, blocks_per_sm: int):
     lib().hisq_mee_fused_shape(int(lag), int(blocks_per_sm))
 
 
-def hisq_mee_fused_wait_test(polls: int, unreachable: bool):
-    lib().hisq_mee_fused_wait_test(int(polls) & 0xFFFFFFFF, int(bool(unreachable)))
+def hisq_mee_fused_wait_test(polls: int, unreachable: int):
+    lib().hisq_mee_fused_wait_test(int(polls) & 0xFFFFFFFF, int(unreachable))
 
 
 def hisq_programmatic_launch(mode: int) -> int:
