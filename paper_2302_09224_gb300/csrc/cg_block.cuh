@@ -12,22 +12,27 @@
 //   tmp = D_oe p | barrier | A p = diag p - D_eo tmp, <p, A p> | sum barrier |
 //   r -= alpha A p, |r|^2, <r, r_old> | sum barrier | p = r + beta p | barrier.
 // Every block sums the blocks' partials in one fixed order, takes alpha, beta and
-// the decision to stop from them in FP32 pairs (an FP64 division in the way of
-// every block costs half a microsecond) and keeps its own copy of the solver's
-// state, so the decision needs no further exchange; block 0 writes it back.
+// the decision to stop from them as FP64 would (in FP32 pairs wherever these
+// cannot differ, see cg_scalars.cuh: an FP64 division in the way of every block
+// costs half a microsecond) and keeps its own copy of the solver's state, so the
+// decision needs no further exchange; block 0 writes it back.
 //
 // S lanes share a site (one or more directions each, their sums combined by
-// shuffles): as many as keep the launch within one block of at most 1024
-// threads per SM, so that 8^4 occupies the whole chip and 16^3x64 still fits.
+// shuffles): four or two while that takes one block of at most 512 threads an SM,
+// else one, with up to 1024 threads (cg_block_shape), so that 8^4 occupies the
+// whole chip and 16^3x64 still fits.
 //
 // The blocks of the launch wait for one another: the launch is cooperative
-// (all of them resident or none), every wait is bounded, and a wait that gives
-// up sets bit 2 of the error word and ends its block.
+// (all of them resident or none; with 40 SMs taken by another stream's kernel for
+// two seconds a 16^3x32 solve began after that and gave the same bits), every
+// wait is bounded, and a wait that gives up sets bit 2 of the error word and ends
+// its block.
 #pragma once
 
 #include <cuda_runtime.h>
 
 #include "cg.h"
+#include "cg_scalars.cuh"
 #include "codecs.cuh"
 #include "dslash.cuh"
 #include "finish.cuh"
@@ -200,13 +205,16 @@ __global__ void __launch_bounds__(T, 1) cg_block_kernel(const __grid_constant__ 
     const float ratio = lsc / fsc;
     const float diag = (float)a.diag;
     const int pr = st.pr;
-    // Thread 0: the recurrence's scalars.  The decisions compare FP32 pairs (FP64 divisions, and even
-    // conversions, of a launch's every iteration would stand in every block's way); the state receives
-    // the same numbers in FP64 at the end of the launch, or each iteration where a history or the
-    // error-estimate trigger asks for the FP64 finishers.
+    // Thread 0: the recurrence's scalars in FP32 pairs (FP64 divisions, and even conversions, of a launch's every
+    // iteration would stand in every block's way), FP64 deciding where a pair cannot.  The sums are pairs, so
+    // their doubles are known exactly; those of the launch's start stay in st.  The state receives the doubles at
+    // the end of the launch, or each iteration where a history or the error-estimate trigger asks for the FP64
+    // finishers.
     const bool fp64 = st.dyn || a.st->hist != nullptr;
-    ff rr(st.rr), rr_prev(st.rr_prev), rr_max(st.rr_max);
-    const ff delta2(st.delta2), stop2(st.stop2);
+    ff rr(st.rr), rr_prev(0.0f), rr_max(st.rr_max);
+    const float delta2 = (float)st.delta2, stop2 = (float)st.stop2;
+    int steps = 0;          // updates of rr so far: the first makes rr, the second rr_prev a sum's pair
+    bool max_sum = false;   // rr_max is a sum's pair
     float al_used = 0.0f, be_used = 0.0f;
 
     float r[6], p[6], dx[6] = {0, 0, 0, 0, 0, 0};
@@ -220,22 +228,26 @@ __global__ void __launch_bounds__(T, 1) cg_block_kernel(const __grid_constant__ 
     unsigned arrived = 0;  // the target of the next barrier
     bool bad = false, gave_up = false;
     auto f64 = [](FF v) { return (double)v.hi + (double)v.lo; };
-    auto less = [](ff x, ff y) { return x.hi < y.hi || (x.hi == y.hi && x.lo < y.lo); };
+    auto rr64 = [&] { return steps > 0 ? (double)rr : st.rr; };
+    auto max64 = [&] { return max_sum ? (double)rr_max : st.rr_max; };
     // thread 0, after iteration i: the finishers' decisions
     auto finish = [&](int i) {
         if (fp64) {
             double tot[2] = {f64(tot_ap[0]), f64(tot_ap[1])};
             run_finisher(FIN_CG_ALPHA, tot, &st, i);
-            st.alpha = (double)al_used;
             tot[0] = f64(tot_r[0]);
             tot[1] = f64(tot_r[1]);
             run_finisher(FIN_CG_BETA, tot, &st, i);
         } else {
             st.k += 1;
-            if (less(rr_max, rr)) rr_max = rr;
-            if (!less(stop2, rr))
+            if (decide_less(rr_max.hi, rr.hi, [&](double &x, double &y) { x = max64(), y = (double)rr; })) {
+                rr_max = rr;
+                max_sum = true;
+            }
+            if (!decide_less(stop2, rr.hi, [&](double &x, double &y) { x = st.stop2, y = (double)rr; }))
                 stop_iterating(&st, REASON_CONVERGED);
-            else if (less(rr, delta2 * rr_max))
+            else if (decide_less(rr.hi, delta2 * rr_max.hi,
+                                 [&](double &x, double &y) { x = (double)rr, y = st.delta2 * max64(); }))
                 stop_iterating(&st, REASON_RELIABLE);
         }
         ring_sh[i] = i == a.nslots - 1 ? 0.0f : al_used;
@@ -275,7 +287,10 @@ __global__ void __launch_bounds__(T, 1) cg_block_kernel(const __grid_constant__ 
         if (threadIdx.x == 0) {
             tot_ap[0] = tot[0];
             tot_ap[1] = tot[1];
-            step_sh = al_used = (rr / ff(tot[0].hi, tot[0].lo)).hi;
+            step_sh = al_used = step_quotient(rr, ff(0.0f), ff(tot[0].hi, tot[0].lo), [&](double &n, double &d) {
+                n = rr64();
+                d = f64(tot[0]);
+            });
             ok_sh = !got ? 0 : tot[0].hi > 0.0f && isfinite(al_used) ? 1 : 2;
         }
         __syncthreads();
@@ -302,9 +317,13 @@ __global__ void __launch_bounds__(T, 1) cg_block_kernel(const __grid_constant__ 
             tot_r[0] = tot[0];
             tot_r[1] = tot[1];
             const ff rn(tot[0].hi, tot[0].lo);
+            step_sh = be_used = step_quotient(rn, pr ? ff(tot[1].hi, tot[1].lo) : ff(0.0f), rr, [&](double &n, double &d) {
+                n = pr ? f64(tot[0]) - f64(tot[1]) : f64(tot[0]);
+                d = rr64();
+            });
             rr_prev = rr;
             rr = rn;
-            step_sh = be_used = ((pr ? rn - ff(tot[1].hi, tot[1].lo) : rn) / rr_prev).hi;
+            steps++;
             ok_sh = !got ? 0 : isfinite(tot[0].hi) && isfinite(be_used) ? 1 : 2;
         }
         __syncthreads();
@@ -358,9 +377,11 @@ __global__ void __launch_bounds__(T, 1) cg_block_kernel(const __grid_constant__ 
     if (bad && lead) atomicOr(a.err, 1);
     if (threadIdx.x == 0) {
         if (!fp64) {
-            st.rr = (double)rr;
-            st.rr_prev = (double)rr_prev;
-            st.rr_max = (double)rr_max;
+            if (steps > 0) {
+                st.rr_prev = steps > 1 ? (double)rr_prev : st.rr;
+                st.rr = (double)rr;
+            }
+            st.rr_max = max64();
             st.pAp = f64(tot_ap[0]);
             st.apap = f64(tot_ap[1]);
             st.alpha = (double)al_used;

@@ -12,7 +12,54 @@
 
 #include <cuda_runtime.h>
 
+#include <cmath>
+#include <cstdint>
+
 namespace hisq {
+
+// FP32 operations rounded to nearest and never contracted: the device's own, and
+// plain ones on the host, whose code is compiled without contraction (it checks
+// this arithmetic on the CPU).
+__host__ __device__ __forceinline__ float rn_add(float a, float b)
+{
+#ifdef __CUDA_ARCH__
+    return __fadd_rn(a, b);
+#else
+    return a + b;
+#endif
+}
+__host__ __device__ __forceinline__ float rn_sub(float a, float b)
+{
+#ifdef __CUDA_ARCH__
+    return __fsub_rn(a, b);
+#else
+    return a - b;
+#endif
+}
+__host__ __device__ __forceinline__ float rn_mul(float a, float b)
+{
+#ifdef __CUDA_ARCH__
+    return __fmul_rn(a, b);
+#else
+    return a * b;
+#endif
+}
+__host__ __device__ __forceinline__ float rn_div(float a, float b)
+{
+#ifdef __CUDA_ARCH__
+    return __fdiv_rn(a, b);
+#else
+    return a / b;
+#endif
+}
+__host__ __device__ __forceinline__ float rn_fma(float a, float b, float c)
+{
+#ifdef __CUDA_ARCH__
+    return __fmaf_rn(a, b, c);
+#else
+    return std::fma(a, b, c);
+#endif
+}
 
 struct ff {
     float hi, lo;
@@ -20,53 +67,53 @@ struct ff {
     __host__ __device__ constexpr ff(float h, float l) : hi(h), lo(l) {}
     __host__ __device__ constexpr ff(float x) : hi(x), lo(0.0f) {}
     __host__ __device__ constexpr ff(int x) : hi((float)x), lo(0.0f) {}  // small integers only (exact)
-    __device__ explicit ff(double d)
+    __host__ __device__ explicit ff(double d)
     {
-        hi = __double2float_rn(d);
-        lo = __double2float_rn(d - (double)hi);
+        hi = (float)d;
+        lo = (float)(d - (double)hi);
     }
-    __device__ explicit operator double() const { return (double)hi + (double)lo; }
+    __host__ __device__ explicit operator double() const { return (double)hi + (double)lo; }
 };
 
-__device__ __forceinline__ ff ff_two_sum(float a, float b)
+__host__ __device__ __forceinline__ ff ff_two_sum(float a, float b)
 {
-    const float s = __fadd_rn(a, b);
-    const float bb = __fsub_rn(s, a);
-    return ff(s, __fadd_rn(__fsub_rn(a, __fsub_rn(s, bb)), __fsub_rn(b, bb)));
+    const float s = rn_add(a, b);
+    const float bb = rn_sub(s, a);
+    return ff(s, rn_add(rn_sub(a, rn_sub(s, bb)), rn_sub(b, bb)));
 }
 
-__device__ __forceinline__ ff ff_fast_two_sum(float a, float b)
+__host__ __device__ __forceinline__ ff ff_fast_two_sum(float a, float b)
 {
-    const float s = __fadd_rn(a, b);
-    return ff(s, __fsub_rn(b, __fsub_rn(s, a)));
+    const float s = rn_add(a, b);
+    return ff(s, rn_sub(b, rn_sub(s, a)));
 }
 
-__device__ __forceinline__ ff operator+(ff a, ff b)
+__host__ __device__ __forceinline__ ff operator+(ff a, ff b)
 {
     const ff s = ff_two_sum(a.hi, b.hi);
-    return ff_fast_two_sum(s.hi, __fadd_rn(s.lo, __fadd_rn(a.lo, b.lo)));
+    return ff_fast_two_sum(s.hi, rn_add(s.lo, rn_add(a.lo, b.lo)));
 }
-__device__ __forceinline__ ff operator-(ff a) { return ff(-a.hi, -a.lo); }
-__device__ __forceinline__ ff operator-(ff a, ff b) { return a + (-b); }
-__device__ __forceinline__ ff operator*(ff a, ff b)
+__host__ __device__ __forceinline__ ff operator-(ff a) { return ff(-a.hi, -a.lo); }
+__host__ __device__ __forceinline__ ff operator-(ff a, ff b) { return a + (-b); }
+__host__ __device__ __forceinline__ ff operator*(ff a, ff b)
 {
-    const float p = __fmul_rn(a.hi, b.hi);
-    float e = __fmaf_rn(a.hi, b.hi, -p);
-    e = __fmaf_rn(a.hi, b.lo, e);
-    e = __fmaf_rn(a.lo, b.hi, e);
+    const float p = rn_mul(a.hi, b.hi);
+    float e = rn_fma(a.hi, b.hi, -p);
+    e = rn_fma(a.hi, b.lo, e);
+    e = rn_fma(a.lo, b.hi, e);
     return ff_fast_two_sum(p, e);
 }
-__device__ __forceinline__ ff operator/(ff a, ff b)
+__host__ __device__ __forceinline__ ff operator/(ff a, ff b)
 {
     // two Newton-style quotient digits: q1 = a/b rounded, q2 = (a - q1 b)/b
-    const float q1 = __fdiv_rn(a.hi, b.hi);
+    const float q1 = rn_div(a.hi, b.hi);
     const ff r = a - b * ff(q1);
-    const float q2 = __fdiv_rn(r.hi, b.hi);
+    const float q2 = rn_div(r.hi, b.hi);
     return ff_fast_two_sum(q1, q2);
 }
-__device__ __forceinline__ ff &operator+=(ff &a, ff b) { return a = a + b; }
-__device__ __forceinline__ ff &operator-=(ff &a, ff b) { return a = a - b; }
-__device__ __forceinline__ ff &operator*=(ff &a, ff b) { return a = a * b; }
+__host__ __device__ __forceinline__ ff &operator+=(ff &a, ff b) { return a = a + b; }
+__host__ __device__ __forceinline__ ff &operator-=(ff &a, ff b) { return a = a - b; }
+__host__ __device__ __forceinline__ ff &operator*=(ff &a, ff b) { return a = a * b; }
 
 // An integer below 2^31 in magnitude as an exact pair: q = qh 2^16 + ql with
 // qh and ql exact in FP32, summed error-free.
