@@ -136,9 +136,14 @@ HISQ_API const char *hisq_last_error(hisq_ctx *ctx);
 /* Device bytes of the context in use by gauge fields and running calls.
  * Buffers of finished calls stay with the context for the next call of the same
  * sizes (at most 4 GiB and an eighth of the budget, beside those in use and
- * within the budget; released when an allocation needs the room); they are
- * not counted. */
+ * within the budget; released when an allocation of this context needs the
+ * room, by hisq_release_buffers and by hisq_destroy); they are not counted. */
 HISQ_API size_t hisq_mem_used(hisq_ctx *ctx);
+
+/* Give the buffers kept for later calls (device and pinned host memory) back to
+ * the driver, for a program whose other allocations need the room.  Waits for
+ * the device; the next call of each kind allocates anew. */
+HISQ_API void hisq_release_buffers(hisq_ctx *ctx);
 
 /* Load a gauge configuration (Sec. 2 footnote, Sec. 4: one global scale per
  * fixed-point field).  fat and lng are FP64 in the host gauge layout

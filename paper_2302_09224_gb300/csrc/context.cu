@@ -167,6 +167,15 @@ void pinned_put(hisq_ctx *c, void *p)
     cudaFreeHost(p);
 }
 
+// Everything kept for later calls.
+void release_buffers(hisq_ctx *c)
+{
+    std::lock_guard<std::mutex> lk(c->alloc_mu);
+    release_kept(c, 0);
+    for (void *h : c->pinned) cudaFreeHost(h);
+    c->pinned.clear();
+}
+
 cudaStream_t pick_stream(hisq_ctx *c, void *s) { return s ? (cudaStream_t)s : c->stream; }
 
 bool stream_capturing(cudaStream_t s)
@@ -600,8 +609,7 @@ void hisq_destroy(hisq_ctx *c)
     if (c->scratch) cudaFree(c->scratch);
     if (c->red.partials) cudaFree(c->red.partials);
     if (c->host_flags) cudaFreeHost(c->host_flags);
-    for (auto &k : c->kept) cudaFree(k.first);
-    for (void *h : c->pinned) cudaFreeHost(h);
+    release_buffers(c);
     if (c->stream) cudaStreamDestroy(c->stream);
     delete c;
 }
@@ -613,6 +621,13 @@ const char *hisq_last_error(hisq_ctx *c)
 }
 
 size_t hisq_mem_used(hisq_ctx *c) { return c ? c->used : 0; }
+
+void hisq_release_buffers(hisq_ctx *c)
+{
+    if (!c) return;
+    cudaSetDevice(c->device);
+    release_buffers(c);
+}
 
 hisq_status hisq_load_gauge(hisq_ctx *c, const int dims[4], const double *fat, const double *lng, unsigned flags,
                             hisq_gauge **out)

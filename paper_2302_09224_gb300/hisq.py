@@ -118,6 +118,7 @@ _SIGS = {
     "hisq_destroy": (None, [_P]),
     "hisq_last_error": (ctypes.c_char_p, [_P]),
     "hisq_mem_used": (_SZ, [_P]),
+    "hisq_release_buffers": (None, [_P]),
     "hisq_load_gauge": (_I, [_P, _P, _P, _P, ctypes.c_uint, ctypes.POINTER(_P)]),
     "hisq_free_gauge": (None, [_P, _P]),
     "hisq_gauge_scale": (_D, [_P, _I]),
@@ -237,6 +238,10 @@ def hisq_last_error(ctx) -> str:
 
 def hisq_mem_used(ctx) -> int:
     return int(lib().hisq_mem_used(ctx))
+
+
+def hisq_release_buffers(ctx):
+    lib().hisq_release_buffers(ctx)
 
 
 def hisq_load_gauge(ctx, dims, fat, lng, flags: int = 0):
