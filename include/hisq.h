@@ -347,7 +347,9 @@ HISQ_API int hisq_programmatic_launch(int mode);
 HISQ_API int hisq_cg_split_scalars(int mode);
 /* The shape in use for triplet p on gauge g's lattice (plain pass, or the
  * reducing pass if reduce != 0): the forced one, else the tuned one, else -1
- * when that pair has not been tuned yet. */
+ * when that pair has not been tuned: not used yet, or used only where no shape
+ * applies (FP64 passes of lattices so small that lanes share a site, CG
+ * iterations in one resident launch; these ignore a forced shape too). */
 HISQ_API int hisq_stencil_config_in_use(const hisq_gauge *g, hisq_prec p, int reduce);
 
 /* Kernels this context has launched so far (graph replays add their nodes). */

@@ -685,8 +685,8 @@ hisq_status hisq_load_gauge(hisq_ctx *c, const int dims[4], const double *fat, c
         return st;
     }
     // Device arrays are copied by the scan (16^3x32: 94 us a load, 137 us with copies of their own) where it may
-    // read them.  Host arrays, and whatever else a copy accepts or refuses (memory of
-    // another device, an unaligned address, an array too short), are copied first.
+    // read them.  Host arrays, and whatever else a copy accepts or refuses (memory of another device, an unaligned
+    // address, an array too short), are copied first.
     const bool on_device = (flags & HISQ_GAUGE_ON_DEVICE) != 0;
     const cudaMemcpyKind kind = on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice;
     const bool fat_in_place = on_device && readable_in_place(c, fat, bytes);

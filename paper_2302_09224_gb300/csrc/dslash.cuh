@@ -978,7 +978,8 @@ template <int GF, int SF, typename real, int LREC, bool RED>
 void launch_any(int cfg, const DslashArgs &a, cudaStream_t s)
 {
     if constexpr (!RED && GF == G_F64) {
-        const int lanes = a.dot == nullptr ? f64_lanes((long long)a.g.vh * (a.out64 != nullptr && a.half_bytes ? 2 : 1)) : 1;
+        const int lanes = a.dot == nullptr && !a.one_lane
+                              ? f64_lanes((long long)a.g.vh * (a.out64 != nullptr && a.half_bytes ? 2 : 1)) : 1;
         if (lanes == 4) return launch_lanes<LREC, 4>(a, s);
         if (lanes == 2) return launch_lanes<LREC, 2>(a, s);
     }

@@ -140,6 +140,12 @@ void tune_variant(int gf, int sf, int cf, int lrec, bool red, const DslashArgs &
     DslashArgs a = args;
     a.fin = FIN_NONE;
     a.active = nullptr;
+    if (gf == G_F64 && !red) {
+        // the shapes serve the passes with a thread a site: none on lattices where both the pass over one parity
+        // and the one over both share a site among lanes
+        if (dslash_f64_lanes(args.g.vh) > 1 && dslash_f64_lanes(2LL * args.g.vh) > 1) return;
+        a.one_lane = 1;
+    }
     if (red) {
         a.xpay = 1;
         a.y = a.out;

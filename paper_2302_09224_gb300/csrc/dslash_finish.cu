@@ -12,6 +12,8 @@ unsigned dslash_partials(int gf, int sf, int cf, int long_recon, const Geom &g)
     return (unsigned)((g.vh + b - 1) / b);
 }
 
+int dslash_f64_lanes(long long n) { return f64_lanes(n); }
+
 int dslash_full_rows(int gf, int vh)
 {
     const int b = stencil_threads(4, gf, 2 * vh);

@@ -227,6 +227,7 @@ struct DslashArgs {
     int fin;
     void *st;               // CGState or MSState, per finisher
     int slot;               // ring slot handed to the finisher
+    int one_lane;           // FP64: one lane a site whatever the lattice (timing the launch shapes)
     int defer_finish;       // reducing pass: leave the summing launch to launch_dslash_finish
     // the pass to a caller's array (plain pass only, out unused): the stored value decoded to FP64
     // [site][6]; nothing is written when *bad != 0 (device int); err may be host-mapped
@@ -239,6 +240,8 @@ struct DslashArgs {
 };
 // Blocks of the pass over both parities with dot.
 int dslash_full_rows(int gf, int vh);
+// Lanes a site of an FP64 pass over n sites; with more than one it takes no launch shape.
+int dslash_f64_lanes(long long n);
 
 // The fused M_ee pass (d1: D_oe into tmp; d2: D_eo from tmp with xpay and the
 // reduction), scheduled in t-slices through red.sync.
