@@ -505,6 +505,8 @@ hisq_status BatchSession::setup()
     }
     adapt = cfg.tile == 0 && cfg.kernel == 0;
     if (nr % T) return fail(c, HISQ_EINVAL, "RHS tile %d does not divide nrhs %d", T, nr);
+    // the largest lattices a batch takes: a bound of the reductions' common buffer, kept although the block sums
+    // of the batched passes lie in a work field
     if (!red_fits(vh, kMrhsBlock, 2 * T) || !red_fits(vh, kBlock, 2 * kMaxRHS))
         return fail(c, HISQ_EINVAL, "lattice too large for a batched reduction over a tile of %d", T);
     tune_stencil(c, g->geom, prec_f64(), gv_d, (char *)ax64, (char *)tmp64, s);

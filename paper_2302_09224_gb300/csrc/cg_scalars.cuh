@@ -5,8 +5,11 @@
 // itself, and an FP64 division or conversion there stands in the way of all of
 // them (cg_block.cuh).  Pairs carry some 45 bits, and what leaves is an FP32 step or
 // a comparison, so they decide wherever their error cannot change it; next to a
-// tie, or outside the range where the error bound holds, FP64 does.  The
-// functions run on the host too, where their bounds are checked.
+// tie, or outside the range where the error bound holds, FP64 does.  Microseconds
+// an iteration with the pairs alone and with this (reliable updates included):
+// 20-bit 8^4 10.74 and 10.77, 16^4 17.62 and 17.73, 16^3x64 41.1 and 41.3; 16-bit
+// 8^4 10.63 and 10.77.  The functions run on the host too, where their bounds are
+// checked.
 #pragma once
 
 #include "ff.cuh"

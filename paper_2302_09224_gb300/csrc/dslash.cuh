@@ -148,7 +148,9 @@ __host__ __device__ constexpr int stencil_block(int cfg) { return cfg == 3 ? 256
 // rate, so its time is that of the fullest SM: with few blocks an SM the grid
 // is cut finer (down to 32 threads a block) while that lowers the most sites
 // any SM gets.  16^3x32 (65536 sites, 152 SMs): blocks of 128 leave up to four
-// blocks on an SM where 3.4 is the mean.
+// blocks on an SM where 3.4 is the mean.  (The chip's 152 SMs as a constant, here
+// and in f64_lanes: only the split depends on it, and host code that sizes
+// partials evaluates the same rule.)
 inline int stencil_threads(int cfg, int gf, int vh)
 {
     const int b = stencil_block(cfg);
@@ -856,7 +858,10 @@ __device__ __forceinline__ void dot_records_f64(const int32_t x[6], uint32_t Ex,
 // the two fields took 10 to 20 us).  On a small lattice one launch of both
 // parities also fills the chip better than two of one.  The sums are in the
 // compute precision; those of the FP64-class triplet, whose stencil runs in
-// integers and FP32 pairs, in FP64 from the stored records.
+// integers and FP32 pairs, in FP64 from the stored records (BiCGStab(4), us a
+// matrix application against sums in pairs of the values before their rounding,
+// which were off by 1e-11: 16^4 64.5 and 60.7, 16^3x32 102.8 and 102.6, 24^3x48
+// 408.6 and 415.9).
 template <int GF, int SF, typename real, int LREC, int CFG, bool KEEP>
 __global__ void __launch_bounds__(stencil_block(CFG), stencil_minb(CFG))
     dslash_full_dot_kernel(const __grid_constant__ DslashArgs a)

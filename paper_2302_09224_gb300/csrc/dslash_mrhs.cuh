@@ -484,7 +484,7 @@ __global__ void __launch_bounds__(kMrhsBlock, mrhs_min_blocks(T)) dslash_mrhs_ke
         }
     }
 
-    // block sums, summed by the residual update's blocks: [t0 * blocks + block * T + j]
+    // block sums, summed per right-hand side by a launch of their own: [t0 * blocks + block * T + j]
     if constexpr (RED)
         store_partial_at<2 * T, float>(rv, reinterpret_cast<float *>(a.partials + (size_t)t0 * a.nblocks),
                                        (unsigned)site_block);

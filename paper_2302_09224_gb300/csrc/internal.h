@@ -99,9 +99,12 @@ inline bool red_fits(int64_t n, int block, int nr, int gy = 1)
     return ((n + block - 1) / block) * gy * nr <= (int64_t)kMaxRedBlocks * kMaxRed;
 }
 
-// The single-RHS solvers' reducing launches: the stencil (blocks of 128 or
-// more, 2 values), the BLAS kernels (256, 3) and BiCGStab(l)'s two-parity
-// grids (256, 3, 2 rows).  Holds up to Vh = 2^27 sites.
+// The single-RHS solvers' reducing launches: the stencil (blocks of 128, 2
+// values), the BLAS kernels (256, 3) and BiCGStab(l)'s two-parity grids (256, 3,
+// 2 rows).  Holds up to Vh = 2^27 sites.  Launches with finer blocks stay within
+// it: FP64 stencil blocks go down to 32 threads only where that takes 3 % off the
+// fullest SM (stencil_threads: below half a million sites, some 14 thousand blocks
+// at most), one-site BLAS blocks go down to 64 only under 152 blocks.
 inline bool solver_red_fits(int64_t vh) { return red_fits(vh, 128, 2) && red_fits(vh, 256, 3, 2); }
 
 // ---------------------------------------------------------------------------

@@ -17,7 +17,9 @@
 // hidden.  FP64 CG, 16^3x32: 43.1 ms with the early call, 29.9 without
 // programmatic launches, 29.8 with the late call; BiCGStab(4), 20-bit,
 // 16^3x32: 15.7, 13.9, 13.7; 20-bit CG, 24^3x48 (many waves a pass): 20.5,
-// 21.0, 20.5.  Kernels of a few blocks call it first.
+// 21.0, 20.5.  Kernels of a few blocks call it first, and so do the batched
+// stencil (dslash_mrhs_kernel, many waves a pass) and the multi-shift stage's
+// shift_ring_kernel, for which the two orders have not been compared.
 #pragma once
 
 #include <cuda_runtime.h>
